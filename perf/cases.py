@@ -1,0 +1,580 @@
+"""Timed cases of the solver, through the entry points a program calls.
+
+Four kinds of case:
+  step       one implicit time step of one slab (trt.Solver.step) and the fields it leaves;
+  batch      one time step of many independent slabs together (trt.Batch.step);
+  sweep      one high-order sweep on the caller's own device arrays (trt_k_sweep);
+  mlp_infer  the closure network's prediction for every (cell, group) row;
+  mlp_train  one training step of it (gradient and Adam).
+`listed()` holds the sizes of the repository's own workloads (fc_small, fc_paper, fc_1024,
+fc_4096, batch_256's family, the closure's inference and training batches) and two ragged
+ones; `draw` spreads cases over the same ranges.  `exact` restates the discretised method
+in plain torch, 64 bits throughout.
+"""
+import ctypes
+import math
+
+import numpy as np
+import torch
+
+from paper_2011_05427_gb300 import closure, mlp, trt
+from paper_2011_05427_gb300 import workloads as W
+
+C = 299.792458                                   # cm / sh
+A_RAD = W.A_RAD                                  # GJ / (cm^3 keV^4)
+C_B = 15.0 * A_RAD * C / (2.0 * math.pi ** 4)
+DEV = "cuda"
+F64 = torch.float64
+
+
+# ---------------------------------------------------------------------------
+# the cases
+# ---------------------------------------------------------------------------
+def _step(name, nx, N, G, levels, precision, cycle, l_max, max_outer=100, eps=1e-8, dt=1e-3,
+          length=6.0, nu_a=1e-5, nu_b=1e2, top="inf", tune=True, graded=False, tr=False):
+    """A `step` case.  eps > 0: a converged step; eps < 0: exactly max_outer low-order phases
+    of l_max cycles (a fixed budget of work per time step)."""
+    c = dict(kind="step", nx=nx, N=N, G=G, levels=levels, precision=precision, cycle=cycle,
+             l_max=l_max, max_outer=max_outer, eps=eps, dt=dt, length=length, nu_a=nu_a,
+             nu_b=nu_b, top=top, tune=tune, graded=graded, tr=tr)
+    return dict(c, name=name) if name else c
+
+
+def listed():
+    return [
+        # the smallest production slab, plain FP64: launches and latency
+        _step("step_fc_small", 60, 8, 17, "17,1", "fp64", "V", 4, dt=2e-3, tune=False),
+        # the paper's own test (10 cells, 256 groups, eps 1e-6) with its F cycle on four grids
+        _step("step_fc_paper_F", 10, 8, 256, "256,32,16,1", "fp64", "F", 2, eps=1e-6, dt=2e-3,
+              length=4.0, nu_a=1e-4, nu_b=10.0, top="1e7", tune=False),
+        # the benchmark's slab: plain FP64, V cycle, converged
+        _step("step_fc_1024_fp64_V", 500, 32, 1024, "1024,256,64,16,1", "fp64", "V", 3),
+        # the same slab in a W cycle over its five grids, a fixed budget of phases
+        _step("step_fc_1024_fp64_W", 500, 32, 1024, "1024,256,64,16,1", "fp64", "W", 1,
+              max_outer=6, eps=-1.0),
+        # its fastest form: FP32 sweeps, group systems in FP32 pairs
+        _step("step_fc_1024_pair_V", 500, 32, 1024, "1024,256,64,16,1", "sweep32_lopair", "V", 2),
+        # the largest slab: 4096 groups on seven grids, 128 directions
+        _step("step_fc_4096_pair_W", 1000, 64, 4096, "4096,1024,256,64,16,4,1",
+              "sweep32_lopair", "W", 1, max_outer=4, eps=-1.0),
+        # odd sizes on a graded mesh at the library's default tile, FP32 sweeps
+        _step("step_ragged_sweep32_W", 137, 12, 200, "200,50,10,1", "sweep32", "W", 2,
+              max_outer=5, eps=-1.0, tune=False, graded=True),
+        # opacities at the radiation temperature
+        _step("step_tr_fp64_V", 120, 8, 96, "96,24,6,1", "fp64", "V", 2, max_outer=5, eps=-1.0,
+              dt=2e-3, tune=False, tr=True),
+        # a parameter study: 64 slabs of uneven sizes stepped together
+        dict(name="batch_64_pair_V", kind="batch", n=64, sizes=W.BATCH_SEED,
+             precision="sweep32_lopair", cycle="V", l_max=2, eps=1e-8, dt=1e-3),
+        # one FP64 sweep of a caller with arrays of its own, sizes off every tile
+        dict(name="sweep_fp64_ragged", kind="sweep", nx=333, N=24, G=500, precision="fp64",
+             dt=1e-3),
+        # closure inference over the benchmark slab's 512,000 (cell, group) rows
+        dict(name="mlp_infer_512k", kind="mlp_infer", rows=512000),
+        # one closure training step on the trainer's batch of 8192 rows
+        dict(name="mlp_train_8192", kind="mlp_train", rows=8192),
+    ]
+
+
+def _log_int(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    kind = rng.choice(["step"] * 6 + ["batch", "sweep", "mlp_infer", "mlp_train"])
+    if kind == "mlp_infer":
+        return dict(kind=kind, rows=_log_int(rng, 500, 512000))
+    if kind == "mlp_train":
+        return dict(kind=kind, rows=128 * _log_int(rng, 2, 128))
+    if kind == "batch":
+        return dict(kind=kind, n=_log_int(rng, 4, 64), sizes=rng.randint(1, 10 ** 6), cycle="V",
+                    l_max=2, eps=1e-8, dt=1e-3, precision=rng.choice(["sweep32_lopair", "sweep32", "fp64"]))
+    if kind == "sweep":
+        return dict(kind=kind, nx=_log_int(rng, 20, 700), N=rng.choice([4, 6, 8, 12, 16, 24, 32]),
+                    G=_log_int(rng, 17, 1100), precision=rng.choice(["fp64", "sweep32"]),
+                    dt=rng.choice([1e-3, 2e-3]))
+    factor = rng.choice([2, 4, 8])               # coarsening from the grey grid up
+    depth = rng.randint(1, {2: 5, 4: 4, 8: 3}[factor])
+    levels = [1, rng.choice([3, 4, 5, 7])]
+    while len(levels) < depth + 2 or levels[-1] < 17:    # at least fc_small's group count
+        levels.append(levels[-1] * factor)
+    nx, N = _log_int(rng, 20, 900), rng.choice([4, 6, 8, 12, 16, 32])
+    cycle = rng.choice(["V", "V", "W", "F"])
+    return _step(None, nx, N, levels[-1], ",".join(str(v) for v in reversed(levels)),
+                 rng.choice(["fp64", "fp64", "sweep32", "sweep32_lopair", "lopair", "mixed"]),
+                 cycle, rng.randint(1, 3) if cycle == "V" else 1,
+                 max_outer=rng.randint(3, 6), eps=-1.0, dt=rng.choice([1e-3, 2e-3]),
+                 tune=rng.random() < 0.5, graded=rng.random() < 0.3)
+
+
+# ---------------------------------------------------------------------------
+# inputs, made from the seed
+# ---------------------------------------------------------------------------
+def _problem(case, seed):
+    """A slab's mesh, groups and the physical parameters that a study varies."""
+    r = np.random.default_rng(seed)
+    nx = case["nx"]
+    p = dict(levels=[int(v) for v in case["levels"].split(",")],
+             edges=W.group_edges(case["G"], case["nu_a"], case["nu_b"], float(case["top"])),
+             T_left=float(r.uniform(0.7, 1.3)), scale=float(r.uniform(0.7, 1.4)),
+             T0=0.05 if case["tr"] else 1e-3)
+    x = np.linspace(0.0, case["length"], nx + 1)
+    if case["graded"]:
+        x = np.concatenate([[0.0], np.cumsum(W.random_h(r, nx, case["length"]))])
+    p["x"] = x
+    return p
+
+
+def _batch_slabs(case, seed):
+    """Slabs of the batched family: their sizes belong to the case, the inflow temperatures
+    and opacity scales to the seed."""
+    r = np.random.default_rng(seed)
+    slabs = W.batch_256(case["n"], case["sizes"])
+    for s in slabs:
+        s.T_left, s.opac_scale = float(r.uniform(0.3, 1.5)), float(r.uniform(0.5, 2.0))
+    return slabs
+
+
+def _sweep_inputs(case, seed):
+    """Opacities, emission and intensities of a caller: a hot-to-cold slab, spectra spanning
+    many decades."""
+    nx, M, G = case["nx"], 2 * case["N"], case["G"]
+    g = torch.Generator(device=DEV)
+    g.manual_seed(seed)
+    u = lambda lo, hi, *s: lo + (hi - lo) * torch.rand(s, generator=g, device=DEV, dtype=F64)  # noqa: E731
+    T = torch.exp(u(math.log(1e-3), math.log(1.5), nx))
+    nu = torch.as_tensor(np.geomspace(1e-2, 30.0, G), device=DEV)
+    sig = 27.0 / nu[:, None] ** 3 * -torch.expm1(-nu[:, None] / T[None, :])
+    base = torch.exp(u(-30.0, 2.0, G))
+    emis = sig * base[:, None] * u(0.5, 1.5, G, nx)
+    I = torch.zeros((M, nx, 2, (G + 31) // 32 * 32), dtype=F64, device=DEV)
+    I[..., :G] = base * u(0.2, 1.8, M, nx, 2, G)
+    if case["precision"] == "sweep32":
+        I = I.float()
+    return sig, emis, I
+
+
+def _mlp_inputs(case, seed):
+    """Network parameters as trained runs have them, features and targets in their ranges."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(seed)
+    rnd = lambda *s: torch.rand(s, generator=g, device=DEV)  # noqa: E731
+    P = torch.as_tensor(closure._init(seed), device=DEV)
+    for o in (mlp_off["b1"], mlp_off["b2"], mlp_off["b3"]):
+        P[o:o + 256] = 0.2 * rnd(256) - 0.1
+    x = 3.0 * rnd(case["rows"], 3) - 1.5
+    t = 0.35 + 0.5 * torch.sigmoid(2.0 * x[:, 1] - x[:, 2]) + 0.1 * torch.tanh(x[:, 0])
+    return P, x, t.clamp(0.34, 0.99)
+
+
+mlp_off = dict(W1=0, b1=768, W2=1024, b2=66560, W3=66816, b3=132352, w4=132608, b4=132864)
+
+
+def prepare(case, seed):
+    k = case["kind"]
+    if k == "step":
+        p = _problem(case, seed)
+        s = trt.Solver(case["nx"], case["length"], case["N"], p["edges"], p["levels"], p["scale"],
+                       W.CV_FC, p["T0"], p["T_left"], 0.0, precision=case["precision"],
+                       device="cuda:0", x_edges=p["x"], tr_mode=case["tr"])
+        if case["tune"]:
+            s.autotune(case["dt"], reps=3)
+        return dict(case=case, solver=s, groups=_group_fields(s, s.workspace))
+    if k == "batch":
+        b = trt.Batch(_batch_slabs(case, seed), precision=case["precision"], device="cuda:0")
+        if case["precision"] != "fp64":
+            b.set_tile(16, 4)                    # the tuner's choice for this family
+        views = [b.slab(i) for i in range(case["n"])]
+        return dict(case=case, batch=b, views=views,
+                    groups=[_group_fields(v, b.workspace) for v in views])
+    if k == "sweep":
+        s = trt.Solver(case["nx"], 6.0, case["N"], W.group_edges(case["G"], 1e-5, 1e2),
+                       [case["G"], 1], precision=case["precision"], device="cuda:0")
+        sig, emis, I = _sweep_inputs(case, seed)
+        out = [torch.zeros_like(I), torch.zeros_like(sig)] + \
+              [torch.zeros(case["G"], dtype=F64, device=DEV) for _ in range(4)]
+        return dict(case=case, solver=s, args=(sig, emis, I), out=out)
+    P, x, t = _mlp_inputs(case, seed)
+    net = mlp.MLP(device="cuda:0")
+    net.params.copy_(P)
+    net.refresh()
+    return dict(case=case, net=net, x=x, t=t)
+
+
+def _group_fields(s, workspace):
+    """The solver's E_g and F_g of the last step as tensors over its own device arrays."""
+    lv = trt.trt_level()
+    s._check(trt.lib().trt_level_view(s.h, 0, ctypes.byref(lv)))
+
+    def view(p, shape):
+        at = ctypes.cast(p, ctypes.c_void_p).value - workspace.data_ptr()
+        n = shape[0] * shape[1]
+        return workspace[at:at + 8 * n].view(F64).view(shape)
+
+    return view(lv.E, (s.G, s.nx)), view(lv.F, (s.G, s.nx + 1))
+
+
+# ---------------------------------------------------------------------------
+# one pass
+# ---------------------------------------------------------------------------
+def run(state):
+    case, k = state["case"], state["case"]["kind"]
+    if k == "step":
+        s = state["solver"]
+        s.step(case["dt"], case["cycle"], case["l_max"], case["eps"], max_outer=case["max_outer"])
+        m = s.moments(groups=False)
+        return dict(T=m["T"], E=m["E"], F=m["F"], Eg=state["groups"][0], Fg=state["groups"][1])
+    if k == "batch":
+        state["batch"].step(case["dt"], case["cycle"], case["l_max"], case["eps"])
+        m = [v.moments(groups=False) for v in state["views"]]
+        out = {key: np.concatenate([x[key] for x in m]) for key in ("T", "E", "F")}
+        out["Eg"] = torch.cat([g[0].reshape(-1) for g in state["groups"]])
+        out["Fg"] = torch.cat([g[1].reshape(-1) for g in state["groups"]])
+        return out
+    if k == "sweep":
+        s = state["solver"]
+        s._check(trt.lib().trt_k_sweep(s.h, case["dt"], *[a.data_ptr() for a in state["args"]],
+                                       *[o.data_ptr() for o in state["out"]]))
+        I, f, fb0, fbX, C0, CX = state["out"]
+        return dict(I=I[..., :case["G"]], f=f, fb0=fb0, fbX=fbX, C0=C0, CX=CX)
+    net = state["net"]
+    if k == "mlp_infer":
+        return net.forward_fused(state["x"])
+    loss = net.train_step(state["x"], state["t"], lr=1e-3)
+    return dict(loss=loss, grad=net.grad_buf, params=net.params, m=net.m, v=net.v)
+
+
+# ---------------------------------------------------------------------------
+# what a pass cannot do without
+# ---------------------------------------------------------------------------
+def _step_work(nx, N, G, fp32, levels, cycle, l_max, phases):
+    """Fields read and written once per sweep and cycle; operations per sweep update 23, per
+    group cell of a low-order solve 44, an opacity evaluation 28, a restriction 16."""
+    S = []
+    if cycle == "W":
+        S = [levels[-2]]
+        for n in reversed(levels[1:-2]):
+            S = S + [n] + S
+        S = S if len(levels) > 2 else []
+    elif cycle == "F":
+        S = levels[-2:0:-1]
+    upd, cg = nx * 2 * N * G, nx * G
+    visits = len(S)
+    sweeps, cycles = phases - 1, phases * l_max
+    lo = cg + sum(n * nx for n in S)
+    flops = sweeps * upd * 23 + cycles * (44 * lo + 28 * cg * (1 + visits) + 16 * (cg * (1 + visits)))
+    byt = sweeps * upd * 4 * (4 if fp32 else 8) + cycles * 8 * (10 * lo + 4 * cg * (1 + visits))
+    return dict(bytes=byt, flops=flops)
+
+
+def work(case):
+    k = case["kind"]
+    if k == "mlp_infer":
+        n = case["rows"]
+        return dict(bytes=16 * n + 6 * mlp.NPARAM, flops=2 * n * (3 * 256 + 2 * 65536 + 256))
+    if k == "mlp_train":
+        n = case["rows"]
+        return dict(bytes=16 * n + 4 * 8 * mlp.NPARAM, flops=6 * n * (3 * 256 + 2 * 65536 + 256))
+    if k == "sweep":
+        upd, cg = case["nx"] * 2 * case["N"] * case["G"], case["nx"] * case["G"]
+        b = 4 if case["precision"] == "sweep32" else 8
+        return dict(bytes=upd * 4 * b + cg * 24, flops=23 * upd)
+    fp32 = "sweep32" in case["precision"] or case["precision"] == "mixed"
+    if k == "batch":
+        total = dict(bytes=0, flops=0)
+        for s in W.batch_256(case["n"], case["sizes"]):
+            w = _step_work(s.n_cells, s.N, s.G, fp32, s.levels, "V", case["l_max"], 6)
+            total = {key: total[key] + w[key] for key in w}
+        return total
+    phases = case["max_outer"] if case["eps"] < 0 else 6
+    return _step_work(case["nx"], case["N"], case["G"], fp32,
+                      [int(v) for v in case["levels"].split(",")], case["cycle"], case["l_max"],
+                      phases)
+
+
+# ---------------------------------------------------------------------------
+# the same in plain torch, 64 bits
+# ---------------------------------------------------------------------------
+_GX, _GW = np.polynomial.legendre.leggauss(8)
+
+
+def _quadratures(xa, xb, rho=None):
+    """e^{xa} times the group integrals over [xa, xb] (cut at xa + 64) of t^3/(e^t - 1),
+    t^4 e^t/(e^t - 1)^2, t^7 e^t/((1 - e^{-rho t})(e^t - 1)^2) and (1 - e^{-rho t})/(e^t - 1)
+    by 8-point Gauss rules on panels of width at most 2 (graded towards 0 for rho > 1)."""
+    hi = torch.minimum(xb, xa + 64.0)
+    a = xa.clone()
+    P, Nn, D, J = (torch.zeros_like(xa) for _ in range(4))
+    while bool((a < hi).any()):
+        wmax = torch.full_like(a, 2.0)
+        if rho is not None:
+            wmax = torch.where(rho > 1.0, torch.minimum(wmax, torch.maximum(1.0 / rho, 0.5 * a)), wmax)
+        b = torch.where(hi - a <= 1.5 * wmax, hi, a + wmax)
+        half = 0.5 * (b - a)
+        for gx, gw in zip(_GX, _GW):
+            x = a + half * (1.0 + float(gx))
+            e, om = torch.exp(xa - x), -torch.expm1(-x)
+            orh = om if rho is None else -torch.expm1(-rho * x)
+            wq, x3 = half * float(gw), x * x * x
+            P += wq * x3 * e / om
+            Nn += wq * x3 * x * e / (om * om)
+            D += wq * x3 * x3 * x * e / (orh * om * om)
+            J += wq * e * orh / om
+        a = b
+    return P, Nn, D, J
+
+
+class _Slab:
+    """Algorithm 3 on one slab: simple-corner-balance sweeps, group low-order systems by
+    Thomas elimination, restriction by sums over members, one Newton step per grey visit."""
+
+    def __init__(self, case, seed):
+        p = _problem(case, seed)
+        self.dt, self.case, self.levels, self.s = case["dt"], case, p["levels"], p["scale"]
+        t = lambda a: torch.as_tensor(np.asarray(a, np.float64), device=DEV)  # noqa: E731
+        self.h, self.edges = t(np.diff(p["x"])), t(p["edges"])
+        self.nx, self.G = case["nx"], case["G"]
+        x, w = np.polynomial.legendre.leggauss(case["N"])
+        self.mu, self.w = t(0.5 * (1.0 + x)), t(0.5 * w)      # one half range
+        e = self.edges
+        self.T = torch.full((self.nx,), p["T0"], dtype=F64, device=DEV)
+        B0 = self.planck(p["T0"])
+        self.Iin = self.planck(p["T_left"])
+        n0, n1, n2 = self.w.sum(), (self.w * self.mu).sum(), (self.w * self.mu ** 2).sum()
+        one = torch.ones_like(B0)
+        self.Ein0, self.Fin0, self.zero = n0 * self.Iin / C, n1 * self.Iin, torch.zeros_like(B0)
+        self.Eg = (2 * n0 * B0 / C)[:, None].expand(-1, self.nx).clone()
+        self.Fg = torch.zeros((self.G, self.nx + 1), dtype=F64, device=DEV)
+        self.f = (n2 / n0 * one)[:, None].expand(-1, self.nx).clone()
+        self.fb0 = self.fbX = n2 / n0 * one
+        self.C0, self.CX = -n1 / n0 * one, n1 / n0 * one
+        N = case["N"]
+        self.I = [B0.expand(N, self.nx, 2, self.G).clone() for _ in range(2)]   # mu > 0, mu < 0
+        self.last = bool(torch.isinf(e[-1]))
+        dx = 0.5 * (torch.cat([self.h[:1] * 0, self.h]) + torch.cat([self.h, self.h[:1] * 0]))
+        self.dx = dx                                          # face widths, half cells at the ends
+
+    def planck(self, T):
+        xa, xb = self.edges[:-1] / T, self.edges[1:] / T
+        return C_B * T ** 4 * torch.exp(-xa) * _quadratures(xa, xb)[0]
+
+    def opacities(self, T, E):
+        Tr = T
+        if self.case["tr"]:
+            Tr = torch.where(E > 0, (E / A_RAD) ** 0.25, T)
+        out = []
+        for c in range(0, self.nx, 128):                      # a slice of cells at a time
+            t, r = T[None, c:c + 128], Tr[None, c:c + 128]
+            ya, yb = self.edges[:-1, None] / t, self.edges[1:, None] / t
+            xa, xb = self.edges[:-1, None] / r, self.edges[1:, None] / r
+            P, Nn, D, J = _quadratures(xa, xb, r / t + 0 * xa if self.case["tr"] else None)
+            em = 27.0 * self.s * C_B * t * torch.exp(-ya) * -torch.expm1(ya - yb)
+            k = 27.0 * self.s / r ** 3
+            out.append((k * J / P, em, k * Nn / D))
+        return [torch.cat(v, 1) for v in zip(*out)]
+
+    def sweep(self, sig, em):
+        """The intensities of the new time level and the QD factors."""
+        h, icdt, mu = self.h, 1.0 / (C * self.dt), self.mu[:, None]
+        b = 0.5 * mu
+        new, out = [torch.empty_like(v) for v in self.I], []
+        A0, A2 = torch.zeros_like(sig), torch.zeros_like(sig)
+        for d in range(2):
+            psi = self.Iin.expand(len(self.mu), -1) if d == 0 else torch.zeros_like(self.I[1][:, 0, 0])
+            up, dn = (0, 1) if d == 0 else (1, 0)             # the corner the flow enters, leaves
+            for i in (range(self.nx) if d == 0 else range(self.nx - 1, -1, -1)):
+                a = b + 0.5 * (sig[:, i] + icdt) * h[i]
+                ru = 0.5 * h[i] * (em[:, i] + icdt * self.I0[d][:, i, up]) + mu * psi
+                rd = 0.5 * h[i] * (em[:, i] + icdt * self.I0[d][:, i, dn])
+                det = a * a + b * b
+                pu, psi = (a * ru - b * rd) / det, (a * rd + b * ru) / det
+                new[d][:, i, up], new[d][:, i, dn] = pu, psi
+                S = 0.5 * (pu + psi)
+                A0[:, i] += self.w @ S
+                A2[:, i] += (self.w * self.mu ** 2) @ S
+            out.append(psi)
+        self.I = new
+        q = lambda a, b, z: torch.where(b != 0, a / b, torch.full_like(a, z))  # noqa: E731
+        self.f = q(A2, A0, 1.0 / 3.0)
+        w, m = self.w, self.mu
+        for face, (ins, outs) in enumerate(((self.Iin.expand(len(m), -1), out[1]),
+                                            (torch.zeros_like(out[0]), out[0]))):
+            fb = q((w * m * m) @ (ins + outs), w @ (ins + outs), 1.0 / 3.0)
+            Cb = q((w * m) @ outs, w @ outs, 0.5)
+            if face == 0:
+                self.fb0, self.C0 = fb, -Cb
+            else:
+                self.fbX, self.CX = fb, Cb
+
+    def solve(self, L, a, s):
+        """E, F and the boundary-face energies of every group of a level."""
+        dt, h, dx, icdt = self.dt, self.h, self.dx, 1.0 / (C * self.dt)
+        pl = torch.cat([L["b0"][:, None], L["phi"]], 1) + L["etaL"]
+        pr = torch.cat([L["phi"], L["bX"][:, None]], 1) + L["etaR"]
+        D = dx * (icdt + L["sigR"])
+        Gf = dx * L["Fold"] * icdt
+        D[:, 0] -= pl[:, 0] / L["C0"]
+        D[:, -1] += pr[:, -1] / L["CX"]
+        Gf[:, 0] += pl[:, 0] * (C * L["Ein0"] - L["Fin0"] / L["C0"])
+        Gf[:, -1] += -pr[:, -1] * (C * L["EinX"] - L["FinX"] / L["CX"])
+        PL, PR, GD = C * pl / D, C * pr / D, Gf / D
+        di = (h / dt + h * a + PL[:, 1:] + PR[:, :-1]).T.contiguous()
+        rh = (h * s + h * L["Eold"] / dt - GD[:, 1:] + GD[:, :-1]).T.contiguous()
+        up, lo = (-PR[:, 1:]).T.contiguous(), (-PL[:, :-1]).T.contiguous()
+        di, rh, up, lo = ([*v.unbind(0)] for v in (di, rh, up, lo))
+        for i in range(1, self.nx):
+            k = lo[i] / di[i - 1]
+            di[i] = di[i] - k * up[i - 1]
+            rh[i] = rh[i] - k * rh[i - 1]
+        E = [rh[-1] / di[-1]]
+        for i in range(self.nx - 2, -1, -1):
+            E.append((rh[i] - up[i] * E[-1]) / di[i])
+        E = torch.stack(E[::-1], 1)
+        z = torch.zeros_like(E[:, :1])
+        F = GD + PL * torch.cat([z, E], 1) - PR * torch.cat([E, z], 1)
+        L["E"], L["F"] = E, F
+        L["Eb0"] = L["Ein0"] + (F[:, 0] - L["Fin0"]) / (C * L["C0"])
+        L["EbX"] = L["EinX"] + (F[:, -1] - L["FinX"]) / (C * L["CX"])
+        return L
+
+    def restrict(self, A, n):
+        g = lambda v: v.reshape(n, -1, *v.shape[1:])  # noqa: E731
+
+        def mean(v, w):
+            v, w = g(v), g(w)
+            d = w.sum(1)
+            return torch.where(d != 0, (v * w).sum(1) / torch.where(d != 0, d, torch.ones_like(d)),
+                               v.mean(1))
+
+        ER = torch.cat([A["E"], A["EbX"][:, None]], 1)
+        EL = torch.cat([A["Eb0"][:, None], A["E"]], 1)
+        L = dict(phi=mean(A["phi"], A["E"]), sig=mean(A["sig"], A["E"]),
+                 sigR=mean(A["sigR"], A["F"].abs() + 0.5e-6 * C * (EL + ER)),
+                 b0=mean(A["b0"], A["Eb0"]), bX=mean(A["bX"], A["EbX"]),
+                 C0=mean(A["C0"], A["Eb0"] - A["Ein0"]), CX=mean(A["CX"], A["EbX"] - A["EinX"]))
+        for k in ("emis", "Eold", "Fold", "Ein0", "Fin0", "EinX", "FinX"):
+            L[k] = g(A[k]).sum(1)
+        L["Esum"] = g(A["E"]).sum(1)
+        xi = (self.dx * (g(A["sigR"]) - L["sigR"][:, None]) * g(A["F"]) +
+              C * (g(A["etaR"] * ER) - g(A["etaL"] * EL))).sum(1)
+        sR, sL = g(ER).sum(1), g(EL).sum(1)
+        z = torch.zeros_like(xi)
+        L["etaR"] = torch.where((xi > 0) & (sR != 0), xi / (C * sR), z)
+        L["etaL"] = torch.where((xi < 0) & (sL != 0), -xi / (C * sL), z)
+        return L
+
+    def newton(self, L, Tst, prev, cut):
+        cv, dt = W.CV_FC, self.dt
+        e0 = self.edges[0] / Tst
+        dQ = (1.0 + e0) * torch.exp(-e0)
+        if not self.last:
+            eX = self.edges[-1] / Tst
+            dQ = dQ - (1.0 + eX) * torch.exp(-eX)
+        dQ, Q = 54.0 * self.s * C_B * dQ, 2.0 * L["emis"][0]
+        sig, Es = L["sig"][0], L["Esum"][0]
+        D = torch.zeros_like(Q)
+        if prev is not None:
+            dT = Tst - prev[1]
+            ok = (dT != 0) & (dT.abs() > cut * Tst)
+            D = torch.where(ok, (sig - prev[0]) / torch.where(ok, dT, torch.ones_like(dT)), D)
+        base = cv / dt + dQ
+        lam = torch.maximum(base - C * D * Es, 0.5 * base)
+        w, m = (cv / dt) / lam, cv * (Tst - self.Told) / dt
+        self.solve(L, (w * C * sig)[None], (w * Q - (1.0 - w) * m)[None])
+        return Tst + (C * sig * L["E"][0] - Q - m) / lam
+
+    def fine(self, sig, em, sR):
+        h, z = self.h, torch.zeros((self.G, self.nx + 1), dtype=F64, device=DEV)
+        mid = (sR[:, :-1] * h[:-1] + sR[:, 1:] * h[1:]) / (h[:-1] + h[1:])
+        return dict(phi=self.f, sig=sig, emis=em, Eold=self.Eg0, Fold=self.Fg0, etaR=z, etaL=z,
+                    sigR=torch.cat([sR[:, :1], mid, sR[:, -1:]], 1), b0=self.fb0, bX=self.fbX,
+                    C0=self.C0, CX=self.CX, Ein0=self.Ein0, Fin0=self.Fin0, EinX=self.zero,
+                    FinX=self.zero)
+
+    def step(self):
+        c = self.case
+        S, lv = [], self.levels
+        if c["cycle"] == "W" and len(lv) > 2:
+            S = [lv[-2]]
+            for n in reversed(lv[1:-2]):
+                S = S + [n] + S
+        elif c["cycle"] == "F":
+            S = lv[-2:0:-1]
+        self.Told, self.Eg0, self.Fg0, self.I0 = self.T, self.Eg, self.Fg, self.I
+        T, prev, fixed = self.T, None, c["eps"] < 0
+        E = Eph = self.Eg0.sum(0)
+        same = lambda a, b, tol: bool((a - b).abs().max() <= tol * a.abs().max())  # noqa: E731
+        for phase in range(c["max_outer"]):
+            if phase > 0:
+                self.sweep(*self.opacities(T, E)[:2])
+            Tph, Ec = T, Eph
+            for _ in range(c["l_max"]):
+                Tc = T
+                F = self.fine(*self.opacities(T, E))
+                self.solve(F, C * F["sig"], 2.0 * F["emis"])
+                for k in range(len(S) + 1):
+                    L = F
+                    if k > 0:
+                        L = self.fine(*self.opacities(T, E))
+                        L.update({q: F[q] for q in ("E", "F", "Eb0", "EbX")})
+                        L = self.restrict(L, S[k - 1])
+                        self.solve(L, C * L["sig"], 2.0 * L["emis"])
+                    gr = self.restrict(L, 1)
+                    Tn = self.newton(gr, T, prev, 1e-7 if S else 0.0)
+                    prev, T, E = (gr["sig"][0], T), Tn, gr["E"][0]
+                done = same(T, Tc, 0.1 * c["eps"]) and same(E, Ec, 0.1 * c["eps"])
+                Ec = E
+                if not fixed and done:
+                    break
+            end = same(T, Tph, c["eps"]) and same(E, Eph, c["eps"])
+            Eph = E
+            if not fixed and end:
+                break
+        return dict(T=T, E=E, F=gr["F"][0], Eg=F["E"], Fg=F["F"])
+
+
+def _exact_sweep(case, seed):
+    sig, em, I = _sweep_inputs(case, seed)
+    N, nx, G = case["N"], case["nx"], case["G"]
+    s = _Slab(dict(case, levels="%d,1" % G, nu_a=1e-5, nu_b=1e2, top="inf", tr=False,
+                   graded=False, length=6.0), 0)
+    s.Iin = s.planck(1.0)
+    s.I0 = s.I = [v.double() for v in (I[:N, ..., :G], I[N:, ..., :G])]
+    s.sweep(sig, em)
+    return dict(I=torch.cat(s.I, 0), f=s.f, fb0=s.fb0, fbX=s.fbX, C0=s.C0, CX=s.CX)
+
+
+def _exact_mlp(case, seed):
+    P, x, t = (v.double() for v in _mlp_inputs(case, seed))
+    o = mlp_off
+    W1, W2, W3 = P[:768].view(256, 3), P[o["W2"]:o["b2"]].view(256, 256), \
+        P[o["W3"]:o["b3"]].view(256, 256)
+    b1, b2, b3, w4 = (P[o[k]:o[k] + 256] for k in ("b1", "b2", "b3", "w4"))
+    h1 = torch.relu(x @ W1.T + b1)
+    h2 = torch.relu(h1 @ W2.T + b2)
+    h3 = torch.relu(h2 @ W3.T + b3)
+    y = torch.sigmoid(h3 @ w4 + P[o["b4"]])
+    if case["kind"] == "mlp_infer":
+        return y
+    dz = 2.0 / len(x) * (y - t) * y * (1.0 - y)
+    d3 = dz[:, None] * w4 * (h3 > 0)
+    d2 = d3 @ W3 * (h2 > 0)
+    d1 = d2 @ W2 * (h1 > 0)
+    grad = torch.zeros_like(P)
+    for k, v in (("W1", d1.T @ x), ("b1", d1.sum(0)), ("W2", d2.T @ h1), ("b2", d2.sum(0)),
+                 ("W3", d3.T @ h2), ("b3", d3.sum(0)), ("w4", dz @ h3), ("b4", dz.sum())):
+        grad[o[k]:o[k] + v.numel()] = v.reshape(-1)
+    m, v = 0.1 * grad, 0.001 * grad * grad
+    params = P - 1e-3 * (m / 0.1) / (torch.sqrt(v / 0.001) + 1e-8)
+    return dict(loss=((y - t) ** 2).mean()[None], grad=grad, params=params, m=m, v=v)
+
+
+def exact(case, seed):
+    if case["kind"].startswith("mlp"):
+        return _exact_mlp(case, seed)
+    if case["kind"] == "sweep":
+        return _exact_sweep(case, seed)
+    # the largest slabs, 64 slabs of a batch: minutes of host-driven elimination
+    if case["kind"] == "batch" or case["nx"] * case["N"] * case["G"] > 2e7:
+        return None
+    return _Slab(case, seed).step()
