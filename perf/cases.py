@@ -85,7 +85,7 @@ def draw(rng):
     if kind == "mlp_infer":
         return dict(kind=kind, rows=_log_int(rng, 500, 512000))
     if kind == "mlp_train":
-        return dict(kind=kind, rows=128 * _log_int(rng, 2, 128))
+        return dict(kind=kind, rows=128 * _log_int(rng, 4, 128))
     if kind == "batch":
         return dict(kind=kind, n=_log_int(rng, 4, 64), sizes=rng.randint(1, 10 ** 6), cycle="V",
                     l_max=2, eps=1e-8, dt=1e-3, precision=rng.choice(["sweep32_lopair", "sweep32", "fp64"]))
