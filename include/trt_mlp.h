@@ -76,7 +76,7 @@ int trt_mlp_refresh(const float *params, void *w16, void *stream);
 int trt_mlp_forward(int rows, const float *x, const float *params, const void *w16,
                     void *scratch, size_t scratch_bytes, float *y, void *stream);
 
-/* Inference in one persistent kernel (one CTA per SM in clusters of two, 256 rows per
+/* Inference in one persistent kernel (one CTA per SM, 256 rows per
  * iteration as two 128-row groups half a period apart, both hidden layers on the tensor
  * cores with the activations kept in shared memory and the weights streamed in 32-wide K
  * chunks from the image trt_mlp_refresh keeps in w16); same arithmetic and result as

@@ -98,13 +98,14 @@ __device__ inline uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
            ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
 }
 
+template <uint32_t kDesc = IDESC>
 __device__ inline void umma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(IDESC), "r"(acc));
+        "l"(a), "l"(b), "r"(kDesc), "r"(acc));
 }
 
 __device__ inline void umma_commit(uint64_t *bar)
@@ -169,15 +170,10 @@ struct Epi {
     float *out32;
     bf16 *out16, *out16T;
     int ldT;
-    // head: z = sum_n act[n] w[n] + b, y = sigmoid(z); with a target, also
-    // dz = scale (y - t) y (1 - y), sq = (y - t)^2, dact = dz w[n] [act > 0]
+    // head: z = sum_n act[n] w[n] + b, y = sigmoid(z)
     const float *head_w;
     const float *head_b;   // device pointer to the head's bias
     float *head_y;
-    const float *target;
-    float scale;
-    float *dz, *sq;
-    bf16 *dact16, *dact16T;
 };
 
 __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const bf16 *__restrict__ A,
@@ -326,34 +322,9 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const bf16 *_
                 for (int j = 0; j < 32; ++j) dot = fmaf(v[j], e.head_w[nb + j], dot);
             }
         }
-        float dz = 0.f;
         if (e.head_w && row < M) {
             const float z = dot + *e.head_b;
-            const float y = 1.f / (1.f + __expf(-z));
-            if (e.head_y) e.head_y[row] = y;
-            if (e.target) {
-                const float d = y - e.target[row];
-                dz = e.scale * d * y * (1.f - y);
-                e.dz[row] = dz;
-                e.sq[row] = 0.5f * e.scale * d * d;
-            }
-        }
-        if (e.head_w && e.target) {
-            // second pass over the accumulator (all threads: the loads are warp-collective)
-            // for the gradient of the last hidden layer, dz w4 [h3 > 0]
-            for (int ch = 0; ch < BN / 32; ++ch) {
-                float v[32];
-                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + ch * 32, v);
-                if (row >= M) continue;
-                const int nb = n0 + ch * 32;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float a = v[j] + (e.bias ? e.bias[nb + j] : 0.f);
-                    const bf16 gb = __float2bfloat16_rn((a > 0.f) ? dz * e.head_w[nb + j] : 0.f);
-                    e.dact16[(size_t)row * N + nb + j] = gb;
-                    e.dact16T[(size_t)(nb + j) * e.ldT + row] = gb;
-                }
-            }
+            e.head_y[row] = 1.f / (1.f + __expf(-z));
         }
     }
     tc_before();
@@ -446,6 +417,64 @@ __device__ inline uint32_t relu_bf16x2(float2 v)
     return d;
 }
 
+// element (row, K group k8) of an activation tile: core matrix (row / 8, k8), row % 8 at
+// 16 bytes
+__device__ inline uint32_t a_off(int row, int k8)
+{
+    return (uint32_t)((row >> 3) * FA_SBO + k8 * 128 + (row & 7) * 16);
+}
+
+// layer 1 of one row, h1 = relu(W1 x + b1), columns 8 k0 .. 8 k1 - 1 into the activation
+// tile: 8 columns per step, W1^T rows and b1 as broadcast float4 reads of shared memory,
+// pairs of columns by packed FP32 FMAs, ReLU fused in the BF16 pack.  kMax: clamp first by
+// fmax, which turns a NaN into 0 as the GEMM epilogue does (the pack's ReLU keeps it)
+template <bool kMax>
+__device__ inline void layer1_row(const float *sP, float x0, float x1, float x2,
+                                  unsigned char *A, int r, int k0, int k1)
+{
+    const float2 X0 = make_float2(x0, x0), X1 = make_float2(x1, x1), X2 = make_float2(x2, x2);
+    const float4 *pw0 = reinterpret_cast<const float4 *>(sP + FP_W1);
+    const float4 *pw1 = reinterpret_cast<const float4 *>(sP + FP_W1 + 256);
+    const float4 *pw2 = reinterpret_cast<const float4 *>(sP + FP_W1 + 512);
+    const float4 *pb = reinterpret_cast<const float4 *>(sP + FP_B1);
+#pragma unroll 4
+    for (int k8 = k0; k8 < k1; ++k8) {
+        uint4 u;
+        uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 b = pb[k8 * 2 + h], w0 = pw0[k8 * 2 + h], w1 = pw1[k8 * 2 + h],
+                         w2 = pw2[k8 * 2 + h];
+            float2 a = make_float2(b.x, b.y), c = make_float2(b.z, b.w);
+            a = fma2(make_float2(w0.x, w0.y), X0, a);
+            c = fma2(make_float2(w0.z, w0.w), X0, c);
+            a = fma2(make_float2(w1.x, w1.y), X1, a);
+            c = fma2(make_float2(w1.z, w1.w), X1, c);
+            a = fma2(make_float2(w2.x, w2.y), X2, a);
+            c = fma2(make_float2(w2.z, w2.w), X2, c);
+            if (kMax) {
+                a = make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+                c = make_float2(fmaxf(c.x, 0.f), fmaxf(c.y, 0.f));
+            }
+            hw[2 * h] = relu_bf16x2(a);
+            hw[2 * h + 1] = relu_bf16x2(c);
+        }
+        *reinterpret_cast<uint4 *>(A + a_off(r, k8)) = u;
+    }
+}
+
+// small parameters into shared memory (W1 transposed, b1, b2, b3, w4, b4) by threads
+// 0 .. 255; P of any alignment
+__device__ inline void stage_params(float *sP, const float *P, int tid)
+{
+    for (int k = 0; k < 3; ++k) sP[FP_W1 + k * 256 + tid] = __ldg(P + TRT_MLP_W1 + 3 * tid + k);
+    sP[FP_B1 + tid] = __ldg(P + TRT_MLP_B1 + tid);
+    sP[FP_B2 + tid] = __ldg(P + TRT_MLP_B2 + tid);
+    sP[FP_B3 + tid] = __ldg(P + TRT_MLP_B3 + tid);
+    sP[FP_W4 + tid] = __ldg(P + TRT_MLP_W4 + tid);
+    if (tid == 0) sP[FP_B4] = __ldg(P + TRT_MLP_B4);
+}
+
 // one contiguous bulk copy global -> this CTA's shared memory, completing (bytes) on `bar`
 __device__ inline void bulk_copy(void *dst, const void *src, unsigned bytes, uint64_t *bar)
 {
@@ -493,15 +522,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
                      "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (tid < 256) {   // small parameters (W1 transposed; float4 runs b1, b2, b3 + w4)
-        const float4 *gp = reinterpret_cast<const float4 *>(P);
-        float4 *d = reinterpret_cast<float4 *>(sP);
-        for (int k = 0; k < 3; ++k) sP[FP_W1 + k * 256 + tid] = __ldg(P + TRT_MLP_W1 + 3 * tid + k);
-        if (tid < 64) d[FP_B1 / 4 + tid] = __ldg(gp + TRT_MLP_B1 / 4 + tid);     // b1
-        if (tid < 64) d[FP_B2 / 4 + tid] = __ldg(gp + TRT_MLP_B2 / 4 + tid);     // b2
-        if (tid < 128) d[FP_B3 / 4 + tid] = __ldg(gp + TRT_MLP_B3 / 4 + tid);    // b3, w4
-        if (tid == 0) sP[FP_B4] = __ldg(P + TRT_MLP_B4);
-    }
+    if (tid < 256) stage_params(sP, P, tid);
     tc_before();
     __syncthreads();
     tc_after();
@@ -569,8 +590,6 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
         const int g = warp >> 2, r = tid & 127;
         unsigned char *myA = sm + g * FA_BYTES;
         const uint32_t tb = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * 256);
-        // A tile element (row, k) offset: core matrix (row / 8, k / 8), row % 8 at 16 bytes
-        auto a_off = [](int row, int k8) { return (row >> 3) * FA_SBO + k8 * 128 + (row & 7) * 16; };
         unsigned pacc = 0;
         auto wait_acc = [&]() {
             if (!mbar_wait(&acc[g], pacc)) {
@@ -598,37 +617,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
         for (int it = 0; it < mine && ok; ++it) {
             const int row = ((int)blockIdx.x + it * (int)gridDim.x) * 256 + g * 128 + r;
             const bool rv = row < rows;
-            // ---- layer 1: h1 = relu(W1 x + b1) ----
-            {
-                const float2 X0 = make_float2(xn0, xn0), X1 = make_float2(xn1, xn1),
-                             X2 = make_float2(xn2, xn2);
-                // 8 columns per step: W1^T rows and b1 as broadcast float4 reads of shared
-                // memory, pairs of columns by packed FP32 FMAs, ReLU fused in the BF16 pack
-                const float4 *pw0 = reinterpret_cast<const float4 *>(sP + FP_W1);
-                const float4 *pw1 = reinterpret_cast<const float4 *>(sP + FP_W1 + 256);
-                const float4 *pw2 = reinterpret_cast<const float4 *>(sP + FP_W1 + 512);
-                const float4 *pb = reinterpret_cast<const float4 *>(sP + FP_B1);
-#pragma unroll 4
-                for (int k8 = 0; k8 < 32; ++k8) {
-                    uint4 u;
-                    uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float4 b = pb[k8 * 2 + h], w0 = pw0[k8 * 2 + h],
-                                     w1 = pw1[k8 * 2 + h], w2 = pw2[k8 * 2 + h];
-                        float2 a = make_float2(b.x, b.y), c = make_float2(b.z, b.w);
-                        a = fma2(make_float2(w0.x, w0.y), X0, a);
-                        c = fma2(make_float2(w0.z, w0.w), X0, c);
-                        a = fma2(make_float2(w1.x, w1.y), X1, a);
-                        c = fma2(make_float2(w1.z, w1.w), X1, c);
-                        a = fma2(make_float2(w2.x, w2.y), X2, a);
-                        c = fma2(make_float2(w2.z, w2.w), X2, c);
-                        hw[2 * h] = relu_bf16x2(a);
-                        hw[2 * h + 1] = relu_bf16x2(c);
-                    }
-                    *reinterpret_cast<uint4 *>(myA + a_off(r, k8)) = u;
-                }
-            }
+            layer1_row<false>(sP, xn0, xn1, xn2, myA, r, 0, 32);
             // the next tile's inputs, in flight during the two layers
             {
                 const int nrow = row + (int)gridDim.x * 256;
@@ -713,6 +702,506 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
     }
 }
 
+// ---- training: forward, backward and weight gradients of 128 rows per CTA ----
+// One CTA takes 128 rows through the whole step: the activations and layer gradients stay
+// in two 64 KB shared-memory tiles (core-matrix layout of the fused inference kernel), the
+// accumulators in tensor memory, and only the CTA's partial parameter gradients (FP32, one
+// value per parameter) go to global memory; k_train_reduce adds the CTAs' partials in a
+// fixed order.  Products per CTA (M 128, K 16 per instruction, BF16 in, FP32 accumulate):
+//   h2 = relu(h1 W2^T), h3 = relu(h2 W3^T)          weights K-major from the streaming image
+//   d2 = (d3 W3) [h2 > 0], d1 = (d2 W2) [h1 > 0]    the same image read MN-major: a K chunk
+//                                                   (32 outputs) is 32 pieces of 512 bytes
+//   dW3 = d3^T h2, dW2 = d2^T h1                    both operands MN-major from the tiles
+// The weight gradients are 256 x 256: two halves of 128 output features, one in the
+// accumulator columns of the layers (0 .. 255), one in columns 256 .. 511.
+// Warps 0-7 (thread = tensor-memory lane of quadrant warp & 3, columns 128 (warp >> 2) ..)
+// run the epilogues, warp 8 streams weights through a ring of F_TSLOTS chunks, warp 9
+// issues the MMAs.  h1 is formed twice (3 FMAs a value) because three tiles would leave the
+// ring too small.  The loss head sums a row's 256 terms in column order in one chain, as
+// the inference GEMM's epilogue does.
+// What bounds it: 8192 rows are 64 CTAs of the 152 SMs, each a serial chain of 4 layer
+// products (1 us each at the tensor rate) with their epilogues; the floor at the measured
+// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 46 us against 1249 us
+// for one GEMM launch per product, whose two weight gradients ran on two CTAs over K = 8192
+// (500 us) and whose column sums ran on 8 and 1 CTAs (520 us).
+constexpr int F_TSLOTS = 5;
+constexpr int F_TRING = F_TSLOTS * FW_BYTES;
+constexpr int TNBAR = 2 * F_TSLOTS + 3;   // full, empty, act, acc0, acc1
+constexpr int T_SMEM = 2 * FA_BYTES + F_TRING + FP_BYTES + 128 * 16 + 3 * 128 * 4 + 8 * TNBAR + 32;
+constexpr uint32_t IDESC_BT = IDESC | (1u << 16);                  // B MN-major
+constexpr uint32_t IDESC_ABT = IDESC | (1u << 15) | (1u << 16);    // A and B MN-major
+// one CTA's partials: dW2 and dW3 as float4 [i / 4][o] (stored by lanes that own o), then the
+// other gradients at their parameter offsets less the matrices, b4, the loss
+constexpr int TP_DW2 = 0, TP_DW3 = 65536, TP_W1 = 131072, TP_B1 = TP_W1 + 768, TP_B2 = TP_B1 + 256,
+              TP_B3 = TP_B2 + 256, TP_W4 = TP_B3 + 256, TP_B4 = TP_W4 + 256, TP_LOSS = TP_B4 + 1,
+              TP_N = TP_B4 + 4;
+
+__device__ inline void bar_epi() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+// sums over the 128 rows of the tile's 256 columns (each row times wr[row], or 1): warp w
+// takes K groups 4 w .. 4 w + 3, lane = (K group & 3) * 8 + row % 8 (conflict-free 16-byte
+// reads), 16 rows per lane, then the 8 lanes of a K group
+template <bool kW>
+__device__ inline void tile_colsum(const unsigned char *A, int warp, int lane, const float *wr,
+                                   float *out)
+{
+    const int kg = warp * 4 + (lane >> 3), r8 = lane & 7;
+    float s[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] = 0.f;
+#pragma unroll 4
+    for (int rg = 0; rg < 16; ++rg) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(A + a_off(rg * 8 + r8, kg));
+        const float f = kW ? wr[rg * 8 + r8] : 1.f;
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float lo = __uint_as_float(w[j] << 16), hi = __uint_as_float(w[j] & 0xffff0000u);
+            s[2 * j] = kW ? fmaf(lo, f, s[2 * j]) : s[2 * j] + lo;
+            s[2 * j + 1] = kW ? fmaf(hi, f, s[2 * j + 1]) : s[2 * j + 1] + hi;
+        }
+    }
+    float v = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
+        if (r8 == j) v = s[j];
+    }
+    out[kg * 8 + r8] = v;
+}
+
+__global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const float *__restrict__ x,
+                                                            const float *__restrict__ target,
+                                                            const float *__restrict__ P,
+                                                            const bf16 *__restrict__ Wimg,
+                                                            float *__restrict__ part)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *A0 = sm, *A1 = sm + FA_BYTES, *ring = sm + 2 * FA_BYTES;
+    float *sP = reinterpret_cast<float *>(ring + F_TRING);
+    float4 *sx = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sP) + FP_BYTES);
+    float *sdot = reinterpret_cast<float *>(sx + 128), *sdz = sdot + 128, *ssq = sdz + 128;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(ssq + 128);
+    uint64_t *full = bar, *empty = bar + F_TSLOTS, *act = bar + 2 * F_TSLOTS, *acc = act + 1;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + TNBAR);
+    volatile int *sfail = reinterpret_cast<int *>(tslot + 1);
+    volatile int *sprod = sfail + 1, *scons = sfail + 2;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int row0 = blockIdx.x * 128;
+    float *pt = part + (size_t)blockIdx.x * TP_N;
+
+    if (tid == 0) {
+        for (int k = 0; k < F_TSLOTS; ++k) {
+            mbar_init_n(&full[k], 1);
+            mbar_init_n(&empty[k], 1);
+        }
+        mbar_init_n(act, 256);
+        mbar_init_n(&acc[0], 1);
+        mbar_init_n(&acc[1], 1);
+        *sfail = 0;
+        *sprod = 0;
+        *scons = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         su32(tslot)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    griddep_wait();   // the parameters and their image are the previous step's
+    if (tid < 256) stage_params(sP, P, tid);
+    if (tid < 128) {
+        const size_t r = (size_t)(row0 + tid) * 3;
+        sx[tid] = make_float4(x[r], x[r + 1], x[r + 2], 0.f);
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const uint32_t tmem = *tslot;
+    bool ok = true;
+
+    constexpr int Q = 4 * FNC;   // chunks: W2, W3 (forward), W3, W2 (backward)
+    if (warp == 8) {
+        // ---------------- producer warp ----------------
+        int q = 0;
+        for (; q < Q; ++q) {
+            const int slot = q % F_TSLOTS, job = q / FNC, c = q % FNC;
+            // a warp-uniform outcome (the lanes time out each for itself)
+            if (!__all_sync(0xffffffffu, q < F_TSLOTS ||
+                                             mbar_wait(&empty[slot], ((q - F_TSLOTS) / F_TSLOTS) & 1))) {
+                *sfail = 1;
+                break;
+            }
+            const bf16 *img = Wimg + (job == 1 || job == 2 ? 65536 : 0);
+            unsigned char *dst = ring + slot * FW_BYTES;
+            if (lane == 0) mbar_expect(&full[slot], FW_BYTES);
+            __syncwarp();
+            if (job < 2) {
+                if (lane == 0) bulk_copy(dst, img + c * (FW_BYTES / 2), FW_BYTES, &full[slot]);
+            } else {   // inputs 8 lane .. 8 lane + 7 of outputs 32 c .. 32 c + 31
+                bulk_copy(dst + lane * 512, img + lane * 2048 + c * 256, 512, &full[slot]);
+            }
+        }
+        if (lane == 0) *sprod = q;
+    } else if (warp == 9) {
+        // ---------------- MMA thread ----------------
+        if (lane == 0) {
+            int q = 0;
+            unsigned pact = 0;
+            const uint32_t a0 = su32(A0), a1 = su32(A1);
+            auto wait_act = [&]() {
+                if (ok && !mbar_wait(act, pact)) ok = false;
+                pact ^= 1u;
+                tc_after();
+            };
+            // one layer product into columns 0 .. 255: A = a tile (K-major), B = 8 chunks
+            auto layer = [&](uint32_t a, bool back) {
+                for (int c = 0; c < FNC && ok; ++c, ++q) {
+                    const int slot = q % F_TSLOTS;
+                    if (!mbar_wait(&full[slot], (q / F_TSLOTS) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t w = su32(ring + slot * FW_BYTES);
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk) {
+                        const uint64_t ad = sdesc(a + (c * 4 + kk * 2) * 128, LBO, FA_SBO);
+                        if (back)   // outputs (K) 8 apart at 128 bytes, inputs (N) at 512
+                            umma<IDESC_BT>(tmem, ad, sdesc(w + kk * 256, 128, 512), (c | kk) != 0);
+                        else
+                            umma(tmem, ad, sdesc(w + kk * 2 * FW_LBO, FW_LBO, FW_SBO), (c | kk) != 0);
+                    }
+                    umma_commit(&empty[slot]);
+                }
+                if (ok) umma_commit(&acc[0]);
+            };
+            // half hf (output features 128 hf ..) of d^T h over the tile's 128 rows
+            auto wgrad = [&](uint32_t d, uint32_t h, int hf, uint32_t col, uint64_t *done) {
+                if (!ok) return;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)   // rows 16 kk ..: row groups 4096 bytes apart
+                    umma<IDESC_ABT>(tmem + col, sdesc(d + hf * 2048 + kk * 8192, FA_SBO, 128),
+                                    sdesc(h + kk * 8192, FA_SBO, 128), kk != 0);
+                umma_commit(done);
+            };
+            wait_act();             // h1 in A0
+            layer(a0, false);
+            wait_act();             // h2 in A1
+            layer(a1, false);
+            wait_act();             // d3 in A0
+            wgrad(a0, a1, 1, 0, &acc[0]);
+            wgrad(a0, a1, 0, 256, &acc[1]);
+            wait_act();             // columns 0 .. 255 read
+            layer(a0, true);
+            wait_act();             // d2 in A0, h1 in A1, every column read
+            layer(a0, true);
+            wgrad(a0, a1, 0, 256, &acc[1]);
+            wait_act();             // columns 0 .. 255 read
+            wgrad(a0, a1, 1, 0, &acc[0]);
+            if (!ok) *sfail = 1;
+            *scons = q;
+        }
+    } else {
+        // ---------------- epilogue warps ----------------
+        const int qd = warp & 3, hf = warp >> 2;
+        const int r = qd * 32 + lane;       // the tile row, or the output feature of a gradient
+        const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16);
+        unsigned p0 = 0, p1 = 0;
+        auto wait_acc = [&](int k, unsigned &ph) {
+            if (ok && !mbar_wait(&acc[k], ph)) {
+                ok = false;
+                *sfail = 1;
+            }
+            ph ^= 1u;
+            __syncwarp();
+            tc_after();
+        };
+        auto hand_off = [&]() {
+            tc_before();
+            fence_async_smem();
+            mbar_arrive(act);
+        };
+        auto load32 = [&](uint32_t col, uint32_t (&v)[32]) {
+            tmem_ld32_issue(tb + col, v);
+            tmem_wait_tied(v);
+        };
+        // this thread's 128 columns of feature 128 half + r of a weight gradient
+        auto drain = [&](int tp, int half, uint32_t col) {
+            float4 *o = reinterpret_cast<float4 *>(pt + tp) + half * 128 + r;
+#pragma unroll 1
+            for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
+                uint32_t v[32];
+                load32(col + ch * 32, v);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    o[(size_t)(ch * 8 + j) * 256] =
+                        make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                    __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+            }
+        };
+        const float4 X = sx[r];
+        layer1_row<true>(sP, X.x, X.y, X.z, A0, r, 16 * hf, 16 * hf + 16);
+        hand_off();
+        // ---- h2 = relu(acc + b2) ----
+        wait_acc(0, p0);
+#pragma unroll 1
+        for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
+            uint32_t v[32];
+            load32(ch * 32, v);
+#pragma unroll
+            for (int qq = 0; qq < 4; ++qq) {
+                uint4 u;
+                uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 b = *reinterpret_cast<const float2 *>(sP + FP_B2 + ch * 32 + qq * 8 + 2 * j);
+                    const float2 a = add2(make_float2(__uint_as_float(v[qq * 8 + 2 * j]),
+                                                      __uint_as_float(v[qq * 8 + 2 * j + 1])), b);
+                    hw[j] = relu_bf16x2(make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f)));
+                }
+                *reinterpret_cast<uint4 *>(A1 + a_off(r, ch * 4 + qq)) = u;
+            }
+        }
+        hand_off();
+        // ---- h3 = relu(acc + b3) into A0, the head in column order: the first half's
+        // threads take columns 0 .. 127, the second half's go on from their sums ----
+        wait_acc(0, p0);
+        float dot = 0.f;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+            for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
+                if (pass == 1 && hf == 0) break;
+                uint32_t v[32];
+                load32(ch * 32, v);
+                float a[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    a[j] = fmaxf(__uint_as_float(v[j]) + sP[FP_B3 + ch * 32 + j], 0.f);
+                if (pass == 0) {
+#pragma unroll
+                    for (int qq = 0; qq < 4; ++qq) {
+                        uint4 u;
+                        uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            hw[j] = relu_bf16x2(make_float2(a[qq * 8 + 2 * j], a[qq * 8 + 2 * j + 1]));
+                        *reinterpret_cast<uint4 *>(A0 + a_off(r, ch * 4 + qq)) = u;
+                    }
+                }
+                if (pass == hf) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) dot = fmaf(a[j], sP[FP_W4 + ch * 32 + j], dot);
+                }
+            }
+            if (pass == 0) {
+                if (hf == 0) sdot[r] = dot;
+                bar_epi();
+                if (hf == 1) dot = sdot[r];
+            }
+        }
+        if (hf == 1) {
+            const float scale = 2.f / rows;
+            const float z = dot + sP[FP_B4];
+            const float y = 1.f / (1.f + __expf(-z));
+            const float d = y - target[row0 + r];
+            sdz[r] = scale * d * y * (1.f - y);
+            ssq[r] = 0.5f * scale * d * d;
+        }
+        bar_epi();
+        tile_colsum<true>(A0, warp, lane, sdz, pt + TP_W4);   // dw4 = sum dz h3
+        if (warp == 0) {
+            float s = (sdz[lane] + sdz[lane + 32]) + (sdz[lane + 64] + sdz[lane + 96]);
+            float t = (ssq[lane] + ssq[lane + 32]) + (ssq[lane + 64] + ssq[lane + 96]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, o);
+                t += __shfl_xor_sync(0xffffffffu, t, o);
+            }
+            if (lane == 0) {
+                pt[TP_B4] = s;
+                pt[TP_LOSS] = t;
+            }
+        }
+        bar_epi();
+        // ---- d3 = dz w4 [h3 > 0] over h3 ----
+        {
+            const float dz = sdz[r];
+#pragma unroll 4
+            for (int k8 = 16 * hf; k8 < 16 * hf + 16; ++k8) {
+                uint4 *p = reinterpret_cast<uint4 *>(A0 + a_off(r, k8));
+                uint4 u = *p;
+                uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {   // h3 >= 0: positive where not zero
+                    const float2 w = *reinterpret_cast<const float2 *>(sP + FP_W4 + k8 * 8 + 2 * j);
+                    const __nv_bfloat162 g = __floats2bfloat162_rn((hw[j] & 0x7fffu) ? dz * w.x : 0.f,
+                                                                   (hw[j] & 0x7fff0000u) ? dz * w.y : 0.f);
+                    hw[j] = *reinterpret_cast<const uint32_t *>(&g);
+                }
+                *p = u;
+            }
+        }
+        hand_off();
+        bar_epi();
+        tile_colsum<false>(A0, warp, lane, nullptr, pt + TP_B3);
+        // ---- dW3 ----
+        wait_acc(0, p0);
+        drain(TP_DW3, 1, 0);
+        hand_off();
+        wait_acc(1, p1);
+        drain(TP_DW3, 0, 256);
+        // ---- d2 = acc [h2 > 0] over d3, h1 again over h2 ----
+        wait_acc(0, p0);
+#pragma unroll 1
+        for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
+            uint32_t v[32];
+            load32(ch * 32, v);
+#pragma unroll
+            for (int qq = 0; qq < 4; ++qq) {
+                const uint4 m = *reinterpret_cast<const uint4 *>(A1 + a_off(r, ch * 4 + qq));
+                const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
+                uint4 u;
+                uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const __nv_bfloat162 g = __floats2bfloat162_rn(
+                        (mw[j] & 0x7fffu) ? __uint_as_float(v[qq * 8 + 2 * j]) : 0.f,
+                        (mw[j] & 0x7fff0000u) ? __uint_as_float(v[qq * 8 + 2 * j + 1]) : 0.f);
+                    hw[j] = *reinterpret_cast<const uint32_t *>(&g);
+                }
+                *reinterpret_cast<uint4 *>(A0 + a_off(r, ch * 4 + qq)) = u;
+            }
+        }
+        layer1_row<true>(sP, X.x, X.y, X.z, A1, r, 16 * hf, 16 * hf + 16);
+        hand_off();
+        bar_epi();
+        tile_colsum<false>(A0, warp, lane, nullptr, pt + TP_B2);
+        // ---- d1 = acc [h1 > 0] (FP32): its column sums, plain (b1) and times x (W1).  The
+        // ring is free (the last layer product has read it): a warp stages 32 rows x 32
+        // columns, lane = column sums its 32 rows, then the four row quadrants meet ----
+        wait_acc(0, p0);
+        float *stage = reinterpret_cast<float *>(ring) + warp * (32 * 33);
+        float *quad = reinterpret_cast<float *>(ring) + 8 * 32 * 33;   // [4 sums][4 quadrants][256]
+#pragma unroll 1
+        for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
+            uint32_t v[32];
+            load32(ch * 32, v);
+#pragma unroll
+            for (int qq = 0; qq < 4; ++qq) {
+                const uint4 m = *reinterpret_cast<const uint4 *>(A1 + a_off(r, ch * 4 + qq));
+                const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    stage[lane * 33 + qq * 8 + 2 * j] =
+                        (mw[j] & 0x7fffu) ? __uint_as_float(v[qq * 8 + 2 * j]) : 0.f;
+                    stage[lane * 33 + qq * 8 + 2 * j + 1] =
+                        (mw[j] & 0x7fff0000u) ? __uint_as_float(v[qq * 8 + 2 * j + 1]) : 0.f;
+                }
+            }
+            __syncwarp();
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 8
+            for (int k = 0; k < 32; ++k) {
+                const float dv = stage[k * 33 + lane];
+                const float4 xr = sx[qd * 32 + k];
+                s0 += dv;
+                s1 = fmaf(dv, xr.x, s1);
+                s2 = fmaf(dv, xr.y, s2);
+                s3 = fmaf(dv, xr.z, s3);
+            }
+            const int c = ch * 32 + lane;
+            quad[(0 * 4 + qd) * 256 + c] = s0;
+            quad[(1 * 4 + qd) * 256 + c] = s1;
+            quad[(2 * 4 + qd) * 256 + c] = s2;
+            quad[(3 * 4 + qd) * 256 + c] = s3;
+            __syncwarp();
+        }
+        hand_off();
+        bar_epi();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float *qs = quad + k * 1024 + tid;
+            const float s = (qs[0] + qs[256]) + (qs[512] + qs[768]);
+            if (k == 0) pt[TP_B1 + tid] = s;
+            else pt[TP_W1 + 3 * tid + k - 1] = s;
+        }
+        // ---- dW2 ----
+        wait_acc(1, p1);
+        drain(TP_DW2, 0, 256);
+        wait_acc(0, p0);
+        drain(TP_DW2, 1, 0);
+    }
+    tc_before();
+    __syncthreads();
+    if (*sfail && tid == 0) {
+        atomicExch(&g_mlp_err, TRT_ETIMEOUT);
+        for (int q = *scons; q < *sprod; ++q)   // the copies in flight land (bounded)
+            mbar_wait(&full[q % F_TSLOTS], (q / F_TSLOTS) & 1);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        tc_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    }
+}
+
+// grad and loss from the CTAs' partials: 64 float4 positions x 4 slices per block, slice s
+// adds CTAs s, s + 4, ..., then the slices in order (fixed order, deterministic)
+__global__ void __launch_bounds__(256) k_train_reduce(int nt, const float *__restrict__ part,
+                                                      float *__restrict__ grad,
+                                                      float *__restrict__ loss)
+{
+    __shared__ float4 red[4][64];
+    griddep_wait();
+    const int l = threadIdx.x & 63, sl = threadIdx.x >> 6;
+    const int p = blockIdx.x * 64 + l;   // float4 index
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p < TP_N / 4) {
+        const float4 *src = reinterpret_cast<const float4 *>(part) + p;
+#pragma unroll 8
+        for (int t = sl; t < nt; t += 4) {
+            const float4 v = __ldcg(src + (size_t)t * (TP_N / 4));
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    }
+    red[sl][l] = s;
+    __syncthreads();
+    if (sl != 0 || p >= TP_N / 4) return;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+        const float4 v = red[k][l];
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+    if (p < TP_W1 / 4) {   // a matrix: float4 i4 of output o
+        const int m = p >> 14, i4 = (p >> 8) & 63, o = p & 255;
+        float *g = grad + (m ? TRT_MLP_W3 : TRT_MLP_W2) + o * 256 + i4 * 4;
+        g[0] = s.x;
+        g[1] = s.y;
+        g[2] = s.z;
+        g[3] = s.w;
+        return;
+    }
+    const float v[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int k = 4 * p + j;
+        if (k < TP_B2) grad[TRT_MLP_W1 + k - TP_W1] = v[j];              // W1, then b1
+        else if (k < TP_B3) grad[TRT_MLP_B2 + k - TP_B2] = v[j];
+        else if (k < TP_LOSS) grad[TRT_MLP_B3 + k - TP_B3] = v[j];       // b3, w4, b4
+        else if (k == TP_LOSS) *loss = v[j];
+    }
+}
+
 int g_num_sms = 0;
 
 cudaError_t mlp_fused(int rows, const float *x, const float *P, const bf16 *W, float *y,
@@ -754,9 +1243,9 @@ cudaError_t gemm(int M, int N, int K, const bf16 *A, const bf16 *B, const Epi &e
 
 // ---- MLP pieces on CUDA cores ----
 
-// h1 = relu(W1 x + b1) per row (FP32), stored BF16 row-major and optionally transposed
+// h1 = relu(W1 x + b1) per row (FP32), stored BF16 row-major
 __global__ void k_layer1(int R, const float *__restrict__ x, const float *__restrict__ P,
-                         bf16 *__restrict__ h1, bf16 *__restrict__ h1T, int ldT)
+                         bf16 *__restrict__ h1)
 {
     __shared__ float w[TRT_MLP_HIDDEN * 4];
     for (int i = threadIdx.x; i < TRT_MLP_HIDDEN; i += blockDim.x) {
@@ -781,62 +1270,15 @@ __global__ void k_layer1(int R, const float *__restrict__ x, const float *__rest
             a = fmaf(w[4 * c + 1], x1, a);
             a = fmaf(w[4 * c + 2], x2, a);
             hb[j] = __float2bfloat16_rn(fmaxf(a, 0.f));
-            if (h1T) h1T[(size_t)c * ldT + r] = hb[j];
         }
         o[q] = u;
     }
 }
 
-// out[c] = sum_r a[r][c] * (wr ? wr[r * ws + wo] : 1), c < ncol; a is BF16 or FP32 with row
-// stride lda; fixed summation order: 8 row slices per column, then the slices in order
-template <typename T>
-__global__ void k_colsum(int R, int ncol, const T *__restrict__ a, int lda,
-                         const float *__restrict__ wr, int ws, int wo, float *__restrict__ out)
-{
-    __shared__ float part[8][33];
-    const int cl = threadIdx.x & 31, sl = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + cl;
-    float s = 0.f;
-    if (c < ncol)
-        for (int r = sl; r < R; r += 8) {
-            const float v = (float)a[(size_t)r * lda + c];
-            s = fmaf(v, wr ? wr[(size_t)r * ws + wo] : 1.f, s);
-        }
-    part[sl][cl] = s;
-    __syncthreads();
-    if (sl == 0 && c < ncol) {
-        float t = 0.f;
-        for (int k = 0; k < 8; ++k) t += part[k][cl];
-        out[c] = t;
-    }
-}
-
-// dW1[c][k] = sum_r d1[r][c] x[r][k]: one column sum per (c, k), written at stride 3
-__global__ void k_dw1(int R, const float *__restrict__ d1, const float *__restrict__ x,
-                      float *__restrict__ g)
-{
-    __shared__ float part[8][33];
-    const int cl = threadIdx.x & 31, sl = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + cl, k = blockIdx.y;
-    float s = 0.f;
-    for (int r = sl; r < R; r += 8) s = fmaf(d1[(size_t)r * TRT_MLP_HIDDEN + c], x[3 * r + k], s);
-    part[sl][cl] = s;
-    __syncthreads();
-    if (sl == 0) {
-        float t = 0.f;
-        for (int q = 0; q < 8; ++q) t += part[q][cl];
-        g[TRT_MLP_W1 + 3 * c + k] = t;
-    }
-}
-
 // W2, W3 (BF16), their transposes and their streaming images (the 16 KB chunks of the
 // fused kernel, each laid out as it lands in shared memory) from the FP32 parameters
-__global__ void k_refresh(const float *__restrict__ P, bf16 *__restrict__ w16)
+__device__ inline void store_w16(bf16 *w16, int layer, int o, int i, float v)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;   // 2 x 65536
-    if (idx >= 2 * 65536) return;
-    const int layer = idx >> 16, o = (idx >> 8) & 255, i = idx & 255;
-    const float v = P[(layer ? TRT_MLP_W3 : TRT_MLP_W2) + o * 256 + i];
     const bf16 b = __float2bfloat16_rn(v);
     w16[layer * 65536 + o * 256 + i] = b;                 // W [out][in]
     w16[(2 + layer) * 65536 + i * 256 + o] = b;           // W^T [in][out]
@@ -844,10 +1286,21 @@ __global__ void k_refresh(const float *__restrict__ P, bf16 *__restrict__ w16)
     w16[(4 + layer) * 65536 + c * 8192 + kg * 2048 + o * 8 + j] = b;
 }
 
+__global__ void k_refresh(const float *__restrict__ P, bf16 *__restrict__ w16)
+{
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;   // 2 x 65536
+    if (idx >= 2 * 65536) return;
+    const int layer = idx >> 16, o = (idx >> 8) & 255, i = idx & 255;
+    store_w16(w16, layer, o, i, P[(layer ? TRT_MLP_W3 : TRT_MLP_W2) + o * 256 + i]);
+}
+
+// one Adam step, and the BF16 copies of the matrix elements it updated (k_refresh's, saving
+// its launch and its read of the parameters)
 __global__ void k_adam(int n, float *__restrict__ P, const float *__restrict__ g,
                        float *__restrict__ m, float *__restrict__ v, float lr, float b1,
-                       float b2, float eps, float c1, float c2)
+                       float b2, float eps, float c1, float c2, bf16 *__restrict__ w16)
 {
+    griddep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -855,7 +1308,11 @@ __global__ void k_adam(int n, float *__restrict__ P, const float *__restrict__ g
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float p = P[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    P[i] = p;
+    const int layer = i >= TRT_MLP_W3 ? 1 : 0;
+    const int e = i - (layer ? TRT_MLP_W3 : TRT_MLP_W2);
+    if (e >= 0 && e < 65536) store_w16(w16, layer, e >> 8, e & 255, p);
 }
 
 __global__ void k_features(int nx, int G, const double *__restrict__ T,
@@ -876,8 +1333,8 @@ __global__ void k_features(int nx, int G, const double *__restrict__ T,
 inline size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct Scratch {
-    bf16 *h1, *h1T, *h2, *h2T, *h3, *d3, *d3T, *d2, *d2T;
-    float *d1, *dz, *sq;
+    bf16 *h1, *h2;   // inference
+    float *part;     // training: the CTAs' partial gradients
     size_t bytes;
 };
 
@@ -886,21 +1343,12 @@ Scratch carve_scratch(void *base, int R, int training)
     Scratch s{};
     char *p = reinterpret_cast<char *>(base);
     size_t o = 0;
-    const size_t hb = al256((size_t)R * TRT_MLP_HIDDEN * sizeof(bf16));
-    auto take = [&](size_t n) { char *q = p ? p + o : nullptr; o += n; return q; };
-    s.h1 = reinterpret_cast<bf16 *>(take(hb));
-    s.h2 = reinterpret_cast<bf16 *>(take(hb));
+    auto take = [&](size_t n) { char *q = p ? p + o : nullptr; o += al256(n); return q; };
     if (training) {
-        s.h1T = reinterpret_cast<bf16 *>(take(hb));
-        s.h2T = reinterpret_cast<bf16 *>(take(hb));
-        s.h3 = reinterpret_cast<bf16 *>(take(hb));
-        s.d3 = reinterpret_cast<bf16 *>(take(hb));
-        s.d3T = reinterpret_cast<bf16 *>(take(hb));
-        s.d2 = reinterpret_cast<bf16 *>(take(hb));
-        s.d2T = reinterpret_cast<bf16 *>(take(hb));
-        s.d1 = reinterpret_cast<float *>(take(al256((size_t)R * TRT_MLP_HIDDEN * sizeof(float))));
-        s.dz = reinterpret_cast<float *>(take(al256((size_t)R * sizeof(float))));
-        s.sq = reinterpret_cast<float *>(take(al256((size_t)R * sizeof(float))));
+        s.part = reinterpret_cast<float *>(take((size_t)((R + 127) / 128) * TP_N * sizeof(float)));
+    } else {
+        s.h1 = reinterpret_cast<bf16 *>(take((size_t)R * TRT_MLP_HIDDEN * sizeof(bf16)));
+        s.h2 = reinterpret_cast<bf16 *>(take((size_t)R * TRT_MLP_HIDDEN * sizeof(bf16)));
     }
     s.bytes = o;
     return s;
@@ -969,7 +1417,7 @@ int trt_mlp_forward(int rows, const float *x, const float *params, const void *w
     if (scratch_bytes < s.bytes || !al16(scratch)) return TRT_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const bf16 *W = reinterpret_cast<const bf16 *>(w16);
-    k_layer1<<<(rows + 127) / 128, 128, 0, st>>>(rows, x, params, s.h1, nullptr, 0);
+    k_layer1<<<(rows + 127) / 128, 128, 0, st>>>(rows, x, params, s.h1);
     if (cudaGetLastError() != cudaSuccess) return TRT_ECUDA;
     Epi e2{};
     e2.bias = params + TRT_MLP_B2;
@@ -996,63 +1444,16 @@ int trt_mlp_grad(int rows, const float *x, const float *target, const float *par
     Scratch s = carve_scratch(scratch, rows, 1);
     if (scratch_bytes < s.bytes || !al16(scratch)) return TRT_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const bf16 *W = reinterpret_cast<const bf16 *>(w16);
-    const bf16 *W2 = W, *W3 = W + 65536, *W2T = W + 2 * 65536, *W3T = W + 3 * 65536;
-#define CKL(x)                                            \
-    do {                                                  \
-        if ((x) != cudaSuccess) return TRT_ECUDA;         \
-    } while (0)
-    k_layer1<<<(rows + 127) / 128, 128, 0, st>>>(rows, x, params, s.h1, s.h1T, rows);
-    CKL(cudaGetLastError());
-    Epi e2{};
-    e2.bias = params + TRT_MLP_B2;
-    e2.relu = 1;
-    e2.out16 = s.h2;
-    e2.out16T = s.h2T;
-    e2.ldT = rows;
-    CKL(gemm(rows, 256, 256, s.h1, W2, e2, st));
-    Epi e3{};
-    e3.bias = params + TRT_MLP_B3;
-    e3.relu = 1;
-    e3.out16 = s.h3;
-    e3.head_w = params + TRT_MLP_W4;
-    e3.head_b = params + TRT_MLP_B4;
-    e3.target = target;
-    e3.scale = 2.f / rows;
-    e3.dz = s.dz;
-    e3.sq = s.sq;
-    e3.dact16 = s.d3;
-    e3.dact16T = s.d3T;
-    e3.ldT = rows;
-    CKL(gemm(rows, 256, 256, s.h2, W3, e3, st));
-    // d2 = (d3 W3) [h2 > 0];  dW3 = d3^T h2
-    Epi eb{};
-    eb.mask = s.h2;
-    eb.out16 = s.d2;
-    eb.out16T = s.d2T;
-    eb.ldT = rows;
-    CKL(gemm(rows, 256, 256, s.d3, W3T, eb, st));
-    Epi ew{};
-    ew.out32 = grad + TRT_MLP_W3;
-    CKL(gemm(256, 256, rows, s.d3T, s.h2T, ew, st));
-    // d1 = (d2 W2) [h1 > 0];  dW2 = d2^T h1
-    Epi e1{};
-    e1.mask = s.h1;
-    e1.out32 = s.d1;
-    CKL(gemm(rows, 256, 256, s.d2, W2T, e1, st));
-    Epi ew2{};
-    ew2.out32 = grad + TRT_MLP_W2;
-    CKL(gemm(256, 256, rows, s.d2T, s.h1T, ew2, st));
-    // biases, W1, w4, b4, loss: fixed-order column sums over the rows
-    k_colsum<bf16><<<8, 256, 0, st>>>(rows, 256, s.d3, 256, nullptr, 0, 0, grad + TRT_MLP_B3);
-    k_colsum<bf16><<<8, 256, 0, st>>>(rows, 256, s.d2, 256, nullptr, 0, 0, grad + TRT_MLP_B2);
-    k_colsum<float><<<8, 256, 0, st>>>(rows, 256, s.d1, 256, nullptr, 0, 0, grad + TRT_MLP_B1);
-    k_colsum<bf16><<<8, 256, 0, st>>>(rows, 256, s.h3, 256, s.dz, 1, 0, grad + TRT_MLP_W4);
-    k_colsum<float><<<1, 256, 0, st>>>(rows, 1, s.dz, 1, nullptr, 0, 0, grad + TRT_MLP_B4);
-    k_colsum<float><<<1, 256, 0, st>>>(rows, 1, s.sq, 1, nullptr, 0, 0, loss);
-    k_dw1<<<dim3(8, 3), 256, 0, st>>>(rows, s.d1, x, grad);
-    CKL(cudaGetLastError());
-#undef CKL
+    const bf16 *img = reinterpret_cast<const bf16 *>(w16) + 4 * 65536;
+    if (!al16(w16)) return TRT_EINVAL;
+    const int nt = rows / 128;
+    if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, T_SMEM) !=
+            cudaSuccess ||
+        launch_pdl(k_mlp_train, dim3(nt), dim3(F_THREADS), T_SMEM, st, rows, x, target, params, img,
+                   s.part) != cudaSuccess ||
+        launch_pdl(k_train_reduce, dim3((TP_N / 4 + 63) / 64), dim3(256), 0, st, nt,
+                   (const float *)s.part, grad, loss) != cudaSuccess)
+        return TRT_ECUDA;
     return TRT_OK;
 }
 
@@ -1062,10 +1463,11 @@ int trt_mlp_adam(float *params, const float *grad, float *m, float *v, int t, fl
     if (!params || !grad || !m || !v || t < 1 || !w16) return TRT_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const float c1 = 1.f - powf(beta1, (float)t), c2 = 1.f - powf(beta2, (float)t);
-    k_adam<<<(TRT_MLP_NPARAM + 255) / 256, 256, 0, st>>>(TRT_MLP_NPARAM, params, grad, m, v, lr,
-                                                         beta1, beta2, eps, c1, c2);
-    if (cudaGetLastError() != cudaSuccess) return TRT_ECUDA;
-    return trt_mlp_refresh(params, w16, stream);
+    return launch_pdl(k_adam, dim3((TRT_MLP_NPARAM + 255) / 256), dim3(256), 0, st, TRT_MLP_NPARAM,
+                      params, grad, m, v, lr, beta1, beta2, eps, c1, c2,
+                      reinterpret_cast<bf16 *>(w16)) == cudaSuccess
+               ? TRT_OK
+               : TRT_ECUDA;
 }
 
 int trt_mlp_features(int nx, int G, const double *T, const double *sigE, const double *Eg,

@@ -127,6 +127,32 @@ def test_mlp_gradient_vs_oracle(env):
     assert mlp.MLP.status() == 0
 
 
+@pytest.mark.parametrize("rows", [128, 384, 19584])
+def test_mlp_gradient_row_tiles(env, rows):
+    """One 128-row tile, a few, and one more tile than the GPU has SMs: every block of the
+    gradient against the oracle with BF16 rounding at the same points.  The bound is the
+    element bound of test_mlp_gradient_vs_oracle, 5e-4 of the block's largest gradient,
+    doubled for the longer FP32 sums (up to 19584 terms)."""
+    torch, mlp = env
+    r = np.random.default_rng(rows)
+    p = OM.init_params(70) + OM.pack({"b1": r.normal(0, 0.1, 256), "b2": r.normal(0, 0.1, 256),
+                                      "b3": r.normal(0, 0.1, 256), "b4": -0.1})
+    p32 = p.astype(np.float32).astype(np.float64)
+    x = r.normal(0, 1, (rows, 3)).astype(np.float32)
+    t = r.uniform(0.3, 1.0, rows).astype(np.float32)
+    net = mlp.MLP(p32)
+    g, L = net.grad(x, t)
+    g = g.cpu().numpy().astype(np.float64)
+    gr, Lr = OM.grad(p32, x.astype(np.float64), t.astype(np.float64), "bf16")
+    assert L.item() == pytest.approx(Lr, rel=1e-3)
+    for name, n in (("W1", 768), ("b1", 256), ("W2", 65536), ("b2", 256), ("W3", 65536),
+                    ("b3", 256), ("w4", 256), ("b4", 1)):
+        o = OM.OFF[name]
+        a, b = g[o:o + n], gr[o:o + n]
+        assert np.max(np.abs(a - b)) <= 1e-3 * np.abs(b).max(), name
+    assert mlp.MLP.status() == 0
+
+
 def test_adam_step_vs_oracle(env):
     torch, mlp = env
     r = np.random.default_rng(41)
