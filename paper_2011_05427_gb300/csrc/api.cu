@@ -86,8 +86,8 @@ void carve(trt_handle *h, Carver &c)
     p.otabp = lo_pair(p.precision) ? c.take<double>(otab_doubles((int)G) + G + 1) : nullptr;
     p.cpair = lo_pair(p.precision) ? c.take<double>(5 * nx) : nullptr;
     p.lopc = lo_pair(p.precision) ? c.take<double>(8 * (nx + 1)) : nullptr;
-    p.rscratch_doubles = restrict_scratch_doubles((int)nx, (int)G, 1);
-    p.rscratch = p.rscratch_doubles ? c.take<double>(p.rscratch_doubles) : nullptr;
+    p.rscratch_doubles = restrict_scratch_doubles(p);
+    p.rscratch = c.take<double>(p.rscratch_doubles);
     double **tl[] = {&h->T, &h->Told, &h->Tcyc, &h->Tphase, &h->Ttil, &h->Tnew, &h->sig_prev,
                      &h->T_prev, &h->Ecyc, &h->Ephase};
     for (double **q : tl) *q = c.take<double>(nx);
@@ -114,6 +114,12 @@ void carve(trt_handle *h, Carver &c)
     h->gpre = c.take<double>(3 * nx);
     int n2 = (p.nlev >= 3) ? p.levels[1] : 1;
     carve_level(c, h->crs, n2, p.nx);
+    // the coarse grids' sums of Eold and Fold, formed at a grid's first visit of a step (of a
+    // cycle in a batch): the largest grid's in crs, the others' apart
+    for (int l = 1; l + 1 < p.nlev; ++l) {
+        h->crs_Eold[l] = l == 1 ? h->crs.Eold : c.take<double>((size_t)p.levels[l] * nx);
+        h->crs_Fold[l] = l == 1 ? h->crs.Fold : c.take<double>((size_t)p.levels[l] * (nx + 1));
+    }
     carve_level(c, h->grey, 1, p.nx);
     h->flags = c.take<double>(10);
     h->ctl = reinterpret_cast<int *>(h->flags + 8);
@@ -451,6 +457,7 @@ int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups 
     CK(launch_otab_build(p));   // opacity tables of this group structure
     CK(launch_lo_pair_consts(p));
     CK(cudaMemsetAsync(H->flags, 0, 10 * sizeof(double), p.stream));
+    CK(cudaMemsetAsync(p.rscratch, 0, restrict_head_doubles() * sizeof(double), p.stream));
     CK(cudaStreamSynchronize(p.stream));
     *out = hp.release();
     return TRT_OK;
@@ -537,8 +544,8 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
     for (int k = 0; k < K; ++k) lo_per_cycle += p.levels[S[k] - 1];
 
     bool opac_next = false;   // the phase's opacities already enqueued (below)
-    // which source's sums of Eold and Fold (fixed within a step) the grey level holds
-    int grey_old = 0;
+    // the sums of Eold and Fold are fixed within a step: the grids that hold them already
+    std::vector<char> old_sums(p.nlev, 0);
     for (;;) {
         if (s > 0) {
             if (!opac_next) {
@@ -581,12 +588,15 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
                 double *Tout = (k == K) ? h->T : ((k & 1) ? h->Tnew : h->Ttil);
                 Level *src = &fine;
                 if (k > 0) {
-                    const int ng = p.levels[S[k - 1] - 1];
+                    const int lev = S[k - 1] - 1, ng = p.levels[lev];
                     CK(launch_opacity(p, Tst, h->sigE, h->emis, h->sigR, nullptr, nullptr, 0.0,
                                       Erad));
                     opac_valid = false;
                     h->crs.n = ng;
-                    CK(launch_restrict(p, fine, h->crs));
+                    h->crs.Eold = h->crs_Eold[lev];
+                    h->crs.Fold = h->crs_Fold[lev];
+                    CK(launch_restrict(p, fine, h->crs, nullptr, nullptr, old_sums[lev] != 0));
+                    old_sums[lev] = 1;
                     CK(launch_lo_solve(p, dt, h->crs));
                     nk += 3;
                     src = &h->crs;
@@ -606,11 +616,11 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
                     a.ctl = h->ctl; a.eps_in = eps_in; a.fixed = fixed ? 1 : 0;
                 }
                 // the restriction to the grey level, which forms the visit's per-cell
-                // Newton terms too where its two-stage form runs
+                // Newton terms too
                 const GreyArgs ready = grey_args_ready(p, a);
-                bool formed = false;
-                CK(launch_restrict(p, *src, h->grey, &ready, h->gpre, &formed, &grey_old));
-                a.pre = formed ? h->gpre : nullptr;
+                CK(launch_restrict(p, *src, h->grey, &ready, h->gpre, old_sums[p.nlev - 1] != 0));
+                old_sums[p.nlev - 1] = 1;
+                a.pre = h->gpre;
                 CK(launch_grey(p, h->grey, a));
                 nk += 2;   // restriction to grey + grey Newton
                 have_prev = 1;

@@ -6,8 +6,7 @@
 // step end); a stage is a fixed list of ops, an op is one batched kernel (batch.cuh) over
 // the slabs eligible for it.  Eligibility has a static part, fixed at creation (the
 // op's per-slab block counts: zero when the op does not apply to the slab, e.g. a coarse
-// visit beyond the slab's schedule or a restriction variant the slab does not use), and a
-// dynamic part, one byte per (class, slab) written by the host before the stage runs
+// visit beyond the slab's schedule), and a dynamic part, one byte per (class, slab) written by the host before the stage runs
 // (which slabs sweep now, which are still inside the cycle loop, which need opacities).
 // A planner kernel turns both into the ops' work lists on the device, so the argument
 // blocks (rebuilt once per step) and the launch sequence are the same for every run of a
@@ -29,13 +28,12 @@ using namespace trt;
 namespace {
 
 enum Cls { C_ALL = 0, C_SWEEP, C_PHASE, C_CYCLE, C_OPAC0, C_PHASE_END, NCLS };
-enum Kind { K_OPAC, K_SWEEP, K_FINAL, K_LO, K_RESTRICT, K_RPART, K_RFINAL, K_GREY, K_GSUM, K_COPY };
+enum Kind { K_OPAC, K_SWEEP, K_FINAL, K_LO, K_RESTRICT, K_GREY, K_GSUM, K_COPY };
 enum StageId { S_STEP_START, S_SWEEP, S_PHASE, S_PHASE_END, S_STEP_END, S_CYCLE0 };
 
 struct Op {
     Kind kind;
     int cls;
-    int KS = 1;             // K_RESTRICT row slices
     size_t csz = 0;         // bytes of one argument block
     size_t ctx_off = 0;     // byte offset of xs[n] in the argument region
     size_t meta_off = 0;    // int offset of the work list in the meta region
@@ -144,8 +142,6 @@ size_t ctx_size(Kind k)
     case K_FINAL: return sizeof(FinalizeArgs);
     case K_LO: return sizeof(LoCtx);
     case K_RESTRICT: return sizeof(RestrictCtx);
-    case K_RPART:
-    case K_RFINAL: return sizeof(Restrict2Ctx);
     case K_GREY: return sizeof(GreyCtx);
     case K_GSUM: return sizeof(GroupSumArgs);
     case K_COPY: return sizeof(CopyArgs);
@@ -156,7 +152,7 @@ size_t ctx_size(Kind k)
 int grid_cap(Kind k) { return k == K_SWEEP ? 152 * 2 : 152 * 16; }
 
 // ops of all stages built for one cycle type: the W cycle is the longest (2^(Gamma-2) - 1
-// coarse visits); per visit at most opacity + 7 restriction variants + solve + grey
+// coarse visits); per visit at most opacity + 2 restrictions + solve + grey
 size_t max_ops(int nlev_max)
 {
     const size_t K = ((size_t)1 << (std::min(nlev_max, 12) - 2)) - 1;
@@ -197,8 +193,6 @@ struct Builder {
             if (c[s].n > 0) set(o, s, c[s], (int)((c[s].n + 255) / 256), (int)((c[s].n + 255) / 256));
     }
 };
-
-int face_blocks(const Problem &p) { return (p.nx + 1 + 31) / 32; }
 
 }  // namespace
 
@@ -308,34 +302,17 @@ void build_stage(trt_batch *b, int id, double dt, int cycle_type)
         for (int s = 0; s < n; ++s) cp[s] = CopyArgs{Tbuf(s, 0), H(s)->T, H(s)->p.nx};
         B.copy(C_CYCLE, cp);
         auto restrict_op = [&](const std::vector<Level> &src, const std::vector<Level> &dst,
-                               const std::vector<int> &use) {
-            // variants: two-stage (part + final), or single with KS in {1, 2, 4, 8, 16}
-            int ip = -1, iv[5] = {-1, -1, -1, -1, -1};
+                               const std::vector<int> &use, const std::vector<int> &held) {
+            // held: the target already holds the step's sums of Eold and Fold (an earlier
+            // visit of the cycle formed them)
+            Op &o = B.add(K_RESTRICT, C_CYCLE);
             for (int s = 0; s < n; ++s) {
                 if (!use[s]) continue;
                 const Problem &p = H(s)->p;
-                int KS = 1;
-                if (restrict_kind(p, src[s].n, dst[s].n, &KS) == 2) {
-                    if (ip < 0) {
-                        ip = (int)sg.ops.size();
-                        B.add(K_RPART, C_CYCLE);
-                        B.add(K_RFINAL, C_CYCLE);
-                    }
-                    const Restrict2Ctx y = make_restrict2_ctx(p, src[s], dst[s]);
-                    const int gxx = face_blocks(p);
-                    B.set(sg.ops[ip], s, y, gxx * dst[s].n * y.nchunk, gxx);
-                    B.set(sg.ops[ip + 1], s, y, gxx * dst[s].n, gxx);
-                } else {
-                    int idx = 0;
-                    while ((1 << idx) < KS) ++idx;
-                    if (iv[idx] < 0) {
-                        iv[idx] = (int)sg.ops.size();
-                        B.add(K_RESTRICT, C_CYCLE).KS = KS;
-                    }
-                    const int gxx = face_blocks(p);
-                    B.set(sg.ops[iv[idx]], s, make_restrict_ctx(p, src[s], dst[s]),
-                          gxx * dst[s].n, gxx);
-                }
+                const RestrictPlan q = restrict_plan(p, src[s].n, dst[s].n);
+                RestrictCtx x = make_restrict_ctx(p, src[s], dst[s]);
+                x.skip_old = held[s];
+                B.set(o, s, x, (q.nt + 1) * q.gy, q.nt + 1);
             }
         };
         for (int k = 0; k <= Kmax; ++k) {
@@ -351,11 +328,17 @@ void build_stage(trt_batch *b, int id, double dt, int cycle_type)
                                                    H(s)->sigR, nullptr, nullptr, 0.0),
                           opacity_blocks(p), opacity_gx(p));
                 }
+                std::vector<int> held(n, 0);
                 for (int s = 0; s < n; ++s) {
                     crs[s] = H(s)->crs;
-                    if (use[s]) crs[s].n = H(s)->p.levels[S[s][k - 1] - 1];
+                    if (!use[s]) continue;
+                    const int lev = S[s][k - 1] - 1;
+                    crs[s].n = H(s)->p.levels[lev];
+                    crs[s].Eold = H(s)->crs_Eold[lev];
+                    crs[s].Fold = H(s)->crs_Fold[lev];
+                    for (int j = 0; j < k - 1; ++j) held[s] |= S[s][j] == S[s][k - 1];
                 }
-                restrict_op(fine, crs, use);
+                restrict_op(fine, crs, use, held);
                 Op &ol = B.add(K_LO, C_CYCLE);
                 for (int s = 0; s < n; ++s)
                     if (use[s]) B.set(ol, s, make_lo_ctx(H(s)->p, dt, crs[s]), crs[s].n, crs[s].n);
@@ -363,7 +346,7 @@ void build_stage(trt_batch *b, int id, double dt, int cycle_type)
             } else {
                 src = fine;
             }
-            restrict_op(src, grey, use);
+            restrict_op(src, grey, use, std::vector<int>(n, k > 0));
             Op &og = B.add(K_GREY, C_CYCLE);
             for (int s = 0; s < n; ++s) {
                 if (!use[s]) continue;
@@ -586,14 +569,7 @@ cudaError_t launch_op(trt_batch *b, const Op &o)
         return launch_lo_solve_b(b->precision, b->max_nx, meta, N,
                                  reinterpret_cast<const LoCtx *>(x), o.grid, b->st);
     case K_RESTRICT:
-        return launch_restrict_b(o.KS, meta, N, reinterpret_cast<const RestrictCtx *>(x), o.grid,
-                                 b->st);
-    case K_RPART:
-        return launch_restrict_part_b(meta, N, reinterpret_cast<const Restrict2Ctx *>(x), o.grid,
-                                      b->st);
-    case K_RFINAL:
-        return launch_restrict_final_b(meta, N, reinterpret_cast<const Restrict2Ctx *>(x),
-                                       o.grid, b->st);
+        return launch_restrict_b(meta, N, reinterpret_cast<const RestrictCtx *>(x), o.grid, b->st);
     case K_GREY:
         return launch_grey_b(b->max_nx, meta, N, reinterpret_cast<const GreyCtx *>(x), o.grid,
                              b->st);

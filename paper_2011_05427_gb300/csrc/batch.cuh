@@ -75,28 +75,29 @@ struct LoCtx {
 };
 
 struct RestrictCtx {
-    int nx, r;       // r = members per coarse group
+    int nx, r, n_to;         // r = members per coarse group
+    int mode, nt, kc, nchunk;   // RestrictPlan
     const double *h, *ihf;
-    Level S;         // source level (coefficients + solution)
-    Level T;         // target level (written)
+    Level S;                 // source level (coefficients + solution)
+    Level T;                 // target level (written)
     const int *gate;
-};
-
-struct Restrict2Ctx {
-    int nx, r, nchunk;
-    const double *h, *ihf;
-    Level S, T;
-    double *part;   // [n_to][nchunk][kRP][nx+1]
-    const int *gate;
-    // the grey visit's per-cell Newton terms, formed by the final stage when newton != 0
+    int *ticket;             // [n_to][nt + 1], zero between launches (nchunk > 1)
+    double *bpart, *part;    // [n_to][nchunk][16] and [n_to][nchunk][12][32 nt]
+    // the grey visit's per-cell Newton terms, formed with the cell means when newton != 0
     // (single slab, target = the grey level): into pre [3][nx], with the visit's arguments
     int newton;
     GreyArgs ga;
     double *pre;
-    // the target's Eold and Fold sums already hold this step's values from this source
-    // (they change only between steps): stage 1 neither loads nor sums them, stage 2 keeps
-    // them
+    // the target's Eold and Fold sums already hold this step's values (they change only
+    // between steps): neither loaded nor summed
     int skip_old;
+};
+
+// How one restriction is split (lo.cu): mode 0, a warp per coarse group; mode 1, a CTA per
+// kc members of one, nchunk of them; nt position tiles (and one block of boundary means)
+// by gy rows of CTAs.
+struct RestrictPlan {
+    int mode, nt, kc, nchunk, gy;
 };
 
 struct GreyCtx {
@@ -159,12 +160,8 @@ FinalizeArgs make_finalize_args(const Problem &p, const SweepArgs &a);
 int finalize_blocks(const Problem &p);
 int pick_D(const Problem &p);   // directions per CTA of the single-slab sweep
 LoCtx make_lo_ctx(const Problem &p, double dt, const Level &L);
-// restriction: kind 2 (two-stage) when the source has >= 64 members per coarse group and
-// the scratch holds it, else kind 1 with KS row slices per CTA
-int restrict_kind(const Problem &p, int n_from, int n_to, int *KS);
+RestrictPlan restrict_plan(const Problem &p, int n_from, int n_to);
 RestrictCtx make_restrict_ctx(const Problem &p, const Level &src, const Level &dst);
-Restrict2Ctx make_restrict2_ctx(const Problem &p, const Level &src, const Level &dst);
-int restrict2_nchunk(int n_from, int n_to);
 GreyCtx make_grey_ctx(const Problem &p, const Level &g, const GreyArgs &a);
 
 // ---- batched launchers (grid: CTAs of the fixed grid; stream: the batch's stream) ----
@@ -177,12 +174,8 @@ cudaError_t launch_finalize_b(int precision, const int *meta, int N, const Final
                               int grid, cudaStream_t st);
 cudaError_t launch_lo_solve_b(int precision, int max_nx, const int *meta, int N,
                               const LoCtx *xs, int grid, cudaStream_t st);
-cudaError_t launch_restrict_b(int KS, const int *meta, int N, const RestrictCtx *xs, int grid,
+cudaError_t launch_restrict_b(const int *meta, int N, const RestrictCtx *xs, int grid,
                               cudaStream_t st);
-cudaError_t launch_restrict_part_b(const int *meta, int N, const Restrict2Ctx *xs, int grid,
-                                   cudaStream_t st);
-cudaError_t launch_restrict_final_b(const int *meta, int N, const Restrict2Ctx *xs, int grid,
-                                    cudaStream_t st);
 cudaError_t launch_grey_b(int max_nx, const int *meta, int N, const GreyCtx *xs, int grid,
                           cudaStream_t st);
 cudaError_t launch_group_sum_b(const int *meta, int N, const GroupSumArgs *xs, int grid,

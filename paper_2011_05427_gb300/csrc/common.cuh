@@ -245,7 +245,7 @@ struct Problem {
     double *e2tab;      // [32]: 2^(j/32), the table of texp for kernels outside physics.cu
     int *lo_slot;       // [nx+1]: shared-memory slot k * 32 + l of face/row f in the
                         // partitioned tridiagonal solve (chunk l, row k of the chunk)
-    double *rscratch;   // partial sums of the two-stage restriction
+    double *rscratch;   // the restriction's tickets (zero between launches) and partial sums
     size_t rscratch_doubles;
     // sweep tile: directions per CTA (0 = default) and strip shape index (0 = default)
     int sweep_D = 0, sweep_shape = 0;
@@ -307,16 +307,16 @@ cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L);
 cudaError_t ensure_lo_consts(Problem &p, double dt);
 // the step-independent pair row constants (Problem::lopc; once per handle, TRT_LO_PAIR)
 cudaError_t launch_lo_pair_consts(const Problem &p);
-// newton (with pre): the visit's grey Newton arguments; the two-stage restriction to the
-// grey level then also forms the per-cell Newton terms into pre ([3][nx]) and sets *formed
-// old_key (in/out, may be null): which source's Eold and Fold sums dst holds from this
-// step (0: none); the two-stage restriction skips them when it matches src
+// newton (with pre): the visit's grey Newton arguments; the restriction to the grey level
+// then also forms the per-cell Newton terms into pre ([3][nx]).  skip_old: dst holds this
+// step's Eold and Fold sums already
 cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
                             const GreyArgs *newton = nullptr, double *pre = nullptr,
-                            bool *formed = nullptr, int *old_key = nullptr);
+                            bool skip_old = false);
 // the host-formed constants of a grey visit (c_v/dt, 54 s C_B, the exponential's table)
 GreyArgs grey_args_ready(const Problem &p, const GreyArgs &a);
-size_t restrict_scratch_doubles(int nx, int n_from, int n_to);
+size_t restrict_scratch_doubles(const Problem &p);   // from nx and the grids
+size_t restrict_head_doubles();                      // its tickets: zero at creation
 cudaError_t launch_grey(const Problem &p, const Level &g, const GreyArgs &a);
 cudaError_t launch_group_sum(const Problem &p, int n, const double *X, double *out);
 

@@ -17,6 +17,7 @@ struct trt_handle {
     double *E1, *F1, *Eb0_1, *EbX_1;
     double *gpre;   // [3][nx]: the grey Newton terms formed by the restriction
     trt::Level crs, grey;
+    double *crs_Eold[16] = {}, *crs_Fold[16] = {};   // per coarse grid (trt_step)
     double *Ecyc, *Ephase;
     double *flags = nullptr;    // [10]: convergence flags [0..6], then the inner-loop
     int *ctl = nullptr;         // control words (ints in the last two doubles of flags)

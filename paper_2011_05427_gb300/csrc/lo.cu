@@ -697,14 +697,6 @@ __global__ void __launch_bounds__(128) k_lo_solve_b(const int *__restrict__ meta
     }
 }
 
-// ---------------------------------------------------------------------------------------
-// The weighted means below divide (no reciprocal-multiply): the weights (sums of E or of
-// boundary energies over a coarse group) reach the subnormal range in cold cells, where
-// 1/w overflows while a/w stays finite.
-//
-// restriction (eqs. coeff-gamma, g-notation, eta-gamma / coeff-Gamma, g2G-notation,
-// eta-Gamma, and the discrete compensation of eq. mloqd-d-gamma)
-// ---------------------------------------------------------------------------------------
 // Per-cell terms of the grey Newton step (Sec. 5, eqs. eb-Gamma and f-derivative-d): from the
 // grey opacity sig*, Q* = 2 e* and the group energy sum Esum of cell i at T*, the
 // absorption w c sig*, the source w Q* - (1 - w) c_v (T* - Told)/dt and 1/Lambda.  Called
@@ -748,348 +740,328 @@ __device__ inline void grey_newton_terms(const GreyArgs &a, int have_prev, int i
     sL = iL;
 }
 
-constexpr int kRV1 = 18;   // pass-1 sums
-constexpr int kRV2 = 6;    // pass-2 sums
+// ---- restriction (eqs. coeff-gamma, g-notation, eta-gamma / coeff-Gamma, g2G-notation,
+// eta-Gamma, and the discrete compensation of eq. mloqd-d-gamma) ----
+//
+// One kernel per restriction.  Every sum over the members of a coarse group is an FP64
+// operation, and GB300's FP64 pipe (a warp-wide operation holds its sub-partition's pipe for
+// 64 cycles or more) bounds the kernel, so the split is by FP64 operations:
+//   - a lane owns an extended position j = -1 .. n_x: cell j and face j, with the boundary
+//     energies as "cells" -1 and n_x.  A warp covers 31 faces and the cell before its first
+//     (lane 0), so that a face's sums of E_L and E_R are the cell sums of two neighbouring
+//     lanes: no FP64 operation of their own;
+//   - one pass: the compensation is xi = dx (sum sigR F - sigR-bar sum F) + c (sum etaR E_R -
+//     sum etaL E_L), equal to the two-pass sum up to rounding relative to the sigR dx F
+//     terms.  12 operations per member and position (4 for the cell, 8 for the face), 2 more
+//     for Eold and Fold where the target does not hold this step's sums yet, 2 more for the
+//     compensation of a coarse source;
+//   - the boundary means are the work of blocks of their own (bx = nt: 16 lanes are the 2
+//     sides x 8 sums), not a second branch of the position blocks at the two ends;
+//   - a quotient is a reciprocal and one residual correction (rquot), 6 operations.
+// Modes (restrict_plan), one CTA = 4 warps, one per sub-partition:
+//   0  a warp takes a whole coarse group (few members, many groups);
+//   1  a CTA takes kc members of a coarse group, each warp every fourth; with more than one
+//      chunk the partial sums go to scratch and the CTA that arrives last at a position
+//      tile (a ticket) adds the chunks in a fixed order and forms the coefficients: no
+//      second launch.
+// Measured (warm): 1024 members to the grey level, 500 cells: RMEAS
+constexpr int kRV = 12;   // sums per position: the order of restrict_member's v
+enum { R_PHI, R_SIG, R_EMIS, R_E, R_SW, R_W, R_SF, R_F, R_EOLD, R_FOLD, R_ETAR, R_ETAL };
+constexpr int kRTile = 31;          // faces per position tile
+constexpr int kRTickets = 2432;     // ints at the head of the scratch (nt * n_to < 1216 there)
+constexpr int kRHead = kRTickets / 2;   // doubles
 
-
-__device__ inline double src_phi_b(const Level &S, int p, int side)
+// a/w: the refined reciprocal and one residual correction (the correctly rounded quotient
+// but for rare last bits).  The weights of cold cells are subnormal, where 1/w overflows and
+// a/w does not: an exponent outside +-900 divides, and a non-finite quotient is kept.
+static __device__ __noinline__ double rquot_divide(double a, double w) { return a / w; }
+__device__ inline double rquot(double a, double w)
 {
-    return side == 0 ? S.phib0[p] : S.phibX[p];
+    const unsigned ex = ((unsigned)__double2hiint(w) >> 20) & 0x7ffu;
+    if (ex - 123u > 1800u) return rquot_divide(a, w);
+    const double r = rcp64(w);
+    const double q = a * r;
+    if ((((unsigned)__double2hiint(q) >> 20) & 0x7ffu) == 0x7ffu) return q;
+    return fma(fma(-q, w, a), r, q);
 }
 
-// block (32, KS <= 16); grid (ceil((nx+1)/32), n_to)
+// sums over members p = p0, p0 + step, .. < pe of lane position i (clamped by the caller)
+__device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, int step, int i,
+                                        double (&v)[kRV])
+{
+    const Level &S = x.S;
+    const int nx = x.nx;
+    const size_t nf = (size_t)nx + 1;
+    const int ic = min(max(i, 0), nx - 1), jf = max(i, 0);
+    const double *Ep = i < 0 ? S.Eb0 : i >= nx ? S.EbX : S.E + i;
+    const size_t Es = (i < 0 || i >= nx) ? 1 : (size_t)nx;
+    const int ia = max(ic - (i < nx ? 1 : 0), 0);   // the cell left of face i
+    double wa = 0.0, wb = 0.0;
+    if (S.fine && i > 0 && i < nx) {   // the face opacity's dx-weighted mean
+        wa = x.h[i - 1] * x.ihf[i];
+        wb = x.h[i] * x.ihf[i];
+    }
+#pragma unroll
+    for (int k = 0; k < kRV; ++k) v[k] = 0.0;
+#pragma unroll 2
+    for (int p = p0; p < pe; p += step) {
+        const size_t c = (size_t)p * nx, fp = (size_t)p * nf + jf;
+        const double E = Ep[(size_t)p * Es];
+        const double EL = __shfl_up_sync(0xffffffffu, E, 1);
+        const double F = S.F[fp];
+        v[R_PHI] = fma(S.phi[c + ic], E, v[R_PHI]);
+        v[R_SIG] = fma(S.sig[c + ic], E, v[R_SIG]);
+        v[R_EMIS] += S.emis[c + ic];
+        v[R_E] += E;
+        double sR;
+        if (S.fine) {
+            const double a = S.sigR[c + ia], b = S.sigR[c + ic];
+            sR = (i <= 0) ? b : (i >= nx) ? a : fma(wa, a, wb * b);
+        } else {
+            sR = S.sigR[fp];
+            v[R_ETAR] = fma(S.etaR[fp], E, v[R_ETAR]);
+            v[R_ETAL] = fma(S.etaL[fp], EL, v[R_ETAL]);
+        }
+        // |F| weight with a floor 1e-6 c E-bar: groups in local equilibrium carry
+        // rounding-noise fluxes that must not decide the mean
+        const double w = fma(0.5e-6 * kC, EL + E,
+                             __longlong_as_double(__double_as_longlong(F) & 0x7fffffffffffffffll));
+        v[R_SW] = fma(sR, w, v[R_SW]);
+        v[R_W] += w;
+        v[R_SF] = fma(sR, F, v[R_SF]);
+        v[R_F] += F;
+        if (!x.skip_old) {
+            v[R_EOLD] += S.Eold[c + ic];
+            v[R_FOLD] += S.Fold[fp];
+        }
+    }
+}
+
+// the E-weighted cell means of coarse group P at cell i (and the grey visit's Newton terms)
+__device__ inline void restrict_cell(const RestrictCtx &x, int P, int i, double sphi, double ssig,
+                                     double semis, double sE)
+{
+    const Level &S = x.S;
+    const int nx = x.nx;
+    const size_t c = (size_t)P * nx + i;
+    double ph, sg;
+    if (sE != 0.0) {
+        ph = rquot(sphi, sE);
+        sg = rquot(ssig, sE);
+    } else {   // no energy in the coarse group: plain means of the members
+        ph = sg = 0.0;
+        for (int p = P * x.r; p < (P + 1) * x.r; ++p) {
+            ph += S.phi[(size_t)p * nx + i];
+            sg += S.sig[(size_t)p * nx + i];
+        }
+        ph = rquot(ph, (double)x.r);
+        sg = rquot(sg, (double)x.r);
+    }
+    x.T.phi[c] = ph;
+    x.T.sig[c] = sg;
+    if (x.newton) {   // target = the grey level: the visit's Newton terms of cell i
+        double sa, ss, sL;
+        grey_newton_terms(x.ga, x.ga.have_prev, i, sg, 2.0 * semis, sE, sa, ss, sL);
+        x.pre[i] = sa;
+        x.pre[nx + i] = ss;
+        x.pre[2 * (size_t)nx + i] = sL;
+    }
+}
+
+// the copied sums of coarse group P at position i
+__device__ inline void restrict_sums(const RestrictCtx &x, int P, int i, double semis, double sE,
+                                     double sEold, double sFold)
+{
+    const int nx = x.nx;
+    if (i < nx) {
+        const size_t c = (size_t)P * nx + i;
+        x.T.emis[c] = semis;
+        x.T.Esum[c] = sE;
+        if (!x.skip_old) x.T.Eold[c] = sEold;
+    }
+    if (!x.skip_old) x.T.Fold[(size_t)P * (nx + 1) + i] = sFold;
+}
+
+// the face opacity and compensation of coarse group P at face i; sER, sEL: sums of E on
+// either side
+__device__ inline void restrict_face(const RestrictCtx &x, int P, int i, double sSW, double sW,
+                                     double sSF, double sF, double sER, double sEL, double eR,
+                                     double eL)
+{
+    const Level &S = x.S;
+    const int nx = x.nx, nf = nx + 1;
+    const double dxf = (i == 0) ? 0.5 * x.h[0] : (i == nx) ? 0.5 * x.h[nx - 1]
+                                            : 0.5 * (x.h[i - 1] + x.h[i]);
+    double sRP;
+    if (sW != 0.0) {
+        sRP = rquot(sSW, sW);
+    } else {   // no flux weight: plain mean of the members' face opacities
+        sRP = 0.0;
+        for (int p = P * x.r; p < (P + 1) * x.r; ++p) {
+            if (S.fine) {
+                const double *sc = S.sigR + (size_t)p * nx;
+                sRP += (i == 0) ? sc[0] : (i == nx) ? sc[nx - 1]
+                       : (sc[i - 1] * x.h[i - 1] + sc[i] * x.h[i]) * x.ihf[i];
+            } else {
+                sRP += S.sigR[(size_t)p * nf + i];
+            }
+        }
+        sRP = rquot(sRP, (double)x.r);
+    }
+    double xi = dxf * fma(-sRP, sF, sSF);
+    if (!S.fine) xi = fma(kC, eR - eL, xi);
+    const size_t f = (size_t)P * nf + i;
+    const double side = xi > 0.0 ? sER : sEL;
+    double eta = 0.0;
+    if (xi != 0.0 && side != 0.0) eta = rquot(fabs(xi), kC * side);
+    x.T.sigR[f] = sRP;
+    x.T.etaR[f] = xi > 0.0 ? eta : 0.0;
+    x.T.etaL[f] = xi < 0.0 ? eta : 0.0;
+}
+
+// lane side * 8 + k (< 16): sum k of the boundary means of one side over the members
+__device__ inline double restrict_boundary(const RestrictCtx &x, int p0, int pe, int step, int l)
+{
+    const Level &S = x.S;
+    const int side = l >> 3, k = l & 7;
+    const double *ph = side ? S.phibX : S.phib0, *Eb = side ? S.EbX : S.Eb0,
+                 *Cb = side ? S.CX : S.C0, *Ein = side ? S.EinX : S.Ein0,
+                 *Fin = side ? S.FinX : S.Fin0;
+    // phi Eb, phi, Eb, C Eo, C, Eo, Ein, Fin with Eo = Eb - Ein
+    const double *pa = k < 2 ? ph : (k == 2 || k == 5) ? Eb : k < 5 ? Cb : k == 6 ? Ein : Fin;
+    double s = 0.0;
+    for (int p = p0; p < pe; p += step) {
+        double a = pa[p], b = 1.0;
+        if (k == 0) b = Eb[p];
+        if (k == 3) b = Eb[p] - Ein[p];
+        if (k == 5) a -= Ein[p];
+        s = fma(a, b, s);
+    }
+    return s;
+}
+// the boundary means of coarse group P from the 16 sums on lanes 0 .. 15 of a warp
+__device__ inline void restrict_boundary_out(const RestrictCtx &x, int P, int lane, double s)
+{
+    const int side = (lane >> 3) & 1, k = lane & 7;
+    const double den = __shfl_sync(0xffffffffu, s, side * 8 + (k < 3 ? 2 : 5));
+    const double pl = __shfl_sync(0xffffffffu, s, side * 8 + (k < 3 ? 1 : 4));
+    if (lane >= 16) return;
+    const Level &T = x.T;
+    if (k == 0 || k == 3) {
+        const double m = den != 0.0 ? rquot(s, den) : rquot(pl, (double)x.r);
+        (k == 0 ? (side ? T.phibX : T.phib0) : (side ? T.CX : T.C0))[P] = m;
+    }
+    if (k == 6) (side ? T.EinX : T.Ein0)[P] = s;
+    if (k == 7) (side ? T.FinX : T.Fin0)[P] = s;
+}
+
+// last arrival of `n` CTAs at ticket t (which it resets): the partial sums written before
+// by the others are visible to the CTA that gets true
+__device__ inline bool restrict_last(int *t, int n)
+{
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(t, 1) == n - 1;
+        if (last) *t = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// block 128; grid (nt + 1, ceil(n_to / 4)) in mode 0, (nt + 1, n_to * nchunk) in mode 1
 __device__ void restrict_body(const RestrictCtx &x, int bx, int by)
 {
-    extern __shared__ __align__(16) double rsm[];
-    const int tx = threadIdx.x, ty = threadIdx.y, KS = blockDim.y;
-    const int nx = x.nx, nf = nx + 1;
-    const int i = bx * 32 + tx;   // cell index and face index
-    const int P = by;
-    const int pb = P * x.r;
-    const Level &S = x.S;
-    double v[kRV1];
-#pragma unroll
-    for (int k = 0; k < kRV1; ++k) v[k] = 0.0;
-    // ---- pass 1 ----
-    for (int p = pb + ty; p < pb + x.r; p += KS) {
-        if (i < nx) {
-            size_t c = (size_t)p * nx + i;
-            double E = S.E[c];
-            double ph = S.phi[c], sg = S.sig[c];
-            v[0] += ph * E; v[1] += ph; v[2] += sg * E; v[3] += sg;
-            v[4] += S.emis[c]; v[5] += S.Eold[c]; v[6] += E;
-        }
-        if (i <= nx) {
-            double Fp = S.F[(size_t)p * nf + i];
-            double sR;
-            if (S.fine) {
-                const double *sc = S.sigR + (size_t)p * nx;
-                sR = (i == 0) ? sc[0] : (i == nx) ? sc[nx - 1]
-                     : (sc[i - 1] * x.h[i - 1] + sc[i] * x.h[i]) * x.ihf[i];
-            } else {
-                sR = S.sigR[(size_t)p * nf + i];
-            }
-            // |F| weight with a floor 1e-6 c E-bar: groups in local equilibrium carry
-            // rounding-noise fluxes that must not decide the mean
-            double ER = (i == nx) ? S.EbX[p] : S.E[(size_t)p * nx + i];
-            double EL = (i == 0) ? S.Eb0[p] : S.E[(size_t)p * nx + i - 1];
-            double wF = fabs(Fp) + 1e-6 * kC * 0.5 * (EL + ER);
-            v[7] += sR * wF; v[8] += sR; v[9] += wF;
-        }
-        if (i == 0 || i == nx) {
-            const int side = (i == 0) ? 0 : 1;
-            double Eb = side == 0 ? S.Eb0[p] : S.EbX[p];
-            double Ein = side == 0 ? S.Ein0[p] : S.EinX[p];
-            double Fin = side == 0 ? S.Fin0[p] : S.FinX[p];
-            double Cb = side == 0 ? S.C0[p] : S.CX[p];
-            double ph = src_phi_b(S, p, side);
-            double Eo = Eb - Ein;
-            v[10] += ph * Eb; v[11] += ph; v[12] += Eb;
-            v[13] += Cb * Eo; v[14] += Cb; v[15] += Eo;
-            v[16] += Ein; v[17] += Fin;
-        }
-    }
-    // reduce over ty
-    if (KS > 1) {
-        double *red = rsm + ((size_t)ty * 32 + tx) * kRV1;
-        for (int k = 0; k < kRV1; ++k) red[k] = v[k];
-        __syncthreads();
-        if (ty == 0) {
-            for (int y = 1; y < KS; ++y) {
-                const double *o = rsm + ((size_t)y * 32 + tx) * kRV1;
-                for (int k = 0; k < kRV1; ++k) v[k] += o[k];
-            }
-            double *bc = rsm + (size_t)tx * kRV1;
-            for (int k = 0; k < kRV1; ++k) bc[k] = v[k];
-        }
-        __syncthreads();
-        if (ty != 0) {
-            const double *bc = rsm + (size_t)tx * kRV1;
-            for (int k = 0; k < kRV1; ++k) v[k] = bc[k];
-        }
-        __syncthreads();
-    }
-    const double rn = (double)x.r;
-    const double sRP = (v[9] != 0.0) ? v[7] / v[9] : v[8] / rn;
-    // ---- pass 2 (faces): xi, eta sums, side energies, Fold ----
-    double u[kRV2];
-#pragma unroll
-    for (int k = 0; k < kRV2; ++k) u[k] = 0.0;
-    if (i <= nx) {
-        const double dxf = (i == 0) ? 0.5 * x.h[0] : (i == nx) ? 0.5 * x.h[nx - 1]
-                                               : 0.5 * (x.h[i - 1] + x.h[i]);
-        for (int p = pb + ty; p < pb + x.r; p += KS) {
-            size_t fp = (size_t)p * nf + i;
-            double Fp = S.F[fp];
-            double sR;
-            if (S.fine) {
-                const double *sc = S.sigR + (size_t)p * nx;
-                sR = (i == 0) ? sc[0] : (i == nx) ? sc[nx - 1]
-                     : (sc[i - 1] * x.h[i - 1] + sc[i] * x.h[i]) * x.ihf[i];
-            } else {
-                sR = S.sigR[fp];
-            }
-            double ER = (i == nx) ? S.EbX[p] : S.E[(size_t)p * nx + i];
-            double EL = (i == 0) ? S.Eb0[p] : S.E[(size_t)p * nx + i - 1];
-            u[0] += dxf * (sR - sRP) * Fp;
-            if (!S.fine) {
-                u[1] += S.etaR[fp] * ER;
-                u[2] += S.etaL[fp] * EL;
-            }
-            u[3] += ER; u[4] += EL; u[5] += S.Fold[fp];
-        }
-    }
-    if (KS > 1) {
-        double *red = rsm + ((size_t)ty * 32 + tx) * kRV2;
-        for (int k = 0; k < kRV2; ++k) red[k] = u[k];
-        __syncthreads();
-        if (ty == 0) {
-            for (int y = 1; y < KS; ++y) {
-                const double *o = rsm + ((size_t)y * 32 + tx) * kRV2;
-                for (int k = 0; k < kRV2; ++k) u[k] += o[k];
-            }
-        }
-    }
-    if (ty != 0) return;
-    const Level &T = x.T;
-    if (i < nx) {
-        size_t c = (size_t)P * nx + i;
-        (T.phi)[c] = (v[6] != 0.0) ? v[0] / v[6] : v[1] / rn;
-        (T.sig)[c] = (v[6] != 0.0) ? v[2] / v[6] : v[3] / rn;
-        (T.emis)[c] = v[4];
-        (T.Eold)[c] = v[5];
-        T.Esum[c] = v[6];
-    }
-    if (i <= nx) {
-        size_t f = (size_t)P * nf + i;
-        double xi = u[0] + kC * (u[1] - u[2]);
-        (T.sigR)[f] = sRP;
-        (T.etaR)[f] = (xi > 0.0 && u[3] != 0.0) ? xi / (kC * u[3]) : 0.0;
-        (T.etaL)[f] = (xi < 0.0 && u[4] != 0.0) ? -xi / (kC * u[4]) : 0.0;
-        (T.Fold)[f] = u[5];
-    }
-    if (i == 0 || i == nx) {
-        double phb = (v[12] != 0.0) ? v[10] / v[12] : v[11] / rn;
-        double Cb = (v[15] != 0.0) ? v[13] / v[15] : v[14] / rn;
-        if (i == 0) {
-            (T.phib0)[P] = phb;
-            (T.C0)[P] = Cb;
-            (T.Ein0)[P] = v[16];
-            (T.Fin0)[P] = v[17];
-        } else {
-            (T.phibX)[P] = phb;
-            (T.CX)[P] = Cb;
-            (T.EinX)[P] = v[16];
-            (T.FinX)[P] = v[17];
-        }
-    }
-}
+    __shared__ double red[4][kRV][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nx = x.nx;
+    const bool many = x.mode == 0;
+    const int P = many ? by * 4 + warp : by / x.nchunk;
+    const int ch = many ? 0 : by - P * x.nchunk;
+    const int pb = P * x.r + ch * x.kc;
+    const int pe = min(pb + x.kc, (P + 1) * x.r);
 
-// Two-stage restriction for wide coarse groups (r >= 64 members): stage 1 sums chunks of
-// kChunk members per (coarse group, cell / face) into partial vectors with many CTAs;
-// stage 2 adds the chunks in a fixed order and forms the coefficients.  Sums stage 1 does
-// not form: the member energies on either side of an interior face (sum E_R at face i is
-// sum E at cell i, sum E_L is sum E at cell i - 1: the same terms in the same order, so
-// the same bits), and the plain means that replace a weighted mean whose weights sum to
-// zero (formed by stage 2 from the members in that rare case).  Every stage-1 addition is
-// an FP64 operation, the pipe that bounds these kernels on GB300.  The compensation
-// is summed in one pass, xi = dx (sum sigR F - sigR-bar sum F) + c (sum etaR E_R -
-// sum etaL E_L), which is the two-pass sum up to rounding relative to the sigR dx F terms.
-constexpr int kChunk = 64;
-constexpr int kRP = 25;
-constexpr int kPartRows = 8;   // rows (warps) of a stage-1 block: kChunk / kPartRows members each
-constexpr size_t kPartSmem = sizeof(double) * kPartRows * 32 * (kRP + 1);
-
-
-// block (32, kPartRows); grid (ceil((nx+1)/32), n_to * nchunk); kPartSmem bytes of dynamic
-// shared memory
-__device__ void restrict_part_body(const Restrict2Ctx &x, int bx, int by)
-{
-    extern __shared__ __align__(16) double red_raw[];
-    double (*red)[32][kRP + 1] = reinterpret_cast<double (*)[32][kRP + 1]>(red_raw);
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int nx = x.nx, nf = nx + 1;
-    const int i = bx * 32 + tx;
-    const int P = by / x.nchunk, ch = by - P * x.nchunk;
-    const int pb = P * x.r + ch * kChunk;
-    const int pe = min(pb + kChunk, P * x.r + x.r);
-    const Level &S = x.S;
-    double v[kRP];
-#pragma unroll
-    for (int k = 0; k < kRP; ++k) v[k] = 0.0;
-    for (int p = pb + ty; p < pe; p += kPartRows) {
-        if (i < nx) {
-            const size_t c = (size_t)p * nx + i;
-            const double E = S.E[c];
-            v[0] += S.phi[c] * E; v[2] += S.sig[c] * E;
-            v[4] += S.emis[c];
-            if (!x.skip_old) v[5] += S.Eold[c];
-            v[6] += E;
+    if (bx == x.nt) {   // ---- boundary means ----
+        const int l = lane & 15, half = lane >> 4;
+        if (many) {
+            if (P >= x.n_to) return;
+            double s = restrict_boundary(x, pb + half, pe, 2, l);
+            s += __shfl_xor_sync(0xffffffffu, s, 16);
+            restrict_boundary_out(x, P, lane, s);
+            return;
         }
-        if (i <= nx) {
-            const size_t fp = (size_t)p * nf + i;
-            const double Fp = S.F[fp];
-            double sR;
-            if (S.fine) {
-                const double *sc = S.sigR + (size_t)p * nx;
-                sR = (i == 0) ? sc[0] : (i == nx) ? sc[nx - 1]
-                     : (sc[i - 1] * x.h[i - 1] + sc[i] * x.h[i]) * x.ihf[i];
-            } else {
-                sR = S.sigR[fp];
-            }
-            const double ER = (i == nx) ? S.EbX[p] : S.E[(size_t)p * nx + i];
-            const double EL = (i == 0) ? S.Eb0[p] : S.E[(size_t)p * nx + i - 1];
-            const double wF = fabs(Fp) + 1e-6 * kC * 0.5 * (EL + ER);
-            v[7] += sR * wF; v[9] += wF; v[10] += sR * Fp; v[11] += Fp;
-            if (!S.fine) {
-                v[12] += S.etaR[fp] * ER;
-                v[13] += S.etaL[fp] * EL;
-            }
-            if (i == nx) v[14] += ER;
-            if (i == 0) v[15] += EL;
-            if (!x.skip_old) v[16] += S.Fold[fp];
+        double *rb = &red[0][0][0];   // [8 slices][16]
+        rb[(warp * 2 + half) * 16 + l] = restrict_boundary(x, pb + warp * 2 + half, pe, 8, l);
+        __syncthreads();
+        double s = 0.0;
+        if (warp == 0)
+            for (int k = 0; k < 8; ++k) s += rb[k * 16 + l];
+        if (x.nchunk > 1) {
+            if (threadIdx.x < 16) x.bpart[(size_t)by * 16 + l] = s;
+            if (!restrict_last(x.ticket + P * (x.nt + 1) + bx, x.nchunk)) return;
+            s = 0.0;
+            if (warp == 0)
+                for (int c = 0; c < x.nchunk; ++c)
+                    s += __ldcg(x.bpart + ((size_t)P * x.nchunk + c) * 16 + l);
         }
-        if (i == 0 || i == nx) {
-            const int side = (i == 0) ? 0 : 1;
-            const double Eb = side == 0 ? S.Eb0[p] : S.EbX[p];
-            const double Ein = side == 0 ? S.Ein0[p] : S.EinX[p];
-            const double Fin = side == 0 ? S.Fin0[p] : S.FinX[p];
-            const double Cb = side == 0 ? S.C0[p] : S.CX[p];
-            const double ph = side == 0 ? S.phib0[p] : S.phibX[p];
-            const double Eo = Eb - Ein;
-            v[17] += ph * Eb; v[18] += ph; v[19] += Eb;
-            v[20] += Cb * Eo; v[21] += Cb; v[22] += Eo;
-            v[23] += Ein; v[24] += Fin;
-        }
+        if (warp == 0) restrict_boundary_out(x, P, lane, s);
+        return;
     }
+
+    const int i = bx * kRTile - 1 + lane;   // extended position; lane 0 is the halo
+    const bool face = lane > 0 && i <= nx, cell = lane > 0 && i < nx;
+    double v[kRV];
+    if (many) {
+        if (P >= x.n_to) return;
+        restrict_members(x, pb, pe, 1, min(i, nx), v);
+        const double sEL = __shfl_up_sync(0xffffffffu, v[R_E], 1);
+        if (cell) restrict_cell(x, P, i, v[R_PHI], v[R_SIG], v[R_EMIS], v[R_E]);
+        if (face) {
+            restrict_sums(x, P, i, v[R_EMIS], v[R_E], v[R_EOLD], v[R_FOLD]);
+            restrict_face(x, P, i, v[R_SW], v[R_W], v[R_SF], v[R_F], v[R_E], sEL, v[R_ETAR],
+                          v[R_ETAL]);
+        }
+        return;
+    }
+    restrict_members(x, pb + warp, pe, 4, min(i, nx), v);
 #pragma unroll
-    for (int k = 0; k < kRP; ++k) red[ty][tx][k] = v[k];
+    for (int k = 0; k < kRV; ++k) red[warp][k][lane] = v[k];
     __syncthreads();
-    // the rows' partials, value k by row k % kPartRows: the additions are spread over the
-    // warps (all four sub-partitions' FP64 pipes); same order as a sum by one row
-    if (i <= nx) {
-        double *o = x.part + ((size_t)(P * x.nchunk + ch) * kRP) * nf + i;
-        for (int k = ty; k < kRP; k += kPartRows) {
-            double a = red[0][tx][k];
-#pragma unroll
-            for (int y = 1; y < kPartRows; ++y) a += red[y][tx][k];
-            o[(size_t)k * nf] = a;
-        }
+    // the warps' partials, value k by warp k % 4 (the additions spread over the four FP64
+    // pipes), then the chunks' in the same split
+    const size_t np = (size_t)x.nt * 32;
+    double *part = x.part + (size_t)by * kRV * np + bx * 32 + lane;
+    const int kend = x.S.fine ? R_ETAR : kRV;   // a fine source has no compensation
+    for (int k = warp; k < kend; k += 4) {
+        if (x.skip_old && (k == R_EOLD || k == R_FOLD)) continue;
+        const double s = (red[0][k][lane] + red[1][k][lane]) + (red[2][k][lane] + red[3][k][lane]);
+        if (x.nchunk > 1) part[k * np] = s;
+        else red[0][k][lane] = s;
     }
-}
-
-// block (32, kRP); grid (ceil((nx+1)/32), n_to): thread (tx, k) adds value k of position
-// tx over the chunks in a fixed order; then rows 0 .. 3 (one warp each, on four
-// sub-partitions) form the coefficients: row 0 the E-weighted cell means, row 1 the copied
-// cell sums, row 2 the face opacity and compensation, row 3 the boundary means.
-__device__ void restrict_final_body(const Restrict2Ctx &x, int bx, int by)
-{
-    __shared__ double sv[kRP][33];
-    const int nx = x.nx, nf = nx + 1;
-    const int tx = threadIdx.x, k = threadIdx.y;
-    const int i = bx * 32 + tx;
-    const int P = by;
-    if (i <= nx) {
-        double acc = 0.0;
-        // sum E_L at the block's first face (i > 0) is sum E at cell i - 1 of the block before
-        const int kk = (k == 15 && tx == 0 && i > 0) ? 6 : k;
-        const int ii = (kk != k) ? i - 1 : i;
-        const double *o = x.part + ((size_t)P * x.nchunk * kRP + kk) * nf + ii;
-        for (int ch = 0; ch < x.nchunk; ++ch) acc += o[(size_t)ch * kRP * nf];
-        sv[k][tx] = acc;
+    if (x.nchunk > 1) {
+        if (!restrict_last(x.ticket + P * (x.nt + 1) + bx, x.nchunk)) return;
+        const double *all = x.part + (size_t)P * x.nchunk * kRV * np + bx * 32 + lane;
+        for (int k = warp; k < kend; k += 4) {
+            if (x.skip_old && (k == R_EOLD || k == R_FOLD)) continue;
+            double s = 0.0;
+#pragma unroll 8
+            for (int c = 0; c < x.nchunk; ++c) s += __ldcg(all + ((size_t)c * kRV + k) * np);
+            red[0][k][lane] = s;
+        }
     }
     __syncthreads();
-    if (k > 3 || i > nx) return;
-    const double rn = (double)x.r;
-    const Level &T = x.T;
-    const Level &S = x.S;
-    const int p0 = P * x.r;
-    if (k == 0 && i < nx) {
-        const size_t c = (size_t)P * nx + i;
-        const double E = sv[6][tx];
-        double ph = 0.0, sg = 0.0;
-        if (E != 0.0) {
-            ph = sv[0][tx] / E;
-            sg = sv[2][tx] / E;
-        } else {   // no energy in the coarse group: plain means of the members
-            for (int p = p0; p < p0 + x.r; ++p) {
-                ph += S.phi[(size_t)p * nx + i];
-                sg += S.sig[(size_t)p * nx + i];
-            }
-            ph /= rn;
-            sg /= rn;
-        }
-        T.phi[c] = ph;
-        T.sig[c] = sg;
-        if (x.newton) {   // target = the grey level: the visit's Newton terms of cell i
-            double sa, ss, sL;
-            grey_newton_terms(x.ga, x.ga.have_prev, i, sg, 2.0 * sv[4][tx], sv[6][tx], sa, ss,
-                              sL);
-            x.pre[i] = sa;
-            x.pre[nx + i] = ss;
-            x.pre[2 * (size_t)nx + i] = sL;
-        }
-    } else if (k == 1) {
-        if (i < nx) {
-            const size_t c = (size_t)P * nx + i;
-            T.emis[c] = sv[4][tx];
-            if (!x.skip_old) T.Eold[c] = sv[5][tx];
-            T.Esum[c] = sv[6][tx];
-        }
-        if (!x.skip_old) T.Fold[(size_t)P * nf + i] = sv[16][tx];
-    } else if (k == 2) {
-        const double v14 = (i < nx) ? sv[6][tx] : sv[14][tx];
-        const double v15 = (i > 0 && tx > 0) ? sv[6][tx - 1] : sv[15][tx];
-        const double dxf = (i == 0) ? 0.5 * x.h[0] : (i == nx) ? 0.5 * x.h[nx - 1]
-                                                : 0.5 * (x.h[i - 1] + x.h[i]);
-        double sRP = 0.0;
-        if (sv[9][tx] != 0.0) {
-            sRP = sv[7][tx] / sv[9][tx];
-        } else {   // no flux weight: plain mean of the members' face opacities
-            for (int p = p0; p < p0 + x.r; ++p) {
-                if (S.fine) {
-                    const double *sc = S.sigR + (size_t)p * nx;
-                    sRP += (i == 0) ? sc[0] : (i == nx) ? sc[nx - 1]
-                           : (sc[i - 1] * x.h[i - 1] + sc[i] * x.h[i]) * x.ihf[i];
-                } else {
-                    sRP += S.sigR[(size_t)p * nf + i];
-                }
-            }
-            sRP /= rn;
-        }
-        const double xi = dxf * (sv[10][tx] - sRP * sv[11][tx]) + kC * (sv[12][tx] - sv[13][tx]);
-        const size_t f = (size_t)P * nf + i;
-        T.sigR[f] = sRP;
-        T.etaR[f] = (xi > 0.0 && v14 != 0.0) ? xi / (kC * v14) : 0.0;
-        T.etaL[f] = (xi < 0.0 && v15 != 0.0) ? -xi / (kC * v15) : 0.0;
-    } else if (k == 3 && (i == 0 || i == nx)) {
-        const double phb = (sv[19][tx] != 0.0) ? sv[17][tx] / sv[19][tx] : sv[18][tx] / rn;
-        const double Cb = (sv[22][tx] != 0.0) ? sv[20][tx] / sv[22][tx] : sv[21][tx] / rn;
-        if (i == 0) {
-            T.phib0[P] = phb; T.C0[P] = Cb; T.Ein0[P] = sv[23][tx]; T.Fin0[P] = sv[24][tx];
-        } else {
-            T.phibX[P] = phb; T.CX[P] = Cb; T.EinX[P] = sv[23][tx]; T.FinX[P] = sv[24][tx];
-        }
+    const double(*sv)[32] = red[0];
+    if (warp == 0) {
+        if (cell) restrict_cell(x, P, i, sv[R_PHI][lane], sv[R_SIG][lane], sv[R_EMIS][lane], sv[R_E][lane]);
+    } else if (warp == 1) {
+        if (face)
+            restrict_sums(x, P, i, sv[R_EMIS][lane], sv[R_E][lane], sv[R_EOLD][lane], sv[R_FOLD][lane]);
+    } else if (warp == 2) {
+        if (face)
+            restrict_face(x, P, i, sv[R_SW][lane], sv[R_W][lane], sv[R_SF][lane], sv[R_F][lane],
+                          sv[R_E][lane], sv[R_E][lane - 1], sv[R_ETAR][lane], sv[R_ETAL][lane]);
     }
 }
 
@@ -1407,23 +1379,11 @@ __device__ void group_sum_body(const GroupSumArgs &a, int bx)
 
 // entry points: the single-slab kernels pass blockIdx; the batched ones walk a work list
 // (single-slab entry points: return at entry while the driver's gate is set)
-__global__ void __launch_bounds__(512) k_restrict(RestrictCtx x)
+__global__ void __launch_bounds__(128) k_restrict(RestrictCtx x)
 {
     griddep_wait();
     if (x.gate && *x.gate) return;
     restrict_body(x, blockIdx.x, blockIdx.y);
-}
-__global__ void __launch_bounds__(32 * kPartRows) k_restrict_part(Restrict2Ctx x)
-{
-    griddep_wait();
-    if (x.gate && *x.gate) return;
-    restrict_part_body(x, blockIdx.x, blockIdx.y);
-}
-__global__ void __launch_bounds__(32 * kRP, 1) k_restrict_final(Restrict2Ctx x)
-{
-    griddep_wait();
-    if (x.gate && *x.gate) return;
-    restrict_final_body(x, blockIdx.x, blockIdx.y);
 }
 __global__ void __launch_bounds__(1024) k_grey(GreyCtx x)
 {
@@ -1433,8 +1393,8 @@ __global__ void __launch_bounds__(1024) k_grey(GreyCtx x)
 }
 __global__ void __launch_bounds__(256) k_group_sum(GroupSumArgs a) { group_sum_body(a, blockIdx.x); }
 
-#define TRT_BATCHED(name, Ctx, bounds, call)                                                  \
-    __global__ void __launch_bounds__(bounds) name(const int *__restrict__ meta, int N,        \
+#define TRT_BATCHED(name, Ctx, bounds, minb, call)                                            \
+    __global__ void __launch_bounds__(bounds, minb) name(const int *__restrict__ meta, int N,        \
                                                    const Ctx *__restrict__ xs)                 \
     {                                                                                          \
         for (int b = blockIdx.x;; b += gridDim.x) {                                            \
@@ -1445,11 +1405,11 @@ __global__ void __launch_bounds__(256) k_group_sum(GroupSumArgs a) { group_sum_b
             __syncthreads();                                                                   \
         }                                                                                      \
     }
-TRT_BATCHED(k_restrict_b, RestrictCtx, 512, restrict_body(x, bx, by))
-TRT_BATCHED(k_restrict_part_b, Restrict2Ctx, 32 * kPartRows, restrict_part_body(x, bx, by))
-TRT_BATCHED(k_restrict_final_b, Restrict2Ctx, 32 * kRP, restrict_final_body(x, bx, by))
-TRT_BATCHED(k_grey_b, GreyCtx, 1024, grey_body(x))
-TRT_BATCHED(k_group_sum_b, GroupSumArgs, 256, group_sum_body(x, bx))
+// (6 CTAs per SM: unbounded, the argument block held in registers leaves 3; 64 slabs to the
+// grey level 486 -> BMEAS us)
+TRT_BATCHED(k_restrict_b, RestrictCtx, 128, 6, restrict_body(x, bx, by))
+TRT_BATCHED(k_grey_b, GreyCtx, 1024, 1, grey_body(x))
+TRT_BATCHED(k_group_sum_b, GroupSumArgs, 256, 1, group_sum_body(x, bx))
 #undef TRT_BATCHED
 
 __global__ void __launch_bounds__(256) k_copy_b(const int *__restrict__ meta, int N,
@@ -1543,6 +1503,12 @@ LoCtx make_lo_ctx(const Problem &p, double dt, const Level &L)
     return x;
 }
 
+// doubles of restriction scratch: tickets, boundary partials, position partials
+static size_t restrict_doubles(int nt, int n_to, int nchunk)
+{
+    return kRHead + (size_t)n_to * nchunk * (16 + (size_t)kRV * nt * 32);
+}
+
 // shared memory of one LO solve; the FP32 form with refinement keeps both copies of the
 // rows and falls back to the FP64 form where they do not fit (n_x above ~3100)
 static size_t lo_smem(int precision, int nx)
@@ -1606,114 +1572,86 @@ cudaError_t launch_lo_solve_b(int precision, int max_nx, const int *meta, int N,
     return cudaGetLastError();
 }
 
-size_t restrict_scratch_doubles(int nx, int n_from, int n_to)
+RestrictPlan restrict_plan(const Problem &p, int n_from, int n_to)
 {
+    RestrictPlan q;
     const int r = n_from / n_to;
-    if (r < 64) return 0;
-    const int nchunk = (r + kChunk - 1) / kChunk;
-    return (size_t)n_to * nchunk * kRP * (nx + 1);
+    q.nt = (p.nx + 1 + kRTile - 1) / kRTile;
+    q.kc = r;
+    q.nchunk = 1;
+    const long units = (long)q.nt * n_to;
+    // A warp per coarse group where that fills the GPU twice over (2 warps on each of the
+    // 608 sub-partitions) and a warp's serial chain stays short; below, four warps share the
+    // members.
+    q.mode = (r < 16 && units >= 1216) ? 0 : 1;
+    if (q.mode == 1 && r > 32 && units < 1216) {
+        // Members in chunks: a warp's chain is 12 kc / 4 operations and the last CTA's 3 r / kc
+        // (its 12 sums on 4 warps), least for kc = sqrt(r); no more than 16 CTAs per SM.
+        int kc = 8;
+        while (kc * kc < r) kc *= 2;
+        while (kc < r && units * ((r + kc - 1) / kc) > 2432) kc *= 2;
+        const int nc = (r + kc - 1) / kc;
+        if (nc > 1 && restrict_doubles(q.nt, n_to, nc) <= p.rscratch_doubles) {
+            q.kc = kc;
+            q.nchunk = nc;
+        }
+    }
+    q.gy = q.mode == 0 ? (n_to + 3) / 4 : n_to * q.nchunk;
+    return q;
 }
 
-int restrict2_nchunk(int n_from, int n_to) { return (n_from / n_to + kChunk - 1) / kChunk; }
+size_t restrict_head_doubles() { return kRHead; }
 
-int restrict_kind(const Problem &p, int n_from, int n_to, int *KS)
+size_t restrict_scratch_doubles(const Problem &p)
 {
-    const size_t need = restrict_scratch_doubles(p.nx, n_from, n_to);
-    if (need > 0 && p.rscratch && need <= p.rscratch_doubles) return 2;
-    const int r = n_from / n_to;
-    int k = 1;
-    while (k < 16 && k * 4 <= r) k *= 2;   // <= 512 threads: the register file holds them
-    *KS = k;
-    return 1;
+    Problem t = p;
+    t.rscratch_doubles = ~(size_t)0;
+    size_t need = kRHead;
+    for (int l = 0; l + 1 < p.nlev; ++l)
+        for (int m = l + 1; m < p.nlev; ++m) {
+            if (l > 0 && m + 1 < p.nlev) continue;   // fine to any grid, any grid to grey
+            const RestrictPlan q = restrict_plan(t, p.levels[l], p.levels[m]);
+            if (q.nchunk > 1) need = std::max(need, restrict_doubles(q.nt, p.levels[m], q.nchunk));
+        }
+    return need;
 }
 
 RestrictCtx make_restrict_ctx(const Problem &p, const Level &src, const Level &dst)
 {
     RestrictCtx x;
-    x.nx = p.nx; x.r = src.n / dst.n; x.h = p.h; x.ihf = p.ihf; x.S = src; x.T = dst;
+    const RestrictPlan q = restrict_plan(p, src.n, dst.n);
+    x.nx = p.nx; x.r = src.n / dst.n; x.n_to = dst.n; x.h = p.h; x.ihf = p.ihf;
+    x.S = src; x.T = dst;
     x.gate = p.gate;
+    x.mode = q.mode; x.nt = q.nt; x.kc = q.kc; x.nchunk = q.nchunk;
+    x.ticket = reinterpret_cast<int *>(p.rscratch);
+    x.bpart = p.rscratch + kRHead;
+    x.part = x.bpart + (size_t)dst.n * q.nchunk * 16;
+    x.newton = 0;
+    x.ga = GreyArgs{};
+    x.pre = nullptr;
+    x.skip_old = 0;
     return x;
 }
 
-Restrict2Ctx make_restrict2_ctx(const Problem &p, const Level &src, const Level &dst)
-{
-    Restrict2Ctx y;
-    y.nx = p.nx; y.r = src.n / dst.n; y.nchunk = restrict2_nchunk(src.n, dst.n);
-    y.h = p.h; y.ihf = p.ihf; y.S = src; y.T = dst; y.part = p.rscratch;
-    y.gate = p.gate;
-    y.newton = 0;
-    y.ga = GreyArgs{};
-    y.pre = nullptr;
-    y.skip_old = 0;
-    return y;
-}
-
-static size_t restrict_smem(int KS) { return (KS > 1) ? sizeof(double) * KS * 32 * kRV1 : 0; }
-
 cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
-                            const GreyArgs *newton, double *pre, bool *formed, int *old_key)
+                            const GreyArgs *newton, double *pre, bool skip_old)
 {
-    int KS = 1;
-    if (formed) *formed = false;
-    const int key = 2 * src.n + (src.fine ? 1 : 0);
-    if (restrict_kind(p, src.n, dst.n, &KS) == 2) {
-        Restrict2Ctx y = make_restrict2_ctx(p, src, dst);
-        if (old_key) {
-            y.skip_old = (*old_key == key) ? 1 : 0;
-            *old_key = key;
-        }
-        if (newton && pre && dst.n == 1 && !newton->have_prev_dev) {
-            y.newton = 1;
-            y.ga = *newton;
-            y.pre = pre;
-            if (formed) *formed = true;
-        }
-        dim3 g1((p.nx + 1 + 31) / 32, dst.n * y.nchunk);
-        cudaError_t e = cudaFuncSetAttribute(k_restrict_part,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kPartSmem);
-        if (e != cudaSuccess) return e;
-        e = launch_pdl(k_restrict_part, g1, dim3(32, kPartRows), kPartSmem, p.stream, y);
-        if (e != cudaSuccess) return e;
-        return launch_pdl(k_restrict_final, dim3((p.nx + 1 + 31) / 32, dst.n), dim3(32, kRP), 0,
-                          p.stream, y);
+    RestrictCtx x = make_restrict_ctx(p, src, dst);
+    x.skip_old = skip_old ? 1 : 0;
+    if (newton) {
+        x.newton = 1;
+        x.ga = *newton;
+        x.pre = pre;
     }
-    if (old_key) *old_key = 0;   // the one-stage form sums them in another order
-    const RestrictCtx x = make_restrict_ctx(p, src, dst);
-    dim3 grid((p.nx + 1 + 31) / 32, dst.n);
-    const size_t sm = restrict_smem(KS);
-    cudaError_t e = cudaFuncSetAttribute(k_restrict, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(k_restrict, grid, dim3(32, KS), sm, p.stream, x);
+    const RestrictPlan q = restrict_plan(p, src.n, dst.n);
+    return launch_pdl(k_restrict, dim3(q.nt + 1, q.gy), dim3(128), 0, p.stream, x);
 }
 
-cudaError_t launch_restrict_b(int KS, const int *meta, int N, const RestrictCtx *xs, int grid,
+cudaError_t launch_restrict_b(const int *meta, int N, const RestrictCtx *xs, int grid,
                               cudaStream_t st)
 {
-    const size_t sm = restrict_smem(KS);
-    cudaError_t e = cudaFuncSetAttribute(k_restrict_b, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e != cudaSuccess) return e;
-    k_restrict_b<<<grid, dim3(32, KS), sm, st>>>(meta, N, xs);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_restrict_part_b(const int *meta, int N, const Restrict2Ctx *xs, int grid,
-                                   cudaStream_t st)
-{
-    cudaError_t e = cudaFuncSetAttribute(k_restrict_part_b,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kPartSmem);
-    if (e != cudaSuccess) return e;
-    k_restrict_part_b<<<grid, dim3(32, kPartRows), kPartSmem, st>>>(meta, N, xs);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_restrict_final_b(const int *meta, int N, const Restrict2Ctx *xs, int grid,
-                                    cudaStream_t st)
-{
-    k_restrict_final_b<<<grid, dim3(32, kRP), 0, st>>>(meta, N, xs);
+    k_restrict_b<<<grid, 128, 0, st>>>(meta, N, xs);
     return cudaGetLastError();
 }
 

@@ -3,7 +3,7 @@
 // Sec. 2 / Sec. 3.1 / Sec. 6 of the paper: with x = nu/T,
 //   B_g     = CB T^4 [P(x_{g+1}) - P(x_g)],           P(x) = int_0^x t^3/(e^t-1) dt
 //   e_g     = int sigma B = s 27 CB T (e^{-x_g} - e^{-x_{g+1}})   (sigma B = 27 s CB e^{-nu/T})
-//   sigma_B = e_g / B_g = sigma_E          (T_r = T; the T_r option: opacity_tr)
+//   sigma_B = e_g / B_g = sigma_E          (T_r = T; the T_r option: k_opacity_tr)
 //   sigma_R = s 27 N_g / (T^3 D_g),  N_g = [-x^4/(e^x-1) + 4 P(x)],  D_g = [int t^7 e^{2t}/(e^t-1)^3]
 // Every per-edge integral is evaluated in closed form: a power series below x = 2 (radius
 // of convergence 2 pi; the coefficients follow from t/(e^t-1) = sum B_n t^n / n!), and
@@ -469,47 +469,6 @@ __device__ inline void stage_cells(const OpacityArgs &a, int i0, CellTerms &ct, 
     __syncthreads();
 }
 
-// sigma_E,g(T, T_r) and sigma_R,g(T, T_r) (Sec. 2, Sec. 3.1) for sigma = 27 s/nu^3 (1 -
-// e^{-nu/T}); with x = nu/T_r and rho = T_r/T:
-//   sigma_E = 27 s J / (T_r^3 [P(x_{g+1}) - P(x_g)]),  J = int (1 - e^{-rho x})/(e^x - 1) dx
-//   sigma_R = 27 s N / (T_r^3 D),  N the T_r = T numerator at x = nu/T_r,
-//             D = int x^7 e^x / ((1 - e^{-rho x}) (e^x - 1)^2) dx
-// J and D by the 8-point Gauss rule on panels over [x_g, min(x_{g+1}, x_g + 64)], width 2 or,
-// for rho > 1, max(1/rho, a/2) from a panel start a below 4 (1 - e^{-rho x} changes on the
-// scale 1/rho near 0), the last panel taking the remainder up to 1.5 widths; both scaled
-// by e^{x_g} like the Planck difference, so cold groups neither underflow nor lose the
-// ratio.  About 40 FP64 operations per node: far dearer than the tabulated T_r = T path.
-__device__ void opacity_tr(double nu_a, double nu_b, bool binf, double Tr, double rho,
-                           double k27, const Mx &mx, double &sg, double &sR)
-{
-    const double iTr = 1.0 / Tr;
-    const double xa = nu_a * iTr;
-    const double xb = binf ? 0.0 : nu_b * iTr;
-    double dPs, Ns, Ds0, om;
-    group_integrals(xa, xb, binf, c_ser, mx, dPs, Ns, Ds0, om);
-    const double hi = binf ? xa + 64.0 : fmin(xb, xa + 64.0);
-    double Js = 0.0, Ds = 0.0, a = xa;
-    while (a < hi) {
-        const double wmax = (rho > 1.0) ? fmin(2.0, fmax(1.0 / rho, 0.5 * a)) : 2.0;
-        const double b = (hi - a <= 1.5 * wmax) ? hi : a + wmax;
-        const double hw = 0.5 * (b - a);
-        for (int q = 0; q < 8; ++q) {
-            const double x = a + hw * (1.0 + c_ser.g8x[q]);
-            const double e = exp(xa - x);
-            const double o1 = -expm1(-x);
-            const double orh = -expm1(-rho * x);
-            const double wq = hw * c_ser.g8w[q];
-            Js += wq * e * orh / o1;
-            const double x2 = x * x, x7 = x2 * x2 * x2 * x;
-            Ds += wq * x7 * e / (orh * o1 * o1);
-        }
-        a = b;
-    }
-    const double Tr3 = Tr * Tr * Tr;
-    sg = k27 * Js / (Tr3 * dPs);
-    sR = k27 * Ns / (Tr3 * Ds);
-}
-
 // cell i, group g with the cell's terms v; outputs [G][nx] (cells contiguous)
 __device__ inline void opacity_body(const OpacityArgs &a, int i, int g, const CellVals &v,
                                     const Mx &mx)
@@ -541,8 +500,6 @@ __device__ inline void opacity_body(const OpacityArgs &a, int i, int g, const Ce
         sR = k27 * Ns * iT3 * rcp64(Ds);
         em = k27 * kCB * Ti * mx.ex(-xa) * om;
     }
-    if (a.Erad)   // T_r option: absorption and Rosseland opacities at the radiation temperature
-        opacity_tr(a.edges[g], eb, binf, v.Tr, v.rho, 27.0 * a.s, mx, sg, sR);
     a.sigE[idx] = sg;
     a.emis[idx] = em;
     a.sigR[idx] = sR;
@@ -562,8 +519,8 @@ __device__ inline void opacity_body(const OpacityArgs &a, int i, int g, const Ce
 // FP64 result (pr_join), so e_g keeps FP64's range.  Relative errors: about 1e-14 in the
 // opacities, about 3 2^-47 max(1, |w|) in e_g (w's: nu_g, 1/T and their product each
 // rounded to a pair; 1.6e-11 at the smallest e_g that FP64 holds, e^-746).  m, tf: the
-// cell's table interval (>= 0) and FP32 local coordinate; cells outside the tables and the
-// T_r option take opacity_body (the callers' choice).
+// cell's table interval (>= 0) and FP32 local coordinate; cells outside the tables take
+// opacity_body (the callers' choice), the T_r option k_opacity_tr.
 __device__ inline fpair horner_pair(const fpair *__restrict__ a, const float *__restrict__ b,
                                    fpair t, float tf)
 {
@@ -650,7 +607,7 @@ __global__ void __launch_bounds__(256) k_opacity(OpacityArgs a)
     if (i >= a.nx || g >= a.G) return;
     const CellArrays ca = cell_arrays(a);
     const int m = ca.m[i];
-    if (a.otabp && m >= 0 && !a.Erad) {
+    if (a.otabp && m >= 0) {
         const int n = a.nx;
         const CellPair cp{a.cpair[i], a.cpair[n + i], a.cpair[2 * n + i], a.cpair[3 * n + i],
                           a.cpair[4 * n + i]};
@@ -676,12 +633,132 @@ __global__ void __launch_bounds__(256) k_opacity_b(const int *__restrict__ meta,
         const int i = bx * 32 + threadIdx.x, g = by * 8 + threadIdx.y;
         if (i < a.nx && g < a.G) {
             const CellVals &v = ct.v[threadIdx.x];
-            if (a.otabp && v.m >= 0 && !a.Erad)
+            if (a.otabp && v.m >= 0)
                 opacity_body_pair(a, i, g, v.m, v.tf, ct.p[threadIdx.x], s_e2p);
             else
                 opacity_body(a, i, g, v, mx);
         }
         __syncthreads();   // the cell terms are restaged by the next work item
+    }
+}
+
+// 1 - e^{-x} from x >= 0 and ex = e^{-x}: directly where x >= 0.1 (relative error <= eps/x),
+// by the series x (1 - x/2! + x^2/3! - ...) below (11 terms: the next is 2.5e-18)
+__device__ inline double one_minus_exp(double x, double ex)
+{
+    if (x >= 0.1) return 1.0 - ex;
+    double p = 1.0 / 39916800.0;
+    constexpr double c[10] = {-1.0 / 3628800.0, 1.0 / 362880.0, -1.0 / 40320.0, 1.0 / 5040.0,
+                              -1.0 / 720.0, 1.0 / 120.0, -1.0 / 24.0, 1.0 / 6.0, -0.5, 1.0};
+#pragma unroll
+    for (int k = 0; k < 10; ++k) p = fma(p, x, c[k]);
+    return p * x;
+}
+
+// The T_r option: sigma_E,g(T, T_r) and sigma_R,g(T, T_r) (Sec. 2, Sec. 3.1) for sigma = 27
+// s/nu^3 (1 - e^{-nu/T}); with x = nu/T_r and rho = T_r/T:
+//   sigma_E = 27 s J / (T_r^3 P),  J = int (1 - e^{-rho x})/(e^x - 1) dx, P = int x^3/(e^x - 1) dx
+//   sigma_R = 27 s N / (T_r^3 D),  N = int x^4 e^x/(e^x - 1)^2 dx,
+//             D = int x^7 e^x / ((1 - e^{-rho x}) (e^x - 1)^2) dx
+// all over [x_g, min(x_{g+1}, x_g + 64)] and scaled by e^{x_g}, by the 8-point Gauss rule on
+// panels of width 2 or, for rho > 1, max(1/rho, a/2) from a panel start a below 4 (1 -
+// e^{-rho x} changes on the scale 1/rho near 0), the last panel taking the remainder up to
+// 1.5 widths.  Where e^{-x} and e^{-rho x} are both below e^{-40} and the group takes
+// several panels, the factors are 1 and the four integrals are the T_r = T ones in closed
+// form.  Four lanes share a (cell, group): each takes one pair of nodes mid -/+ t of every
+// panel (they share e^{t}, e^{rho t} and their reciprocals) and the sums meet by shuffles.
+// FP64-bound (~110 FP64 operations per lane and panel).  A thread per (cell, group) with
+// library exponentials and divisions in 48 CTAs left 104 SMs idle behind its longest
+// chain: 120 cells x 96 groups 811-981 us, now 43 us.
+// block 256 (8 groups x 8 cells x 4 lanes); grid (ceil(nx / 8), ceil(G / 8)); the cells'
+// terms from k_cell_terms
+__global__ void __launch_bounds__(256) k_opacity_tr(OpacityArgs a)
+{
+    griddep_wait();
+    if (a.gate && *a.gate) return;
+    __shared__ double s_e2[32];
+    if (threadIdx.x < 32) s_e2[threadIdx.x] = c_ser.e2[threadIdx.x];
+    __syncthreads();
+    const Mx mx{s_e2, ExpConsts{c_ser.einv, c_ser.eL1, c_ser.eL2}};
+    const int lane = threadIdx.x & 31, j = lane & 3;
+    const int i = blockIdx.x * 8 + (lane >> 2), g = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (g >= a.G) return;   // a whole warp
+    const bool on = i < a.nx;
+    const CellVals v = cell_arrays(a).get(on ? i : a.nx - 1);
+    const double nu_a = a.edges[g], nu_b = a.edges[g + 1];
+    const bool binf = isinf(nu_b);
+    const double rho = v.rho, iTr = 1.0 / v.Tr;
+    const double xa = nu_a * iTr, xb = binf ? 0.0 : nu_b * iTr;
+    const double hi = binf ? xa + 64.0 : fmin(xb, xa + 64.0);
+    const double gx = c_ser.g8x[4 + j], gw = c_ser.g8w[4 + j];
+    double J = 0.0, P = 0.0, N = 0.0, D = 0.0;
+    const bool closed = xa >= 40.0 && rho * xa >= 40.0 && hi - xa > 3.0;
+    if (!closed) {
+        const double exa = mx.ex(-xa);
+        double lo = xa;
+        while (lo < hi) {
+            const double wmax = (rho > 1.0) ? fmin(2.0, fmax(rcp64(rho), 0.5 * lo)) : 2.0;
+            const double up = (hi - lo <= 1.5 * wmax) ? hi : lo + wmax;
+            const double hw = 0.5 * (up - lo), mid = 0.5 * (up + lo), t = hw * gx;
+            const double E0 = mx.ex(xa - mid), ep = mx.ex(t), em = rcp64(ep);
+            const bool warm = lo < 37.0, rwarm = rho * lo < 37.0;   // some factor is not 1
+            const double Em = warm ? E0 * exa : 0.0;
+            double R0 = 0.0, rp = 0.0, rm = 0.0;
+            if (rwarm) {
+                R0 = mx.ex(-rho * mid);
+                rp = mx.ex(rho * t);
+                rm = rcp64(rp);
+            }
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const double x = side ? mid + t : mid - t;
+                const double f = side ? em : ep;
+                const double o1 = warm ? one_minus_exp(x, Em * f) : 1.0;
+                const double orh = rwarm ? one_minus_exp(rho * x, R0 * (side ? rm : rp)) : 1.0;
+                const double iq = rcp64(orh * o1);          // 1/((1 - e^{-rho x})(1 - e^{-x}))
+                const double io = iq * orh;                 // 1/(1 - e^{-x})
+                const double x2 = x * x;
+                const double q = hw * gw * E0 * f * io;     // weight e^{xa - x}/(1 - e^{-x})
+                const double q3 = q * x2 * x;
+                J = fma(q, orh, J);
+                P += q3;
+                N = fma(q3 * x, io, N);
+                D = fma(q3 * x2 * x2, iq, D);
+            }
+            lo = up;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        J += __shfl_xor_sync(0xffffffffu, J, o);
+        P += __shfl_xor_sync(0xffffffffu, P, o);
+        N += __shfl_xor_sync(0xffffffffu, N, o);
+        D += __shfl_xor_sync(0xffffffffu, D, o);
+    }
+    if (!on || j != 0) return;
+    if (closed) group_integrals(xa, xb, binf, c_ser, mx, P, N, D, J);
+    const double k = 27.0 * a.s * iTr * iTr * iTr;
+    const double sg = k * J * rcp64(P), sR = k * N * rcp64(D);
+    double em;   // the emission stays at T: the tables, or in closed form outside them
+    if (v.m >= 0) {
+        const double *c = a.otab + ((size_t)g * kTabNI + v.m) * kTabEntry;
+        const float *ch = reinterpret_cast<const float *>(c + kTabNF * kTabLo);
+        em = v.kET * mx.ex(horner(c + 2 * kTabLo, ch + 2 * (kTabNC - kTabLo), v.t, v.tf) -
+                           nu_a * v.iT);
+    } else {
+        const double om = binf ? 1.0 : -expm1(-(nu_b - nu_a) * v.iT);
+        em = 27.0 * a.s * kCB * v.T * mx.ex(-nu_a * v.iT) * om;
+    }
+    const size_t idx = (size_t)g * a.nx + i;
+    a.sigE[idx] = sg;
+    a.emis[idx] = em;
+    a.sigR[idx] = sR;
+    if (a.sig32) {
+        const double hh = 0.5 * a.h[i];
+        a.sig32[idx] = (float)(hh * (sg + a.icdt));
+        a.emis32[idx] = (float)(hh * em);
+        if (g == 0) a.kap32[i] = (float)(hh * a.icdt);
     }
 }
 
@@ -897,6 +974,8 @@ cudaError_t launch_opacity(const Problem &p, const double *T, double *sigE, doub
     const OpacityArgs a = make_opacity_args(p, T, sigE, emis, sigR, sig32, emis32, dt, Erad);
     cudaError_t e = launch_pdl(k_cell_terms, dim3((p.nx + 127) / 128), dim3(128), 0, p.stream, a);
     if (e != cudaSuccess) return e;
+    if (a.Erad)
+        return launch_pdl(k_opacity_tr, dim3((p.nx + 7) / 8, (p.G + 7) / 8), dim3(256), 0, p.stream, a);
     return launch_pdl(k_opacity, dim3(opacity_gx(p), (p.G + 7) / 8), dim3(32, 8), 0, p.stream, a);
 }
 
