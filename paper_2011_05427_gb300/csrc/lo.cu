@@ -749,7 +749,8 @@ __device__ inline void grey_newton_terms(const GreyArgs &a, int have_prev, int i
 //   - a lane owns an extended position j = -1 .. n_x: cell j and face j, with the boundary
 //     energies as "cells" -1 and n_x.  A warp covers 31 faces and the cell before its first
 //     (lane 0), so that a face's sums of E_L and E_R are the cell sums of two neighbouring
-//     lanes: no FP64 operation of their own;
+//     lanes: no FP64 operation of their own.  A member's E_L is a second load: a shuffle
+//     per member occupies the FP64 pipe as well (counters; 166 against 144 us below);
 //   - one pass: the compensation is xi = dx (sum sigR F - sigR-bar sum F) + c (sum etaR E_R -
 //     sum etaL E_L), equal to the two-pass sum up to rounding relative to the sigR dx F
 //     terms.  12 operations per member and position (4 for the cell, 8 for the face), 2 more
@@ -764,7 +765,10 @@ __device__ inline void grey_newton_terms(const GreyArgs &a, int have_prev, int i
 //      chunk the partial sums go to scratch and the CTA that arrives last at a position
 //      tile (a ticket) adds the chunks in a fixed order and forms the coefficients: no
 //      second launch.
-// Measured (warm): 1024 members to the grey level, 500 cells: RMEAS
+// Measured (warm, with the former two launches' times for the same work): 1024 members to
+// the grey level, 500 cells 27.5 us (35.3 + 8.3); 4096 members to a few groups, 1000 cells
+// 144 us (163 + 50; the FP64 pipe's own time is 106 us); 1024 to 256 groups, 500 cells 31 us
+// (38); 256 members, 10 cells 13 us (21.6 + 5.6).
 constexpr int kRV = 12;   // sums per position: the order of restrict_member's v
 enum { R_PHI, R_SIG, R_EMIS, R_E, R_SW, R_W, R_SF, R_F, R_EOLD, R_FOLD, R_ETAR, R_ETAL };
 constexpr int kRTile = 31;          // faces per position tile
@@ -785,43 +789,41 @@ __device__ inline double rquot(double a, double w)
     return fma(fma(-q, w, a), r, q);
 }
 
-// sums over members p = p0, p0 + step, .. < pe of lane position i (clamped by the caller)
+// sums over members p = p0, p0 + step, .. < pe of lane position i (clamped by the caller);
+// kFine: S is the fine grid; kOld: Eold and Fold are summed too
+template <bool kFine, bool kOld>
 __device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, int step, int i,
                                         double (&v)[kRV])
 {
     const Level &S = x.S;
     const int nx = x.nx;
-    const size_t nf = (size_t)nx + 1;
-    const int ic = min(max(i, 0), nx - 1), jf = max(i, 0);
-    const double *Ep = i < 0 ? S.Eb0 : i >= nx ? S.EbX : S.E + i;
-    const size_t Es = (i < 0 || i >= nx) ? 1 : (size_t)nx;
-    const int ia = max(ic - (i < nx ? 1 : 0), 0);   // the cell left of face i
-    double wa = 0.0, wb = 0.0;
-    if (S.fine && i > 0 && i < nx) {   // the face opacity's dx-weighted mean
-        wa = x.h[i - 1] * x.ihf[i];
-        wb = x.h[i] * x.ihf[i];
+    const int ic = min(max(i, 0), nx - 1);
+    const size_t cs = (size_t)p0 * nx + ic, cd = (size_t)step * nx;
+    const size_t fs = (size_t)p0 * (nx + 1) + max(i, 0), fd = cd + step;
+    const bool in = i >= 0 && i < nx;
+    const double *Ep = in ? S.E + cs : (i < 0 ? S.Eb0 : S.EbX) + p0;
+    const size_t Ed = in ? cd : (size_t)step;
+    const double *Lp = i > 0 ? S.E + (size_t)p0 * nx + i - 1 : S.Eb0 + p0;   // E left of face i
+    const size_t Ld = i > 0 ? cd : (size_t)step;
+    const double *ph = S.phi + cs, *sg = S.sig + cs, *em = S.emis + cs, *Fp = S.F + fs;
+    const double *sb = S.sigR + (kFine ? cs : fs);
+    const double *sa = kFine ? S.sigR + (size_t)p0 * nx + (in ? max(i - 1, 0) : ic) : nullptr;
+    double wa = 0.0, wb = 1.0;
+    if (kFine && i > 0) {   // the face opacity's dx-weighted mean; face n_x: its cell alone
+        wa = i < nx ? x.h[i - 1] * x.ihf[i] : 1.0;
+        wb = i < nx ? x.h[i] * x.ihf[i] : 0.0;
     }
 #pragma unroll
     for (int k = 0; k < kRV; ++k) v[k] = 0.0;
 #pragma unroll 2
     for (int p = p0; p < pe; p += step) {
-        const size_t c = (size_t)p * nx, fp = (size_t)p * nf + jf;
-        const double E = Ep[(size_t)p * Es];
-        const double EL = __shfl_up_sync(0xffffffffu, E, 1);
-        const double F = S.F[fp];
-        v[R_PHI] = fma(S.phi[c + ic], E, v[R_PHI]);
-        v[R_SIG] = fma(S.sig[c + ic], E, v[R_SIG]);
-        v[R_EMIS] += S.emis[c + ic];
+        const double E = *Ep, EL = *Lp, F = *Fp;
+        v[R_PHI] = fma(*ph, E, v[R_PHI]);
+        v[R_SIG] = fma(*sg, E, v[R_SIG]);
+        v[R_EMIS] += *em;
         v[R_E] += E;
-        double sR;
-        if (S.fine) {
-            const double a = S.sigR[c + ia], b = S.sigR[c + ic];
-            sR = (i <= 0) ? b : (i >= nx) ? a : fma(wa, a, wb * b);
-        } else {
-            sR = S.sigR[fp];
-            v[R_ETAR] = fma(S.etaR[fp], E, v[R_ETAR]);
-            v[R_ETAL] = fma(S.etaL[fp], EL, v[R_ETAL]);
-        }
+        double sR = *sb;
+        if (kFine) sR = fma(wa, *sa, wb * sR);
         // |F| weight with a floor 1e-6 c E-bar: groups in local equilibrium carry
         // rounding-noise fluxes that must not decide the mean
         const double w = fma(0.5e-6 * kC, EL + E,
@@ -830,10 +832,29 @@ __device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, in
         v[R_W] += w;
         v[R_SF] = fma(sR, F, v[R_SF]);
         v[R_F] += F;
-        if (!x.skip_old) {
-            v[R_EOLD] += S.Eold[c + ic];
-            v[R_FOLD] += S.Fold[fp];
+        if (!kFine) {
+            const size_t fp = (size_t)p * (nx + 1) + max(i, 0);
+            v[R_ETAR] = fma(S.etaR[fp], E, v[R_ETAR]);
+            v[R_ETAL] = fma(S.etaL[fp], EL, v[R_ETAL]);
         }
+        if (kOld) {
+            v[R_EOLD] += S.Eold[(size_t)p * nx + ic];
+            v[R_FOLD] += S.Fold[(size_t)p * (nx + 1) + max(i, 0)];
+        }
+        Ep += Ed; Lp += Ld; ph += cd; sg += cd; em += cd; Fp += fd;
+        sb += kFine ? cd : fd;
+        if (kFine) sa += cd;
+    }
+}
+__device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, int step, int i,
+                                        double (&v)[kRV])
+{
+    if (x.S.fine) {
+        if (x.skip_old) restrict_members<true, false>(x, p0, pe, step, i, v);
+        else restrict_members<true, true>(x, p0, pe, step, i, v);
+    } else {
+        if (x.skip_old) restrict_members<false, false>(x, p0, pe, step, i, v);
+        else restrict_members<false, true>(x, p0, pe, step, i, v);
     }
 }
 
@@ -1405,8 +1426,8 @@ __global__ void __launch_bounds__(256) k_group_sum(GroupSumArgs a) { group_sum_b
             __syncthreads();                                                                   \
         }                                                                                      \
     }
-// (6 CTAs per SM: unbounded, the argument block held in registers leaves 3; 64 slabs to the
-// grey level 486 -> BMEAS us)
+// (6 CTAs per SM: unbounded, the argument block held in registers leaves 3 and 64 slabs'
+// restriction to the grey level takes 25% longer)
 TRT_BATCHED(k_restrict_b, RestrictCtx, 128, 6, restrict_body(x, bx, by))
 TRT_BATCHED(k_grey_b, GreyCtx, 1024, 1, grey_body(x))
 TRT_BATCHED(k_group_sum_b, GroupSumArgs, 256, 1, group_sum_body(x, bx))

@@ -402,6 +402,46 @@ def test_restrict_parity(trt, orc, n_from, n_to, eta, nx, fine, precision):
     assert rel(got["Esum"], Esum) < 1e-13
 
 
+@pytest.mark.parametrize("fine", [False, True])
+@pytest.mark.parametrize("n_from,n_to,nx", [(40, 40, 1), (3, 1, 2), (60, 4, 29), (64, 1, 30),
+                                            (96, 2, 31), (40, 8, 61), (1300, 1, 62),
+                                            (2560, 1280, 10), (15, 3, 92), (4096, 4, 7)])
+def test_restrict_tiles(trt, orc, n_from, n_to, nx, fine):
+    """The restriction's splits: one cell, position tiles of 31 faces full, one short and one
+    over, fewer members than warps, chunks with a ragged last one, a warp per coarse group.
+    Bounds as in test_restrict_parity; a second call on the same handle gives the same bits
+    (the tickets of the chunked form are back at zero)."""
+    r = W.rng(4800 + n_from + nx)
+    h = W.random_h(r, nx)
+    lv = random_level(r, n_from, nx, eta=not fine)
+    src = dict(lv)
+    if fine:
+        src["sigR"] = np.exp(r.uniform(-3, 3, (n_from, nx)))
+        lv["sigR"] = orc.fine_face_sigR(h, src["sigR"])
+    sol = oracle_level_solve(orc, h, 2e-3, lv)
+    s = solver(trt, nx=nx, N=2, G=max(n_from, 3), h=h, levels=[max(n_from, 3), 1])
+    src.update(sol)
+    got = {k: v.cpu().numpy() for k, v in s.k_restrict(src, n_to, fine=fine).items()}
+    again = {k: v.cpu().numpy() for k, v in s.k_restrict(src, n_to, fine=fine).items()}
+    ref, Esum = orc.restrict(h, lv, sol, np.arange(n_from) // (n_from // n_to), n_to)
+    # the one-pass compensation: rounding relative to the terms it is made of (1e-12 of them)
+    dxf = np.concatenate([[h[0] / 2], (h[:-1] + h[1:]) / 2, [h[-1] / 2]])
+    ER = np.concatenate([sol["E"], sol["EbX"][:, None]], axis=1)
+    EL = np.concatenate([sol["Eb0"][:, None], sol["E"]], axis=1)
+    m = lambda a: a.reshape(n_to, -1, nx + 1).sum(1)
+    terms = m(dxf * np.abs(lv["sigR"] * sol["F"]) + C * (np.abs(lv["etaR"] * ER) + np.abs(lv["etaL"] * EL)))
+    for k in orc.LEVEL_KEYS:
+        assert np.array_equal(got[k], again[k]), k
+        if k in ("etaR", "etaL"):
+            side = m(ER) if k == "etaR" else m(EL)
+            assert np.all(np.abs(got[k] - ref[k]) <= 1e-12 * terms / (C * side)), k
+        elif k == "Fold":
+            assert np.max(np.abs(got[k] - ref[k])) <= 1e-12 * np.abs(ref[k]).max(), k
+        else:
+            assert rel(got[k], ref[k]) < 1e-12, k
+    assert rel(got["Esum"], Esum) < 1e-13
+
+
 @pytest.mark.parametrize("precision", ["fp64", "lopair"])
 @pytest.mark.parametrize("fine", [False, True])
 def test_restrict_wide_range(trt, orc, fine, precision):
