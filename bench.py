@@ -168,11 +168,11 @@ def fp64_peak(trt, local=0):
 # sub-partitions are busy, i.e. the FMA rate trt_fp64_peak measures (~1.056 TFLOP/s, 84%
 # of the nominal 1.25); the instruction-rate fraction below divides by that measured rate.
 # FP64 thread instructions per update (ncu, DFMA + DMUL + DADD over the updates of one
-# fc_1024 launch): the strip sweep 17.6 (11.0 + 4.5 + 2.1), the paired sweep 13.5 (9.0 +
-# 3.0 + 1.5: t and s formed once per pair of directions); the FLOP ceiling of a mix is
-# 23 / (2 x instructions) of the FMA rate.
+# fc_1024 launch): the strip sweep 17.6 (11.0 + 4.5 + 2.1), the paired sweep 13.0 (t and s
+# formed once per pair of directions, the moments of both signs together); the FLOP
+# ceiling of a mix is 23 / (2 x instructions) of the FMA rate.
 FP64_INST_PEAK = 152 * 4 * 2.07e9 / 64 * 32
-FP64_INST_PER_UPDATE = {"strip": 17.6, "pair": 13.5}
+FP64_INST_PER_UPDATE = {"strip": 17.6, "pair": 13.0}
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum, one ncu capture of the
 # sweep and its finalize on the fc_1024 workload), valid while the kernel sources hash to
@@ -212,9 +212,11 @@ def _traffic(key, tile):
 def sweep_kernel(fp32, D, shape):
     """The kernels one sweep launches for tile (D, shape) (the library's shape table)."""
     if not fp32:
+        if D == 0:   # the library default: the paired sweep at its own tile height
+            return "k_prescale64 + k_sweep_pair<default> + k_sweep_finalize<double>"
         if shape in (3, 4):   # paired sweep: its pre-scaled inputs, the sweep, the finalize
             S, NS = {3: (8, 2), 4: (4, 2)}[shape]
-            return f"k_prescale64 + k_sweep_pair<{S},{NS}> + k_sweep_finalize<double>"
+            return f"k_prescale64 + k_sweep_pair<4,{S},{NS}> + k_sweep_finalize<double>"
         S, NS = {0: (8, 2), 1: (16, 2), 2: (8, 3)}[shape]
         return f"k_sweep<double,double,{S},{NS}> + k_sweep_finalize<double>"
     if shape == 6 or D not in (4, 8, 16):   # the strip sweep (tile heights without a lean kernel)
@@ -240,7 +242,7 @@ def sweep_roofline(trt, s, cfg, fp32=False, local=0, reps=20):
                                  device=f"cuda:{local}")
         tile = s.autotune(cfg.dt, reps=10)
     D, shape = s.sweep_tile()
-    if D == 0:   # the library default: the largest power of two <= 8 dividing N
+    if D == 0 and fp32:   # the library default: the largest power of two <= 8 dividing N
         D = max(d for d in (1, 2, 4, 8) if cfg.N % d == 0)
     ms = s.sweep_time(cfg.dt, reps=reps)
     if own:
@@ -257,7 +259,7 @@ def sweep_roofline(trt, s, cfg, fp32=False, local=0, reps=20):
                 "peak_source": f"{src} (MEASURED_PEAKS hbm_gbs, copy)",
                 "updates_per_s": upd / (ms * 1e-3)}
     else:
-        kind64 = "pair" if shape in (3, 4) else "strip"
+        kind64 = "pair" if shape in (3, 4) or D == 0 else "strip"
         flops = FLOP_PER_UPDATE * upd
         ach = flops / (ms * 1e-3) / 1e12
         pk, pk_src = fp64_peak(trt, local)

@@ -285,7 +285,8 @@ int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS);
 int trt_sweep_shapes(const trt_handle *h);
 int trt_set_sweep_tile(trt_handle *h, int D, int shape);
 /* The sweep tile the next step uses (after trt_autotune, trt_set_sweep_tile or neither):
- * *D = directions per CTA (0: the library's default for this problem), *shape = shape index.
+ * *D = directions per CTA (0: the library's default for this problem, which trt_autotune
+ * times too on an FP64 handle and may keep), *shape = shape index.
  * Either pointer may be NULL.  TRT_EINVAL for a NULL handle. */
 int trt_get_sweep_tile(const trt_handle *h, int *D, int *shape);
 

@@ -103,9 +103,11 @@ void carve(trt_handle *h, Carver &c)
     if (sweep_fp32(p.precision)) {
         h->sig32 = c.take<float>(G * nx);
         h->emis32 = c.take<float>(G * nx + nx);   // then h/(2 c dt) per cell (kap32)
-    } else {   // the paired FP64 sweep's t, s and pre-scaled inputs
-        p.ts64 = c.take<double>((size_t)p.N * nx * 2 * p.ldG);
+    } else {   // the paired FP64 sweep's t, s, sums, pre-scaled inputs and hand-over slots
+        p.ts64 = c.take<double>((size_t)p.N * nx * 3 * p.ldG);
         p.tab64 = c.take<double>(2 * nx * (size_t)p.ldG + nx);
+        p.hand64 = c.take<double>(pair_hand_doubles());
+        p.pair64 = true;
     }
     h->part = c.take<double>(std::max(sweep_partial_doubles(p), 4 * nx + 8));
     h->psi_exit = c.take<double>(M * (size_t)p.ldG);
@@ -458,6 +460,7 @@ int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups 
     CK(launch_lo_pair_consts(p));
     CK(cudaMemsetAsync(H->flags, 0, 10 * sizeof(double), p.stream));
     CK(cudaMemsetAsync(p.rscratch, 0, restrict_head_doubles() * sizeof(double), p.stream));
+    if (p.hand64) CK(cudaMemsetAsync(p.hand64, 0, pair_hand_doubles() * sizeof(double), p.stream));
     CK(cudaStreamSynchronize(p.stream));
     *out = hp.release();
     return TRT_OK;
@@ -901,10 +904,11 @@ int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS)
     const int D0 = h->p.sweep_D, sh0 = h->p.sweep_shape;
     float best = 1e30f;
     int bD = D0, bsh = sh0;
-    for (int i = 0; i < nc; ++i) {
-        for (int k = 0; k < ns; ++k) {
-            if (!sweep_tile_ok(h->p.precision, cand[i], k)) continue;
-            h->p.sweep_D = cand[i];
+    // the library's default (D = 0) first: the paired FP64 sweep at its own tile height
+    for (int i = h->p.pair64 ? -1 : 0; i < nc; ++i) {
+        for (int k = 0; k < (i < 0 ? 1 : ns); ++k) {
+            if (i >= 0 && !sweep_tile_ok(h->p.precision, cand[i], k)) continue;
+            h->p.sweep_D = i < 0 ? 0 : cand[i];
             h->p.sweep_shape = k;
             float ms = 0;
             const int rc = trt_sweep_time(h, dt, reps, &ms);
@@ -926,7 +930,7 @@ int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS)
             }
             if (ms < best) {
                 best = ms;
-                bD = cand[i];
+                bD = h->p.sweep_D;
                 bsh = k;
             }
         }

@@ -249,9 +249,12 @@ struct Problem {
     size_t rscratch_doubles;
     // sweep tile: directions per CTA (0 = default) and strip shape index (0 = default)
     int sweep_D = 0, sweep_shape = 0;
-    // scratch of the paired FP64 sweep (FP64 handles; null elsewhere): t, s per (|mu|,
-    // cell, group) [N][nx][2][ldG], and the pre-scaled inputs [2][nx][ldG] + [nx]
-    double *ts64 = nullptr, *tab64 = nullptr;
+    // scratch of the paired FP64 sweep (FP64 handles; null elsewhere): t, s and psi_L + psi_R
+    // per (|mu|, cell, group) [N][nx][3][ldG], the pre-scaled inputs [2][nx][ldG] + [nx], and
+    // the hand-over slots and flags of split jobs (zero between launches); pair64: the handle
+    // has them, and the paired sweep is its default tile
+    double *ts64 = nullptr, *tab64 = nullptr, *hand64 = nullptr;
+    bool pair64 = false;
     // per-group polynomial tables in ln T (Chebyshev fits stored as monomials) of
     // sigma_E T^3, sigma_R T^3 and the emission factor ln(1 - e^{-w}) (null: direct
     // integrals)
@@ -289,6 +292,7 @@ cudaError_t launch_opacity(const Problem &p, const double *T, double *sigE, doub
 cudaError_t launch_prescale32(const Problem &p, double dt, const double *sigE, const double *emis,
                               float *sig32, float *emis32);
 size_t sweep_partial_doubles(const Problem &p);
+size_t pair_hand_doubles();
 int sweep_shape_count(int precision);
 // a kernel exists and fits (shared memory); `batched`: the batched sweep has one too
 bool sweep_tile_ok(int precision, int D, int shape, bool batched = false);

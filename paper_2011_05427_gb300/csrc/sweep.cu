@@ -413,8 +413,9 @@ __global__ void k_sweep_finalize_b(const int *__restrict__ meta, int N,
 // multiple of 4).  Measured at 500 cells x 64 directions x 1024 groups: lean one group per
 // lane D = 16 (8, 4) 0.100 ms with the finalize, (16, 2) 0.104; two groups per lane
 // D = 8 (8, 4) 0.108 (it wins on some batches); the strip sweep D = 8 (16, 2) 0.209.
-// FP64 (strip sweep): (8, 2) 1.26 ms, (16, 2) 1.37, (8, 3) 1.37; the paired sweep of
-// sweep64.cu (single slab, D = 4) as shapes 3 and 4.
+// FP64 (strip sweep): (8, 2) 1.24 ms, (16, 2) 1.37, (8, 3) 1.37; the paired sweep of
+// sweep64.cu (single slab) at D = 4 as shapes 3 and 4 (0.918 and 0.946 ms), and at its own
+// D as the default of a single slab (0.831 ms).
 struct Shape {
     int S, NS, V;   // strip cells, strip buffers, kind (1: strip sweep; 5, 6: lean sweep
                     // with one, two groups per lane; 7: paired FP64 sweep)
@@ -470,9 +471,7 @@ cudaError_t dispatch_shape(int shape, const SweepArgs *a, int M, int ldG, int D,
         return launch_shape<float, float, 16, 2>(a, M, ldG, D, meta, N, xs, grid, st);
     }
     if (D > 8) return cudaErrorInvalidConfiguration;
-    if (kShapes64[shape].V == 7)   // paired sweep: single slab only
-        return a ? launch_sweep_pair(kShapes64[shape].S, kShapes64[shape].NS, *a, M, ldG, st)
-                 : cudaErrorInvalidConfiguration;
+    if (kShapes64[shape].V == 7) return cudaErrorInvalidConfiguration;   // single slabs: launch_sweep
     switch (shape) {
     case 1: return launch_shape<double, double, 16, 2>(a, M, ldG, D, meta, N, xs, grid, st);
     case 2: return launch_shape<double, double, 8, 3>(a, M, ldG, D, meta, N, xs, grid, st);
@@ -481,17 +480,20 @@ cudaError_t dispatch_shape(int shape, const SweepArgs *a, int M, int ldG, int D,
 }
 
 template <typename R>
+cudaError_t launch_finalize(const Problem &p, const SweepArgs &a)
+{
+    const FinalizeArgs fa = make_finalize_args(p, a);
+    return launch_pdl(k_sweep_finalize<R>,
+                      dim3((unsigned)(fa.nb_cell + finalize_bnd_blocks(p.G))), dim3(256), 0,
+                      p.stream, fa);
+}
+
+template <typename R>
 cudaError_t launch_sweep_t(const Problem &p, const SweepArgs &a)
 {
     cudaError_t e = dispatch_shape<R>(p.sweep_shape, &a, p.M, p.ldG, a.D, nullptr, 0, nullptr, 0,
                                       p.stream);
-    if (e != cudaSuccess) return e;
-    const FinalizeArgs fa = make_finalize_args(p, a);
-    cudaError_t ef = launch_pdl(k_sweep_finalize<R>,
-                                dim3((unsigned)(fa.nb_cell + finalize_bnd_blocks(p.G))), dim3(256),
-                                0, p.stream, fa);
-    if (ef != cudaSuccess) return ef;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : launch_finalize<R>(p, a);
 }
 
 }  // namespace
@@ -553,7 +555,9 @@ int sweep_D_candidates(const Problem &p, int *D)
 size_t sweep_partial_doubles(const Problem &p)
 {
     // sized for the smallest direction tile any shape may use
-    return (size_t)(p.M / std::min(base_D(p.N, 4), pick_D(p))) * 2 * p.G * p.nx;
+    int tiles = p.M / std::min(base_D(p.N, 4), pick_D(p));
+    if (p.pair64) tiles = std::max(tiles, p.N / pair_default_D(p.N, p.ldG));
+    return (size_t)tiles * 2 * p.G * p.nx;
 }
 
 SweepArgs make_sweep_args(const Problem &p, double dt, const void *sigE, const void *emis,
@@ -570,8 +574,12 @@ SweepArgs make_sweep_args(const Problem &p, double dt, const void *sigE, const v
     a.f = f; a.fb0 = fb0; a.fbX = fbX; a.C0 = C0; a.CX = CX;
     a.kap32 = nullptr;
     a.dir32 = p.dir32;
+    a.ntile = p.M / D;
     a.ts = p.ts64;
     a.tab64 = p.tab64;
+    a.hand = p.hand64;
+    a.hand_flag = nullptr;
+    a.hand_epoch = 0;
     return a;
 }
 
@@ -579,7 +587,7 @@ FinalizeArgs make_finalize_args(const Problem &p, const SweepArgs &a)
 {
     FinalizeArgs x;
     x.nx = p.nx; x.N = p.N; x.G = p.G; x.ldG = p.ldG;
-    x.ntile = p.M / a.D;
+    x.ntile = a.ntile;
     x.nb_cell = (int)(((long)p.G * p.nx + 255) / 256);
     x.part = a.part; x.psi_exit = a.psi_exit;
     x.mu = p.mu; x.w = p.w; x.Iin0 = p.Iin0; x.IinX = p.IinX;
@@ -599,7 +607,22 @@ cudaError_t launch_sweep(const Problem &p, double dt, const void *sigE, const vo
 {
     SweepArgs a = make_sweep_args(p, dt, sigE, emis, I_old, I_new, part, psi_exit, f, fb0, fbX,
                                   C0, CX, pick_D(p));
-    if (!sweep_fp32(p.precision)) return launch_sweep_t<double>(p, a);
+    if (!sweep_fp32(p.precision)) {
+        // The default of a handle with the paired sweep's scratch is that sweep: 13 FP64
+        // instructions per update against 17.6 of the strip sweep, at any size (with the
+        // finalize, against the strip sweep's best tile: 500 cells x 64 x 1024 0.831 against
+        // 1.239 ms; 333 x 48 x 500 0.319, 0.468; 60 x 16 x 17 0.049, 0.058; 10 x 16 x 256
+        // 0.017, 0.017)
+        const bool def = p.sweep_D == 0 && p.pair64;
+        if (def || kShapes64[p.sweep_shape].V == 7) {
+            if (def) a.D = pair_default_D(p.N, p.ldG);
+            a.ntile = p.N / a.D;   // a tile holds both signs
+            const int S = def ? 4 : kShapes64[p.sweep_shape].S, NS = def ? 2 : kShapes64[p.sweep_shape].NS;
+            cudaError_t e = launch_sweep_pair(a.D, S, NS, a, p.M, p.ldG, p.stream);
+            return e != cudaSuccess ? e : launch_finalize<double>(p, a);
+        }
+        return launch_sweep_t<double>(p, a);
+    }
     if (!sigma_fp32 || !p.dir32) return cudaErrorInvalidValue;   // FP32 sweeps: FP32 inputs
     // the pre-scaled inputs carry h/(2 c dt) after e (launch_opacity, launch_prescale32)
     a.kap32 = reinterpret_cast<const float *>(emis) + (size_t)p.G * p.nx;

@@ -285,6 +285,32 @@ def test_lean_sweep_kernel_parity(trt, orc, nx, N, G):
     assert n >= 12
 
 
+@pytest.mark.parametrize("nx,N,G", [(1, 1, 3), (2, 3, 17), (7, 6, 40), (13, 2, 33), (9, 32, 320),
+                                    (1, 32, 640), (13, 32, 640), (30, 16, 1000), (6, 32, 960)])
+def test_default_fp64_sweep(trt, orc, nx, N, G):
+    """The default FP64 sweep (paired, one or two |mu| per CTA) against the oracle: one cell,
+    fewer cells than a strip, odd direction counts, partial group tiles, fewer jobs than SMs,
+    and more (160, 320, 256 and 480 jobs), where CTAs take shares of the strips and hand psi
+    over inside a job.  Bounds as for the other FP64 shapes; a second call gives the same
+    bits (the hand-over flags are back at zero)."""
+    r, h, sig, em, I_old, TL = sweep_inputs(orc, 2900 + nx + G, nx, N, G, thick=True)
+    edges = W.group_edges(G, 1e-5, 1e2)
+    s = solver(trt, nx=nx, N=N, G=G, h=h, edges=edges, TL=TL, TR=0.3)
+    assert s.sweep_tile()[0] == 0
+    dt = 1.7e-3
+    mu, w = orc.double_gl(N)
+    Iin0 = orc.group_physics(edges, TL)[0]
+    IinX = orc.group_physics(edges, 0.3)[0]
+    ref = orc.sweep(h, mu, w, sig, em, 1.0 / (C * dt), I_old, Iin0, IinX)
+    got = [x.cpu().numpy() for x in s.k_sweep(dt, sig, em, I_old)]
+    again = [x.cpu().numpy() for x in s.k_sweep(dt, sig, em, I_old)]
+    assert pair_err(got[0], ref[0]) < 1e-12
+    for a, b in zip(got[1:], ref[1:]):
+        assert rel(a, b) < 1e-11
+    for a, b in zip(got, again):
+        assert np.array_equal(a, b)
+
+
 def test_autotune_keeps_state(trt):
     """trt_autotune / trt_sweep_time leave T, E_g, F_g, I and the QD factors unchanged and
     keep a candidate tile; steps after tuning match steps without it to round-off."""
