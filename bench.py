@@ -216,7 +216,7 @@ def sweep_kernel(fp32, D, shape):
             return "k_prescale64 + k_sweep_pair<default> + k_sweep_finalize<double>"
         if shape in (3, 4):   # paired sweep: its pre-scaled inputs, the sweep, the finalize
             S, NS = {3: (8, 2), 4: (4, 2)}[shape]
-            return f"k_prescale64 + k_sweep_pair<4,{S},{NS}> + k_sweep_finalize<double>"
+            return f"k_prescale64 + k_sweep_pair<{S},{NS}> + k_sweep_finalize<double>"
         S, NS = {0: (8, 2), 1: (16, 2), 2: (8, 3)}[shape]
         return f"k_sweep<double,double,{S},{NS}> + k_sweep_finalize<double>"
     if shape == 6 or D not in (4, 8, 16):   # the strip sweep (tile heights without a lean kernel)
