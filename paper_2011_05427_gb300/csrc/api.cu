@@ -355,22 +355,8 @@ int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups 
         fwl[f] = hf[f] * ihf[f] * hh[f - 1];
         fwr[f] = hf[f] * ihf[f] * hh[f];
     }
-    std::vector<int> lo_slot(nx + 1, 0);   // chunk layout of the partitioned LO solve
-    if (nx >= 2) {
-        const int P = std::min(32, nx / 2);
-        for (int f = 0; f <= nx; ++f) {
-            int l, k;
-            if (f == nx) {
-                l = P - 1;
-                k = nx - ((P - 1) * nx) / P;
-            } else {
-                l = (f * P) / nx;
-                if (l + 1 < P && ((l + 1) * nx) / P <= f) ++l;
-                k = f - (l * nx) / P;
-            }
-            lo_slot[f] = k * 32 + l;
-        }
-    }
+    std::vector<int> lo_slot(nx + 1, 0);   // row layout of the LO solves
+    lo_slots(nx, lo_slot.data());
     {
         std::vector<double> x(N), wx(N);
         gauss_legendre_host(N, x.data(), wx.data());

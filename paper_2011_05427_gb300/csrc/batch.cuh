@@ -107,7 +107,6 @@ struct RestrictPlan {
 struct GreyCtx {
     LoCtx lo;
     GreyArgs a;
-    int mmax;
 };
 
 struct CopyArgs {
@@ -148,10 +147,6 @@ __device__ inline bool bdecode(const int *__restrict__ meta, int N, int b, int &
 }
 
 // ---- host-side argument builders (the single-slab launchers use the same) ----
-inline int lo_mmax_h(int nx)
-{
-    return nx < 2 ? 1 : (nx + (std::min(32, nx / 2)) - 1) / std::min(32, nx / 2) + 1;
-}
 OpacityArgs make_opacity_args(const Problem &p, const double *T, double *sigE, double *emis,
                               double *sigR, float *sig32, float *emis32, double dt,
                               const double *Erad = nullptr);

@@ -10,15 +10,16 @@
 // face, F_f = GD_f + PL_f E_{f-1} - PR_f E_f, gives a tridiagonal system in E that is
 // column diagonally dominant (the dx/dt term), so elimination needs no pivoting.
 //
-// GB300 mapping.  A warp owns one system.  FP64 throughput on GB300 is a small fraction of
-// FP32, so the solver keeps the FP64 work of plain Thomas elimination (one reciprocal per
-// row) but splits the serial chain: lane l eliminates its chunk of >= 2 consecutive rows
-// (a "modified Thomas" pass down and up the chunk that leaves each row coupled only to the
-// chunk's first and last unknowns), the 2 x 32 chunk-boundary unknowns form a tridiagonal
-// system solved by parallel cyclic reduction in registers with warp shuffles, and every
-// lane back-substitutes its interior rows.  Rows are built on the fly from the level's
-// fields; per-warp shared memory holds the chunk coefficients in a [row-in-chunk][lane]
-// layout (conflict free).
+// GB300 mapping.  A CTA of four warps (one per sub-partition, each with its own FP64 pipe)
+// owns one system.  FP64 throughput on GB300 is a small fraction of FP32, so the solver
+// keeps the FP64 work of plain Thomas elimination (one reciprocal per row) but splits the
+// serial chain: each of P = min(128, n/2) threads eliminates its chunk of >= 2 consecutive
+// rows (a "modified Thomas" pass down and up the chunk that leaves each row coupled only to
+// the chunk's first and last unknowns); the chunks' last rows, then every other first row,
+// are eliminated by cyclic reduction until at most 32 rows are left, which one warp solves
+// by parallel cyclic reduction in registers; back substitution retraces the steps.  Rows are
+// built from the level's fields into shared memory in a [row-in-chunk][chunk] layout
+// (conflict free for the elimination).
 #include <cmath>
 #include "batch.cuh"
 #include "pair.cuh"
@@ -35,6 +36,20 @@ template <>
 __device__ inline float rcpR<float>(float d) { return __frcp_rn(d); }
 template <>
 __device__ inline fpair rcpR<fpair>(fpair d) { return prcp(d); }
+
+// a/w: the refined reciprocal and one residual correction (the correctly rounded quotient
+// but for rare last bits).  The weights of cold cells are subnormal, where 1/w overflows and
+// a/w does not: an exponent outside +-900 divides, and a non-finite quotient is kept.
+static __device__ __noinline__ double rquot_divide(double a, double w) { return a / w; }
+__device__ inline double rquot(double a, double w)
+{
+    const unsigned ex = ((unsigned)__double2hiint(w) >> 20) & 0x7ffu;
+    if (ex - 123u > 1800u) return rquot_divide(a, w);
+    const double r = rcp64(w);
+    const double q = a * r;
+    if ((((unsigned)__double2hiint(q) >> 20) & 0x7ffu) == 0x7ffu) return q;
+    return fma(fma(-q, w, a), r, q);
+}
 
 // Source terms of a group system (Eold, the emission, Fold, the boundary inflows) and its
 // solution (E, F) in the pair form are held scaled by 2^-ks, ks the group's largest source
@@ -183,27 +198,32 @@ __device__ inline void cell_row(const LoCtx &x, int q, int i, R &Ap, R &Dp, int 
     }
 }
 
-// Solve system q with one warp.  sm: 6 * 32 * mmax values of R for this warp.
-// Writes E, F, Eb0, EbX of system q.
-//   phase A (all lanes, coalesced over cells/faces): face coefficients PL, PR, GD and the
-//           row parts dx/dt + dx a, dx s + dx Eold/dt, stored in the chunk layout
-//           [row-in-chunk][lane] so that phase B reads conflict free;
-//   phase B (each lane its chunk): modified Thomas down and up the chunk;
-//   phase C (warp): parallel cyclic reduction of the 2 x 32 chunk-boundary rows;
-//   phase D (each lane): back substitution, then the fluxes of its faces.
+// The layout of a system's rows in shared memory: P chunks, chunk l the rows l n / P ..
+// (l + 1) n / P - 1, its row k in slot k LP + l; face i shares the slot of row i, face n has
+// the slot after all others.  LP is odd in units of 8 so that the staging's stores (threads
+// along the rows) spread over the banks.
+struct TriLayout {
+    int P, LP, S;   // chunks, slots per row-in-chunk, slots
+};
+__host__ __device__ inline TriLayout tri_layout(int n)
+{
+    TriLayout t;
+    t.P = n / 2 < 128 ? n / 2 : 128;
+    if (t.P < 1) t.P = 1;
+    t.LP = (t.P + 31) / 32 * 32 + 8;
+    t.S = t.LP * ((n + t.P - 1) / t.P) + 1;
+    return t;
+}
 
-// Phase A for system q by `nthr` cooperating threads (index `t`): face coefficients and
-// row parts into the chunk layout.  n >= 2.
+// The face coefficients PL, PR, GD and the row parts dx/dt + dx a, dx s + dx Eold/dt of
+// system q into the layout by `nthr` cooperating threads (index `t`).  n >= 2.
 template <typename R>
-__device__ void lo_stage(const LoCtx &x, int q, R *sm, int mmax, int t, int nthr, int ks = 0)
+__device__ void lo_stage(const LoCtx &x, int q, R *sm, int S, int t, int nthr, int ks = 0)
 {
     const int n = x.nx;
-    const int S = 32 * mmax;
     R *PLc = sm, *PRc = sm + S, *GDc = sm + 2 * S, *Ap = sm + 3 * S, *Dp = sm + 5 * S;
     for (int f = t; f <= n; f += nthr) {
-        // slot k * 32 + l (chunk l = the lane whose rows hold f, row k of the chunk;
-        // face n after the last chunk's last row): a table built with the problem
-        const int o = x.lo_slot[f];
+        const int o = x.lo_slot[f];   // TriLayout's slots: a table built with the problem
         R PL, PR, GD;
         face_coef<R>(x, q, f, PL, PR, GD, ks);
         PLc[o] = PL;
@@ -213,7 +233,7 @@ __device__ void lo_stage(const LoCtx &x, int q, R *sm, int mmax, int t, int nthr
     }
 }
 
-// Phase A in the pair form by the CTA (t = threadIdx.x), with the group's source scale
+// The same in the pair form by the CTA (t = threadIdx.x), with the group's source scale
 // (src_in): pass 1 forms the coefficients PL, PR, Ap and the face factor W of Fold (a 7th
 // array after the six of the solve) and parks the raw FP64 sources in slots the
 // elimination fills later (Fold in GD's, Eold in Dp's, the emission in Cp's) while it
@@ -221,10 +241,9 @@ __device__ void lo_stage(const LoCtx &x, int q, R *sm, int mmax, int t, int nthr
 // sources at that scale into GD and Dp (the boundary faces are formed again whole, with
 // their inflow terms).  Each slot is written and read again by one thread, so only the
 // reduction needs a barrier.  Returns ks.  n >= 2.
-__device__ int lo_stage_pair(const LoCtx &x, int q, fpair *sm, int mmax)
+__device__ int lo_stage_pair(const LoCtx &x, int q, fpair *sm, int S)
 {
     const int n = x.nx;
-    const int S = 32 * mmax;
     const int t = threadIdx.x, nthr = blockDim.x;
     fpair *PLc = sm, *PRc = sm + S, *GDc = sm + 2 * S, *Ap = sm + 3 * S, *Cp = sm + 4 * S,
           *Dp = sm + 5 * S, *Wc = sm + 6 * S;
@@ -281,38 +300,43 @@ __device__ int lo_stage_pair(const LoCtx &x, int q, fpair *sm, int mmax)
     return ks;
 }
 
-// Phases B-D of one system by one warp on the staged arrays in sm: the solution x ends in
-// the Dp array (chunk layout); nothing is written to global memory.  n >= 2.
+// One system on the staged arrays in sm (PL, PR, GD, Ap, Cp, Dp of y.S slots each; rb: 3 P
+// more) by the whole block, of which the first P threads work: the solution x ends in Dp.
+// n >= 2; ends with a barrier.
+//   - chunks: rows normalised, row 0 of a chunk coupled to the last unknown of the chunk before
+//     and its own last, the others to the chunk's first and last;
+//   - the last rows are eliminated (a row needs its neighbours' three values: one exchange
+//     through rb), then every other first row at strides 1, 2 until 32 or fewer are left;
+//   - parallel cyclic reduction of those by warp 0 (rows kept with unit diagonals: one
+//     reciprocal per row and level);
+//   - back substitution.
+// On the chain of one thread: 13 operations per chunk row (4 rows at n = 500), 12 per
+// elimination step (3 + 5 there), about 170 in all, where one warp with 16-row chunks and
+// PCR of 64 rows took 430; the operations in all are the same.  Measured against that one-warp
+// form, 500 cells: 16 groups FP64 30.5 -> 20.3 us, 1024 groups FP64 (FP64-bound) 60 -> 61,
+// 1024 groups pair (latency-bound) 41.8 -> 32.2; the grey kernel (four warps with 256 rows of
+// PCR before) 23.0 -> 16.4.
 template <typename R>
-__device__ void tri_solve(R *sm, int n, int mmax)
+__device__ void tri_solve(R *sm, R *rb, int n, const TriLayout &y)
 {
-    const int lane = threadIdx.x & 31;
-    const int P = min(32, n / 2);
-    const bool act = lane < P;
-    const int r0 = act ? (lane * n) / P : n;
-    const int r1 = act ? ((lane + 1) * n) / P : n;
-    const int m = r1 - r0;
-    const int S = 32 * mmax;
+    const int t = threadIdx.x, P = y.P, S = y.S, LP = y.LP;
     R *PLc = sm, *PRc = sm + S, *GDc = sm + 2 * S;
     R *Ap = sm + 3 * S, *Cp = sm + 4 * S, *Dp = sm + 5 * S;
-#define CH(arr, k, l) arr[(k) * 32 + (l)]
-
-    R x0 = 0, x1 = 0;
-    R A0r = 0, C0r = 0, D0r = 0, A1r = 0, C1r = 0, D1r = 0;   // reduced rows
+    R *rA = rb, *rC = rb + P, *rD = rb + 2 * P;
+    const bool act = t < P;
+    const int r0 = act ? (t * n) / P : n;
+    const int r1 = act ? ((t + 1) * n) / P : n;
+    const int m = r1 - r0;
+    R A0 = 0, C0 = 0, D0 = 0, A1 = 0, C1 = 0, D1 = 0;   // the chunk's first and last row
     if (act) {
-        // ---- phase B: rows r0..r1-1, each normalised, coupled to x_{r0} and x_{k+1} ----
-        R PLi = CH(PLc, 0, lane), PRi = CH(PRc, 0, lane), GDi = CH(GDc, 0, lane);
+        R PLi = PLc[t], PRi = PRc[t], GDi = GDc[t];
         R ap = 0, cp = 0, dp = 0;
         for (int k = 0; k < m; ++k) {
-            const int i = r0 + k;
-            R PL1, PR1, GD1;
-            if (k + 1 < m || lane == P - 1) {
-                PL1 = CH(PLc, k + 1, lane); PR1 = CH(PRc, k + 1, lane); GD1 = CH(GDc, k + 1, lane);
-            } else {
-                PL1 = CH(PLc, 0, lane + 1); PR1 = CH(PRc, 0, lane + 1); GD1 = CH(GDc, 0, lane + 1);
-            }
-            const R di = CH(Ap, k, lane) + PL1 + PRi;
-            const R rh = CH(Dp, k, lane) - GD1 + GDi;
+            const int i = r0 + k, o = k * LP + t;
+            const int on = (k + 1 < m) ? o + LP : (t + 1 < P) ? t + 1 : S - 1;   // face i + 1
+            const R PL1 = PLc[on], PR1 = PRc[on], GD1 = GDc[on];
+            const R di = Ap[o] + PL1 + PRi;
+            const R rh = Dp[o] - GD1 + GDi;
             const R lo = (i > 0) ? -PLi : (R)0;
             const R up = (i < n - 1) ? -PR1 : (R)0;
             if (k < 2) {
@@ -326,151 +350,117 @@ __device__ void tri_solve(R *sm, int n, int mmax)
                 ap = -r * lo * ap;
                 cp = r * up;
             }
-            CH(Ap, k, lane) = ap;
-            CH(Cp, k, lane) = cp;
-            CH(Dp, k, lane) = dp;
+            if (k == 0) { A0 = ap; C0 = cp; D0 = dp; }
+            Ap[o] = ap;
+            Cp[o] = cp;
+            Dp[o] = dp;
             PLi = PL1;
             PRi = PR1;
             GDi = GD1;
         }
-        // backward: rows k = m-3..1 coupled to x_{r0} and x_{r1-1}
+        A1 = ap; C1 = cp; D1 = dp;
+        // upwards: rows m-3 .. 1 coupled to the chunk's first and last unknown
         if (m >= 3) {
+            const int o2 = (m - 2) * LP + t;
+            R a = Ap[o2], c = Cp[o2], d = Dp[o2];   // the row below
             for (int k = m - 3; k >= 1; --k) {
-                const R ck = CH(Cp, k, lane);
-                CH(Dp, k, lane) = CH(Dp, k, lane) - ck * CH(Dp, k + 1, lane);
-                CH(Ap, k, lane) = CH(Ap, k, lane) - ck * CH(Ap, k + 1, lane);
-                CH(Cp, k, lane) = -ck * CH(Cp, k + 1, lane);
+                const int o = k * LP + t;
+                const R ck = Cp[o];
+                d = Dp[o] - ck * d;
+                a = Ap[o] - ck * a;
+                c = -ck * c;
+                Dp[o] = d;
+                Ap[o] = a;
+                Cp[o] = c;
             }
-            const R c0 = CH(Cp, 0, lane);
-            const R r = rcpR<R>((R)1 - c0 * CH(Ap, 1, lane));
-            CH(Dp, 0, lane) = r * (CH(Dp, 0, lane) - c0 * CH(Dp, 1, lane));
-            CH(Ap, 0, lane) = r * CH(Ap, 0, lane);
-            CH(Cp, 0, lane) = -r * c0 * CH(Cp, 1, lane);
+            const R r = rcpR<R>((R)1 - C0 * a);
+            D0 = r * (D0 - C0 * d);
+            A0 = r * A0;
+            C0 = -r * C0 * c;
         }
-        A0r = CH(Ap, 0, lane); C0r = CH(Cp, 0, lane); D0r = CH(Dp, 0, lane);
-        A1r = CH(Ap, m - 1, lane); C1r = CH(Cp, m - 1, lane); D1r = CH(Dp, m - 1, lane);
+        rA[t] = A1;
+        rC[t] = C1;
+        rD[t] = D1;
     }
-    // ---- phase C: reduced system rows (first_l, last_l), l = 0..31, PCR with shuffles ----
-    // Every row is kept with a unit diagonal (the reduced rows of phase B already are):
-    // a level eliminates the neighbours at distance s with the factors -A and -C, then
-    // divides the row by its new diagonal -- one reciprocal per row and level instead of
-    // one per neighbour, and no diagonals to exchange.
-    {
-        if (!act) { A0r = C0r = D0r = A1r = C1r = D1r = 0; }
-        const unsigned full = 0xffffffffu;
-        for (int s = 1; s < 64; s <<= 1) {
-            R lA0, lC0, lD0, uA0, uC0, uD0;   // neighbours of slot 0 (unit diagonals)
-            R lA1, lC1, lD1, uA1, uC1, uD1;   // neighbours of slot 1
-            if (s == 1) {
-                R tA = shfl_up(full, A1r, 1), tC = shfl_up(full, C1r, 1);
-                R tD = shfl_up(full, D1r, 1);
-                R vA = shfl_down(full, A0r, 1), vC = shfl_down(full, C0r, 1);
-                R vD = shfl_down(full, D0r, 1);
-                if (lane >= 1) { lA0 = tA; lC0 = tC; lD0 = tD; }
-                else { lA0 = 0; lC0 = 0; lD0 = 0; }
-                uA0 = A1r; uC0 = C1r; uD0 = D1r;
-                lA1 = A0r; lC1 = C0r; lD1 = D0r;
-                if (lane <= 30) { uA1 = vA; uC1 = vC; uD1 = vD; }
-                else { uA1 = 0; uC1 = 0; uD1 = 0; }
-            } else {
-                const int t = s >> 1;
-                R a0 = shfl_up(full, A0r, t), c0 = shfl_up(full, C0r, t);
-                R d0 = shfl_up(full, D0r, t);
-                R a1 = shfl_up(full, A1r, t), c1 = shfl_up(full, C1r, t);
-                R d1 = shfl_up(full, D1r, t);
-                R e0 = shfl_down(full, A0r, t), g0 = shfl_down(full, C0r, t);
-                R h0 = shfl_down(full, D0r, t);
-                R e1 = shfl_down(full, A1r, t), g1 = shfl_down(full, C1r, t);
-                R h1 = shfl_down(full, D1r, t);
-                if (lane >= t) {
-                    lA0 = a0; lC0 = c0; lD0 = d0;
-                    lA1 = a1; lC1 = c1; lD1 = d1;
-                } else {
-                    lA0 = lA1 = 0; lC0 = lC1 = 0; lD0 = lD1 = 0;
-                }
-                if (lane + t <= 31) {
-                    uA0 = e0; uC0 = g0; uD0 = h0;
-                    uA1 = e1; uC1 = g1; uD1 = h1;
-                } else {
-                    uA0 = uA1 = 0; uC0 = uC1 = 0; uD0 = uD1 = 0;
-                }
-            }
-            {
-                const R al = -A0r, ga = -C0r;
-                const R r = rcpR<R>((R)1 + al * lC0 + ga * uA0);
-                const R nA = al * lA0, nC = ga * uC0, nD = D0r + al * lD0 + ga * uD0;
-                A0r = nA * r; C0r = nC * r; D0r = nD * r;
-            }
-            {
-                const R al = -A1r, ga = -C1r;
-                const R r = rcpR<R>((R)1 + al * lC1 + ga * uA1);
-                const R nA = al * lA1, nC = ga * uC1, nD = D1r + al * lD1 + ga * uD1;
-                A1r = nA * r; C1r = nC * r; D1r = nD * r;
-            }
-        }
-        x0 = D0r;
-        x1 = D1r;
-    }
-    // ---- phase D: back substitution (E into Dp), then the fluxes ----
+    __syncthreads();
+    R lA = 0, lC = 0, lD = 0;   // the last row of the chunk before
+    if (act && t > 0) { lA = rA[t - 1]; lC = rC[t - 1]; lD = rD[t - 1]; }
+    __syncthreads();
+    // row j with unit diagonal between rows l and u: A, C, D of the row at twice the distance
+    const auto step = [](R &A, R &C, R &D, R lA, R lC, R lD, R uA, R uC, R uD) {
+        const R al = -A, ga = -C;
+        const R r = rcpR<R>((R)1 + al * lC + ga * uA);
+        A = al * lA * r;
+        C = ga * uC * r;
+        D = (D + al * lD + ga * uD) * r;
+    };
     if (act) {
-        for (int k = 1; k < m - 1; ++k)
-            CH(Dp, k, lane) = CH(Dp, k, lane) - CH(Ap, k, lane) * x0 - CH(Cp, k, lane) * x1;
-        CH(Dp, 0, lane) = x0;
-        CH(Dp, m - 1, lane) = x1;
+        step(A0, C0, D0, lA, lC, lD, A1, C1, D1);
+        rA[t] = A0;
+        rC[t] = C0;
+        rD[t] = D0;
     }
-    __syncwarp();
-#undef CH
-}
-
-// The outputs of system q from the solution in the Dp array and the face coefficients:
-// E, F (F_f = GD_f + PL_f E_{f-1} - PR_f E_f) and the boundary face energies.  n >= 2.
-template <typename R>
-__device__ void lo_outputs(const LoCtx &x, int q, R *sm, int mmax, int ks = 0)
-{
-    const int lane = threadIdx.x & 31;
-    const int n = x.nx;
-    double *E = x.L.E + (size_t)q * n;
-    double *F = x.L.F + (size_t)q * (n + 1);
-    const int P = min(32, n / 2);
-    const bool act = lane < P;
-    const int r0 = act ? (lane * n) / P : n;
-    const int r1 = act ? ((lane + 1) * n) / P : n;
-    const int m = r1 - r0;
-    const int S = 32 * mmax;
-    R *PLc = sm, *PRc = sm + S, *GDc = sm + 2 * S;
-    R *Ap = sm + 3 * S, *Cp = sm + 4 * S, *Dp = sm + 5 * S;
-#define CH(arr, k, l) arr[(k) * 32 + (l)]
-
-    if (act)
-        for (int k = 0; k < m; ++k) E[r0 + k] = sol_out<R>(CH(Dp, k, lane), ks);
-    if (act) {
-        const int mprev = (lane > 0) ? r0 - ((lane - 1) * n) / P : 0;
-        const R Eleft0 = (lane > 0) ? CH(Dp, mprev - 1, lane - 1) : (R)0;
-        const int kend = (lane == P - 1) ? m : m - 1;
-        for (int k = 0; k <= kend; ++k) {
-            const int f = r0 + k;
-            R Fv = CH(GDc, k, lane);
-            if (f > 0) Fv += CH(PLc, k, lane) * ((k == 0) ? Eleft0 : CH(Dp, k - 1, lane));
-            if (f < n) Fv -= CH(PRc, k, lane) * CH(Dp, k, lane);
-            const double Fd = sol_out<R>(Fv, ks);
-            F[f] = Fd;
-            if (f == 0) x.L.Eb0[q] = x.L.Ein0[q] + (Fd - x.L.Fin0[q]) / (kC * x.L.C0[q]);
-            if (f == n) x.L.EbX[q] = x.L.EinX[q] + (Fd - x.L.FinX[q]) / (kC * x.L.CX[q]);
+    __syncthreads();
+    int s = 1;   // stride of the first rows still in play
+    for (; (P + s - 1) / s > 32; s <<= 1) {
+        const int j = t * 2 * s;
+        if (j < P) {
+            R A = rA[j], C = rC[j], D = rD[j];
+            const bool hl = j > 0, hu = j + s < P;
+            step(A, C, D, hl ? rA[j - s] : (R)0, hl ? rC[j - s] : (R)0, hl ? rD[j - s] : (R)0,
+                 hu ? rA[j + s] : (R)0, hu ? rC[j + s] : (R)0, hu ? rD[j + s] : (R)0);
+            rA[j] = A;   // no other thread reads row j: its neighbours are odd multiples of s
+            rC[j] = C;
+            rD[j] = D;
         }
+        __syncthreads();
     }
-#undef CH
+    if (t < 32) {
+        const int nr = (P + s - 1) / s, j = t * s;
+        R A = 0, C = 0, D = 0;
+        if (t < nr) { A = rA[j]; C = rC[j]; D = rD[j]; }
+        for (int d = 1; d < nr; d <<= 1) {
+            R pA = shfl_up(0xffffffffu, A, d), pC = shfl_up(0xffffffffu, C, d), pD = shfl_up(0xffffffffu, D, d);
+            R uA = shfl_down(0xffffffffu, A, d), uC = shfl_down(0xffffffffu, C, d), uD = shfl_down(0xffffffffu, D, d);
+            if (t < d) { pA = 0; pC = 0; pD = 0; }
+            if (t + d > 31) { uA = 0; uC = 0; uD = 0; }
+            step(A, C, D, pA, pC, pD, uA, uC, uD);
+        }
+        if (t < nr) rD[j] = D;
+    }
+    __syncthreads();
+    for (s >>= 1; s >= 1; s >>= 1) {   // the eliminated first rows, odd multiples of s
+        const int j = t * 2 * s + s;
+        if (j < P) {
+            R D = rD[j] - rA[j] * rD[j - s];
+            if (j + s < P) D = D - rC[j] * rD[j + s];
+            rD[j] = D;
+        }
+        __syncthreads();
+    }
+    if (act) {
+        const R x0 = rD[t];
+        R x1 = D1 - A1 * x0;
+        if (t + 1 < P) x1 = x1 - C1 * rD[t + 1];
+        Dp[t] = x0;
+        for (int k = 1; k < m - 1; ++k) {
+            const int o = k * LP + t;
+            Dp[o] = Dp[o] - Ap[o] * x0 - Cp[o] * x1;
+        }
+        Dp[(m - 1) * LP + t] = x1;
+    }
+    __syncthreads();
 }
 
 // The outputs of system q by every thread of the CTA, from the solution (chunk layout, in
 // the Dp array) and the face coefficients: consecutive threads take consecutive cells and
-// faces (coalesced stores), each slot found through the slot table.  The boundary face
-// energies as in lo_outputs (the pair form in pair arithmetic, at the source scale).
-// n >= 2; called after a barrier that follows the elimination.
+// faces (coalesced stores), each slot found through the slot table: F_f = GD_f + PL_f
+// E_{f-1} - PR_f E_f, and the boundary face energies (the pair form in pair arithmetic, at
+// the source scale).  n >= 2; called after a barrier that follows the elimination.
 template <typename R>
-__device__ void lo_outputs_cta(const LoCtx &x, int q, const R *sm, int mmax, int ks)
+__device__ void lo_outputs_cta(const LoCtx &x, int q, const R *sm, int S, int ks)
 {
     const int n = x.nx;
-    const int S = 32 * mmax;
     const R *PLc = sm, *PRc = sm + S, *GDc = sm + 2 * S, *Dp = sm + 5 * S;
     double *E = x.L.E + (size_t)q * n;
     double *F = x.L.F + (size_t)q * (n + 1);
@@ -493,55 +483,30 @@ __device__ void lo_outputs_cta(const LoCtx &x, int q, const R *sm, int mmax, int
                 Eb = pr_join(src_in<R>(Ein, ks) +
                                  (Fv - src_in<R>(Fin, ks)) * rcpR<R>((R)kC * (R)Cb), ks);
             else
-                Eb = Ein + ((double)Fv - Fin) / (kC * Cb);
+                Eb = Ein + rquot((double)Fv - Fin, kC * Cb);
             (f == 0 ? x.L.Eb0 : x.L.EbX)[q] = Eb;
         }
     }
 }
 
-// staged = true: phase A already done (by the whole block) for n >= 2.
+// One cell: the system is one equation, solved by one thread.
 template <typename R>
-__device__ void warp_lo_solve(const LoCtx &x, int q, R *sm, int mmax, bool staged = false,
-                              int ks = 0)
+__device__ void lo_one_cell(const LoCtx &x, int q, int ks = 0)
 {
-    const int lane = threadIdx.x & 31;
-    const int n = x.nx;
-    double *E = x.L.E + (size_t)q * n;
-    double *F = x.L.F + (size_t)q * (n + 1);
-
-    if (n == 1) {
-        if (lane == 0) {
-            R PL0, PR0, GD0, PL1, PR1, GD1, Ap0, Dp0;
-            face_coef<R>(x, q, 0, PL0, PR0, GD0, ks);
-            face_coef<R>(x, q, 1, PL1, PR1, GD1, ks);
-            cell_row<R>(x, q, 0, Ap0, Dp0, ks);
-            R di = Ap0 + PL1 + PR0;
-            R rh = Dp0 - GD1 + GD0;
-            R e0 = rh / di;
-            E[0] = sol_out<R>(e0, ks);
-            R F0 = GD0 - PR0 * e0, F1 = GD1 + PL1 * e0;
-            const double F0d = sol_out<R>(F0, ks), F1d = sol_out<R>(F1, ks);
-            F[0] = F0d;
-            F[1] = F1d;
-            x.L.Eb0[q] = x.L.Ein0[q] + (F0d - x.L.Fin0[q]) / (kC * x.L.C0[q]);
-            x.L.EbX[q] = x.L.EinX[q] + (F1d - x.L.FinX[q]) / (kC * x.L.CX[q]);
-        }
-        return;
-    }
-
-    // ---- phase A ----
-    if (!staged) lo_stage<R>(x, q, sm, mmax, lane, 32, ks);
-    __syncwarp();
-
-    tri_solve<R>(sm, n, mmax);
-    lo_outputs<R>(x, q, sm, mmax, ks);
-#undef CH
-}
-
-__host__ __device__ inline int lo_mmax(int nx)
-{
-    const int P = nx / 2 < 32 ? nx / 2 : 32;
-    return nx < 2 ? 1 : (nx + P - 1) / P + 1;
+    double *E = x.L.E + q, *F = x.L.F + 2 * (size_t)q;
+    R PL0, PR0, GD0, PL1, PR1, GD1, Ap0, Dp0;
+    face_coef<R>(x, q, 0, PL0, PR0, GD0, ks);
+    face_coef<R>(x, q, 1, PL1, PR1, GD1, ks);
+    cell_row<R>(x, q, 0, Ap0, Dp0, ks);
+    const R di = Ap0 + PL1 + PR0;
+    const R rh = Dp0 - GD1 + GD0;
+    const R e0 = rh / di;
+    E[0] = sol_out<R>(e0, ks);
+    const double F0d = sol_out<R>(GD0 - PR0 * e0, ks), F1d = sol_out<R>(GD1 + PL1 * e0, ks);
+    F[0] = F0d;
+    F[1] = F1d;
+    x.L.Eb0[q] = x.L.Ein0[q] + (F0d - x.L.Fin0[q]) / (kC * x.L.C0[q]);
+    x.L.EbX[q] = x.L.EinX[q] + (F1d - x.L.FinX[q]) / (kC * x.L.CX[q]);
 }
 
 // FP32 group solve refined to FP64 accuracy (mixed-precision iterative refinement).  The
@@ -552,116 +517,91 @@ __host__ __device__ inline int lo_mmax(int nx)
 // cond(A) eps_32 (the plain FP32 solve's error: 3.6e-6 in T on fc_1024, ~5e-5 in E on a
 // 1000-cell random level, where one step left 2.6e-9); the eliminations, the part that is
 // serial in cells, run on the FP32 pipes.
-// Shared memory: 6 S doubles + 6 S floats (S = 32 mmax).
+// Shared memory: 6 S doubles, 6 S + 3 P floats.
 constexpr int kLoRefine = 2;
 
-__device__ void lo_solve_refined(const LoCtx &x, int q, int sw)
+__device__ void lo_solve_refined(const LoCtx &x, int q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = x.nx;
-    const int mmax = lo_mmax(n);
-    const int S = 32 * mmax;
-    double *s64 = reinterpret_cast<double *>(smem_raw);
-    float *s32 = reinterpret_cast<float *>(s64 + 6 * S);
+    const int n = x.nx, t = threadIdx.x, nthr = blockDim.x;
     if (n < 2) {   // one cell: the FP64 form
-        if (threadIdx.x < 32) warp_lo_solve<double>(x, q, s64, mmax, false);
+        if (t == 0) lo_one_cell<double>(x, q);
         return;
     }
-    lo_stage<double>(x, q, s64, mmax, threadIdx.x, blockDim.x);
-    __syncthreads();
-    if ((int)(threadIdx.x >> 5) != (sw & ((int)(blockDim.x >> 5) - 1))) return;
-    const int lane = threadIdx.x & 31;
+    const TriLayout y = tri_layout(n);
+    const int S = y.S;
+    double *s64 = reinterpret_cast<double *>(smem_raw);
+    float *s32 = reinterpret_cast<float *>(s64 + 6 * S);
     const double *PL = s64, *PR = s64 + S, *GD = s64 + 2 * S, *Ap = s64 + 3 * S;
-    double *X0 = s64 + 4 * S;   // x0 in FP64 (the unused Cp slot of s64)
+    double *X0 = s64 + 4 * S;   // the solution in FP64 (the unused Cp array of s64)
     double *Dp = s64 + 5 * S;   // right-hand sides, then E
-    float *pl = s32, *pr = s32 + S, *gd = s32 + 2 * S, *ap = s32 + 3 * S, *cp = s32 + 4 * S,
-          *dp = s32 + 5 * S;
-    for (int o = lane; o < S; o += 32) {
+    float *pl = s32, *pr = s32 + S, *gd = s32 + 2 * S, *ap = s32 + 3 * S, *dp = s32 + 5 * S;
+    lo_stage<double>(x, q, s64, S, t, nthr);
+    for (int f = t; f <= n; f += nthr) {   // the slots this thread staged
+        const int o = x.lo_slot[f];
         pl[o] = (float)PL[o];
         pr[o] = (float)PR[o];
         gd[o] = (float)GD[o];
-        ap[o] = (float)Ap[o];
-        dp[o] = (float)Dp[o];
+        if (f < n) {
+            ap[o] = (float)Ap[o];
+            dp[o] = (float)Dp[o];
+        }
     }
-    __syncwarp();
-    tri_solve<float>(s32, n, mmax);   // x0 in dp
-    const int P = min(32, n / 2);
-    const bool act = lane < P;
-    const int r0 = act ? (lane * n) / P : n;
-    const int m = act ? ((lane + 1) * n) / P - r0 : 0;
-#define CH(arr, k, l) arr[(k) * 32 + (l)]
-    for (int k = 0; k < m; ++k) CH(X0, k, lane) = (double)CH(dp, k, lane);
-    __syncwarp();
+    __syncthreads();
+    tri_solve<float>(s32, s32 + 6 * S, n, y);   // x0 in dp
+    for (int i = t; i < n; i += nthr) X0[x.lo_slot[i]] = (double)dp[x.lo_slot[i]];
+    __syncthreads();
     for (int step = 0; step < kLoRefine; ++step) {
-        // residual of row i = r0 + k (face i+1 is the next slot of the chunk, or the first
-        // slot of the next chunk; the last chunk keeps face n in its slot m):
+        // the correction system: the same matrix (its FP32 diagonal parts again: the
+        // elimination overwrote them), the residual of row i as right-hand side, no face
+        // sources:
         //   r = (Dp_i - GD_{i+1} + GD_i) - (Ap_i + PL_{i+1} + PR_i) x_i
         //       + PL_i x_{i-1} + PR_{i+1} x_{i+1}
-        for (int k = 0; k < m; ++k) {
-            const int i = r0 + k;
-            const bool wrap = (k + 1 == m) && lane != P - 1;
-            const int kn = wrap ? 0 : k + 1, ln = wrap ? lane + 1 : lane;
-            const double di = CH(Ap, k, lane) + CH(PL, kn, ln) + CH(PR, k, lane);
-            const double rh = CH(Dp, k, lane) - CH(GD, kn, ln) + CH(GD, k, lane);
-            double r = rh - di * CH(X0, k, lane);
-            if (i > 0) {
-                const int mp = (k > 0) ? 0 : r0 - ((lane - 1) * n) / P;   // rows of the chunk before
-                r = fma(CH(PL, k, lane), (k > 0) ? CH(X0, k - 1, lane) : CH(X0, mp - 1, lane - 1), r);
-            }
-            if (i < n - 1) r = fma(CH(PR, kn, ln), CH(X0, kn, ln), r);
-            CH(cp, k, lane) = (float)r;
+        for (int i = t; i <= n; i += nthr) {
+            const int o = x.lo_slot[i];
+            gd[o] = 0.f;
+            if (i == n) break;
+            const int on = x.lo_slot[i + 1];
+            const double di = Ap[o] + PL[on] + PR[o];
+            const double rh = Dp[o] - GD[on] + GD[o];
+            double r = rh - di * X0[o];
+            if (i > 0) r = fma(PL[o], X0[x.lo_slot[i - 1]], r);
+            if (i < n - 1) r = fma(PR[on], X0[on], r);
+            ap[o] = (float)Ap[o];
+            dp[o] = (float)r;
         }
-        __syncwarp();
-        // the correction system: the same matrix (its FP32 diagonal parts again: the
-        // elimination overwrote them), right-hand side r, no face sources
-        for (int k = 0; k <= m; ++k) {
-            if (k < m) {
-                CH(ap, k, lane) = (float)CH(Ap, k, lane);
-                CH(dp, k, lane) = CH(cp, k, lane);
-            }
-            if (k < m || lane == P - 1) CH(gd, k, lane) = 0.f;
-        }
-        __syncwarp();
-        tri_solve<float>(s32, n, mmax);   // the correction in dp
-        for (int k = 0; k < m; ++k) CH(X0, k, lane) += (double)CH(dp, k, lane);
-        __syncwarp();
+        __syncthreads();
+        tri_solve<float>(s32, s32 + 6 * S, n, y);   // the correction in dp
+        for (int i = t; i < n; i += nthr) X0[x.lo_slot[i]] += (double)dp[x.lo_slot[i]];
+        __syncthreads();
     }
-    for (int k = 0; k < m; ++k) CH(Dp, k, lane) = CH(X0, k, lane);
-    __syncwarp();
-#undef CH
-    lo_outputs<double>(x, q, s64, mmax);
+    for (int i = t; i < n; i += nthr) Dp[x.lo_slot[i]] = X0[x.lo_slot[i]];
+    __syncthreads();
+    lo_outputs_cta<double>(x, q, s64, S, 0);
 }
 
-// One system per CTA: all 4 warps stage the rows (phase A: the parallel part, global
-// loads and the face coefficients), warp `sw` runs the elimination, and all 4 warps form
-// and store the outputs.  The CTA's four warps sit on the SM's four sub-partitions, each
-// with its own FP64 pipe; rotating the eliminating warp with the work item spreads the
-// serial chains of the CTAs resident on an SM over all four (always warp 0 would queue
-// them all on one).
+// One system per CTA of 128 threads: all stage the rows (global loads and the face
+// coefficients), eliminate, and form and store the outputs.
 template <typename R>
-__device__ void lo_solve_body(const LoCtx &x, int q, int sw)
+__device__ void lo_solve_body(const LoCtx &x, int q)
 {
     if constexpr (std::is_same<R, float>::value) {   // FP32 group solves: refined to FP64 accuracy
-        lo_solve_refined(x, q, sw);
+        lo_solve_refined(x, q);
         return;
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *sm = reinterpret_cast<R *>(smem_raw);
-    const int mmax = lo_mmax(x.nx);
-    const bool staged = x.nx >= 2;
-    const bool solver = (int)(threadIdx.x >> 5) == (sw & ((int)(blockDim.x >> 5) - 1));
-    if (staged) {
-        int ks = 0;
-        if constexpr (is_pair<R>) ks = lo_stage_pair(x, q, sm, mmax);
-        else lo_stage<R>(x, q, sm, mmax, threadIdx.x, blockDim.x);
+    int ks = 0;
+    if (x.nx >= 2) {
+        const TriLayout y = tri_layout(x.nx);
+        if constexpr (is_pair<R>) ks = lo_stage_pair(x, q, sm, y.S);
+        else lo_stage<R>(x, q, sm, y.S, threadIdx.x, blockDim.x);
         __syncthreads();
-        if (solver) tri_solve<R>(sm, x.nx, mmax);
-        __syncthreads();
-        lo_outputs_cta<R>(x, q, sm, mmax, ks);
+        tri_solve<R>(sm, sm + 6 * y.S, x.nx, y);
+        lo_outputs_cta<R>(x, q, sm, y.S, ks);
         return;
     }
-    int ks = 0;   // one cell: one lane (the pair form's source scale from every thread)
-    if constexpr (is_pair<R>) {
+    if constexpr (is_pair<R>) {   // one cell: one thread (the source scale from every thread)
         __shared__ int kw[32];
         int m = lo_src_exp(x, q, threadIdx.x, blockDim.x);
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -671,7 +611,7 @@ __device__ void lo_solve_body(const LoCtx &x, int q, int sw)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, kw[w]);
         ks = (m == 0) ? 0 : m - 1023;
     }
-    if (solver) warp_lo_solve<R>(x, q, sm, mmax, false, ks);
+    if (threadIdx.x == 0) lo_one_cell<R>(x, q, ks);
 }
 
 // 7 CTAs per SM (at most 72 registers): one wave of 1064 holds every group of a 1024-group
@@ -681,7 +621,7 @@ __global__ void __launch_bounds__(128, 7) k_lo_solve(LoCtx x)
 {
     griddep_wait();
     if (x.gate && *x.gate) return;   // the phase's inner loop has ended
-    lo_solve_body<R>(x, blockIdx.x, blockIdx.x);
+    lo_solve_body<R>(x, blockIdx.x);
 }
 
 template <typename R>
@@ -692,7 +632,7 @@ __global__ void __launch_bounds__(128) k_lo_solve_b(const int *__restrict__ meta
         int s, bx, by;
         if (!bdecode(meta, N, b, s, bx, by)) break;
         const LoCtx x = xs[s];
-        lo_solve_body<R>(x, bx, b);
+        lo_solve_body<R>(x, bx);
         __syncthreads();
     }
 }
@@ -774,20 +714,6 @@ enum { R_PHI, R_SIG, R_EMIS, R_E, R_SW, R_W, R_SF, R_F, R_EOLD, R_FOLD, R_ETAR, 
 constexpr int kRTile = 31;          // faces per position tile
 constexpr int kRTickets = 2432;     // ints at the head of the scratch (nt * n_to < 1216 there)
 constexpr int kRHead = kRTickets / 2;   // doubles
-
-// a/w: the refined reciprocal and one residual correction (the correctly rounded quotient
-// but for rare last bits).  The weights of cold cells are subnormal, where 1/w overflows and
-// a/w does not: an exponent outside +-900 divides, and a non-finite quotient is kept.
-static __device__ __noinline__ double rquot_divide(double a, double w) { return a / w; }
-__device__ inline double rquot(double a, double w)
-{
-    const unsigned ex = ((unsigned)__double2hiint(w) >> 20) & 0x7ffu;
-    if (ex - 123u > 1800u) return rquot_divide(a, w);
-    const double r = rcp64(w);
-    const double q = a * r;
-    if ((((unsigned)__double2hiint(q) >> 20) & 0x7ffu) == 0x7ffu) return q;
-    return fma(fma(-q, w, a), r, q);
-}
 
 // sums over members p = p0, p0 + step, .. < pe of lane position i (clamped by the caller);
 // kFine: S is the fine grid; kOld: Eold and Fold are summed too
@@ -1137,149 +1063,19 @@ __device__ inline void grey_newton_cell(const GreyArgs &a, const Level &g, int h
     grey_newton_terms(a, have_prev, i, g.sig[i], 2.0 * g.emis[i], g.Esum[i], sa, ss, sL);
 }
 
-// The grey level's tridiagonal system (n >= 2) by P = min(128, n/2, block) threads: GB300
-// runs a warp's FP64 instructions on its own sub-partition's FP64 pipe only, so the group
-// systems' one-warp partitioned elimination (32 chunks of ~16 rows: a serial chain of ~500
-// FP64 instructions at 64 cycles each) would keep the SM's other three pipes idle for
-// ~20 us on the grey level, where a single system is solved at a time.  Here every
-// thread eliminates a chunk of ~4 rows (the modified Thomas pass down and up the chunk of
-// tri_solve: rows coupled only to the chunk's first and last unknowns), the 2P chunk-
-// boundary rows are solved by parallel cyclic reduction in shared memory (rows kept with
-// unit diagonals, ceil(log2 2P) levels of one block barrier each), and every thread
-// back-substitutes its chunk's interior.  sm: PL, PR, GD [n + 1], Ap, Cp, Dp [n], then the
-// reduced rows' A, C, D in two buffers [2][3][2P].  All threads of the block call it; the
-// solution is left in Dp.
-__host__ __device__ inline int grey_chunks(int n, int block)
+// the grey level's outputs from the solution: E, the face fluxes F_f = GD_f + PL_f E_{f-1} -
+// PR_f E_f and the boundary face energies
+__device__ void grey_outputs(const LoCtx &x, const double *sm, int S, int n)
 {
-    int P = n / 2;
-    if (P > 128) P = 128;
-    if (P > block) P = block;
-    return P < 1 ? 1 : P;
-}
-
-__device__ void grey_tri_solve(const LoCtx &x, double *sm, int n)
-{
-    const int P = grey_chunks(n, (int)blockDim.x), nr = 2 * P;
-    double *PL = sm, *PR = PL + (n + 1), *GD = PR + (n + 1);
-    double *Ap = GD + (n + 1), *Cp = Ap + n, *Dp = Cp + n;
-    double *rb = Dp + n;   // [2][3][nr]
-    const int t = threadIdx.x;
-    for (int f = t; f <= n; f += blockDim.x) {
-        double pl, pr, gd;
-        face_coef<double>(x, 0, f, pl, pr, gd);
-        PL[f] = pl;
-        PR[f] = pr;
-        GD[f] = gd;
-        if (f < n) cell_row<double>(x, 0, f, Ap[f], Dp[f]);
-    }
-    __syncthreads();
-    const int r0 = (t < P) ? (int)(((long long)t * n) / P) : n;
-    const int r1 = (t < P) ? (int)(((long long)(t + 1) * n) / P) : n;
-    const int m = r1 - r0;
-    if (t < P) {
-        // down the chunk: row k >= 1 coupled to x_{r0} (a) and x_{r0+k+1} (c); row 0 to
-        // x_{r0-1} and x_{r0+1}
-        double PLi = PL[r0], PRi = PR[r0], GDi = GD[r0];
-        double ap = 0.0, cp = 0.0, dp = 0.0;
-        for (int k = 0; k < m; ++k) {
-            const int i = r0 + k;
-            const double PL1 = PL[i + 1], PR1 = PR[i + 1], GD1 = GD[i + 1];
-            const double di = Ap[i] + PL1 + PRi;
-            const double rh = Dp[i] - GD1 + GDi;
-            const double lo = (i > 0) ? -PLi : 0.0;
-            const double up = (i < n - 1) ? -PR1 : 0.0;
-            if (k < 2) {
-                const double r = rcp64(di);
-                ap = lo * r;
-                cp = up * r;
-                dp = rh * r;
-            } else {
-                const double r = rcp64(di - lo * cp);
-                dp = r * (rh - lo * dp);
-                ap = -r * lo * ap;
-                cp = r * up;
-            }
-            Ap[i] = ap;
-            Cp[i] = cp;
-            Dp[i] = dp;
-            PLi = PL1;
-            PRi = PR1;
-            GDi = GD1;
-        }
-        // up the chunk: rows 1 .. m-2 coupled to x_{r0} and x_{r1-1}; row 0 to x_{r0-1}
-        // and x_{r1-1}
-        if (m >= 3) {
-            for (int k = m - 3; k >= 1; --k) {
-                const int i = r0 + k;
-                const double ck = Cp[i];
-                Dp[i] = Dp[i] - ck * Dp[i + 1];
-                Ap[i] = Ap[i] - ck * Ap[i + 1];
-                Cp[i] = -ck * Cp[i + 1];
-            }
-            const double c0 = Cp[r0];
-            const double r = rcp64(1.0 - c0 * Ap[r0 + 1]);
-            Dp[r0] = r * (Dp[r0] - c0 * Dp[r0 + 1]);
-            Ap[r0] = r * Ap[r0];
-            Cp[r0] = -r * c0 * Cp[r0 + 1];
-        }
-        // reduced rows 2t (the chunk's first row) and 2t + 1 (its last)
-        rb[2 * t] = Ap[r0];
-        rb[nr + 2 * t] = Cp[r0];
-        rb[2 * nr + 2 * t] = Dp[r0];
-        rb[2 * t + 1] = Ap[r1 - 1];
-        rb[nr + 2 * t + 1] = Cp[r1 - 1];
-        rb[2 * nr + 2 * t + 1] = Dp[r1 - 1];
-    }
-    __syncthreads();
-    // parallel cyclic reduction of the 2P reduced rows: a level eliminates the neighbours at
-    // distance s with the factors -A and -C and divides by the new diagonal
-    int cur = 0;
-    for (int s = 1; s < nr; s <<= 1) {
-        const double *A = rb + (size_t)cur * 3 * nr, *C = A + nr, *D = C + nr;
-        double *nA = rb + (size_t)(cur ^ 1) * 3 * nr, *nC = nA + nr, *nD = nC + nr;
-        if (t < P) {
-#pragma unroll
-            for (int j = 2 * t; j <= 2 * t + 1; ++j) {
-                const bool hl = j >= s, hu = j + s < nr;
-                const double lA = hl ? A[j - s] : 0.0, lC = hl ? C[j - s] : 0.0;
-                const double lD = hl ? D[j - s] : 0.0;
-                const double uA = hu ? A[j + s] : 0.0, uC = hu ? C[j + s] : 0.0;
-                const double uD = hu ? D[j + s] : 0.0;
-                const double al = -A[j], ga = -C[j];
-                const double r = rcp64(1.0 + al * lC + ga * uA);
-                nA[j] = al * lA * r;
-                nC[j] = ga * uC * r;
-                nD[j] = (D[j] + al * lD + ga * uD) * r;
-            }
-        }
-        cur ^= 1;
-        __syncthreads();
-    }
-    // back substitution of the chunk's interior rows
-    if (t < P) {
-        const double *D = rb + (size_t)cur * 3 * nr + 2 * nr;
-        const double x0 = D[2 * t], x1 = D[2 * t + 1];
-        for (int k = 1; k < m - 1; ++k) {
-            const int i = r0 + k;
-            Dp[i] = Dp[i] - Ap[i] * x0 - Cp[i] * x1;
-        }
-        Dp[r0] = x0;
-        Dp[r1 - 1] = x1;
-    }
-    __syncthreads();
-}
-
-// the grey level's outputs from the solution in Dp (grey_tri_solve's layout): E, the face
-// fluxes F_f = GD_f + PL_f E_{f-1} - PR_f E_f and the boundary face energies
-__device__ void grey_outputs(const LoCtx &x, const double *sm, int n)
-{
-    const double *PL = sm, *PR = PL + (n + 1), *GD = PR + (n + 1);
-    const double *Dp = GD + (n + 1) + 2 * n;
+    const double *PL = sm, *PR = sm + S, *GD = sm + 2 * S, *Dp = sm + 5 * S;
     for (int f = threadIdx.x; f <= n; f += blockDim.x) {
-        if (f < n) x.L.E[f] = Dp[f];
-        double Fv = GD[f];
-        if (f > 0) Fv += PL[f] * Dp[f - 1];
-        if (f < n) Fv -= PR[f] * Dp[f];
+        const int o = x.lo_slot[f];
+        double Fv = GD[o];
+        if (f > 0) Fv += PL[o] * Dp[x.lo_slot[f - 1]];
+        if (f < n) {
+            x.L.E[f] = Dp[o];
+            Fv -= PR[o] * Dp[o];
+        }
         x.L.F[f] = Fv;
         if (f == 0) x.L.Eb0[0] = x.L.Ein0[0] + (Fv - x.L.Fin0[0]) * rcp64(kC * x.L.C0[0]);
         if (f == n) x.L.EbX[0] = x.L.EinX[0] + (Fv - x.L.FinX[0]) * rcp64(kC * x.L.CX[0]);
@@ -1321,7 +1117,7 @@ __device__ void grey_body(const GreyCtx &x)
     double *ss = sa + nx;        // source w Q* - (1-w) cv (T* - Told)/dt
     double *sL = ss + nx;        // 1 / Lambda
     double *red = sL + nx;       // [kGreyRed] block maxima
-    double *wsm = red + kGreyRed;   // solver scratch (grey_tri_solve)
+    double *wsm = red + kGreyRed;   // the solver's rows (TriLayout) and its 3 P values more
     const GreyArgs &a = x.a;
     const Level &g = x.lo.L;
     for (int i = threadIdx.x; i < nx; i += blockDim.x) {
@@ -1339,19 +1135,21 @@ __device__ void grey_body(const GreyCtx &x)
     LoCtx lc = x.lo;
     lc.a_cell = sa;
     lc.s_cell = ss;
-    const double *Esol = wsm + 3 * (size_t)(nx + 1) + 2 * (size_t)nx;   // grey_tri_solve's Dp
+    const TriLayout y = tri_layout(nx);
     if (nx >= 2) {
-        grey_tri_solve(lc, wsm, nx);
-        grey_outputs(lc, wsm, nx);
-    } else {
-        if (threadIdx.x < 32) warp_lo_solve<double>(lc, 0, wsm, x.mmax, false);
+        lo_stage<double>(lc, 0, wsm, y.S, threadIdx.x, blockDim.x);
         __syncthreads();
-        Esol = g.E;
+        tri_solve<double>(wsm, wsm + 6 * y.S, nx, y);
+        grey_outputs(lc, wsm, y.S, nx);
+    } else {
+        if (threadIdx.x == 0) lo_one_cell<double>(lc, 0);
+        __syncthreads();
     }
+    const double *Esol = nx >= 2 ? wsm + 5 * (size_t)y.S : g.E;
     // v: bad flag, max|T - Tcyc|, max|T|, max|E - Ecyc|, max|E|, max|T - Tphase|,
     // max|E - Ephase| as non-negative encodings (flags[0 .. 6])
     unsigned long long v[kGreyNV] = {};
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) grey_update_cell(a, g, i, sL[i], Esol[i], v);
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) grey_update_cell(a, g, i, sL[i], Esol[nx >= 2 ? lc.lo_slot[i] : i], v);
     block_max_bits(v, reinterpret_cast<unsigned long long *>(red));
     if (threadIdx.x == 0) {
         if (v[0] != 0ull) a.flags[0] = 1.0;
@@ -1530,19 +1328,16 @@ static size_t restrict_doubles(int nt, int n_to, int nchunk)
     return kRHead + (size_t)n_to * nchunk * (16 + (size_t)kRV * nt * 32);
 }
 
-// shared memory of one LO solve; the FP32 form with refinement keeps both copies of the
-// rows and falls back to the FP64 form where they do not fit (n_x above ~3100)
+// shared memory of one LO solve: the rows, the pair form's 7th array (the face factors of
+// Fold, free again when the solver wants its 3 P values), or the refined FP32 form's two
+// copies of the rows
 static size_t lo_smem(int precision, int nx)
 {
-    const size_t S = 32 * (size_t)lo_mmax(nx);
-    if (lo_fp32(precision) && 6 * S * (sizeof(double) + sizeof(float)) <= 227 * 1024)
-        return 6 * S * (sizeof(double) + sizeof(float));
-    if (lo_pair(precision)) return 7 * S * sizeof(double);   // + the face factors of Fold
-    return 6 * S * sizeof(double);
-}
-static bool lo_refined(int precision, int nx)
-{
-    return lo_fp32(precision) && 6 * 32 * (size_t)lo_mmax(nx) * 12 <= 227 * 1024;
+    const TriLayout y = tri_layout(nx);
+    const size_t S = y.S, rb = 3 * (size_t)y.P;
+    if (lo_fp32(precision)) return 6 * S * (sizeof(double) + sizeof(float)) + rb * sizeof(float);
+    if (lo_pair(precision)) return (6 * S + std::max(S, rb)) * sizeof(double);
+    return (6 * S + rb) * sizeof(double);
 }
 
 cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L)
@@ -1556,7 +1351,7 @@ cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L)
                                  (int)sm);
         if (e != cudaSuccess) return e;
         return launch_pdl(k_lo_solve<fpair>, dim3(nb), dim3(128), sm, p.stream, x);
-    } else if (!lo_refined(p.precision, p.nx)) {
+    } else if (!lo_fp32(p.precision)) {
         e = cudaFuncSetAttribute(k_lo_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sm);
         if (e != cudaSuccess) return e;
@@ -1579,7 +1374,7 @@ cudaError_t launch_lo_solve_b(int precision, int max_nx, const int *meta, int N,
                                  (int)sm);
         if (e != cudaSuccess) return e;
         k_lo_solve_b<fpair><<<grid, 128, sm, st>>>(meta, N, xs);
-    } else if (!lo_refined(precision, max_nx)) {
+    } else if (!lo_fp32(precision)) {
         e = cudaFuncSetAttribute(k_lo_solve_b<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sm);
         if (e != cudaSuccess) return e;
@@ -1619,6 +1414,15 @@ RestrictPlan restrict_plan(const Problem &p, int n_from, int n_to)
     }
     q.gy = q.mode == 0 ? (n_to + 3) / 4 : n_to * q.nchunk;
     return q;
+}
+
+// TriLayout's slots of the rows and faces 0 .. nx (uploaded with the problem)
+void lo_slots(int nx, int *slot)
+{
+    const TriLayout y = tri_layout(nx);
+    for (int l = 0; l < y.P; ++l)
+        for (int i = (l * nx) / y.P, k = 0; i < ((l + 1) * nx) / y.P; ++i, ++k) slot[i] = k * y.LP + l;
+    slot[nx] = y.S - 1;
 }
 
 size_t restrict_head_doubles() { return kRHead; }
@@ -1692,16 +1496,15 @@ GreyCtx make_grey_ctx(const Problem &p, const Level &g, const GreyArgs &a)
     GreyCtx x;
     x.lo = make_lo_ctx(p, a.dt, g);
     x.a = grey_args_ready(p, a);
-    x.mmax = lo_mmax(p.nx);
     return x;
 }
 
 static void grey_launch_shape(int nx, int &bs, size_t &sm)
 {
     bs = std::min(1024, std::max(32, (nx + 31) / 32 * 32));
-    // Newton terms, block maxima, then grey_tri_solve's rows and reduced rows
-    sm = sizeof(double) * (3 * (size_t)nx + kGreyRed + 3 * (size_t)(nx + 1) + 3 * (size_t)nx +
-                           6 * 256);
+    // at least the solver's chunks; Newton terms, block maxima, the solver's rows
+    const TriLayout y = tri_layout(nx);
+    sm = sizeof(double) * (3 * (size_t)nx + kGreyRed + 6 * (size_t)y.S + 3 * (size_t)y.P);
 }
 
 cudaError_t launch_grey(const Problem &p, const Level &g, const GreyArgs &a)
