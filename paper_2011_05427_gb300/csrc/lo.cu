@@ -614,10 +614,11 @@ __device__ void lo_solve_body(const LoCtx &x, int q)
     if (threadIdx.x == 0) lo_one_cell<R>(x, q, ks);
 }
 
-// 7 CTAs per SM (at most 72 registers): one wave of 1064 holds every group of a 1024-group
-// level
-template <typename R>
-__global__ void __launch_bounds__(128, 7) k_lo_solve(LoCtx x)
+// T threads.  128: 7 CTAs per SM (at most 72 registers), one wave of 1064 holds every group
+// of a 1024-group level.  512 and 256: levels of few groups, whose staging and outputs (loads
+// and ~60 operations per face) would be a chain of n/128 faces per thread; launch_lo_solve.
+template <typename R, int T>
+__global__ void __launch_bounds__(T, T == 128 ? 7 : T == 256 ? 3 : 1) k_lo_solve(LoCtx x)
 {
     griddep_wait();
     if (x.gate && *x.gate) return;   // the phase's inner loop has ended
@@ -1340,28 +1341,30 @@ static size_t lo_smem(int precision, int nx)
     return (6 * S + rb) * sizeof(double);
 }
 
+template <typename R, int T>
+static cudaError_t lo_launch(const LoCtx &x, unsigned nb, size_t sm, cudaStream_t st)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_lo_solve<R, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sm);
+    return e != cudaSuccess ? e : launch_pdl(k_lo_solve<R, T>, dim3(nb), dim3(T), sm, st, x);
+}
+
 cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L)
 {
     const LoCtx x = make_lo_ctx(p, dt, L);
     const size_t sm = lo_smem(p.precision, p.nx);
-    const unsigned nb = (unsigned)L.n;
-    cudaError_t e;
-    if (lo_pair(p.precision)) {
-        e = cudaFuncSetAttribute(k_lo_solve<fpair>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
-        if (e != cudaSuccess) return e;
-        return launch_pdl(k_lo_solve<fpair>, dim3(nb), dim3(128), sm, p.stream, x);
-    } else if (!lo_fp32(p.precision)) {
-        e = cudaFuncSetAttribute(k_lo_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
-        if (e != cudaSuccess) return e;
-        return launch_pdl(k_lo_solve<double>, dim3(nb), dim3(128), sm, p.stream, x);
-    } else {
-        e = cudaFuncSetAttribute(k_lo_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
-        if (e != cudaSuccess) return e;
-        return launch_pdl(k_lo_solve<float>, dim3(nb), dim3(128), sm, p.stream, x);
-    }
+    // 512 threads where every group has an SM of its own, 256 where the level fits the GPU at
+    // three CTAs per SM, if the rows are more than 128 threads take at once.  128 against more
+    // threads, measured: 16 groups x 500 cells FP64 20.3, 14.7 us; 4 groups x 1000 cells pair
+    // 49.6, 21.4; 256 groups x 1000 cells pair 51.3, 31.8
+    const int T = p.nx <= 128 || L.n > 456 ? 128 : L.n <= 152 ? 512 : 256;
+    const auto go = [&](auto zero) {
+        using R = decltype(zero);
+        return T == 512   ? lo_launch<R, 512>(x, L.n, sm, p.stream)
+               : T == 256 ? lo_launch<R, 256>(x, L.n, sm, p.stream)
+                          : lo_launch<R, 128>(x, L.n, sm, p.stream);
+    };
+    return lo_pair(p.precision) ? go(fpair()) : lo_fp32(p.precision) ? go(0.f) : go(0.0);
 }
 
 cudaError_t launch_lo_solve_b(int precision, int max_nx, const int *meta, int N,
