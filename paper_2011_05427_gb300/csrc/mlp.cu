@@ -13,6 +13,7 @@
 // FP32 accumulator lives in 256 tensor-memory columns; in the epilogue thread t owns row
 // t (tensor-memory lane t) and reads its 256 values 32 at a time with tcgen05.ld.
 #include <algorithm>
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include "common.cuh"
@@ -710,23 +711,27 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
 // fixed order.  Products per CTA (M 128, K 16 per instruction, BF16 in, FP32 accumulate):
 //   h2 = relu(h1 W2^T), h3 = relu(h2 W3^T)          weights K-major from the streaming image
 //   d2 = (d3 W3) [h2 > 0], d1 = (d2 W2) [h1 > 0]    the same image read MN-major: a K chunk
-//                                                   (32 outputs) is 32 pieces of 512 bytes
+//                                                   (32 outputs) is a box of 32 rows of 512
+//                                                   bytes, one tensor-map copy
 //   dW3 = d3^T h2, dW2 = d2^T h1                    both operands MN-major from the tiles
-// The weight gradients are 256 x 256: two halves of 128 output features, one in the
-// accumulator columns of the layers (0 .. 255), one in columns 256 .. 511.
+// The weight gradients are 256 x 256: two halves of 128 output features, one after the other
+// in columns 256 .. 511; the layers' accumulator is columns 0 .. 255.
 // Warps 0-7 (thread = tensor-memory lane of quadrant warp & 3, columns 128 (warp >> 2) ..)
-// run the epilogues, warp 8 streams weights through a ring of F_TSLOTS chunks, warp 9
-// issues the MMAs.  h1 is formed twice (3 FMAs a value) because three tiles would leave the
-// ring too small.  The loss head sums a row's 256 terms in column order in one chain, as
-// the inference GEMM's epilogue does.
+// run the layers' epilogues, warps 8-15 (the same lanes and columns) the column sums of the
+// layer gradients and the weight gradients' way out, off the layers' chain; warp 16 streams
+// weights through a ring of F_TSLOTS chunks, warp 17 issues the MMAs.  h1 is formed twice (3
+// FMAs a value) because three tiles would leave the ring too small.  The loss head sums a
+// row's 256 terms in column order in one chain, as the inference GEMM's epilogue does.
 // What bounds it: 8192 rows are 64 CTAs of the 152 SMs, each a serial chain of 4 layer
 // products (1 us each at the tensor rate) with their epilogues; the floor at the measured
-// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 46 us against 1249 us
-// for one GEMM launch per product, whose two weight gradients ran on two CTAs over K = 8192
-// (500 us) and whose column sums ran on 8 and 1 CTAs (520 us).
+// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 39.5 us against
+// 1249 us for one GEMM launch per product, whose two weight gradients ran on two CTAs over K =
+// 8192 (500 us) and whose column sums ran on 8 and 1 CTAs (520 us); 46 us with the eight
+// warps doing everything and the backward weights copied as 512-byte pieces (6 us a layer).
 constexpr int F_TSLOTS = 5;
 constexpr int F_TRING = F_TSLOTS * FW_BYTES;
-constexpr int TNBAR = 2 * F_TSLOTS + 3;   // full, empty, act, acc0, acc1
+constexpr int T_THREADS = 576;
+constexpr int TNBAR = 2 * F_TSLOTS + 7;   // full, empty, act, acc, wac, drn, w3d, d3r, d2r
 constexpr int T_SMEM = 2 * FA_BYTES + F_TRING + FP_BYTES + 128 * 16 + 3 * 128 * 4 + 8 * TNBAR + 32;
 constexpr uint32_t IDESC_BT = IDESC | (1u << 16);                  // B MN-major
 constexpr uint32_t IDESC_ABT = IDESC | (1u << 15) | (1u << 16);    // A and B MN-major
@@ -771,10 +776,21 @@ __device__ inline void tile_colsum(const unsigned char *A, int warp, int lane, c
     out[kg * 8 + r8] = v;
 }
 
-__global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const float *__restrict__ x,
+// a box of 32 rows of 256 elements of the weight images (tensor map of launch_train), at
+// element x of its rows y ..: one tile copy into shared memory, completing on `bar`
+__device__ inline void tile_copy(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar)
+{
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                 "[%1, {%2, %3}], [%4];" ::"r"(su32(dst)),
+                 "l"(map), "r"(x), "r"(y), "r"(su32(bar))
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(T_THREADS, 1) k_mlp_train(int rows, const float *__restrict__ x,
                                                             const float *__restrict__ target,
                                                             const float *__restrict__ P,
                                                             const bf16 *__restrict__ Wimg,
+                                                            const __grid_constant__ CUtensorMap map,
                                                             float *__restrict__ part)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -783,7 +799,11 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
     float4 *sx = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sP) + FP_BYTES);
     float *sdot = reinterpret_cast<float *>(sx + 128), *sdz = sdot + 128, *ssq = sdz + 128;
     uint64_t *bar = reinterpret_cast<uint64_t *>(ssq + 128);
-    uint64_t *full = bar, *empty = bar + F_TSLOTS, *act = bar + 2 * F_TSLOTS, *acc = act + 1;
+    uint64_t *full = bar, *empty = bar + F_TSLOTS, *act = bar + 2 * F_TSLOTS, *acc = act + 1,
+             *wac = act + 2, *drn = act + 3;   // layer product, weight gradient half, its columns read
+    // single-phase barriers of the two groups of warps, neither of which waits on the other's
+    // every phase: dW3 formed, d3 in A0, d2 in A0
+    uint64_t *w3d = act + 4, *d3r = act + 5, *d2r = act + 6;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + TNBAR);
     volatile int *sfail = reinterpret_cast<int *>(tslot + 1);
     volatile int *sprod = sfail + 1, *scons = sfail + 2;
@@ -798,8 +818,12 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
             mbar_init_n(&empty[k], 1);
         }
         mbar_init_n(act, 256);
-        mbar_init_n(&acc[0], 1);
-        mbar_init_n(&acc[1], 1);
+        mbar_init_n(acc, 1);
+        mbar_init_n(wac, 1);
+        mbar_init_n(drn, 256);
+        mbar_init_n(w3d, 1);
+        mbar_init_n(d3r, 256);
+        mbar_init_n(d2r, 256);
         *sfail = 0;
         *sprod = 0;
         *scons = 0;
@@ -824,37 +848,38 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
     bool ok = true;
 
     constexpr int Q = 4 * FNC;   // chunks: W2, W3 (forward), W3, W2 (backward)
-    if (warp == 8) {
-        // ---------------- producer warp ----------------
+    if (warp == 16) {
+        // ---------------- producer thread ----------------
         int q = 0;
-        for (; q < Q; ++q) {
+        for (; lane == 0 && q < Q; ++q) {
             const int slot = q % F_TSLOTS, job = q / FNC, c = q % FNC;
-            // a warp-uniform outcome (the lanes time out each for itself)
-            if (!__all_sync(0xffffffffu, q < F_TSLOTS ||
-                                             mbar_wait(&empty[slot], ((q - F_TSLOTS) / F_TSLOTS) & 1))) {
+            if (q >= F_TSLOTS && !mbar_wait(&empty[slot], ((q - F_TSLOTS) / F_TSLOTS) & 1)) {
                 *sfail = 1;
                 break;
             }
-            const bf16 *img = Wimg + (job == 1 || job == 2 ? 65536 : 0);
+            const int layer = (job == 1 || job == 2) ? 1 : 0;
             unsigned char *dst = ring + slot * FW_BYTES;
-            if (lane == 0) mbar_expect(&full[slot], FW_BYTES);
-            __syncwarp();
-            if (job < 2) {
-                if (lane == 0) bulk_copy(dst, img + c * (FW_BYTES / 2), FW_BYTES, &full[slot]);
-            } else {   // inputs 8 lane .. 8 lane + 7 of outputs 32 c .. 32 c + 31
-                bulk_copy(dst + lane * 512, img + lane * 2048 + c * 256, 512, &full[slot]);
-            }
+            mbar_expect(&full[slot], FW_BYTES);
+            if (job < 2)
+                bulk_copy(dst, Wimg + layer * 65536 + c * (FW_BYTES / 2), FW_BYTES, &full[slot]);
+            else   // inputs 8 i .. 8 i + 7 (box row i) of outputs 32 c .. 32 c + 31
+                tile_copy(dst, &map, c * 256, layer * 32, &full[slot]);
         }
         if (lane == 0) *sprod = q;
-    } else if (warp == 9) {
+    } else if (warp == 17) {
         // ---------------- MMA thread ----------------
         if (lane == 0) {
             int q = 0;
-            unsigned pact = 0;
+            unsigned pact = 0, pdrn = 0;
             const uint32_t a0 = su32(A0), a1 = su32(A1);
             auto wait_act = [&]() {
                 if (ok && !mbar_wait(act, pact)) ok = false;
                 pact ^= 1u;
+                tc_after();
+            };
+            auto wait_drn = [&]() {
+                if (ok && !mbar_wait(drn, pdrn)) ok = false;
+                pdrn ^= 1u;
                 tc_after();
             };
             // one layer product into columns 0 .. 255: A = a tile (K-major), B = 8 chunks
@@ -876,42 +901,44 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
                     }
                     umma_commit(&empty[slot]);
                 }
-                if (ok) umma_commit(&acc[0]);
+                if (ok) umma_commit(acc);
             };
-            // half hf (output features 128 hf ..) of d^T h over the tile's 128 rows
-            auto wgrad = [&](uint32_t d, uint32_t h, int hf, uint32_t col, uint64_t *done) {
+            // half hf (output features 128 hf ..) of A0^T A1 over the tile's 128 rows
+            auto wgrad = [&](int hf) {
                 if (!ok) return;
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)   // rows 16 kk ..: row groups 4096 bytes apart
-                    umma<IDESC_ABT>(tmem + col, sdesc(d + hf * 2048 + kk * 8192, FA_SBO, 128),
-                                    sdesc(h + kk * 8192, FA_SBO, 128), kk != 0);
-                umma_commit(done);
+                    umma<IDESC_ABT>(tmem + 256, sdesc(a0 + hf * 2048 + kk * 8192, FA_SBO, 128),
+                                    sdesc(a1 + kk * 8192, FA_SBO, 128), kk != 0);
+                umma_commit(wac);
             };
             wait_act();             // h1 in A0
             layer(a0, false);
             wait_act();             // h2 in A1
             layer(a1, false);
             wait_act();             // d3 in A0
-            wgrad(a0, a1, 1, 0, &acc[0]);
-            wgrad(a0, a1, 0, 256, &acc[1]);
-            wait_act();             // columns 0 .. 255 read
+            wgrad(0);
             layer(a0, true);
-            wait_act();             // d2 in A0, h1 in A1, every column read
+            wait_drn();             // columns 256 .. 511 read
+            wgrad(1);
+            if (ok) umma_commit(w3d);
+            wait_act();             // d2 in A0, h1 in A1
             layer(a0, true);
-            wgrad(a0, a1, 0, 256, &acc[1]);
-            wait_act();             // columns 0 .. 255 read
-            wgrad(a0, a1, 1, 0, &acc[0]);
+            wait_drn();
+            wgrad(0);
+            wait_drn();
+            wgrad(1);
             if (!ok) *sfail = 1;
             *scons = q;
         }
     } else {
         // ---------------- epilogue warps ----------------
-        const int qd = warp & 3, hf = warp >> 2;
+        const bool side = warp >= 8;   // the column sums and weight gradients
+        const int qd = warp & 3, hf = (warp >> 2) & 1;
         const int r = qd * 32 + lane;       // the tile row, or the output feature of a gradient
         const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16);
-        unsigned p0 = 0, p1 = 0;
-        auto wait_acc = [&](int k, unsigned &ph) {
-            if (ok && !mbar_wait(&acc[k], ph)) {
+        auto wait_bar = [&](uint64_t *b, unsigned &ph) {
+            if (ok && !mbar_wait(b, ph)) {
                 ok = false;
                 *sfail = 1;
             }
@@ -919,6 +946,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
             __syncwarp();
             tc_after();
         };
+        unsigned pacc = 0, pwac = 0, pw3 = 0, pd3 = 0, pd2 = 0;
         auto hand_off = [&]() {
             tc_before();
             fence_async_smem();
@@ -929,24 +957,37 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
             tmem_wait_tied(v);
         };
         // this thread's 128 columns of feature 128 half + r of a weight gradient
-        auto drain = [&](int tp, int half, uint32_t col) {
+        auto drain = [&](int tp, int half) {
+            wait_bar(wac, pwac);
             float4 *o = reinterpret_cast<float4 *>(pt + tp) + half * 128 + r;
 #pragma unroll 1
             for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
                 uint32_t v[32];
-                load32(col + ch * 32, v);
+                load32(256 + ch * 32, v);
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     o[(size_t)(ch * 8 + j) * 256] =
                         make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
                                     __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
             }
+            tc_before();
+            mbar_arrive(drn);
         };
+        if (side) {
+            wait_bar(d3r, pd3);
+            tile_colsum<false>(A0, warp - 8, lane, nullptr, pt + TP_B3);
+            drain(TP_DW3, 0);
+            drain(TP_DW3, 1);
+            wait_bar(d2r, pd2);
+            tile_colsum<false>(A0, warp - 8, lane, nullptr, pt + TP_B2);
+            drain(TP_DW2, 0);
+            drain(TP_DW2, 1);
+        } else {
         const float4 X = sx[r];
         layer1_row<true>(sP, X.x, X.y, X.z, A0, r, 16 * hf, 16 * hf + 16);
         hand_off();
         // ---- h2 = relu(acc + b2) ----
-        wait_acc(0, p0);
+        wait_bar(acc, pacc);
 #pragma unroll 1
         for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
             uint32_t v[32];
@@ -968,7 +1009,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
         hand_off();
         // ---- h3 = relu(acc + b3) into A0, the head in column order: the first half's
         // threads take columns 0 .. 127, the second half's go on from their sums ----
-        wait_acc(0, p0);
+        wait_bar(acc, pacc);
         float dot = 0.f;
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
@@ -1045,17 +1086,12 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
                 *p = u;
             }
         }
+        mbar_arrive(d3r);
         hand_off();
-        bar_epi();
-        tile_colsum<false>(A0, warp, lane, nullptr, pt + TP_B3);
-        // ---- dW3 ----
-        wait_acc(0, p0);
-        drain(TP_DW3, 1, 0);
-        hand_off();
-        wait_acc(1, p1);
-        drain(TP_DW3, 0, 256);
-        // ---- d2 = acc [h2 > 0] over d3, h1 again over h2 ----
-        wait_acc(0, p0);
+        // ---- d2 = acc [h2 > 0] over d3, h1 again over h2, once dW3 has read both (its second
+        // half follows the column sums' read of d3) ----
+        wait_bar(acc, pacc);
+        wait_bar(w3d, pw3);
 #pragma unroll 1
         for (int ch = 4 * hf; ch < 4 * hf + 4; ++ch) {
             uint32_t v[32];
@@ -1076,14 +1112,13 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
                 *reinterpret_cast<uint4 *>(A0 + a_off(r, ch * 4 + qq)) = u;
             }
         }
+        mbar_arrive(d2r);
         layer1_row<true>(sP, X.x, X.y, X.z, A1, r, 16 * hf, 16 * hf + 16);
         hand_off();
-        bar_epi();
-        tile_colsum<false>(A0, warp, lane, nullptr, pt + TP_B2);
         // ---- d1 = acc [h1 > 0] (FP32): its column sums, plain (b1) and times x (W1).  The
         // ring is free (the last layer product has read it): a warp stages 32 rows x 32
         // columns, lane = column sums its 32 rows, then the four row quadrants meet ----
-        wait_acc(0, p0);
+        wait_bar(acc, pacc);
         float *stage = reinterpret_cast<float *>(ring) + warp * (32 * 33);
         float *quad = reinterpret_cast<float *>(ring) + 8 * 32 * 33;   // [4 sums][4 quadrants][256]
 #pragma unroll 1
@@ -1120,7 +1155,6 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
             quad[(3 * 4 + qd) * 256 + c] = s3;
             __syncwarp();
         }
-        hand_off();
         bar_epi();
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -1129,11 +1163,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_train(int rows, const floa
             if (k == 0) pt[TP_B1 + tid] = s;
             else pt[TP_W1 + 3 * tid + k - 1] = s;
         }
-        // ---- dW2 ----
-        wait_acc(1, p1);
-        drain(TP_DW2, 0, 256);
-        wait_acc(0, p0);
-        drain(TP_DW2, 1, 0);
+        }
     }
     tc_before();
     __syncthreads();
@@ -1200,6 +1230,33 @@ __global__ void __launch_bounds__(256) k_train_reduce(int nt, const float *__res
         else if (k < TP_LOSS) grad[TRT_MLP_B3 + k - TP_B3] = v[j];       // b3, w4, b4
         else if (k == TP_LOSS) *loss = v[j];
     }
+}
+
+// the weight images as a matrix of 64 rows (32 input groups of W2, then of W3; 4096 bytes: 256
+// outputs x 8 inputs) for boxes of 32 rows x 32 outputs
+cudaError_t image_map(const bf16 *img, CUtensorMap *map)
+{
+    typedef CUresult (*Encode)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                               const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
+                               CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                               CUtensorMapFloatOOBfill);
+    static Encode encode = nullptr;   // the driver's entry point, the same for every device
+    if (!encode) {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
+                                                         cudaEnableDefault, &q);
+        if (e != cudaSuccess) return e;
+        if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
+        encode = reinterpret_cast<Encode>(fn);
+    }
+    const cuuint64_t dim[2] = {2048, 64}, pitch[1] = {4096};
+    const cuuint32_t box[2] = {256, 32}, one[2] = {1, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(img), dim,
+                              pitch, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 int g_num_sms = 0;
@@ -1447,10 +1504,12 @@ int trt_mlp_grad(int rows, const float *x, const float *target, const float *par
     const bf16 *img = reinterpret_cast<const bf16 *>(w16) + 4 * 65536;
     if (!al16(w16)) return TRT_EINVAL;
     const int nt = rows / 128;
-    if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, T_SMEM) !=
+    CUtensorMap map;
+    if (image_map(img, &map) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, T_SMEM) !=
             cudaSuccess ||
-        launch_pdl(k_mlp_train, dim3(nt), dim3(F_THREADS), T_SMEM, st, rows, x, target, params, img,
-                   s.part) != cudaSuccess ||
+        launch_pdl(k_mlp_train, dim3(nt), dim3(T_THREADS), T_SMEM, st, rows, x, target, params, img,
+                   map, s.part) != cudaSuccess ||
         launch_pdl(k_train_reduce, dim3((TP_N / 4 + 63) / 64), dim3(256), 0, st, nt,
                    (const float *)s.part, grad, loss) != cudaSuccess)
         return TRT_ECUDA;
