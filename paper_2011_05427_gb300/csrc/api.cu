@@ -327,6 +327,8 @@ int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups 
     {
         cudaError_t e = ensure_tables();
         if (e != cudaSuccess) return fail(nullptr, TRT_ECUDA, cudaGetErrorString(e));
+        p.ser = series_device();
+        if (!p.ser) return fail(nullptr, TRT_ECUDA, "no address of the series tables");
     }
     Carver c{reinterpret_cast<char *>(opt->workspace), 0};
     trt_handle *H = hp.get();
@@ -562,13 +564,16 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
         // its last grey visit on the device, so the host waits once per phase.
         p.gate = h->ctl;
         for (int l = 0; l < cyc->l_max; ++l) {
-            if (!opac_valid) {
+            // the opacities at T where the sweep did not form them: inside the solve (the
+            // T_r option: a kernel of their own)
+            const bool form = !opac_valid;
+            if (form && p.tr_mode) {
                 CK(launch_opacity(p, h->T, h->sigE, h->emis, h->sigR, nullptr, nullptr, 0.0,
                                   Erad));
                 ++nk;
             }
             opac_valid = true;
-            CK(launch_lo_solve(p, dt, fine));
+            CK(launch_lo_solve(p, dt, fine, form && !p.tr_mode ? h->T : nullptr));
             ++nk;
             // grey visit k reads T~^[k] and writes T~^[k+1]: T~^[0] = T, the last visit
             // writes T, the ones between alternate over Ttil and Tnew
@@ -578,16 +583,20 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
                 Level *src = &fine;
                 if (k > 0) {
                     const int lev = S[k - 1] - 1, ng = p.levels[lev];
-                    CK(launch_opacity(p, Tst, h->sigE, h->emis, h->sigR, nullptr, nullptr, 0.0,
-                                      Erad));
+                    if (p.tr_mode) {
+                        CK(launch_opacity(p, Tst, h->sigE, h->emis, h->sigR, nullptr, nullptr, 0.0,
+                                          Erad));
+                        ++nk;
+                    }
                     opac_valid = false;
                     h->crs.n = ng;
                     h->crs.Eold = h->crs_Eold[lev];
                     h->crs.Fold = h->crs_Fold[lev];
-                    CK(launch_restrict(p, fine, h->crs, nullptr, nullptr, old_sums[lev] != 0));
+                    CK(launch_restrict(p, fine, h->crs, nullptr, nullptr, old_sums[lev] != 0,
+                                       p.tr_mode ? nullptr : Tst));
                     old_sums[lev] = 1;
                     CK(launch_lo_solve(p, dt, h->crs));
-                    nk += 3;
+                    nk += 2;
                     src = &h->crs;
                 }
                 GreyArgs a{};

@@ -37,6 +37,10 @@ struct OpacityArgs {
     const fpair *otabp;
     fpair *cpair;
     float icdt_h, icdt_l;
+    // for evaluations outside physics.cu: the integrals' tables on the device, and texp's
+    const SeriesTables *ser;
+    const double *e2;
+    ExpConsts ec;
 };
 
 struct SweepArgs {
@@ -150,6 +154,7 @@ __device__ inline bool bdecode(const int *__restrict__ meta, int N, int b, int &
 OpacityArgs make_opacity_args(const Problem &p, const double *T, double *sigE, double *emis,
                               double *sigR, float *sig32, float *emis32, double dt,
                               const double *Erad = nullptr);
+cudaError_t launch_cell_terms(const Problem &p, const OpacityArgs &a);   // k_cell_terms
 int opacity_blocks(const Problem &p);
 int opacity_gx(const Problem &p);   // blocks along the cells (32 cells x 8 groups each)
 SweepArgs make_sweep_args(const Problem &p, double dt, const void *sigE, const void *emis,

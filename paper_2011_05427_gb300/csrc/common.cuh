@@ -144,6 +144,7 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
 const SeriesTables &host_series();   // host copy (built once)
 void gauss_legendre_host(int n, double *x, double *w);   // nodes / weights on [-1, 1]
 cudaError_t ensure_tables();         // upload the tables to the current device (once)
+const SeriesTables *series_device();  // their address there
 cudaError_t launch_fastmath(int n, const double *x, double *ex, double *rc, cudaStream_t st);
 // FP64 FMA rate probe: one timed launch of `reps` FMA steps per chain; FMAs executed in *fmas
 cudaError_t fp64_probe(int reps, cudaStream_t st, float *ms, long long *fmas);
@@ -259,6 +260,7 @@ struct Problem {
     // sigma_E T^3, sigma_R T^3 and the emission factor ln(1 - e^{-w}) (null: direct
     // integrals)
     double *otab = nullptr;
+    const SeriesTables *ser = nullptr;   // the integrals' tables on the device
     // with TRT_LO_PAIR: the tables with their FP64 coefficients as FP32 pairs, then the G+1
     // group edges as pairs (otab_doubles(G) + G + 1 doubles), and per-cell pair terms of the
     // opacity evaluation [5][nx] (t, 1/T, 1/T^3, 27 s C_B T, h/2); null otherwise
@@ -306,17 +308,20 @@ cudaError_t launch_sweep(const Problem &p, double dt, const void *sigE, const vo
                          bool sigma_fp32, const void *I_old, void *I_new, double *part,
                          double *psi_exit, double *f, double *fb0, double *fbX, double *C0,
                          double *CX);
-cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L);
+// Topac (fine levels; may be null): the opacities at these temperatures are formed first, into
+// the level's arrays (not with the T_r option)
+cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L,
+                            const double *Topac = nullptr);
 // h/dt and hf/(c dt) of the LO rows for step length dt (a launch when dt changed)
 cudaError_t ensure_lo_consts(Problem &p, double dt);
 // the step-independent pair row constants (Problem::lopc; once per handle, TRT_LO_PAIR)
 cudaError_t launch_lo_pair_consts(const Problem &p);
 // newton (with pre): the visit's grey Newton arguments; the restriction to the grey level
 // then also forms the per-cell Newton terms into pre ([3][nx]).  skip_old: dst holds this
-// step's Eold and Fold sums already
+// step's Eold and Fold sums already.  Topac as in launch_lo_solve, for a fine src
 cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
                             const GreyArgs *newton = nullptr, double *pre = nullptr,
-                            bool skip_old = false);
+                            bool skip_old = false, const double *Topac = nullptr);
 // the host-formed constants of a grey visit (c_v/dt, 54 s C_B, the exponential's table)
 GreyArgs grey_args_ready(const Problem &p, const GreyArgs &a);
 size_t restrict_scratch_doubles(const Problem &p);   // from nx and the grids

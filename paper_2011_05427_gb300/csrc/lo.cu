@@ -21,8 +21,7 @@
 // built from the level's fields into shared memory in a [row-in-chunk][chunk] layout
 // (conflict free for the elimination).
 #include <cmath>
-#include "batch.cuh"
-#include "pair.cuh"
+#include "opacity.cuh"
 
 namespace trt {
 
@@ -614,6 +613,63 @@ __device__ void lo_solve_body(const LoCtx &x, int q)
     if (threadIdx.x == 0) lo_one_cell<R>(x, q, ks);
 }
 
+// The exponentials' tables in shared memory by the block (ends with a barrier).
+__device__ inline Mx stage_exp(const OpacityArgs &a, double *e2, fpair *e2p)
+{
+    if (threadIdx.x < 32) {
+        e2[threadIdx.x] = a.e2[threadIdx.x];
+        e2p[threadIdx.x] = fpair(a.e2[threadIdx.x]);
+    }
+    __syncthreads();
+    return Mx{e2, a.ec};
+}
+// where an evaluation takes its per-cell terms: 1, formed here (k_cell_terms did not run)
+enum { OP_NONE = 0, OP_ARRAYS = 1, OP_HERE = 2 };
+template <bool kPair>
+__device__ inline void cell_terms(const OpacityArgs &a, int op, int i, CellVals &v, CellPair &cp)
+{
+    if (op == OP_HERE) {
+        v = cell_vals(a, i);
+        if (kPair) cp = cell_pair(a, i, v);
+    } else {
+        v = cell_arrays(a).get(i);
+        if (kPair) cp = cell_pair_at(a, i);
+    }
+}
+// sigma_E, e_g, sigma_R of group g in the cell
+template <bool kPair>
+__device__ inline OpacVals cell_opacities(const OpacityArgs &a, int g, const CellVals &v,
+                                          const CellPair &cp, const Mx &mx, const fpair *e2p)
+{
+    if (kPair && v.m >= 0) {
+        fpair sg, em, sR;
+        int k;
+        opacity_vals_pair(a, g, v.m, v.tf, cp, e2p, sg, em, k, sR);
+        return OpacVals{pr_join(sg, 0), pr_join(em, k), pr_join(sR, 0)};
+    }
+    return opacity_vals(a, g, v, mx);
+}
+// the opacities of group g in every cell by the CTA, into the fine grid's arrays (ends with
+// a barrier)
+template <bool kPair>
+__device__ void group_opacities(const OpacityArgs &a, int op, int g)
+{
+    __shared__ double e2[32];
+    __shared__ fpair e2p[32];
+    const Mx mx = stage_exp(a, e2, e2p);
+    for (int i = threadIdx.x; i < a.nx; i += blockDim.x) {
+        CellVals v;
+        CellPair cp;
+        cell_terms<kPair>(a, op, i, v, cp);
+        const OpacVals o = cell_opacities<kPair>(a, g, v, cp, mx, e2p);
+        const size_t idx = (size_t)g * a.nx + i;
+        a.sigE[idx] = o.sg;
+        a.emis[idx] = o.em;
+        a.sigR[idx] = o.sR;
+    }
+    __syncthreads();
+}
+
 // T threads.  128: 7 CTAs per SM (at most 72 registers), one wave of 1064 holds every group
 // of a 1024-group level.  512 and 256: levels of few groups, whose staging and outputs (loads
 // and ~60 operations per face) would be a chain of n/128 faces per thread; launch_lo_solve.
@@ -622,6 +678,20 @@ __global__ void __launch_bounds__(T, T == 128 ? 7 : T == 256 ? 3 : 1) k_lo_solve
 {
     griddep_wait();
     if (x.gate && *x.gate) return;   // the phase's inner loop has ended
+    lo_solve_body<R>(x, blockIdx.x);
+}
+// a fine grid whose opacities at a.T the CTA forms first, its own group's: a launch and a pass
+// over the fields less than k_opacity and k_lo_solve (1024 groups x 500 cells FP64 84 us for
+// both against 61 + 33; pair 40 against 32 + 15; 17 groups x 60 cells 12 against 9 + 6 + 3
+// with k_cell_terms).  A kernel of its own: in one kernel the pair form's plain solve was 30%
+// slower.
+template <typename R, int T>
+__global__ void __launch_bounds__(T, T == 128 ? 7 : T == 256 ? 3 : 1) k_lo_solve_opac(LoCtx x, OpacityArgs a,
+                                                                                    int op)
+{
+    griddep_wait();
+    if (x.gate && *x.gate) return;
+    group_opacities<is_pair<R>>(a, op, blockIdx.x);
     lo_solve_body<R>(x, blockIdx.x);
 }
 
@@ -785,6 +855,68 @@ __device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, in
     }
 }
 
+// The same over a fine source whose opacities at a.T are formed here, per member and cell,
+// instead of read (and stored for the other readers of the fine grid's arrays): the lane's
+// per-cell terms stay in registers over the members.  A face's left opacity is the lane
+// before's, through shared memory (xch: two rows of 33 for the warp, by turns).
+template <bool kOld, bool kPair>
+__device__ inline void restrict_members_opac(const RestrictCtx &x, const OpacityArgs &a, int op,
+                                             double (*xch)[33], const Mx &mx, const fpair *e2p,
+                                             int p0, int pe, int step, int i, double (&v)[kRV])
+{
+    const Level &S = x.S;
+    const int nx = x.nx, lane = threadIdx.x & 31;
+    const int ic = min(max(i, 0), nx - 1);
+    const size_t cd = (size_t)step * nx;
+    size_t c = (size_t)p0 * nx + ic;
+    const bool in = i >= 0 && i < nx, own = in && lane > 0;
+    const double *Ep = in ? S.E + c : (i < 0 ? S.Eb0 : S.EbX) + p0;
+    const size_t Ed = in ? cd : (size_t)step;
+    const double *Lp = i > 0 ? S.E + (size_t)p0 * nx + i - 1 : S.Eb0 + p0;   // E left of face i
+    const size_t Ld = i > 0 ? cd : (size_t)step;
+    size_t f = (size_t)p0 * (nx + 1) + max(i, 0);
+    double wa = 0.0, wb = 1.0;
+    if (i > 0) {   // the face opacity's dx-weighted mean; face n_x: its cell alone
+        wa = i < nx ? x.h[i - 1] * x.ihf[i] : 1.0;
+        wb = i < nx ? x.h[i] * x.ihf[i] : 0.0;
+    }
+    CellVals cv;
+    CellPair cp;
+    cell_terms<kPair>(a, op, ic, cv, cp);
+#pragma unroll
+    for (int k = 0; k < kRV; ++k) v[k] = 0.0;
+    int par = 0;
+    for (int p = p0; p < pe; p += step) {
+        const double E = *Ep, EL = *Lp, F = S.F[f], ph = S.phi[c];
+        const OpacVals o = cell_opacities<kPair>(a, p, cv, cp, mx, e2p);
+        xch[par][lane] = o.sR;
+        if (own) {
+            S.sig[c] = o.sg;
+            S.emis[c] = o.em;
+            S.sigR[c] = o.sR;
+        }
+        __syncwarp();
+        const double left = xch[par][max(lane - 1, 0)];
+        par ^= 1;
+        const double sR = fma(wa, left, wb * o.sR);
+        v[R_PHI] = fma(ph, E, v[R_PHI]);
+        v[R_SIG] = fma(o.sg, E, v[R_SIG]);
+        v[R_EMIS] += o.em;
+        v[R_E] += E;
+        const double w = fma(0.5e-6 * kC, EL + E,
+                             __longlong_as_double(__double_as_longlong(F) & 0x7fffffffffffffffll));
+        v[R_SW] = fma(sR, w, v[R_SW]);
+        v[R_W] += w;
+        v[R_SF] = fma(sR, F, v[R_SF]);
+        v[R_F] += F;
+        if (kOld) {
+            v[R_EOLD] += S.Eold[c];
+            v[R_FOLD] += S.Fold[f];
+        }
+        Ep += Ed; Lp += Ld; c += cd; f += cd + step;
+    }
+}
+
 // the E-weighted cell means of coarse group P at cell i (and the grey visit's Newton terms)
 __device__ inline void restrict_cell(const RestrictCtx &x, int P, int i, double sphi, double ssig,
                                      double semis, double sE)
@@ -800,7 +932,7 @@ __device__ inline void restrict_cell(const RestrictCtx &x, int P, int i, double 
         ph = sg = 0.0;
         for (int p = P * x.r; p < (P + 1) * x.r; ++p) {
             ph += S.phi[(size_t)p * nx + i];
-            sg += S.sig[(size_t)p * nx + i];
+            sg += __ldcg(S.sig + (size_t)p * nx + i);   // of this launch, perhaps
         }
         ph = rquot(ph, (double)x.r);
         sg = rquot(sg, (double)x.r);
@@ -848,8 +980,8 @@ __device__ inline void restrict_face(const RestrictCtx &x, int P, int i, double 
         for (int p = P * x.r; p < (P + 1) * x.r; ++p) {
             if (S.fine) {
                 const double *sc = S.sigR + (size_t)p * nx;
-                sRP += (i == 0) ? sc[0] : (i == nx) ? sc[nx - 1]
-                       : (sc[i - 1] * x.h[i - 1] + sc[i] * x.h[i]) * x.ihf[i];
+                sRP += (i == 0) ? __ldcg(sc) : (i == nx) ? __ldcg(sc + nx - 1)
+                       : (__ldcg(sc + i - 1) * x.h[i - 1] + __ldcg(sc + i) * x.h[i]) * x.ihf[i];
             } else {
                 sRP += S.sigR[(size_t)p * nf + i];
             }
@@ -919,8 +1051,10 @@ __device__ inline bool restrict_last(int *t, int n)
     return last;
 }
 
-// block 128; grid (nt + 1, ceil(n_to / 4)) in mode 0, (nt + 1, n_to * nchunk) in mode 1
-__device__ void restrict_body(const RestrictCtx &x, int bx, int by)
+// block 128; grid (nt + 1, ceil(n_to / 4)) in mode 0, (nt + 1, n_to * nchunk) in mode 1;
+// members(p0, pe, step, i, v): the sums over members
+template <class Members>
+__device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Members &members)
 {
     __shared__ double red[4][kRV][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -963,7 +1097,7 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by)
     double v[kRV];
     if (many) {
         if (P >= x.n_to) return;
-        restrict_members(x, pb, pe, 1, min(i, nx), v);
+        members(pb, pe, 1, min(i, nx), v);
         const double sEL = __shfl_up_sync(0xffffffffu, v[R_E], 1);
         if (cell) restrict_cell(x, P, i, v[R_PHI], v[R_SIG], v[R_EMIS], v[R_E]);
         if (face) {
@@ -973,7 +1107,7 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by)
         }
         return;
     }
-    restrict_members(x, pb + warp, pe, 4, min(i, nx), v);
+    members(pb + warp, pe, 4, min(i, nx), v);
 #pragma unroll
     for (int k = 0; k < kRV; ++k) red[warp][k][lane] = v[k];
     __syncthreads();
@@ -1199,11 +1333,37 @@ __device__ void group_sum_body(const GroupSumArgs &a, int bx)
 
 // entry points: the single-slab kernels pass blockIdx; the batched ones walk a work list
 // (single-slab entry points: return at entry while the driver's gate is set)
+__device__ inline void restrict_run(const RestrictCtx &x, int bx, int by)
+{
+    restrict_body(x, bx, by, [&](int p0, int pe, int step, int i, double (&v)[kRV]) {
+        restrict_members(x, p0, pe, step, i, v);
+    });
+}
 __global__ void __launch_bounds__(128) k_restrict(RestrictCtx x)
 {
     griddep_wait();
     if (x.gate && *x.gate) return;
-    restrict_body(x, blockIdx.x, blockIdx.y);
+    restrict_run(x, blockIdx.x, blockIdx.y);
+}
+// fine source, its opacities at a.T formed on the way (a coarse visit: every fine group's
+// opacities, then the restriction onto the visit's grid).  The pair form's evaluation runs on
+// the FP32 pipes under the sums' FP64 operations; one launch and a pass over three fields
+// less than k_opacity and k_restrict: 4096 groups x 1000 cells pair 196 us against 89 + 147;
+// FP64 (all of it on the FP64 pipe) 62 against 34 + 29
+template <bool kPair>
+__global__ void __launch_bounds__(128) k_restrict_opac(RestrictCtx x, OpacityArgs a, int op)
+{
+    griddep_wait();
+    if (x.gate && *x.gate) return;
+    __shared__ double e2[32], xch[4][2][33];
+    __shared__ fpair e2p[32];
+    const Mx mx = stage_exp(a, e2, e2p);
+    restrict_body(x, blockIdx.x, blockIdx.y, [&](int p0, int pe, int step, int i, double (&v)[kRV]) {
+        if (x.skip_old)
+            restrict_members_opac<false, kPair>(x, a, op, xch[threadIdx.x >> 5], mx, e2p, p0, pe, step, i, v);
+        else
+            restrict_members_opac<true, kPair>(x, a, op, xch[threadIdx.x >> 5], mx, e2p, p0, pe, step, i, v);
+    });
 }
 __global__ void __launch_bounds__(1024) k_grey(GreyCtx x)
 {
@@ -1227,7 +1387,7 @@ __global__ void __launch_bounds__(256) k_group_sum(GroupSumArgs a) { group_sum_b
     }
 // (6 CTAs per SM: unbounded, the argument block held in registers leaves 3 and 64 slabs'
 // restriction to the grey level takes 25% longer)
-TRT_BATCHED(k_restrict_b, RestrictCtx, 128, 6, restrict_body(x, bx, by))
+TRT_BATCHED(k_restrict_b, RestrictCtx, 128, 6, restrict_run(x, bx, by))
 TRT_BATCHED(k_grey_b, GreyCtx, 1024, 1, grey_body(x))
 TRT_BATCHED(k_group_sum_b, GroupSumArgs, 256, 1, group_sum_body(x, bx))
 #undef TRT_BATCHED
@@ -1342,16 +1502,37 @@ static size_t lo_smem(int precision, int nx)
 }
 
 template <typename R, int T>
-static cudaError_t lo_launch(const LoCtx &x, unsigned nb, size_t sm, cudaStream_t st)
+static cudaError_t lo_launch(const LoCtx &x, const OpacityArgs &a, int op, unsigned nb, size_t sm,
+                             cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_lo_solve<R, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    return e != cudaSuccess ? e : launch_pdl(k_lo_solve<R, T>, dim3(nb), dim3(T), sm, st, x);
+    const auto go = [&](auto kern, auto... more) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        return e != cudaSuccess ? e : launch_pdl(kern, dim3(nb), dim3(T), sm, st, x, more...);
+    };
+    return op == OP_NONE ? go(k_lo_solve<R, T>) : go(k_lo_solve_opac<R, T>, a, op);
 }
 
-cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L)
+// The opacities of a fine level inside a low-order kernel: its arguments, and the per-cell
+// terms from k_cell_terms or, where `ctas` CTAs cannot fill the GPU and a launch costs more
+// than a logarithm more per cell and CTA (3 us against 2), formed in place.
+static cudaError_t fused_opacity(const Problem &p, const double *T, const Level &fine, long ctas,
+                                 OpacityArgs &a, int &op)
+{
+    a = OpacityArgs{};
+    op = OP_NONE;
+    if (!T) return cudaSuccess;
+    a = make_opacity_args(p, T, fine.sig, fine.emis, fine.sigR, nullptr, nullptr, 0.0);
+    op = ctas <= 152 && p.nx <= 128 ? OP_HERE : OP_ARRAYS;
+    return op == OP_HERE ? cudaSuccess : launch_cell_terms(p, a);
+}
+
+cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L, const double *Topac)
 {
     const LoCtx x = make_lo_ctx(p, dt, L);
+    OpacityArgs a;
+    int op;
+    const cudaError_t eo = fused_opacity(p, Topac, L, L.n, a, op);
+    if (eo != cudaSuccess) return eo;
     const size_t sm = lo_smem(p.precision, p.nx);
     // 512 threads where every group has an SM of its own, 256 where the level fits the GPU at
     // three CTAs per SM, if the rows are more than 128 threads take at once.  128 against more
@@ -1360,9 +1541,9 @@ cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L)
     const int T = p.nx <= 128 || L.n > 456 ? 128 : L.n <= 152 ? 512 : 256;
     const auto go = [&](auto zero) {
         using R = decltype(zero);
-        return T == 512   ? lo_launch<R, 512>(x, L.n, sm, p.stream)
-               : T == 256 ? lo_launch<R, 256>(x, L.n, sm, p.stream)
-                          : lo_launch<R, 128>(x, L.n, sm, p.stream);
+        return T == 512   ? lo_launch<R, 512>(x, a, op, L.n, sm, p.stream)
+               : T == 256 ? lo_launch<R, 256>(x, a, op, L.n, sm, p.stream)
+                          : lo_launch<R, 128>(x, a, op, L.n, sm, p.stream);
     };
     return lo_pair(p.precision) ? go(fpair()) : lo_fp32(p.precision) ? go(0.f) : go(0.0);
 }
@@ -1463,7 +1644,7 @@ RestrictCtx make_restrict_ctx(const Problem &p, const Level &src, const Level &d
 }
 
 cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
-                            const GreyArgs *newton, double *pre, bool skip_old)
+                            const GreyArgs *newton, double *pre, bool skip_old, const double *Topac)
 {
     RestrictCtx x = make_restrict_ctx(p, src, dst);
     x.skip_old = skip_old ? 1 : 0;
@@ -1473,7 +1654,14 @@ cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
         x.pre = pre;
     }
     const RestrictPlan q = restrict_plan(p, src.n, dst.n);
-    return launch_pdl(k_restrict, dim3(q.nt + 1, q.gy), dim3(128), 0, p.stream, x);
+    const dim3 grid(q.nt + 1, q.gy);
+    if (!Topac) return launch_pdl(k_restrict, grid, dim3(128), 0, p.stream, x);
+    OpacityArgs a;
+    int op;
+    const cudaError_t e = fused_opacity(p, Topac, src, (long)q.nt * q.gy, a, op);
+    if (e != cudaSuccess) return e;
+    return a.otabp ? launch_pdl(k_restrict_opac<true>, grid, dim3(128), 0, p.stream, x, a, op)
+                   : launch_pdl(k_restrict_opac<false>, grid, dim3(128), 0, p.stream, x, a, op);
 }
 
 cudaError_t launch_restrict_b(const int *meta, int N, const RestrictCtx *xs, int grid,
