@@ -121,6 +121,8 @@ void carve(trt_handle *h, Carver &c)
     for (int l = 1; l + 1 < p.nlev; ++l) {
         h->crs_Eold[l] = l == 1 ? h->crs.Eold : c.take<double>((size_t)p.levels[l] * nx);
         h->crs_Fold[l] = l == 1 ? h->crs.Fold : c.take<double>((size_t)p.levels[l] * (nx + 1));
+        // (a W cycle visits every grid but the finest coarse one again)
+        h->crs_fix[l] = l >= 2 ? c.take<double>(restrict_fix_doubles((int)nx, p.levels[l])) : nullptr;
     }
     carve_level(c, h->grey, 1, p.nx);
     h->flags = c.take<double>(10);
@@ -577,6 +579,7 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
             ++nk;
             // grey visit k reads T~^[k] and writes T~^[k+1]: T~^[0] = T, the last visit
             // writes T, the ones between alternate over Ttil and Tnew
+            std::vector<char> seen(p.nlev, 0);   // grids visited in this cycle
             for (int k = 0; k <= K; ++k) {
                 double *Tst = (k == 0) ? h->T : (((k - 1) & 1) ? h->Tnew : h->Ttil);
                 double *Tout = (k == K) ? h->T : ((k & 1) ? h->Tnew : h->Ttil);
@@ -593,7 +596,8 @@ int trt_step(trt_handle *h, double dt, const trt_cycle *cyc, trt_stats *stats)
                     h->crs.Eold = h->crs_Eold[lev];
                     h->crs.Fold = h->crs_Fold[lev];
                     CK(launch_restrict(p, fine, h->crs, nullptr, nullptr, old_sums[lev] != 0,
-                                       p.tr_mode ? nullptr : Tst));
+                                       p.tr_mode ? nullptr : Tst, h->crs_fix[lev], seen[lev] ? 2 : 1));
+                    seen[lev] = 1;
                     old_sums[lev] = 1;
                     CK(launch_lo_solve(p, dt, h->crs));
                     nk += 2;

@@ -99,6 +99,8 @@ struct RestrictCtx {
     // the target's Eold and Fold sums already hold this step's values (they change only
     // between steps): neither loaded nor summed
     int skip_old;
+    int fixed;     // sums kept between the visits of a cycle: 1 store them in fix, 2 take them
+    double *fix;   // [n_to][4][32 nt]
 };
 
 // How one restriction is split (lo.cu): mode 0, a warp per coarse group; mode 1, a CTA per

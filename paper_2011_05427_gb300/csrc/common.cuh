@@ -318,10 +318,14 @@ cudaError_t ensure_lo_consts(Problem &p, double dt);
 cudaError_t launch_lo_pair_consts(const Problem &p);
 // newton (with pre): the visit's grey Newton arguments; the restriction to the grey level
 // then also forms the per-cell Newton terms into pre ([3][nx]).  skip_old: dst holds this
-// step's Eold and Fold sums already.  Topac as in launch_lo_solve, for a fine src
+// step's Eold and Fold sums already.  Topac as in launch_lo_solve, for a fine src;
+// with it, fixed = 1 stores the sums that depend on the fine solution alone in fix
+// (restrict_fix_doubles), 2 takes them from there (a later visit of the grid in the cycle)
 cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
                             const GreyArgs *newton = nullptr, double *pre = nullptr,
-                            bool skip_old = false, const double *Topac = nullptr);
+                            bool skip_old = false, const double *Topac = nullptr,
+                            double *fix = nullptr, int fixed = 0);
+size_t restrict_fix_doubles(int nx, int n_to);
 // the host-formed constants of a grey visit (c_v/dt, 54 s C_B, the exponential's table)
 GreyArgs grey_args_ready(const Problem &p, const GreyArgs &a);
 size_t restrict_scratch_doubles(const Problem &p);   // from nx and the grids

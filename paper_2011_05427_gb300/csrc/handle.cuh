@@ -18,6 +18,7 @@ struct trt_handle {
     double *gpre;   // [3][nx]: the grey Newton terms formed by the restriction
     trt::Level crs, grey;
     double *crs_Eold[16] = {}, *crs_Fold[16] = {};   // per coarse grid (trt_step)
+    double *crs_fix[16] = {};                          // per coarse grid: launch_restrict's fix
     double *Ecyc, *Ephase;
     double *flags = nullptr;    // [10]: convergence flags [0..6], then the inner-loop
     int *ctl = nullptr;         // control words (ints in the last two doubles of flags)

@@ -859,7 +859,9 @@ __device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, in
 // instead of read (and stored for the other readers of the fine grid's arrays): the lane's
 // per-cell terms stay in registers over the members.  A face's left opacity is the lane
 // before's, through shared memory (xch: two rows of 33 for the warp, by turns).
-template <bool kOld, bool kPair>
+// kFix: the sums that do not depend on the opacities (kFixed) are the caller's, from an
+// earlier visit of the cycle.
+template <bool kOld, bool kPair, bool kFix>
 __device__ inline void restrict_members_opac(const RestrictCtx &x, const OpacityArgs &a, int op,
                                              double (*xch)[33], const Mx &mx, const fpair *e2p,
                                              int p0, int pe, int step, int i, double (&v)[kRV])
@@ -887,7 +889,9 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
     for (int k = 0; k < kRV; ++k) v[k] = 0.0;
     int par = 0;
     for (int p = p0; p < pe; p += step) {
-        const double E = *Ep, EL = *Lp, F = S.F[f], ph = S.phi[c];
+        const double E = *Ep, EL = *Lp, F = S.F[f];
+        double ph = 0.0;
+        if (!kFix) ph = S.phi[c];
         const OpacVals o = cell_opacities<kPair>(a, p, cv, cp, mx, e2p);
         xch[par][lane] = o.sR;
         if (own) {
@@ -899,16 +903,20 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
         const double left = xch[par][max(lane - 1, 0)];
         par ^= 1;
         const double sR = fma(wa, left, wb * o.sR);
-        v[R_PHI] = fma(ph, E, v[R_PHI]);
         v[R_SIG] = fma(o.sg, E, v[R_SIG]);
         v[R_EMIS] += o.em;
-        v[R_E] += E;
+        if (!kFix) {
+            v[R_PHI] = fma(ph, E, v[R_PHI]);
+            v[R_E] += E;
+        }
         const double w = fma(0.5e-6 * kC, EL + E,
                              __longlong_as_double(__double_as_longlong(F) & 0x7fffffffffffffffll));
         v[R_SW] = fma(sR, w, v[R_SW]);
-        v[R_W] += w;
         v[R_SF] = fma(sR, F, v[R_SF]);
-        v[R_F] += F;
+        if (!kFix) {
+            v[R_W] += w;
+            v[R_F] += F;
+        }
         if (kOld) {
             v[R_EOLD] += S.Eold[c];
             v[R_FOLD] += S.Fold[f];
@@ -1035,6 +1043,22 @@ __device__ inline void restrict_boundary_out(const RestrictCtx &x, int P, int la
     if (k == 7) (side ? T.FinX : T.Fin0)[P] = s;
 }
 
+// The sums that a later visit of the same grid in the same cycle would form again from the
+// same fine solution (sum phi E, sum E, sum of the weights, sum F): x.fixed 1 stores them in
+// x.fix ([n_to][4][32 nt]), 2 takes them from there.
+__device__ inline int fixed_index(int k)
+{
+    return k == R_PHI ? 0 : k == R_E ? 1 : k == R_W ? 2 : k == R_F ? 3 : -1;
+}
+__device__ inline void restrict_fixed(const RestrictCtx &x, int P, int bx, int lane, int k, double &v)
+{
+    const int j = fixed_index(k);
+    if (!x.fixed || j < 0) return;
+    double *p = x.fix + ((size_t)P * 4 + j) * x.nt * 32 + bx * 32 + lane;
+    if (x.fixed == 1) *p = v;
+    else v = *p;
+}
+
 // last arrival of `n` CTAs at ticket t (which it resets): the partial sums written before
 // by the others are visible to the CTA that gets true
 __device__ inline bool restrict_last(int *t, int n)
@@ -1098,6 +1122,8 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
     if (many) {
         if (P >= x.n_to) return;
         members(pb, pe, 1, min(i, nx), v);
+#pragma unroll
+        for (int k = 0; k < kRV; ++k) restrict_fixed(x, P, bx, lane, k, v[k]);
         const double sEL = __shfl_up_sync(0xffffffffu, v[R_E], 1);
         if (cell) restrict_cell(x, P, i, v[R_PHI], v[R_SIG], v[R_EMIS], v[R_E]);
         if (face) {
@@ -1118,6 +1144,7 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
     const int kend = x.S.fine ? R_ETAR : kRV;   // a fine source has no compensation
     for (int k = warp; k < kend; k += 4) {
         if (x.skip_old && (k == R_EOLD || k == R_FOLD)) continue;
+        if (x.fixed == 2 && fixed_index(k) >= 0) continue;
         const double s = (red[0][k][lane] + red[1][k][lane]) + (red[2][k][lane] + red[3][k][lane]);
         if (x.nchunk > 1) part[k * np] = s;
         else red[0][k][lane] = s;
@@ -1127,12 +1154,15 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
         const double *all = x.part + (size_t)P * x.nchunk * kRV * np + bx * 32 + lane;
         for (int k = warp; k < kend; k += 4) {
             if (x.skip_old && (k == R_EOLD || k == R_FOLD)) continue;
+            if (x.fixed == 2 && fixed_index(k) >= 0) continue;
             double s = 0.0;
 #pragma unroll 8
             for (int c = 0; c < x.nchunk; ++c) s += __ldcg(all + ((size_t)c * kRV + k) * np);
             red[0][k][lane] = s;
         }
     }
+    if (x.fixed)   // each value by the warp that summed it
+        for (int k = warp; k < kend; k += 4) restrict_fixed(x, P, bx, lane, k, red[0][k][lane]);
     __syncthreads();
     const double(*sv)[32] = red[0];
     if (warp == 0) {
@@ -1348,7 +1378,7 @@ __global__ void __launch_bounds__(128) k_restrict(RestrictCtx x)
 // fine source, its opacities at a.T formed on the way (a coarse visit: every fine group's
 // opacities, then the restriction onto the visit's grid).  The pair form's evaluation runs on
 // the FP32 pipes under the sums' FP64 operations; one launch and a pass over three fields
-// less than k_opacity and k_restrict: 4096 groups x 1000 cells pair 196 us against 89 + 147;
+// less than k_opacity and k_restrict: 4096 groups x 1000 cells pair 196 us against 89 + 147 (178 on average with the sums kept between the visits of a cycle);
 // FP64 (all of it on the FP64 pipe) 62 against 34 + 29
 template <bool kPair>
 __global__ void __launch_bounds__(128) k_restrict_opac(RestrictCtx x, OpacityArgs a, int op)
@@ -1359,10 +1389,13 @@ __global__ void __launch_bounds__(128) k_restrict_opac(RestrictCtx x, OpacityArg
     __shared__ fpair e2p[32];
     const Mx mx = stage_exp(a, e2, e2p);
     restrict_body(x, blockIdx.x, blockIdx.y, [&](int p0, int pe, int step, int i, double (&v)[kRV]) {
-        if (x.skip_old)
-            restrict_members_opac<false, kPair>(x, a, op, xch[threadIdx.x >> 5], mx, e2p, p0, pe, step, i, v);
+        double(*xc)[33] = xch[threadIdx.x >> 5];
+        if (x.fixed == 2)   // not the first visit: the target holds the step's Eold, Fold sums
+            restrict_members_opac<false, kPair, true>(x, a, op, xc, mx, e2p, p0, pe, step, i, v);
+        else if (x.skip_old)
+            restrict_members_opac<false, kPair, false>(x, a, op, xc, mx, e2p, p0, pe, step, i, v);
         else
-            restrict_members_opac<true, kPair>(x, a, op, xch[threadIdx.x >> 5], mx, e2p, p0, pe, step, i, v);
+            restrict_members_opac<true, kPair, false>(x, a, op, xc, mx, e2p, p0, pe, step, i, v);
     });
 }
 __global__ void __launch_bounds__(1024) k_grey(GreyCtx x)
@@ -1640,14 +1673,24 @@ RestrictCtx make_restrict_ctx(const Problem &p, const Level &src, const Level &d
     x.ga = GreyArgs{};
     x.pre = nullptr;
     x.skip_old = 0;
+    x.fixed = 0;
+    x.fix = nullptr;
     return x;
 }
 
+size_t restrict_fix_doubles(int nx, int n_to)
+{
+    return (size_t)n_to * 4 * 32 * ((nx + 1 + kRTile - 1) / kRTile);
+}
+
 cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
-                            const GreyArgs *newton, double *pre, bool skip_old, const double *Topac)
+                            const GreyArgs *newton, double *pre, bool skip_old, const double *Topac,
+                            double *fix, int fixed)
 {
     RestrictCtx x = make_restrict_ctx(p, src, dst);
     x.skip_old = skip_old ? 1 : 0;
+    x.fix = fix;
+    x.fixed = fix && Topac ? fixed : 0;
     if (newton) {
         x.newton = 1;
         x.ga = *newton;
