@@ -96,72 +96,54 @@ __device__ inline int lo_src_exp(const LoCtx &x, int q, int t, int nthr)
 }
 
 
-__device__ inline double sigR_face(const LoCtx &x, int q, int f)
-{
-    const int nx = x.nx;
-    if (!x.L.fine) return x.L.sigR[(size_t)q * (nx + 1) + f];
-    const double *sc = x.L.sigR + (size_t)q * nx;
-    if (f == 0) return sc[0];
-    if (f == nx) return sc[nx - 1];
-    return (sc[f - 1] * x.h[f - 1] + sc[f] * x.h[f]) * x.ihf[f];
-}
-
 // F_f = GD + PL E_{f-1} - PR E_f  (boundary faces: the face energy already eliminated).
 // kW: GD is instead W = dx/(c dt) / D, the factor of Fold in GD, without the boundary
 // inflow terms (the first pass of the pair staging, before the source scale is known).
+// Every load comes before the arithmetic, the two boundaries in one branch: on a level of a
+// few cells or groups a second round trip to L2, and a warp that holds both boundary faces
+// taking two branches in turn, were a third of the staging's time.
 template <typename R, bool kW = false>
 __device__ inline void face_coef(const LoCtx &x, int q, int f, R &PL, R &PR, R &GD, int ks = 0)
 {
     const int nx = x.nx;
-    const double *phi = x.L.phi + (size_t)q * nx;
-    const R dx = lc<R>(x, 0, f, x.hf);
-    R phiL, phiR;
-    if (f == 0) {
-        phiL = (R)x.L.phib0[q];
-        phiR = (R)phi[0];
-    } else if (f == nx) {
-        phiL = (R)phi[nx - 1];
-        phiR = (R)x.L.phibX[q];
-    } else {
-        phiL = (R)phi[f - 1];
-        phiR = (R)phi[f];
-    }
-    if (!x.L.fine) {
-        phiL += (R)x.L.etaL[(size_t)q * (nx + 1) + f];
-        phiR += (R)x.L.etaR[(size_t)q * (nx + 1) + f];
-    }
-    const R c = (R)kC;
-    R D, Gf;
-    if constexpr (!std::is_same<R, float>::value) {
-        // dx (1/(c dt) + sigma_R,face) and dx Fold/(c dt) from the row constants: the face
-        // opacity's dx-weighted mean folded into one FMA per cell opacity
-        const R dxi = lc<R>(x, 1, f, x.dxicdt);
-        if (!x.L.fine) {
-            D = fma(dx, (R)x.L.sigR[(size_t)q * (nx + 1) + f], dxi);
-        } else {
-            const double *sc = x.L.sigR + (size_t)q * nx;
-            D = (f == 0)    ? fma(dx, (R)sc[0], dxi)
-                : (f == nx) ? fma(dx, (R)sc[nx - 1], dxi)
-                            : fma(lc<R>(x, 2, f, x.fwl), (R)sc[f - 1],
-                                  fma(lc<R>(x, 3, f, x.fwr), (R)sc[f], dxi));
+    const bool lo = f == 0, hi = f == nx;
+    const size_t fq = (size_t)q * (nx + 1) + f, cq = (size_t)q * nx;
+    const double vL = *(lo ? x.L.phib0 + q : x.L.phi + cq + f - 1);
+    const double vR = *(hi ? x.L.phibX + q : x.L.phi + cq + f);
+    double Cb = 0.0, Ein = 0.0, Fin = 0.0, Fo = 0.0;
+    if (lo || hi) {
+        Cb = (lo ? x.L.C0 : x.L.CX)[q];
+        if constexpr (!kW) {
+            Ein = (lo ? x.L.Ein0 : x.L.EinX)[q];
+            Fin = (lo ? x.L.Fin0 : x.L.FinX)[q];
         }
-        if constexpr (kW) Gf = dxi;
-        else Gf = src_in<R>(x.L.Fold[(size_t)q * (nx + 1) + f], ks) * dxi;
-    } else {
-        const R icdt = (R)x.icdt;
-        D = dx * (icdt + (R)sigR_face(x, q, f));
-        Gf = dx * (R)x.L.Fold[(size_t)q * (nx + 1) + f] * icdt;
     }
-    if (f == 0) {
-        const R iC0 = rcpR<R>((R)x.L.C0[q]);
-        D -= phiL * iC0;
-        if constexpr (!kW)
-            Gf += c * phiL * src_in<R>(x.L.Ein0[q], ks) - phiL * src_in<R>(x.L.Fin0[q], ks) * iC0;
-    } else if (f == nx) {
-        const R iCX = rcpR<R>((R)x.L.CX[q]);
-        D += phiR * iCX;
-        if constexpr (!kW)
-            Gf += -c * phiR * src_in<R>(x.L.EinX[q], ks) + phiR * src_in<R>(x.L.FinX[q], ks) * iCX;
+    if constexpr (!kW) Fo = x.L.Fold[fq];
+    const R dx = lc<R>(x, 0, f, x.hf);
+    // dx (1/(c dt) + sigma_R,face) and dx Fold/(c dt) from the row constants: the face
+    // opacity's dx-weighted mean folded into one FMA per cell opacity
+    const R dxi = lc<R>(x, 1, f, x.dxicdt);
+    R phiL = (R)vL, phiR = (R)vR, D;
+    if (!x.L.fine) {
+        const double eL = x.L.etaL[fq], eR = x.L.etaR[fq];
+        D = fma(dx, (R)x.L.sigR[fq], dxi);
+        phiL += (R)eL;
+        phiR += (R)eR;
+    } else {
+        const double *sc = x.L.sigR + cq;
+        const double sl = sc[max(f - 1, 0)], sr = sc[min(f, nx - 1)];
+        D = lo || hi ? fma(dx, (R)(lo ? sr : sl), dxi)
+                     : fma(lc<R>(x, 2, f, x.fwl), (R)sl, fma(lc<R>(x, 3, f, x.fwr), (R)sr, dxi));
+    }
+    R Gf;
+    if constexpr (kW) Gf = dxi;
+    else Gf = src_in<R>(Fo, ks) * dxi;
+    const R c = (R)kC;
+    if (lo || hi) {   // E_face = E_in + (F - F_in)/(c C)
+        const R iC = rcpR<R>((R)Cb);
+        const R s = lo ? phiL : -phiR;
+        D -= s * iC;
+        if constexpr (!kW) Gf += s * (c * src_in<R>(Ein, ks) - src_in<R>(Fin, ks) * iC);
     }
     const R iD = rcpR<R>(D);
     const R ciD = c * iD;
@@ -170,30 +152,21 @@ __device__ inline void face_coef(const LoCtx &x, int q, int f, R &PL, R &PR, R &
     GD = Gf * iD;
 }
 
-// row i of the cell equation: Ap = h (1/dt + a), Dp = h (s + Eold/dt)
+// row i of the cell equation, from the row constants h/dt, c h, 2 h: Ap = h (1/dt + a), Dp =
+// h (s + Eold/dt)
 template <typename R>
 __device__ inline void cell_row(const LoCtx &x, int q, int i, R &Ap, R &Dp, int ks = 0)
 {
-    const R Eo = src_in<R>(x.L.Eold[(size_t)q * x.nx + i], ks);
-    if constexpr (!std::is_same<R, float>::value) {   // from the row constants h/dt, c h, 2 h
-        const R hidt = lc<R>(x, 4, i, x.hidt);
-        if (x.a_cell) {
-            const R hc = lc<R>(x, 7, i, x.h);
-            Ap = fma(hc, (R)x.a_cell[i], hidt);
-            Dp = fma(hidt, Eo, hc * src_in<R>(x.s_cell[i], ks));
-        } else {
-            Ap = fma(lc<R>(x, 5, i, x.hc), (R)x.L.sig[(size_t)q * x.nx + i], hidt);
-            Dp = fma(hidt, Eo, lc<R>(x, 6, i, x.h2) * src_in<R>(x.L.emis[(size_t)q * x.nx + i], ks));
-        }
-        return;
-    }
-    const R hi = (R)x.h[i], idt = (R)x.idt;
+    const size_t c = (size_t)q * x.nx + i;
+    const R Eo = src_in<R>(x.L.Eold[c], ks);
+    const R hidt = lc<R>(x, 4, i, x.hidt);
     if (x.a_cell) {
-        Ap = hi * (idt + (R)x.a_cell[i]);
-        Dp = hi * fma(Eo, idt, (R)x.s_cell[i]);
+        const R hc = lc<R>(x, 7, i, x.h);
+        Ap = fma(hc, (R)x.a_cell[i], hidt);
+        Dp = fma(hidt, Eo, hc * src_in<R>(x.s_cell[i], ks));
     } else {
-        Ap = hi * fma((R)kC, (R)x.L.sig[(size_t)q * x.nx + i], idt);
-        Dp = hi * fma(Eo, idt, (R)2 * (R)x.L.emis[(size_t)q * x.nx + i]);
+        Ap = fma(lc<R>(x, 5, i, x.hc), (R)x.L.sig[c], hidt);
+        Dp = fma(hidt, Eo, lc<R>(x, 6, i, x.h2) * src_in<R>(x.L.emis[c], ks));
     }
 }
 
@@ -713,41 +686,59 @@ __global__ void __launch_bounds__(128) k_lo_solve_b(const int *__restrict__ meta
 // absorption w c sig*, the source w Q* - (1 - w) c_v (T* - Told)/dt and 1/Lambda.  Called
 // by the grey kernel on the grey level's arrays, or by the restriction's second stage on
 // the same values it writes there (the same operations, the same bits).
-__device__ inline void grey_newton_terms(const GreyArgs &a, int have_prev, int i, double sig,
-                                         double Q, double Esum, double &sa, double &ss,
-                                         double &sL)
+// In two parts: what does not need the restricted sums (base = c_v/dt + Q'(T*), mT = c_v (T* -
+// Told)/dt, rdT = 1/(T* - T_prev) or 0 without a secant), and the rest.
+struct GreyNewtonIn {   // the cell's inputs of the first part
+    double Ts, Told, Tp, sp;
+};
+__device__ inline GreyNewtonIn grey_newton_load(const GreyArgs &a, int have_prev, int i)
+{
+    GreyNewtonIn c;
+    c.Ts = a.Tstar[i];
+    c.Told = a.Told[i];
+    c.Tp = have_prev ? a.T_prev[i] : c.Ts;
+    c.sp = have_prev ? a.sig_prev[i] : 0.0;
+    return c;
+}
+__device__ inline void grey_newton_first(const GreyArgs &a, const GreyNewtonIn &c, double &base,
+                                         double &mT, double &rdT)
 {
     const double cvdt = a.cvdt;
     const double k54 = a.k54;
-    const double Ts = a.Tstar[i];
-    const double iTs = rcp64(Ts);
+    const double Ts = c.Ts;
     double dQ = k54;   // first edge at 0: (1 + x) e^{-x} = 1
-    if (a.nu_first != 0.0) {
-        const double x1 = a.nu_first * iTs;
-        dQ = k54 * (1.0 + x1) * texp(-x1, a.e2, a.ec);
+    if (a.nu_first != 0.0 || !isinf(a.nu_last)) {
+        const double iTs = rcp64(Ts);
+        if (a.nu_first != 0.0) {
+            const double x1 = a.nu_first * iTs;
+            dQ = k54 * (1.0 + x1) * texp(-x1, a.e2, a.ec);
+        }
+        if (!isinf(a.nu_last)) {
+            const double xL = a.nu_last * iTs;
+            dQ -= k54 * (1.0 + xL) * texp(-xL, a.e2, a.ec);
+        }
     }
-    if (!isinf(a.nu_last)) {
-        const double xL = a.nu_last * iTs;
-        dQ -= k54 * (1.0 + xL) * texp(-xL, a.e2, a.ec);
-    }
-    double D = 0.0;
-    if (have_prev) {
-        const double Tp = a.T_prev[i];
-        // T* != T_prev on the encodings (positive finite values: integer instructions, not
-        // an FP64 compare); across grids only where |dT| is far above rounding (relative
-        // noise ~ eps T/|dT|)
-        const bool moved = __double_as_longlong(Ts) != __double_as_longlong(Tp);
-        const bool cut = __double_as_longlong(a.secant_cut) != 0ll;
-        if (moved && (!cut || fabs(Ts - Tp) > a.secant_cut * Ts))
-            D = (sig - a.sig_prev[i]) * rcp64(Ts - Tp);
-    }
-    const double base = cvdt + dQ;
-    double L = base - kC * D * Esum;
+    // T* != T_prev on the encodings (positive finite values: integer instructions, not an
+    // FP64 compare); across grids only where |dT| is far above rounding (relative noise ~ eps
+    // T/|dT|)
+    rdT = 0.0;
+    const bool moved = __double_as_longlong(Ts) != __double_as_longlong(c.Tp);
+    const bool cut = __double_as_longlong(a.secant_cut) != 0ll;
+    if (moved && (!cut || fabs(Ts - c.Tp) > a.secant_cut * Ts)) rdT = rcp64(Ts - c.Tp);
+    base = cvdt + dQ;
+    mT = cvdt * (Ts - c.Told);
+}
+__device__ inline void grey_newton_rest(const GreyArgs &a, double base, double mT, double rdT,
+                                        double sp, double sig, double Q, double Esum, double &sa,
+                                        double &ss, double &sL)
+{
+    double L = base;
+    if (__double_as_longlong(rdT) != 0ll) L = base - kC * ((sig - sp) * rdT) * Esum;
     if (L < 0.5 * base) L = 0.5 * base;
     const double iL = rcp64(L);
-    const double w = cvdt * iL;
+    const double w = a.cvdt * iL;
     sa = w * kC * sig;
-    ss = w * Q - (1.0 - w) * cvdt * (Ts - a.Told[i]);
+    ss = w * Q - (1.0 - w) * mT;
     sL = iL;
 }
 
@@ -925,14 +916,14 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
     }
 }
 
-// the E-weighted cell means of coarse group P at cell i (and the grey visit's Newton terms)
+// the E-weighted cell means of coarse group P at cell i
 __device__ inline void restrict_cell(const RestrictCtx &x, int P, int i, double sphi, double ssig,
-                                     double semis, double sE)
+                                     double sE, double &sg)
 {
     const Level &S = x.S;
     const int nx = x.nx;
     const size_t c = (size_t)P * nx + i;
-    double ph, sg;
+    double ph;
     if (sE != 0.0) {
         ph = rquot(sphi, sE);
         sg = rquot(ssig, sE);
@@ -947,13 +938,6 @@ __device__ inline void restrict_cell(const RestrictCtx &x, int P, int i, double 
     }
     x.T.phi[c] = ph;
     x.T.sig[c] = sg;
-    if (x.newton) {   // target = the grey level: the visit's Newton terms of cell i
-        double sa, ss, sL;
-        grey_newton_terms(x.ga, x.ga.have_prev, i, sg, 2.0 * semis, sE, sa, ss, sL);
-        x.pre[i] = sa;
-        x.pre[nx + i] = ss;
-        x.pre[2 * (size_t)nx + i] = sL;
-    }
 }
 
 // the copied sums of coarse group P at position i
@@ -1125,7 +1109,8 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
 #pragma unroll
         for (int k = 0; k < kRV; ++k) restrict_fixed(x, P, bx, lane, k, v[k]);
         const double sEL = __shfl_up_sync(0xffffffffu, v[R_E], 1);
-        if (cell) restrict_cell(x, P, i, v[R_PHI], v[R_SIG], v[R_EMIS], v[R_E]);
+        double sg;
+        if (cell) restrict_cell(x, P, i, v[R_PHI], v[R_SIG], v[R_E], sg);
         if (face) {
             restrict_sums(x, P, i, v[R_EMIS], v[R_E], v[R_EOLD], v[R_FOLD]);
             restrict_face(x, P, i, v[R_SW], v[R_W], v[R_SF], v[R_F], v[R_E], sEL, v[R_ETAR],
@@ -1133,6 +1118,9 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
         }
         return;
     }
+    // the grey visit's Newton terms are formed with the cell means: their inputs early
+    GreyNewtonIn nin{};
+    if (x.newton && warp == 3 && cell) nin = grey_newton_load(x.ga, x.ga.have_prev, i);
     members(pb + warp, pe, 4, min(i, nx), v);
 #pragma unroll
     for (int k = 0; k < kRV; ++k) red[warp][k][lane] = v[k];
@@ -1165,8 +1153,32 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
         for (int k = warp; k < kend; k += 4) restrict_fixed(x, P, bx, lane, k, red[0][k][lane]);
     __syncthreads();
     const double(*sv)[32] = red[0];
+    // the coefficients by four warps; warp 3 forms the first part of the Newton terms for warp 0
     if (warp == 0) {
-        if (cell) restrict_cell(x, P, i, sv[R_PHI][lane], sv[R_SIG][lane], sv[R_EMIS][lane], sv[R_E][lane]);
+        double sg = 0.0;
+        if (cell) restrict_cell(x, P, i, sv[R_PHI][lane], sv[R_SIG][lane], sv[R_E][lane], sg);
+        if (x.newton) {
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+            if (cell) {
+                double sa, ss, sL;
+                grey_newton_rest(x.ga, red[1][0][lane], red[1][1][lane], red[1][2][lane],
+                                 red[1][3][lane], sg, 2.0 * sv[R_EMIS][lane], sv[R_E][lane], sa, ss,
+                                 sL);
+                x.pre[i] = sa;
+                x.pre[nx + i] = ss;
+                x.pre[2 * (size_t)nx + i] = sL;
+            }
+        }
+    } else if (warp == 3) {
+        if (x.newton) {
+            double base = 0.0, mT = 0.0, rdT = 0.0;
+            if (cell) grey_newton_first(x.ga, nin, base, mT, rdT);
+            red[1][0][lane] = base;
+            red[1][1][lane] = mT;
+            red[1][2][lane] = rdT;
+            red[1][3][lane] = nin.sp;
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+        }
     } else if (warp == 1) {
         if (face)
             restrict_sums(x, P, i, sv[R_EMIS][lane], sv[R_E][lane], sv[R_EOLD][lane], sv[R_FOLD][lane]);
@@ -1222,12 +1234,6 @@ __device__ inline void block_max_bits(unsigned long long (&v)[kGreyNV], unsigned
     }
 }
 
-__device__ inline void grey_newton_cell(const GreyArgs &a, const Level &g, int have_prev, int i,
-                                        double &sa, double &ss, double &sL)
-{
-    grey_newton_terms(a, have_prev, i, g.sig[i], 2.0 * g.emis[i], g.Esum[i], sa, ss, sL);
-}
-
 // the grey level's outputs from the solution: E, the face fluxes F_f = GD_f + PL_f E_{f-1} -
 // PR_f E_f and the boundary face energies
 __device__ void grey_outputs(const LoCtx &x, const double *sm, int S, int n)
@@ -1247,26 +1253,46 @@ __device__ void grey_outputs(const LoCtx &x, const double *sm, int S, int n)
     }
 }
 
+// what the update of a cell reads (loaded before the solve, whose chain hides the latency)
+struct GreyCell {
+    double Ts, Told, sig, emis, Tc, Ec, Tp, Ep;
+};
+__device__ inline GreyCell grey_cell_load(const GreyArgs &a, const Level &g, int i)
+{
+    GreyCell c{};
+    c.Ts = a.Tstar[i];
+    c.Told = a.Told[i];
+    c.sig = g.sig[i];
+    c.emis = g.emis[i];
+    if (a.want_norms) {
+        c.Tc = a.Tcyc[i];
+        c.Ec = a.Ecyc[i];
+        c.Tp = a.Tphase[i];
+        c.Ep = a.Ephase[i];
+    }
+    return c;
+}
+
 // T at cell i from the grey solution E; the bad-value test and the norms' terms
-__device__ inline void grey_update_cell(const GreyArgs &a, const Level &g, int i, double sL,
+__device__ inline void grey_update_cell(const GreyArgs &a, const GreyCell &c, int i, double sL,
                                         double E, unsigned long long (&v)[kGreyNV])
 {
     const unsigned long long kInfBits = 0x7ff0000000000000ull;
     const double cvdt = a.cvdt;
-    const double Ts = a.Tstar[i];
-    const double T = Ts + (kC * g.sig[i] * E - 2.0 * g.emis[i] - cvdt * (Ts - a.Told[i])) * sL;
+    const double Ts = c.Ts;
+    const double T = Ts + (kC * c.sig * E - 2.0 * c.emis - cvdt * (Ts - c.Told)) * sL;
     a.T[i] = T;
     const long long tb = __double_as_longlong(T);
     const unsigned long long eb = (unsigned long long)__double_as_longlong(E) & 0x7fffffffffffffffull;
     // T > 0 and finite: sign clear, not zero, below the infinity encoding
     if (tb <= 0 || (unsigned long long)tb >= kInfBits || eb >= kInfBits) v[0] = 1ull;
     if (a.want_norms) {
-        v[1] = umax64(v[1], nn_bits(fabs(T - a.Tcyc[i])));
+        v[1] = umax64(v[1], nn_bits(fabs(T - c.Tc)));
         v[2] = umax64(v[2], nn_bits(fabs(T)));
-        v[3] = umax64(v[3], nn_bits(fabs(E - a.Ecyc[i])));
+        v[3] = umax64(v[3], nn_bits(fabs(E - c.Ec)));
         v[4] = umax64(v[4], nn_bits(fabs(E)));
-        v[5] = umax64(v[5], nn_bits(fabs(T - a.Tphase[i])));
-        v[6] = umax64(v[6], nn_bits(fabs(E - a.Ephase[i])));
+        v[5] = umax64(v[5], nn_bits(fabs(T - c.Tp)));
+        v[6] = umax64(v[6], nn_bits(fabs(E - c.Ep)));
         if (a.T_out) a.T_out[i] = T;
         if (a.Tcyc_out) a.Tcyc_out[i] = T;
         if (a.Ecyc_out) a.Ecyc_out[i] = E;
@@ -1285,13 +1311,25 @@ __device__ void grey_body(const GreyCtx &x)
     double *wsm = red + kGreyRed;   // the solver's rows (TriLayout) and its 3 P values more
     const GreyArgs &a = x.a;
     const Level &g = x.lo.L;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+    const int t = threadIdx.x;
+    GreyCell mine{};             // the thread's first cell
+    if (t < nx) mine = grey_cell_load(a, g, t);
+    double bad_before = 0.0;     // what thread 0 will test at the end
+    int cycles = 0;
+    if (t == 0 && a.want_norms && a.ctl) {
+        bad_before = a.flags[0];
+        cycles = a.ctl[1];
+    }
+    for (int i = t; i < nx; i += blockDim.x) {
         if (a.pre) {   // formed by the restriction before this kernel
             sa[i] = a.pre[i];
             ss[i] = a.pre[nx + i];
             sL[i] = a.pre[2 * (size_t)nx + i];
         } else {
-            grey_newton_cell(a, g, have_prev, i, sa[i], ss[i], sL[i]);
+            const GreyNewtonIn c = grey_newton_load(a, have_prev, i);
+            double base, mT, rdT;
+            grey_newton_first(a, c, base, mT, rdT);
+            grey_newton_rest(a, base, mT, rdT, c.sp, g.sig[i], 2.0 * g.emis[i], g.Esum[i], sa[i], ss[i], sL[i]);
         }
         a.sig_prev_out[i] = g.sig[i];
         a.T_prev_out[i] = a.Tstar[i];
@@ -1302,21 +1340,24 @@ __device__ void grey_body(const GreyCtx &x)
     lc.s_cell = ss;
     const TriLayout y = tri_layout(nx);
     if (nx >= 2) {
-        lo_stage<double>(lc, 0, wsm, y.S, threadIdx.x, blockDim.x);
+        lo_stage<double>(lc, 0, wsm, y.S, t, blockDim.x);
         __syncthreads();
         tri_solve<double>(wsm, wsm + 6 * y.S, nx, y);
         grey_outputs(lc, wsm, y.S, nx);
     } else {
-        if (threadIdx.x == 0) lo_one_cell<double>(lc, 0);
+        if (t == 0) lo_one_cell<double>(lc, 0);
         __syncthreads();
     }
     const double *Esol = nx >= 2 ? wsm + 5 * (size_t)y.S : g.E;
     // v: bad flag, max|T - Tcyc|, max|T|, max|E - Ecyc|, max|E|, max|T - Tphase|,
     // max|E - Ephase| as non-negative encodings (flags[0 .. 6])
     unsigned long long v[kGreyNV] = {};
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) grey_update_cell(a, g, i, sL[i], Esol[nx >= 2 ? lc.lo_slot[i] : i], v);
+    for (int i = t; i < nx; i += blockDim.x) {
+        if (i != t) mine = grey_cell_load(a, g, i);
+        grey_update_cell(a, mine, i, sL[i], Esol[nx >= 2 ? lc.lo_slot[i] : i], v);
+    }
     block_max_bits(v, reinterpret_cast<unsigned long long *>(red));
-    if (threadIdx.x == 0) {
+    if (t == 0) {
         if (v[0] != 0ull) a.flags[0] = 1.0;
         if (a.want_norms) {
             a.flags[1] = __longlong_as_double((long long)v[1]);
@@ -1331,13 +1372,13 @@ __device__ void grey_body(const GreyCtx &x)
                 const double f3 = __longlong_as_double((long long)v[3]);
                 const double f4 = __longlong_as_double((long long)v[4]);
                 const bool conv_in = f1 <= a.eps_in * f2 && f3 <= a.eps_in * f4;
-                a.ctl[1] += 1;
+                a.ctl[1] = cycles + 1;
                 // a bad temperature of this visit or of an earlier visit of the cycle
-                if (v[0] != 0ull || a.flags[0] != 0.0 || (!a.fixed && conv_in)) a.ctl[0] = 1;
+                if (v[0] != 0ull || bad_before != 0.0 || (!a.fixed && conv_in)) a.ctl[0] = 1;
             }
         }
     }
-    if (a.have_prev_dev && threadIdx.x == 0) *a.have_prev_dev = 1;   // after the reduction's barriers
+    if (a.have_prev_dev && t == 0) *a.have_prev_dev = 1;   // after the reduction's barriers
 }
 
 // out_i = sum_q X[q][i]: block of 256 threads = 32 cells x 8 rows; row y sums the groups
