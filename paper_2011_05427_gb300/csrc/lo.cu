@@ -598,29 +598,53 @@ __device__ inline Mx stage_exp(const OpacityArgs &a, double *e2, fpair *e2p)
 }
 // where an evaluation takes its per-cell terms: 1, formed here (k_cell_terms did not run)
 enum { OP_NONE = 0, OP_ARRAYS = 1, OP_HERE = 2 };
+// the terms of a cell that the tabulated evaluation reads, and no more of CellVals: a lane
+// keeps them over its members
 template <bool kPair>
-__device__ inline void cell_terms(const OpacityArgs &a, int op, int i, CellVals &v, CellPair &cp)
+struct OpacCell {
+    double t, iT, iT3, kET;
+    float tf;
+    int m;
+};
+template <>
+struct OpacCell<true> {
+    CellPair cp;
+    float tf;
+    int m;
+};
+template <bool kPair>
+__device__ inline OpacCell<kPair> cell_terms(const OpacityArgs &a, int op, int i)
 {
-    if (op == OP_HERE) {
-        v = cell_vals(a, i);
-        if (kPair) cp = cell_pair(a, i, v);
+    const CellVals v = op == OP_HERE ? cell_vals(a, i) : cell_arrays(a).get(i);
+    OpacCell<kPair> c;
+    if constexpr (kPair) {
+        c.cp = op == OP_HERE ? cell_pair(a, i, v) : cell_pair_at(a, i);
     } else {
-        v = cell_arrays(a).get(i);
-        if (kPair) cp = cell_pair_at(a, i);
+        c.t = v.t; c.iT = v.iT; c.iT3 = v.iT3; c.kET = v.kET;
     }
+    c.tf = v.tf;
+    c.m = v.m;
+    return c;
 }
-// sigma_E, e_g, sigma_R of group g in the cell
-template <bool kPair>
-__device__ inline OpacVals cell_opacities(const OpacityArgs &a, int g, const CellVals &v,
-                                          const CellPair &cp, const Mx &mx, const fpair *e2p)
+// sigma_E, e_g, sigma_R of group g in cell i with terms c; kIn: the cell is inside the tables
+template <bool kPair, bool kIn = false>
+__device__ inline OpacVals cell_opacities(const OpacityArgs &a, int g, int i, const OpacCell<kPair> &c,
+                                          const Mx &mx, const fpair *e2p)
 {
-    if (kPair && v.m >= 0) {
+    if (!kIn && c.m < 0) {   // outside the tables: the temperature and its powers again (cell_vals' operations)
+        const double T = a.T[i], iT = rcp64(T);
+        return opacity_direct(a.edges[g], a.edges[g + 1], a.s, T, iT, iT * iT * iT, a.ser, mx);
+    }
+    if constexpr (kPair) {
         fpair sg, em, sR;
         int k;
-        opacity_vals_pair(a, g, v.m, v.tf, cp, e2p, sg, em, k, sR);
+        opacity_vals_pair(a, g, c.m, c.tf, c.cp, e2p, sg, em, k, sR);
         return OpacVals{pr_join(sg, 0), pr_join(em, k), pr_join(sR, 0)};
+    } else {
+        CellVals v;
+        v.t = c.t; v.iT = c.iT; v.iT3 = c.iT3; v.kET = c.kET; v.tf = c.tf; v.m = c.m;
+        return opacity_vals(a, g, v, mx);
     }
-    return opacity_vals(a, g, v, mx);
 }
 // the opacities of group g in every cell by the CTA, into the fine grid's arrays (ends with
 // a barrier)
@@ -631,10 +655,7 @@ __device__ void group_opacities(const OpacityArgs &a, int op, int g)
     __shared__ fpair e2p[32];
     const Mx mx = stage_exp(a, e2, e2p);
     for (int i = threadIdx.x; i < a.nx; i += blockDim.x) {
-        CellVals v;
-        CellPair cp;
-        cell_terms<kPair>(a, op, i, v, cp);
-        const OpacVals o = cell_opacities<kPair>(a, g, v, cp, mx, e2p);
+        const OpacVals o = cell_opacities<kPair>(a, g, i, cell_terms<kPair>(a, op, i), mx, e2p);
         const size_t idx = (size_t)g * a.nx + i;
         a.sigE[idx] = o.sg;
         a.emis[idx] = o.em;
@@ -851,11 +872,12 @@ __device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, in
 // per-cell terms stay in registers over the members.  A face's left opacity is the lane
 // before's, through shared memory (xch: two rows of 33 for the warp, by turns).
 // kFix: the sums that do not depend on the opacities (kFixed) are the caller's, from an
-// earlier visit of the cycle.
-template <bool kOld, bool kPair, bool kFix>
+// earlier visit of the cycle.  kIn: every lane's cell is inside the tables.
+template <bool kOld, bool kPair, bool kFix, bool kIn>
 __device__ inline void restrict_members_opac(const RestrictCtx &x, const OpacityArgs &a, int op,
-                                             double (*xch)[33], const Mx &mx, const fpair *e2p,
-                                             int p0, int pe, int step, int i, double (&v)[kRV])
+                                             const OpacCell<kPair> &cc, double (*xch)[33],
+                                             const Mx &mx, const fpair *e2p, int p0, int pe,
+                                             int step, int i, double (&v)[kRV])
 {
     const Level &S = x.S;
     const int nx = x.nx, lane = threadIdx.x & 31;
@@ -873,9 +895,6 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
         wa = i < nx ? x.h[i - 1] * x.ihf[i] : 1.0;
         wb = i < nx ? x.h[i] * x.ihf[i] : 0.0;
     }
-    CellVals cv;
-    CellPair cp;
-    cell_terms<kPair>(a, op, ic, cv, cp);
 #pragma unroll
     for (int k = 0; k < kRV; ++k) v[k] = 0.0;
     int par = 0;
@@ -883,7 +902,7 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
         const double E = *Ep, EL = *Lp, F = S.F[f];
         double ph = 0.0;
         if (!kFix) ph = S.phi[c];
-        const OpacVals o = cell_opacities<kPair>(a, p, cv, cp, mx, e2p);
+        const OpacVals o = cell_opacities<kPair, kIn>(a, p, ic, cc, mx, e2p);
         xch[par][lane] = o.sR;
         if (own) {
             S.sig[c] = o.sg;
@@ -914,6 +933,21 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
         }
         Ep += Ed; Lp += Ld; c += cd; f += cd + step;
     }
+}
+
+// The form for a warp with a cell outside the tables, out of line: the direct integrals' call
+// in the loop would cost every lane 32 to 48 registers.
+template <bool kOld, bool kPair, bool kFix>
+__device__ __noinline__ void restrict_members_direct(const RestrictCtx &x, const OpacityArgs &a,
+                                                     int op, double (*xch)[33], const double *e2,
+                                                     const fpair *e2p, int p0, int pe, int step,
+                                                     int i, double *u)
+{
+    double v[kRV];
+    const OpacCell<kPair> cc = cell_terms<kPair>(a, op, min(max(i, 0), x.nx - 1));
+    restrict_members_opac<kOld, kPair, kFix, false>(x, a, op, cc, xch, Mx{e2, a.ec}, e2p, p0, pe, step,
+                                                    i, v);
+    for (int k = 0; k < kRV; ++k) u[k] = v[k];
 }
 
 // the E-weighted cell means of coarse group P at cell i
@@ -1419,10 +1453,17 @@ __global__ void __launch_bounds__(128) k_restrict(RestrictCtx x)
 // fine source, its opacities at a.T formed on the way (a coarse visit: every fine group's
 // opacities, then the restriction onto the visit's grid).  The pair form's evaluation runs on
 // the FP32 pipes under the sums' FP64 operations; one launch and a pass over three fields
-// less than k_opacity and k_restrict: 4096 groups x 1000 cells pair 196 us against 89 + 147 (178 on average with the sums kept between the visits of a cycle);
-// FP64 (all of it on the FP64 pipe) 62 against 34 + 29
-template <bool kPair>
-__global__ void __launch_bounds__(128) k_restrict_opac(RestrictCtx x, OpacityArgs a, int op)
+// less than k_opacity and k_restrict.  A member is a chain of table loads and dependent
+// operations, so the warps in flight decide: a kernel per form of the sums, the direct
+// integrals out of line and only the terms that the tables need kept per lane (168 -> 96
+// registers, 3 -> 5 CTAs per SM).  4096 groups x 1000 cells pair 163 us on a later visit of a
+// cycle (FP64 pipe's own time 93), 198 us with the sums of phi E, E and the weights too,
+// against 89 + 147 for the two kernels and 203 / 260 at 168 registers; 6 CTAs at 80 registers
+// 168 / 192, 4 at 128 169 / 213.  1024 groups x 500 cells FP64 (all of it on the FP64 pipe)
+// 59 us against 34 + 29, 63 with 3 CTAs and 57 to 60 with 5.
+template <bool kPair, bool kOld, bool kFix>
+__global__ void __launch_bounds__(128, kPair ? 5 : 4)
+    k_restrict_opac(const __grid_constant__ RestrictCtx x, const __grid_constant__ OpacityArgs a, int op)
 {
     griddep_wait();
     if (x.gate && *x.gate) return;
@@ -1431,12 +1472,15 @@ __global__ void __launch_bounds__(128) k_restrict_opac(RestrictCtx x, OpacityArg
     const Mx mx = stage_exp(a, e2, e2p);
     restrict_body(x, blockIdx.x, blockIdx.y, [&](int p0, int pe, int step, int i, double (&v)[kRV]) {
         double(*xc)[33] = xch[threadIdx.x >> 5];
-        if (x.fixed == 2)   // not the first visit: the target holds the step's Eold, Fold sums
-            restrict_members_opac<false, kPair, true>(x, a, op, xc, mx, e2p, p0, pe, step, i, v);
-        else if (x.skip_old)
-            restrict_members_opac<false, kPair, false>(x, a, op, xc, mx, e2p, p0, pe, step, i, v);
-        else
-            restrict_members_opac<true, kPair, false>(x, a, op, xc, mx, e2p, p0, pe, step, i, v);
+        const OpacCell<kPair> cc = cell_terms<kPair>(a, op, min(max(i, 0), x.nx - 1));
+        if (__all_sync(0xffffffffu, cc.m >= 0)) {
+            restrict_members_opac<kOld, kPair, kFix, true>(x, a, op, cc, xc, mx, e2p, p0, pe, step, i, v);
+        } else {
+            double u[kRV];
+            restrict_members_direct<kOld, kPair, kFix>(x, a, op, xc, e2, e2p, p0, pe, step, i, u);
+#pragma unroll
+            for (int k = 0; k < kRV; ++k) v[k] = u[k];
+        }
     });
 }
 __global__ void __launch_bounds__(1024) k_grey(GreyCtx x)
@@ -1744,8 +1788,15 @@ cudaError_t launch_restrict(const Problem &p, const Level &src, Level &dst,
     int op;
     const cudaError_t e = fused_opacity(p, Topac, src, (long)q.nt * q.gy, a, op);
     if (e != cudaSuccess) return e;
-    return a.otabp ? launch_pdl(k_restrict_opac<true>, grid, dim3(128), 0, p.stream, x, a, op)
-                   : launch_pdl(k_restrict_opac<false>, grid, dim3(128), 0, p.stream, x, a, op);
+    // a later visit of the cycle finds the step's Eold and Fold sums in the target too
+    const int form = x.fixed == 2 ? 2 : x.skip_old ? 1 : 0;
+    auto k = a.otabp ? (form == 2 ? k_restrict_opac<true, false, true>
+                        : form == 1 ? k_restrict_opac<true, false, false>
+                                    : k_restrict_opac<true, true, false>)
+                     : (form == 2 ? k_restrict_opac<false, false, true>
+                        : form == 1 ? k_restrict_opac<false, false, false>
+                                    : k_restrict_opac<false, true, false>);
+    return launch_pdl(k, grid, dim3(128), 0, p.stream, x, a, op);
 }
 
 cudaError_t launch_restrict_b(const int *meta, int N, const RestrictCtx *xs, int grid,

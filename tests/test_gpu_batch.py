@@ -65,6 +65,27 @@ def test_batch_equals_single_slabs(trt, cycle, lmax, eps, max_outer, precision):
     B.close()
 
 
+@pytest.mark.parametrize("precision", ["fp64", "sweep32_lopair"])
+@pytest.mark.parametrize("nx,G,lv", [(70, 64, [64, 4, 1]), (33, 256, [256, 1])])
+def test_restriction_opacities_outside_tables(trt, precision, nx, G, lv):
+    """A slab whose cold cells lie below the opacity tables' lowest temperature and whose
+    heated ones lie inside: the restriction that forms the opacities on the way gives the
+    results of the batch's separate kernels bit for bit (warps of either kind and mixed)."""
+    c = dataclasses.replace(W.scaled(W.fc_small(), nx, 4, G, levels=lv, name="cold"),
+                            T0=5e-5, T_left=0.8)
+    B = trt.Batch([c], precision=precision, T0=5e-5)
+    s = trt.Solver.from_slab(c, precision=precision)
+    s.set_sweep_tile(4, 0)
+    for step in range(2):
+        B.step(1e-4, "W", 1, -1.0, max_outer=3)
+        s.step(1e-4, "W", 1, -1.0, max_outer=3)
+        m = s.moments()
+        assert same(B.slab(0).moments(), m), step
+    assert m["T"].min() < 9.6e-5 < m["T"].max()
+    s.close()
+    B.close()
+
+
 def test_batch_uniform_equilibrium_and_tile(trt):
     """Equilibrium slabs stay put in a batch; a changed sweep tile keeps the results of
     the single-slab path with the same tile; the batched sweep timer leaves the state."""
