@@ -337,16 +337,17 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const bf16 *_
 }
 
 // ---- fused inference: the whole network in one persistent kernel ----
-// One CTA per SM, 320 threads: two groups of four warps, a producer warp and an MMA warp.
-// Each iteration takes 256 rows; group g (warps 4g .. 4g+3, thread = row = tensor-memory
-// lane) owns rows 128 g .. 128 g + 127 of it, its activation tile A_g in shared memory and
-// its 128 x 256 FP32 accumulator in tensor-memory columns 256 g .. 256 g + 255.  One thread
-// (warp 8) streams the weights; one thread (warp 9) issues every MMA, in the order
+// One CTA per SM, 576 threads: two groups of eight warps, a producer warp and an MMA warp.
+// Each iteration takes 256 rows; group g (warps 8g .. 8g+7, thread = row = tensor-memory
+// lane, four warps on columns 0 .. 127 and four on 128 .. 255) owns rows 128 g .. 128 g + 127
+// of it, its activation tile A_g in shared memory and its 128 x 256 FP32 accumulator in
+// tensor-memory columns 256 g .. 256 g + 255.  One thread (warp 16) streams the weights; one
+// elected lane of warp 17 issues every MMA, in the order
 //   layer 2 of group 0, layer 2 of group 1, layer 3 of group 0, layer 3 of group 1,
 // so that while the tensor core multiplies for one group the other group's warps run its
 // CUDA-core phase (layer 1, a ReLU/bias epilogue, the sigmoid head): the two groups work
 // half a period apart and the MMAs of one hide the epilogues of the other.
-//   Weights: 32-wide K chunks (16 KB, 256 rows x 32 K of W2 or W3) through a four-slot
+//   Weights: 32-wide K chunks (16 KB, 256 rows x 32 K of W2 or W3) through a five-slot
 // ring.  trt_mlp_refresh stores each chunk contiguously in the order the tensor core
 // reads it (core matrices of 8 rows x 16 bytes; K groups 4096 bytes apart, row groups 128
 // bytes apart), so one cp.async.bulk of 16 KB moves a chunk and completes on the slot's
@@ -355,7 +356,17 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const bf16 *_
 // streamed twice per 256 rows (from L2: the whole 256 KB image stays resident there).
 //   The MMA thread never waits for a slot to drain (that is the producer's wait), so the
 // tensor core always has the next chunk's MMAs queued behind the running ones.
-//   Hand-offs: a group arrives on act[g] (128 arrivals) when A_g holds the next layer's
+//   What bounds it: shared memory.  The MMAs read 12 KB per 128 cycles and the epilogues'
+// parameter reads (16 bytes broadcast to a warp cost two wavefronts or more) compete with
+// them: without the epilogues' work the same MMA stream takes 67 us for 512,000 rows, without
+// the weight copies it takes as long as with them.  So layer 1 reads each parameter once for
+// four rows (a lane's rows 32 apart, 32 columns per warp) instead of once per row.  512,000
+// rows: 137 us with one row per parameter read, four warps per group, four slots and every
+// MMA operand moved from one thread's registers; 121 us with eight warps, five slots and the
+// byte counts expected by the producer, 117 with the MMA warp's operands uniform, 102 with
+// the four-row layer 1 (floor at the measured BF16 GEMM rate 71 us).  Chunks of 16 K 152 us,
+// of 64 K with two slots 113.
+//   Hand-offs: a group arrives on act[g] (256 arrivals) when A_g holds the next layer's
 // input (after a proxy fence: the MMAs read it through the async proxy); the MMA thread
 // commits the last MMA of a layer to acc[g], which the group waits on before it reads
 // the accumulator.  Small parameters (layer-1 weights, biases, head) sit in shared
@@ -365,15 +376,15 @@ constexpr int FA_BYTES = 128 * 256 * 2;   // one activation tile
 constexpr int FK = 32;                    // K width of a weight chunk
 constexpr int FNC = 256 / FK;             // chunks per layer
 constexpr int FW_BYTES = 256 * FK * 2;    // one weight chunk
-constexpr int F_SLOTS = 4;
+constexpr int F_SLOTS = 5;
 constexpr uint32_t FW_LBO = 4096, FW_SBO = 128;   // weight chunk: K groups, row groups
 // small parameters in shared memory: W1^T [3][256], b1, b2, b3, w4, b4 (1793 floats)
 constexpr int FP_W1 = 0, FP_B1 = 768, FP_B2 = 1024, FP_B3 = 1280, FP_W4 = 1536, FP_B4 = 1792;
 constexpr int FP_BYTES = 1796 * 4;
-constexpr int F_NBAR = 2 * F_SLOTS + 4;   // full[S], empty[S], act[2], acc[2]
-constexpr int F_SMEM = 2 * FA_BYTES + F_SLOTS * FW_BYTES + FP_BYTES + 8 * F_NBAR + 32;
+constexpr int F_NBAR = 2 * F_SLOTS + 6;   // full[S], empty[S], act[2], acc[2], dotb[2]
+constexpr int F_SMEM = 2 * FA_BYTES + F_SLOTS * FW_BYTES + FP_BYTES + 8 * F_NBAR + 32 + 2 * 128 * 4;
 constexpr uint32_t FA_SBO = 4096;         // activation tiles: 32 K groups per row group
-constexpr int F_THREADS = 320;
+constexpr int F_THREADS = 576;
 
 __device__ inline void mbar_init_n(uint64_t *bar, unsigned count)
 {
@@ -427,9 +438,8 @@ __device__ inline uint32_t a_off(int row, int k8)
 
 // layer 1 of one row, h1 = relu(W1 x + b1), columns 8 k0 .. 8 k1 - 1 into the activation
 // tile: 8 columns per step, W1^T rows and b1 as broadcast float4 reads of shared memory,
-// pairs of columns by packed FP32 FMAs, ReLU fused in the BF16 pack.  kMax: clamp first by
-// fmax, which turns a NaN into 0 as the GEMM epilogue does (the pack's ReLU keeps it)
-template <bool kMax>
+// pairs of columns by packed FP32 FMAs, clamped by fmax, which turns a NaN into 0 as the
+// GEMM epilogue does (the BF16 pack's ReLU keeps it)
 __device__ inline void layer1_row(const float *sP, float x0, float x1, float x2,
                                   unsigned char *A, int r, int k0, int k1)
 {
@@ -453,14 +463,45 @@ __device__ inline void layer1_row(const float *sP, float x0, float x1, float x2,
             c = fma2(make_float2(w1.z, w1.w), X1, c);
             a = fma2(make_float2(w2.x, w2.y), X2, a);
             c = fma2(make_float2(w2.z, w2.w), X2, c);
-            if (kMax) {
-                a = make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
-                c = make_float2(fmaxf(c.x, 0.f), fmaxf(c.y, 0.f));
-            }
+            a = make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+            c = make_float2(fmaxf(c.x, 0.f), fmaxf(c.y, 0.f));
             hw[2 * h] = relu_bf16x2(a);
             hw[2 * h + 1] = relu_bf16x2(c);
         }
         *reinterpret_cast<uint4 *>(A + a_off(r, k8)) = u;
+    }
+}
+
+// inference: the four rows r, r + 32, r + 64, r + 96 with inputs v, each parameter read once
+// for the four, ReLU in the BF16 pack alone
+__device__ inline void layer1_rows4(const float *sP, const float (&v)[4][3], unsigned char *A, int r,
+                                    int k0, int k1)
+{
+    const float4 *pw = reinterpret_cast<const float4 *>(sP + FP_W1);
+    const float4 *pb = reinterpret_cast<const float4 *>(sP + FP_B1);
+    for (int k8 = k0; k8 < k1; ++k8) {
+        uint4 u[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = k8 * 2 + h;
+            const float4 b = pb[k], w0 = pw[k], w1 = pw[64 + k], w2 = pw[128 + k];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 X0 = make_float2(v[j][0], v[j][0]), X1 = make_float2(v[j][1], v[j][1]),
+                             X2 = make_float2(v[j][2], v[j][2]);
+                float2 a = make_float2(b.x, b.y), c = make_float2(b.z, b.w);
+                a = fma2(make_float2(w0.x, w0.y), X0, a);
+                c = fma2(make_float2(w0.z, w0.w), X0, c);
+                a = fma2(make_float2(w1.x, w1.y), X1, a);
+                c = fma2(make_float2(w1.z, w1.w), X1, c);
+                a = fma2(make_float2(w2.x, w2.y), X2, a);
+                c = fma2(make_float2(w2.z, w2.w), X2, c);
+                (h ? u[j].z : u[j].x) = relu_bf16x2(a);
+                (h ? u[j].w : u[j].y) = relu_bf16x2(c);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4 *>(A + a_off(r + 32 * j, k8)) = u[j];
     }
 }
 
@@ -474,6 +515,14 @@ __device__ inline void stage_params(float *sP, const float *P, int tid)
     sP[FP_B3 + tid] = __ldg(P + TRT_MLP_B3 + tid);
     sP[FP_W4 + tid] = __ldg(P + TRT_MLP_W4 + tid);
     if (tid == 0) sP[FP_B4] = __ldg(P + TRT_MLP_B4);
+}
+
+// one lane of a converged warp, the same at every call
+__device__ inline bool elect_one()
+{
+    unsigned p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
 // one contiguous bulk copy global -> this CTA's shared memory, completing (bytes) on `bar`
@@ -498,6 +547,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + F_NBAR);
     int *sfail = reinterpret_cast<int *>(tslot + 1);
     int *sprod = sfail + 1, *scons = sfail + 2;   // chunks copied / expected (failure drain)
+    uint64_t *dotb = acc + 2;
+    float *sdot = reinterpret_cast<float *>(bar + F_NBAR) + 8;   // [2][128] head sums of columns 128 ..
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const int ntiles = (rows + 255) / 256;
@@ -509,8 +560,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
             mbar_init_n(&empty[k], 1);   // the commit of the MMAs that read the slot
         }
         for (int g = 0; g < 2; ++g) {
-            mbar_init_n(&act[g], 128);
+            mbar_init_n(&act[g], 256);
             mbar_init_n(&acc[g], 1);
+            mbar_init_n(&dotb[g], 128);
         }
         *sfail = 0;
         *sprod = 0;
@@ -531,67 +583,78 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
     bool ok = true;
 
     const int Q = 4 * FNC * mine;   // weight chunks: 4 layer-jobs of FNC chunks per iteration
-    if (warp == 8) {
+    if (warp == 16) {
         // ---------------- producer thread ----------------
         if ((tid & 31) == 0) {
-            int q = 0;
-            for (; q < Q; ++q) {   // chunk q: job q / FNC, K chunk q % FNC, slot q % S
-                if (q >= F_SLOTS && !mbar_wait(&empty[q % F_SLOTS], ((q - F_SLOTS) / F_SLOTS) & 1)) {
+            int q = 0, slot = 0;
+            unsigned ph = 1;   // the slot's reuse waits for the phase before
+            for (; q < Q; ++q) {   // chunk q: job q / FNC, K chunk q % FNC
+                if (q >= F_SLOTS && !mbar_wait(&empty[slot], ph)) {
                     *sfail = 1;
                     break;
                 }
                 const int layer = (q / FNC) % 4 >= 2 ? 1 : 0;
-                bulk_copy(sW + (q % F_SLOTS) * FW_BYTES,
+                mbar_expect(&full[slot], FW_BYTES);
+                bulk_copy(sW + slot * FW_BYTES,
                           Wimg + layer * 65536 + (q % FNC) * (FW_BYTES / 2), FW_BYTES,
-                          &full[q % F_SLOTS]);
+                          &full[slot]);
+                if (++slot == F_SLOTS) {
+                    slot = 0;
+                    ph ^= 1u;
+                }
             }
             *sprod = q;
         }
-    } else if (warp == 9) {
-        // ---------------- MMA thread ----------------
-        if ((tid & 31) == 0) {
-            unsigned pact = 0;   // bit g: parity of act[g]'s next phase
-            int q = 0;
-            for (int it = 0; it < mine && ok; ++it) {
-                for (int job = 0; job < 4 && ok; ++job) {
-                    const int g = job & 1;
-                    if (!mbar_wait(&act[g], (pact >> g) & 1u)) { ok = false; break; }
-                    pact ^= 1u << g;
-                    tc_after();
-                    const uint32_t a0 = su32(sm + g * FA_BYTES);
-                    const uint32_t d = tmem + (uint32_t)(g * 256);
-                    for (int c = 0; c < FNC; ++c, ++q) {
-                        // chunk q's bytes (the copy may land first: the phase completes
-                        // once both the arrival and the bytes are in)
-                        mbar_expect(&full[q % F_SLOTS], FW_BYTES);
-                        if (!mbar_wait(&full[q % F_SLOTS], (q / F_SLOTS) & 1)) {
-                            ok = false;
-                            ++q;
-                            break;
-                        }
-                        const uint32_t w0 = su32(sW + (q % F_SLOTS) * FW_BYTES);
+    } else if (warp == 17) {
+        // ---------------- MMA warp: one elected lane issues ----------------
+        // the warp walks the chunks together, so that addresses and descriptors are uniform
+        // values (a branch for one thread makes every operand of an MMA a register move)
+        const bool lead = elect_one();
+        unsigned pact = 0, ph = 0;   // bit g: parity of act[g]'s next phase; of the ring's
+        int q = 0, slot = 0;
+        const uint64_t wd = sdesc(su32(sW), FW_LBO, FW_SBO);
+        for (int it = 0; it < mine && ok; ++it) {
+            for (int job = 0; job < 4 && ok; ++job) {
+                const int g = job & 1;
+                if (!__all_sync(0xffffffffu, mbar_wait(&act[g], (pact >> g) & 1u))) { ok = false; break; }
+                pact ^= 1u << g;
+                tc_after();
+                const uint64_t ad = sdesc(su32(sm + g * FA_BYTES), LBO, FA_SBO);
+                const uint32_t d = tmem + (uint32_t)(g * 256);
 #pragma unroll
-                        for (int kk = 0; kk < FK / 16; ++kk) {
-                            const uint64_t bd = sdesc(w0 + kk * 2 * FW_LBO, FW_LBO, FW_SBO);
-                            const uint32_t ka = (c * (FK / 8) + kk * 2) * 128;
-                            umma(d, sdesc(a0 + ka, LBO, FA_SBO), bd, (c | kk) != 0);
-                        }
-                        // the slot is free for chunk q + S once the MMAs reading it are done
-                        umma_commit(&empty[q % F_SLOTS]);
+                for (int c = 0; c < FNC; ++c, ++q) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[slot], ph))) {
+                        ok = false;
+                        break;
                     }
-                    if (!ok) break;
-                    umma_commit(&acc[g]);   // the group's accumulator is complete
+                    const uint64_t bd = wd + (uint64_t)(slot * (FW_BYTES >> 4));
+                    if (lead) {
+#pragma unroll
+                        for (int kk = 0; kk < FK / 16; ++kk)
+                            umma(d, ad + (uint64_t)(((c * (FK / 8) + kk * 2) * 128) >> 4),
+                                 bd + (uint64_t)((kk * 2 * FW_LBO) >> 4), (c | kk) != 0);
+                        // the slot is free for chunk q + S once the MMAs reading it are done
+                        umma_commit(&empty[slot]);
+                    }
+                    if (++slot == F_SLOTS) {
+                        slot = 0;
+                        ph ^= 1u;
+                    }
                 }
+                if (!ok) break;
+                if (lead) umma_commit(&acc[g]);   // the group's accumulator is complete
             }
+        }
+        if (lead) {
             if (!ok) *sfail = 1;
-            *scons = q;   // chunks whose bytes this CTA has expected
+            *scons = q;   // chunks that have landed
         }
     } else {
-        // ---------------- a group of four warps: 128 rows ----------------
-        const int g = warp >> 2, r = tid & 127;
+        // -------- a group of eight warps: 128 rows, columns 128 half .. 128 half + 127 --------
+        const int g = warp >> 3, half = (warp >> 2) & 1, r = tid & 127;
         unsigned char *myA = sm + g * FA_BYTES;
         const uint32_t tb = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * 256);
-        unsigned pacc = 0;
+        unsigned pacc = 0, pdot = 0;
         auto wait_acc = [&]() {
             if (!mbar_wait(&acc[g], pacc)) {
                 *sfail = 1;
@@ -606,43 +669,39 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
             fence_async_smem();
             mbar_arrive(&act[g]);
         };
-        float xn0 = 0.f, xn1 = 0.f, xn2 = 0.f;   // this tile's inputs (0 past the last row)
-        {
-            const int row = (int)blockIdx.x * 256 + g * 128 + r;
-            if (mine > 0 && row < rows) {
-                xn0 = x[3 * row];
-                xn1 = x[3 * row + 1];
-                xn2 = x[3 * row + 2];
+        // layer 1: rows lane + 32 j, columns 32 w8 .. 32 w8 + 31 (w8: the warp within its group)
+        const int lane = tid & 31, w8 = warp & 7;
+        float xn[4][3];   // the tile's inputs (0 past the last row)
+        auto load_x = [&](int base) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int row = base + lane + 32 * j;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) xn[j][k] = row < rows ? x[3 * row + k] : 0.f;
             }
-        }
+        };
+        if (mine > 0) load_x((int)blockIdx.x * 256 + g * 128);
         for (int it = 0; it < mine && ok; ++it) {
-            const int row = ((int)blockIdx.x + it * (int)gridDim.x) * 256 + g * 128 + r;
+            const int base = ((int)blockIdx.x + it * (int)gridDim.x) * 256 + g * 128, row = base + r;
             const bool rv = row < rows;
-            layer1_row<false>(sP, xn0, xn1, xn2, myA, r, 0, 32);
+            layer1_rows4(sP, xn, myA, lane, 4 * w8, 4 * w8 + 4);
             // the next tile's inputs, in flight during the two layers
-            {
-                const int nrow = row + (int)gridDim.x * 256;
-                if (it + 1 < mine && nrow < rows) {
-                    xn0 = x[3 * nrow];
-                    xn1 = x[3 * nrow + 1];
-                    xn2 = x[3 * nrow + 2];
-                }
-            }
+            if (it + 1 < mine) load_x(base + (int)gridDim.x * 256);
             hand_off();
             if (!(ok = wait_acc())) break;
             // ---- epilogue of layer 2: h2 = relu(acc + b2) over h1 ----
-            for (int ch = 0; ch < 8; ch += 2) {   // 64 columns per tensor-memory wait
+            for (int ch = 4 * half; ch < 4 * half + 4; ch += 2) {   // 64 columns per tensor-memory wait
                 uint32_t ra[32], rb[32];
                 tmem_ld32_issue(tb + ch * 32, ra);
                 tmem_ld32_issue(tb + ch * 32 + 32, rb);
                 tmem_wait_tied(ra);
                 reg_tie(rb);
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const uint32_t *rr = half ? rb : ra;
+                for (int k = 0; k < 2; ++k) {
+                    const uint32_t *rr = k ? rb : ra;
 #pragma unroll
                     for (int qq = 0; qq < 4; ++qq) {
-                        const float4 *b2 = reinterpret_cast<const float4 *>(sP + FP_B2) + (ch + half) * 8 + qq * 2;
+                        const float4 *b2 = reinterpret_cast<const float4 *>(sP + FP_B2) + (ch + k) * 8 + qq * 2;
                         const float4 p0 = b2[0], p1 = b2[1];
                         const uint32_t *vq = rr + qq * 8;
                         uint4 u;
@@ -650,7 +709,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
                         u.y = relu_bf16x2(add2(make_float2(__uint_as_float(vq[2]), __uint_as_float(vq[3])), make_float2(p0.z, p0.w)));
                         u.z = relu_bf16x2(add2(make_float2(__uint_as_float(vq[4]), __uint_as_float(vq[5])), make_float2(p1.x, p1.y)));
                         u.w = relu_bf16x2(add2(make_float2(__uint_as_float(vq[6]), __uint_as_float(vq[7])), make_float2(p1.z, p1.w)));
-                        *reinterpret_cast<uint4 *>(myA + a_off(r, (ch + half) * 4 + qq)) = u;
+                        *reinterpret_cast<uint4 *>(myA + a_off(r, (ch + k) * 4 + qq)) = u;
                     }
                 }
             }
@@ -658,19 +717,19 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
             if (!(ok = wait_acc())) break;
             // ---- epilogue of layer 3 and the head: y = sigmoid(w4 . relu(acc + b3) + b4) ----
             float2 dot = make_float2(0.f, 0.f);   // even and odd columns
-            for (int ch = 0; ch < 8; ch += 2) {   // 64 columns per tensor-memory wait
+            for (int ch = 4 * half; ch < 4 * half + 4; ch += 2) {   // 64 columns per tensor-memory wait
                 uint32_t ra[32], rb[32];
                 tmem_ld32_issue(tb + ch * 32, ra);
                 tmem_ld32_issue(tb + ch * 32 + 32, rb);
                 tmem_wait_tied(ra);
                 reg_tie(rb);
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const uint32_t *rr = half ? rb : ra;
+                for (int k = 0; k < 2; ++k) {
+                    const uint32_t *rr = k ? rb : ra;
 #pragma unroll
                     for (int j4 = 0; j4 < 8; ++j4) {
-                        const float4 b3 = reinterpret_cast<const float4 *>(sP + FP_B3)[(ch + half) * 8 + j4];
-                        const float4 w4 = reinterpret_cast<const float4 *>(sP + FP_W4)[(ch + half) * 8 + j4];
+                        const float4 b3 = reinterpret_cast<const float4 *>(sP + FP_B3)[(ch + k) * 8 + j4];
+                        const float4 w4 = reinterpret_cast<const float4 *>(sP + FP_W4)[(ch + k) * 8 + j4];
                         float2 a = add2(make_float2(__uint_as_float(rr[4 * j4]), __uint_as_float(rr[4 * j4 + 1])),
                                         make_float2(b3.x, b3.y));
                         float2 c = add2(make_float2(__uint_as_float(rr[4 * j4 + 2]), __uint_as_float(rr[4 * j4 + 3])),
@@ -682,19 +741,29 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
                     }
                 }
             }
-            if (rv) y[row] = 1.f / (1.f + __expf(-((dot.x + dot.y) + sP[FP_B4])));
+            // the other half's sum through shared memory: its next write is a layer hand-off
+            // later, which this half joins after it has read
+            if (half) {
+                sdot[g * 128 + r] = dot.x + dot.y;
+                mbar_arrive(&dotb[g]);
+            } else {
+                if (!mbar_wait(&dotb[g], pdot)) {
+                    *sfail = 1;
+                    ok = false;
+                    break;
+                }
+                pdot ^= 1u;
+                const float z = (dot.x + dot.y) + sdot[g * 128 + r];
+                if (rv) y[row] = 1.f / (1.f + __expf(-(z + sP[FP_B4])));
+            }
         }
     }
     tc_before();
     __syncthreads();
     if (*sfail && tid == 0) {
         atomicExch(&g_mlp_err, TRT_ETIMEOUT);
-        // let the producer's copies in flight land (bounded): expect what the MMA thread
-        // did not, then wait
-        for (int r = *scons; r < *sprod; ++r) {
-            mbar_expect(&full[r % F_SLOTS], FW_BYTES);
-            mbar_wait(&full[r % F_SLOTS], (r / F_SLOTS) & 1);
-        }
+        // let the producer's copies in flight land (bounded)
+        for (int r = *scons; r < *sprod; ++r) mbar_wait(&full[r % F_SLOTS], (r / F_SLOTS) & 1);
     }
     __syncthreads();   // the drain above ends before TMEM is released
     if (warp == 0) {
@@ -984,7 +1053,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_mlp_train(int rows, const floa
             drain(TP_DW2, 1);
         } else {
         const float4 X = sx[r];
-        layer1_row<true>(sP, X.x, X.y, X.z, A0, r, 16 * hf, 16 * hf + 16);
+        layer1_row(sP, X.x, X.y, X.z, A0, r, 16 * hf, 16 * hf + 16);
         hand_off();
         // ---- h2 = relu(acc + b2) ----
         wait_bar(acc, pacc);
@@ -1113,7 +1182,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_mlp_train(int rows, const floa
             }
         }
         mbar_arrive(d2r);
-        layer1_row<true>(sP, X.x, X.y, X.z, A1, r, 16 * hf, 16 * hf + 16);
+        layer1_row(sP, X.x, X.y, X.z, A1, r, 16 * hf, 16 * hf + 16);
         hand_off();
         // ---- d1 = acc [h1 > 0] (FP32): its column sums, plain (b1) and times x (W1).  The
         // ring is free (the last layer product has read it): a warp stages 32 rows x 32

@@ -95,6 +95,21 @@ def test_mlp_fused_forward(env, rows):
     assert mlp.MLP.status() == 0
 
 
+@pytest.mark.parametrize("rows", [31, 127, 129, 255, 257, 128 * 305 + 33])
+def test_mlp_fused_row_edges(env, rows):
+    """Edges of the fused kernel's 128-row groups and four-row lanes against the three-launch
+    path: the head's 256 terms are summed in another order, at most 256 ulps of a sum of
+    order one through the sigmoid's slope 1/4: 4e-6."""
+    torch, mlp = env
+    r = np.random.default_rng(63)
+    p = OM.init_params(64) + OM.pack({"b1": r.normal(0, 0.1, 256), "b2": r.normal(0, 0.1, 256),
+                                      "b3": r.normal(0, 0.1, 256), "b4": 0.2})
+    x = r.normal(0, 1, (rows, 3)).astype(np.float32)
+    net = mlp.MLP(p.astype(np.float32).astype(np.float64))
+    assert np.max(np.abs(net.forward_fused(x).cpu().numpy() - net.forward(x).cpu().numpy())) < 4e-6
+    assert mlp.MLP.status() == 0
+
+
 def test_mlp_gradient_vs_oracle(env):
     """Gradients of the tensor-core backward pass against the oracle's backward pass with
     BF16 rounding at the same points, element by element: every element within 5e-4 of its
