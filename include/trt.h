@@ -151,7 +151,7 @@ int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups 
                trt_handle **out);
 
 /* One implicit time step of length dt_sh with Algorithm 3.  Blocks on the stream once per
- * cycle to read the convergence flags.  stats may be NULL. */
+ * phase (a sweep and the cycles after it) to read the convergence flags.  stats may be NULL. */
 int trt_step(trt_handle *h, double dt_sh, const trt_cycle *cycle, trt_stats *stats);
 
 /* Copy the state at the current time level to host arrays (any may be NULL):
