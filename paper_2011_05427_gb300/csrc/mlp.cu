@@ -436,44 +436,12 @@ __device__ inline uint32_t a_off(int row, int k8)
     return (uint32_t)((row >> 3) * FA_SBO + k8 * 128 + (row & 7) * 16);
 }
 
-// layer 1 of one row, h1 = relu(W1 x + b1), columns 8 k0 .. 8 k1 - 1 into the activation
-// tile: 8 columns per step, W1^T rows and b1 as broadcast float4 reads of shared memory,
-// pairs of columns by packed FP32 FMAs, clamped by fmax, which turns a NaN into 0 as the
-// GEMM epilogue does (the BF16 pack's ReLU keeps it)
-__device__ inline void layer1_row(const float *sP, float x0, float x1, float x2,
-                                  unsigned char *A, int r, int k0, int k1)
-{
-    const float2 X0 = make_float2(x0, x0), X1 = make_float2(x1, x1), X2 = make_float2(x2, x2);
-    const float4 *pw0 = reinterpret_cast<const float4 *>(sP + FP_W1);
-    const float4 *pw1 = reinterpret_cast<const float4 *>(sP + FP_W1 + 256);
-    const float4 *pw2 = reinterpret_cast<const float4 *>(sP + FP_W1 + 512);
-    const float4 *pb = reinterpret_cast<const float4 *>(sP + FP_B1);
-#pragma unroll 4
-    for (int k8 = k0; k8 < k1; ++k8) {
-        uint4 u;
-        uint32_t *hw = reinterpret_cast<uint32_t *>(&u);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float4 b = pb[k8 * 2 + h], w0 = pw0[k8 * 2 + h], w1 = pw1[k8 * 2 + h],
-                         w2 = pw2[k8 * 2 + h];
-            float2 a = make_float2(b.x, b.y), c = make_float2(b.z, b.w);
-            a = fma2(make_float2(w0.x, w0.y), X0, a);
-            c = fma2(make_float2(w0.z, w0.w), X0, c);
-            a = fma2(make_float2(w1.x, w1.y), X1, a);
-            c = fma2(make_float2(w1.z, w1.w), X1, c);
-            a = fma2(make_float2(w2.x, w2.y), X2, a);
-            c = fma2(make_float2(w2.z, w2.w), X2, c);
-            a = make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
-            c = make_float2(fmaxf(c.x, 0.f), fmaxf(c.y, 0.f));
-            hw[2 * h] = relu_bf16x2(a);
-            hw[2 * h + 1] = relu_bf16x2(c);
-        }
-        *reinterpret_cast<uint4 *>(A + a_off(r, k8)) = u;
-    }
-}
-
-// inference: the four rows r, r + 32, r + 64, r + 96 with inputs v, each parameter read once
-// for the four, ReLU in the BF16 pack alone
+// layer 1, h1 = relu(W1 x + b1), of the four rows r, r + 32, r + 64, r + 96 with inputs v,
+// columns 8 k0 .. 8 k1 - 1 into the activation tile: W1^T rows and b1 as broadcast float4
+// reads of shared memory, once for the four rows, pairs of columns by packed FP32 FMAs, ReLU
+// fused in the BF16 pack.  kMax: clamped first by fmax, which turns a NaN into 0 as the GEMM
+// epilogue does (the pack's ReLU keeps it)
+template <bool kMax>
 __device__ inline void layer1_rows4(const float *sP, const float (&v)[4][3], unsigned char *A, int r,
                                     int k0, int k1)
 {
@@ -496,6 +464,10 @@ __device__ inline void layer1_rows4(const float *sP, const float (&v)[4][3], uns
                 c = fma2(make_float2(w1.z, w1.w), X1, c);
                 a = fma2(make_float2(w2.x, w2.y), X2, a);
                 c = fma2(make_float2(w2.z, w2.w), X2, c);
+                if (kMax) {
+                    a = make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+                    c = make_float2(fmaxf(c.x, 0.f), fmaxf(c.y, 0.f));
+                }
                 (h ? u[j].z : u[j].x) = relu_bf16x2(a);
                 (h ? u[j].w : u[j].y) = relu_bf16x2(c);
             }
@@ -684,7 +656,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
         for (int it = 0; it < mine && ok; ++it) {
             const int base = ((int)blockIdx.x + it * (int)gridDim.x) * 256 + g * 128, row = base + r;
             const bool rv = row < rows;
-            layer1_rows4(sP, xn, myA, lane, 4 * w8, 4 * w8 + 4);
+            layer1_rows4<false>(sP, xn, myA, lane, 4 * w8, 4 * w8 + 4);
             // the next tile's inputs, in flight during the two layers
             if (it + 1 < mine) load_x(base + (int)gridDim.x * 256);
             hand_off();
@@ -793,10 +765,11 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
 // row's 256 terms in column order in one chain, as the inference GEMM's epilogue does.
 // What bounds it: 8192 rows are 64 CTAs of the 152 SMs, each a serial chain of 4 layer
 // products (1 us each at the tensor rate) with their epilogues; the floor at the measured
-// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 39.5 us against
+// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 38.7 us against
 // 1249 us for one GEMM launch per product, whose two weight gradients ran on two CTAs over K =
 // 8192 (500 us) and whose column sums ran on 8 and 1 CTAs (520 us); 46 us with the eight
-// warps doing everything and the backward weights copied as 512-byte pieces (6 us a layer).
+// warps doing everything and the backward weights copied as 512-byte pieces (6 us a layer),
+// 39.5 with layer 1 reading its parameters once per row.
 constexpr int F_TSLOTS = 5;
 constexpr int F_TRING = F_TSLOTS * FW_BYTES;
 constexpr int T_THREADS = 576;
@@ -1052,8 +1025,19 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_mlp_train(int rows, const floa
             drain(TP_DW2, 0);
             drain(TP_DW2, 1);
         } else {
-        const float4 X = sx[r];
-        layer1_row(sP, X.x, X.y, X.z, A0, r, 16 * hf, 16 * hf + 16);
+        // layer 1: rows lane + 32 j, columns 32 warp .. 32 warp + 31
+        const auto layer1 = [&](unsigned char *A) {
+            float xr[4][3];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 X = sx[lane + 32 * j];
+                xr[j][0] = X.x;
+                xr[j][1] = X.y;
+                xr[j][2] = X.z;
+            }
+            layer1_rows4<true>(sP, xr, A, lane, 4 * warp, 4 * warp + 4);
+        };
+        layer1(A0);
         hand_off();
         // ---- h2 = relu(acc + b2) ----
         wait_bar(acc, pacc);
@@ -1182,8 +1166,10 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_mlp_train(int rows, const floa
             }
         }
         mbar_arrive(d2r);
-        layer1_row(sP, X.x, X.y, X.z, A1, r, 16 * hf, 16 * hf + 16);
+        bar_epi();   // every row's h2 has been read
+        layer1(A1);
         hand_off();
+        bar_epi();   // h1 of every row is in place for the mask below
         // ---- d1 = acc [h1 > 0] (FP32): its column sums, plain (b1) and times x (W1).  The
         // ring is free (the last layer product has read it): a warp stages 32 rows x 32
         // columns, lane = column sums its 32 rows, then the four row quadrants meet ----
