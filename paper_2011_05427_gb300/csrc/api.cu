@@ -25,6 +25,7 @@
 #include <string>
 #include <vector>
 #include "handle.cuh"
+#include "tri_layout.cuh"
 #include "../../include/trt_mlp.h"
 
 using namespace trt;

@@ -87,7 +87,8 @@ struct SlabState {
 }  // namespace
 
 struct trt_batch {
-    int n = 0, precision = 0, D = 1, shape = 0, max_nx = 1;
+    int n = 0, precision = 0, D = 1, shape = 0;
+    BatchSmem smem;                           // of the solves, over the slabs
     cudaStream_t st = nullptr;
     std::vector<trt_handle *> h;
     std::vector<int> K;                       // per slab: levels, for schedules
@@ -440,7 +441,7 @@ int trt_create_batch(int n, const trt_grid *grids, const trt_angles *angles,
         if (rc != TRT_OK) return rc;
         b->h.push_back(x);
         off += (w + 255) / 256 * 256;
-        b->max_nx = std::max(b->max_nx, grids[s].n_cells);
+        b->smem.add(b->precision, grids[s].n_cells);
     }
     // directions per CTA of the batched sweep: one D for every slab (a divisor of every N,
     // and no smaller than any slab's smallest candidate: its partial-moment scratch holds
@@ -566,12 +567,12 @@ cudaError_t launch_op(trt_batch *b, const Op &o)
         return launch_finalize_b(b->precision, meta, N, reinterpret_cast<const FinalizeArgs *>(x),
                                  o.grid, b->st);
     case K_LO:
-        return launch_lo_solve_b(b->precision, b->max_nx, meta, N,
+        return launch_lo_solve_b(b->precision, b->smem, meta, N,
                                  reinterpret_cast<const LoCtx *>(x), o.grid, b->st);
     case K_RESTRICT:
         return launch_restrict_b(meta, N, reinterpret_cast<const RestrictCtx *>(x), o.grid, b->st);
     case K_GREY:
-        return launch_grey_b(b->max_nx, meta, N, reinterpret_cast<const GreyCtx *>(x), o.grid,
+        return launch_grey_b(b->smem, meta, N, reinterpret_cast<const GreyCtx *>(x), o.grid,
                              b->st);
     case K_GSUM:
         return launch_group_sum_b(meta, N, reinterpret_cast<const GroupSumArgs *>(x), o.grid,

@@ -14,6 +14,7 @@
 #include <algorithm>
 #include "common.cuh"
 #include "pair.cuh"
+#include "tri_layout.cuh"
 
 namespace trt {
 
@@ -178,11 +179,11 @@ cudaError_t launch_sweep_b(int precision, bool sigma_fp32, int D, int shape, con
                            int N, const SweepArgs *xs, int grid, cudaStream_t st);
 cudaError_t launch_finalize_b(int precision, const int *meta, int N, const FinalizeArgs *xs,
                               int grid, cudaStream_t st);
-cudaError_t launch_lo_solve_b(int precision, int max_nx, const int *meta, int N,
+cudaError_t launch_lo_solve_b(int precision, const BatchSmem &bs, const int *meta, int N,
                               const LoCtx *xs, int grid, cudaStream_t st);
 cudaError_t launch_restrict_b(const int *meta, int N, const RestrictCtx *xs, int grid,
                               cudaStream_t st);
-cudaError_t launch_grey_b(int max_nx, const int *meta, int N, const GreyCtx *xs, int grid,
+cudaError_t launch_grey_b(const BatchSmem &bs, const int *meta, int N, const GreyCtx *xs, int grid,
                           cudaStream_t st);
 cudaError_t launch_group_sum_b(const int *meta, int N, const GroupSumArgs *xs, int grid,
                                cudaStream_t st);

@@ -245,7 +245,7 @@ struct Problem {
     float *dir32;       // [M][4]: |mu|, |mu|/2, w/2, w mu^2/2 rounded once to FP32 (FP32 sweeps)
     double *e2tab;      // [32]: 2^(j/32), the table of texp for kernels outside physics.cu
     int *lo_slot;       // [nx+1]: shared-memory slot of face/row f in the partitioned
-                        // tridiagonal solve (lo.cu, TriLayout)
+                        // tridiagonal solve (tri_layout.cuh)
     double *rscratch;   // the restriction's tickets (zero between launches) and partial sums
     size_t rscratch_doubles;
     // sweep tile: directions per CTA (0 = default) and strip shape index (0 = default)
@@ -329,7 +329,6 @@ size_t restrict_fix_doubles(int nx, int n_to);
 // the host-formed constants of a grey visit (c_v/dt, 54 s C_B, the exponential's table)
 GreyArgs grey_args_ready(const Problem &p, const GreyArgs &a);
 size_t restrict_scratch_doubles(const Problem &p);   // from nx and the grids
-void lo_slots(int nx, int *slot);                    // Problem::lo_slot
 size_t restrict_head_doubles();                      // its tickets: zero at creation
 cudaError_t launch_grey(const Problem &p, const Level &g, const GreyArgs &a);
 cudaError_t launch_group_sum(const Problem &p, int n, const double *X, double *out);

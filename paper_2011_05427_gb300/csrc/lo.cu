@@ -170,23 +170,6 @@ __device__ inline void cell_row(const LoCtx &x, int q, int i, R &Ap, R &Dp, int 
     }
 }
 
-// The layout of a system's rows in shared memory: P chunks, chunk l the rows l n / P ..
-// (l + 1) n / P - 1, its row k in slot k LP + l; face i shares the slot of row i, face n has
-// the slot after all others.  LP is odd in units of 8 so that the staging's stores (threads
-// along the rows) spread over the banks.
-struct TriLayout {
-    int P, LP, S;   // chunks, slots per row-in-chunk, slots
-};
-__host__ __device__ inline TriLayout tri_layout(int n)
-{
-    TriLayout t;
-    t.P = n / 2 < 128 ? n / 2 : 128;
-    if (t.P < 1) t.P = 1;
-    t.LP = (t.P + 31) / 32 * 32 + 8;
-    t.S = t.LP * ((n + t.P - 1) / t.P) + 1;
-    return t;
-}
-
 // The face coefficients PL, PR, GD and the row parts dx/dt + dx a, dx s + dx Eold/dt of
 // system q into the layout by `nthr` cooperating threads (index `t`).  n >= 2.
 template <typename R>
@@ -1233,8 +1216,6 @@ __device__ void restrict_body(const RestrictCtx &x, int bx, int by, const Member
 // cycles on GB300).  NaN maps to 0, the value fmax would keep.  red: kGreyRed slots, at
 // least 32 per value; the maxima are returned to thread 0 (each warp reduces its lanes by
 // shuffles, then warp 0 reduces the warps' results the same way).
-constexpr int kGreyNV = 7;
-constexpr int kGreyRed = 32 * kGreyNV;
 
 __device__ inline unsigned long long nn_bits(double v)
 {
@@ -1607,18 +1588,6 @@ static size_t restrict_doubles(int nt, int n_to, int nchunk)
     return kRHead + (size_t)n_to * nchunk * (16 + (size_t)kRV * nt * 32);
 }
 
-// shared memory of one LO solve: the rows, the pair form's 7th array (the face factors of
-// Fold, free again when the solver wants its 3 P values), or the refined FP32 form's two
-// copies of the rows
-static size_t lo_smem(int precision, int nx)
-{
-    const TriLayout y = tri_layout(nx);
-    const size_t S = y.S, rb = 3 * (size_t)y.P;
-    if (lo_fp32(precision)) return 6 * S * (sizeof(double) + sizeof(float)) + rb * sizeof(float);
-    if (lo_pair(precision)) return (6 * S + std::max(S, rb)) * sizeof(double);
-    return (6 * S + rb) * sizeof(double);
-}
-
 template <typename R, int T>
 static cudaError_t lo_launch(const LoCtx &x, const OpacityArgs &a, int op, unsigned nb, size_t sm,
                              cudaStream_t st)
@@ -1666,10 +1635,10 @@ cudaError_t launch_lo_solve(const Problem &p, double dt, const Level &L, const d
     return lo_pair(p.precision) ? go(fpair()) : lo_fp32(p.precision) ? go(0.f) : go(0.0);
 }
 
-cudaError_t launch_lo_solve_b(int precision, int max_nx, const int *meta, int N,
+cudaError_t launch_lo_solve_b(int precision, const BatchSmem &bs, const int *meta, int N,
                               const LoCtx *xs, int grid, cudaStream_t st)
 {
-    const size_t sm = lo_smem(precision, max_nx);
+    const size_t sm = bs.lo;
     cudaError_t e;
     if (lo_pair(precision)) {
         e = cudaFuncSetAttribute(k_lo_solve_b<fpair>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1716,15 +1685,6 @@ RestrictPlan restrict_plan(const Problem &p, int n_from, int n_to)
     }
     q.gy = q.mode == 0 ? (n_to + 3) / 4 : n_to * q.nchunk;
     return q;
-}
-
-// TriLayout's slots of the rows and faces 0 .. nx (uploaded with the problem)
-void lo_slots(int nx, int *slot)
-{
-    const TriLayout y = tri_layout(nx);
-    for (int l = 0; l < y.P; ++l)
-        for (int i = (l * nx) / y.P, k = 0; i < ((l + 1) * nx) / y.P; ++i, ++k) slot[i] = k * y.LP + l;
-    slot[nx] = y.S - 1;
 }
 
 size_t restrict_head_doubles() { return kRHead; }
@@ -1825,36 +1785,27 @@ GreyCtx make_grey_ctx(const Problem &p, const Level &g, const GreyArgs &a)
     return x;
 }
 
-static void grey_launch_shape(int nx, int &bs, size_t &sm)
-{
-    bs = std::min(1024, std::max(32, (nx + 31) / 32 * 32));
-    // at least the solver's chunks; Newton terms, block maxima, the solver's rows
-    const TriLayout y = tri_layout(nx);
-    sm = sizeof(double) * (3 * (size_t)nx + kGreyRed + 6 * (size_t)y.S + 3 * (size_t)y.P);
-}
+// at least the solver's chunks (<= nx / 2), a warp at least
+static int grey_threads(int nx) { return std::min(1024, std::max(32, (nx + 31) / 32 * 32)); }
 
 cudaError_t launch_grey(const Problem &p, const Level &g, const GreyArgs &a)
 {
     const GreyCtx x = make_grey_ctx(p, g, a);
-    int bs;
-    size_t sm;
-    grey_launch_shape(p.nx, bs, sm);
+    const size_t sm = grey_smem(p.nx);
     cudaError_t e = cudaFuncSetAttribute(k_grey, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_grey, dim3(1), dim3(bs), sm, p.stream, x);
+    return launch_pdl(k_grey, dim3(1), dim3(grey_threads(p.nx)), sm, p.stream, x);
 }
 
-cudaError_t launch_grey_b(int max_nx, const int *meta, int N, const GreyCtx *xs, int grid,
+cudaError_t launch_grey_b(const BatchSmem &bs, const int *meta, int N, const GreyCtx *xs, int grid,
                           cudaStream_t st)
 {
-    int bs;
-    size_t sm;
-    grey_launch_shape(max_nx, bs, sm);
+    const size_t sm = bs.grey;
     cudaError_t e = cudaFuncSetAttribute(k_grey_b, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
     if (e != cudaSuccess) return e;
-    k_grey_b<<<grid, bs, sm, st>>>(meta, N, xs);
+    k_grey_b<<<grid, grey_threads(bs.max_nx), sm, st>>>(meta, N, xs);
     return cudaGetLastError();
 }
 

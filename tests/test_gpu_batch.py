@@ -184,3 +184,24 @@ def test_batch_slabs_match_oracle(trt, orc, cycle, lmax):
             eE = np.max(np.abs(g["Eg"] - r["Eg"]) / r["Eg"].sum(0)[None, :])
             assert eT < 1e-10 and eE < 1e-10, (step, k, eT, eE)
     B.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "lopair", "mixed"])
+@pytest.mark.parametrize("sizes", [(60, 59, 58), (200, 199, 7)])
+def test_batch_of_even_and_odd_cell_counts(trt, precision, sizes):
+    """Slabs whose solves need more shared memory than the largest slab's do (an odd cell
+    count below an even one of at most 256): results of single slabs bit for bit."""
+    cs = [dataclasses.replace(W.scaled(W.fc_small(), n, 4, 34, levels=[34, 17, 1], name=f"s{n}"),
+                              T_left=0.6 + 0.1 * k, dt=1e-3) for k, n in enumerate(sizes)]
+    B = trt.Batch(cs, precision=precision)
+    ss = [trt.Solver.from_slab(c, precision=precision) for c in cs]
+    for s in ss:
+        s.set_sweep_tile(4, 0)
+    for step in range(2):
+        B.step(1e-3, "W", 2, -1.0, max_outer=3)
+        for k, s in enumerate(ss):
+            s.step(1e-3, "W", 2, -1.0, max_outer=3)
+            assert same(B.slab(k).moments(), s.moments()), (step, k)
+    for s in ss:
+        s.close()
+    B.close()
