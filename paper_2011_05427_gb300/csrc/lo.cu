@@ -853,7 +853,10 @@ __device__ inline void restrict_members(const RestrictCtx &x, int p0, int pe, in
 // The same over a fine source whose opacities at a.T are formed here, per member and cell,
 // instead of read (and stored for the other readers of the fine grid's arrays): the lane's
 // per-cell terms stay in registers over the members.  A face's left opacity is the lane
-// before's, through shared memory (xch: two rows of 33 for the warp, by turns).
+// before's, through shared memory (xch: two rows of 33 for the warp, by turns).  The halo
+// lane stores its cell's sigma_R too (the value that the tile before stores there): the
+// plain mean of a face without flux weight (restrict_face) reads the members' sigma_R back,
+// at the tile's first face the halo cell's, and nothing orders it after another tile's store.
 // kFix: the sums that do not depend on the opacities (kFixed) are the caller's, from an
 // earlier visit of the cycle.  kIn: every lane's cell is inside the tables.
 template <bool kOld, bool kPair, bool kFix, bool kIn>
@@ -887,10 +890,10 @@ __device__ inline void restrict_members_opac(const RestrictCtx &x, const Opacity
         if (!kFix) ph = S.phi[c];
         const OpacVals o = cell_opacities<kPair, kIn>(a, p, ic, cc, mx, e2p);
         xch[par][lane] = o.sR;
+        if (in) S.sigR[c] = o.sR;
         if (own) {
             S.sig[c] = o.sg;
             S.emis[c] = o.em;
-            S.sigR[c] = o.sR;
         }
         __syncwarp();
         const double left = xch[par][max(lane - 1, 0)];

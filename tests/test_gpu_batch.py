@@ -205,3 +205,32 @@ def test_batch_of_even_and_odd_cell_counts(trt, precision, sizes):
     for s in ss:
         s.close()
     B.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "sweep32_lopair"])
+@pytest.mark.parametrize("nx,G,lv", [(70, 64, [64, 16, 4, 1]), (95, 256, [256, 4, 1]),
+                                     (64, 2048, [2048, 1024, 1])])
+def test_restriction_opacities_without_flux_weight(trt, precision, nx, G, lv):
+    """Groups far above the slab's temperatures hold no energy and no flux (their spectra
+    underflow to exact zeros), so the coarse groups made of them take the plain means of the
+    members' opacities on every face, those at the edges of the position tiles (31, 62, 93)
+    among them: the last coarse grid's fields after a step of the restriction that forms the
+    opacities on the way are those of the batch's separate kernels bit for bit."""
+    c = dataclasses.replace(W.scaled(W.fc_small(), nx, 4, G, levels=lv, name="dark"),
+                            T_left=0.8, nu_a=1e-4, nu_b=1e7)   # nu / T > 745 from 600 keV on
+    B = trt.Batch([c], precision=precision)
+    s = trt.Solver.from_slab(c, precision=precision)
+    s.set_sweep_tile(4, 0)
+    for step in range(3):
+        B.step(1e-3, "W", 1, -1.0, max_outer=3)
+        s.step(1e-3, "W", 1, -1.0, max_outer=3)
+        a, b = B.slab(0).level_view(1), s.level_view(1)
+        n = b["n"]   # (a batch's view keeps the largest coarse grid's n)
+        assert n == lv[-2] <= a["n"]
+        for k in ("sigR", "sig", "phi", "emis", "etaR", "etaL", "E", "F"):
+            assert np.array_equal(a[k][:n], b[k]), (step, k)
+    dark = ~(b["F"].any(axis=1) | b["E"].any(axis=1))
+    assert dark.any() and not dark.all()
+    assert np.isfinite(b["sigR"]).all()
+    s.close()
+    B.close()
