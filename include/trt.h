@@ -194,7 +194,9 @@ int trt_k_opacity(trt_handle *h, const double *T, double *sigE, double *emis, do
  * direction with sigma_t = sigE + 1/(c dt) and corner sources emis + I_old/(c dt), inflow
  * from the handle's boundary temperatures, followed by the QD factors (eqs. f_g, c_g).
  * I_old / I_new: [M][nx][2][ldG] in the handle's sweep precision (float when the
- * precision has TRT_SWEEP_FP32, else double).  f [G][nx]; fb0, fbX, C0, CX [G]; all FP64.
+ * precision has TRT_SWEEP_FP32, else double), aligned to their elements; an I_old not
+ * aligned to 16 bytes or an I_new not aligned to 8 takes the strip sweep whatever the tile
+ * (the others copy 16 bytes at a time and store pairs).  f [G][nx]; fb0, fbX, C0, CX [G]; all FP64.
  * With TRT_SWEEP_FP32 the FP64 sigE and emis are first rounded once to the step's FP32
  * sweep inputs (sigma_t h/2, h e/2 and h/(2 c dt), in the handle's scratch), so the sweep
  * runs the same kernel and tile on the same inputs as a step would. */

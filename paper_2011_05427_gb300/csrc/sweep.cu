@@ -489,9 +489,9 @@ cudaError_t launch_finalize(const Problem &p, const SweepArgs &a)
 }
 
 template <typename R>
-cudaError_t launch_sweep_t(const Problem &p, const SweepArgs &a)
+cudaError_t launch_sweep_t(const Problem &p, const SweepArgs &a, int shape)
 {
-    cudaError_t e = dispatch_shape<R>(p.sweep_shape, &a, p.M, p.ldG, a.D, nullptr, 0, nullptr, 0,
+    cudaError_t e = dispatch_shape<R>(shape, &a, p.M, p.ldG, a.D, nullptr, 0, nullptr, 0,
                                       p.stream);
     return e != cudaSuccess ? e : launch_finalize<R>(p, a);
 }
@@ -605,28 +605,34 @@ cudaError_t launch_sweep(const Problem &p, double dt, const void *sigE, const vo
                          double *psi_exit, double *f, double *fb0, double *fbX, double *C0,
                          double *CX)
 {
+    // The paired and the lean sweeps copy I_old in pieces of 16 bytes, and the lean sweep of two
+    // groups per lane stores pairs.  Callers' arrays that are aligned to their elements only
+    // take the strip sweep, which reads and writes element by element.
+    const bool wide = ((reinterpret_cast<uintptr_t>(I_old) & 15) | (reinterpret_cast<uintptr_t>(I_new) & 7)) == 0;
+    const int kind = (sweep_fp32(p.precision) ? kShapes32 : kShapes64)[p.sweep_shape].V;
+    const int shape = wide || kind == 1 ? p.sweep_shape : sweep_fp32(p.precision) ? kStrip32 : 0;
     SweepArgs a = make_sweep_args(p, dt, sigE, emis, I_old, I_new, part, psi_exit, f, fb0, fbX,
-                                  C0, CX, pick_D(p));
+                                  C0, CX, wide ? pick_D(p) : std::min(pick_D(p), 8));
     if (!sweep_fp32(p.precision)) {
         // The default of a handle with the paired sweep's scratch is that sweep: 13 FP64
         // instructions per update against 17.6 of the strip sweep, at any size (with the
         // finalize, against the strip sweep's best tile: 500 cells x 64 x 1024 0.831 against
         // 1.239 ms; 333 x 48 x 500 0.319, 0.468; 60 x 16 x 17 0.049, 0.058; 10 x 16 x 256
         // 0.017, 0.017)
-        const bool def = p.sweep_D == 0 && p.pair64;
-        if (def || kShapes64[p.sweep_shape].V == 7) {
+        const bool def = p.sweep_D == 0 && p.pair64 && wide;
+        if (def || kShapes64[shape].V == 7) {
             if (def) a.D = pair_default_D(p.N, p.ldG);
             a.ntile = p.N / a.D;   // a tile holds both signs
-            const int S = def ? 4 : kShapes64[p.sweep_shape].S, NS = def ? 2 : kShapes64[p.sweep_shape].NS;
+            const int S = def ? 4 : kShapes64[shape].S, NS = def ? 2 : kShapes64[shape].NS;
             cudaError_t e = launch_sweep_pair(a.D, S, NS, a, p.M, p.ldG, p.stream);
             return e != cudaSuccess ? e : launch_finalize<double>(p, a);
         }
-        return launch_sweep_t<double>(p, a);
+        return launch_sweep_t<double>(p, a, shape);
     }
     if (!sigma_fp32 || !p.dir32) return cudaErrorInvalidValue;   // FP32 sweeps: FP32 inputs
     // the pre-scaled inputs carry h/(2 c dt) after e (launch_opacity, launch_prescale32)
     a.kap32 = reinterpret_cast<const float *>(emis) + (size_t)p.G * p.nx;
-    return launch_sweep_t<float>(p, a);
+    return launch_sweep_t<float>(p, a, shape);
 }
 
 cudaError_t launch_sweep_b(int precision, bool sigma_fp32, int D, int shape, const int *meta,

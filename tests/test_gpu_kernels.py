@@ -311,6 +311,45 @@ def test_default_fp64_sweep(trt, orc, nx, N, G):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("precision,tile,strip", [("fp64", None, (8, 0)), ("fp64", (4, 3), (4, 0)),
+                                                  ("sweep32", None, (8, 6)),
+                                                  ("sweep32", (16, 0), (8, 6)),
+                                                  ("sweep32", (8, 4), (8, 6))])
+def test_sweep_of_unaligned_intensity(trt, orc, precision, tile, strip):
+    """An I_old that is aligned to its elements but not to 16 bytes (or, in FP32, such an
+    I_new): the strip sweep's result bit for bit, whatever the handle's tile."""
+    import torch
+    nx, N, G = 21, 16, 40
+    r, h, sig, em, I_old, TL = sweep_inputs(orc, 3100, nx, N, G, thick=True)
+    s = solver(trt, nx=nx, N=N, G=G, h=h, edges=W.group_edges(G, 1e-5, 1e2), TL=TL, TR=0.3,
+               precision=precision)
+    rdt = torch.float32 if precision == "sweep32" else torch.float64
+    flat = torch.zeros(2 * N * nx * 2 * 64 + 1, dtype=rdt, device="cuda")
+    Ip = flat[1:].view(2 * N, nx, 2, 64)
+    Ip[..., :G] = torch.as_tensor(I_old, device="cuda").to(rdt)
+    assert Ip.data_ptr() % 16 == Ip.element_size()
+    sd, ed = (torch.as_tensor(a, device="cuda", dtype=torch.float64) for a in (sig, em))
+
+    def run(I, J):
+        out = [J] + [torch.zeros(n, dtype=torch.float64, device="cuda")
+                                        for n in (G * nx, G, G, G, G)]
+        s._check(trt.lib().trt_k_sweep(s.h, 1.7e-3, sd.data_ptr(), ed.data_ptr(), I.data_ptr(),
+                                       *[o.data_ptr() for o in out]))
+        return out
+
+    if tile:
+        s.set_sweep_tile(*tile)
+    off = lambda: torch.zeros_like(flat)[1:].view(Ip.shape)  # noqa: E731
+    got = [run(Ip, torch.zeros_like(Ip)), run(Ip, off())]
+    if precision == "sweep32":
+        got.append(run(Ip.clone(), off()))
+    s.set_sweep_tile(*strip)
+    ref = run(Ip.clone(), torch.zeros_like(Ip))
+    for g in got:
+        for a, b in zip(g, ref):
+            assert torch.equal(a, b)
+
+
 def test_autotune_keeps_state(trt):
     """trt_autotune / trt_sweep_time leave T, E_g, F_g, I and the QD factors unchanged and
     keep a candidate tile; steps after tuning match steps without it to round-off."""
