@@ -22,7 +22,9 @@
  *
  * Ownership: every pointer is caller-owned device memory; nothing is allocated; all work
  * is enqueued on `stream` (cudaStream_t as void*, NULL = legacy stream) and the calls
- * return without synchronising.  Return codes are those of trt.h (TRT_EINVAL for bad
+ * return without synchronising.  trt_mlp_forward, trt_mlp_forward_fused and trt_mlp_grad
+ * copy w16 (and scratch, where they take one) in pieces of 16 bytes and return TRT_EINVAL for
+ * one that is not aligned to 16 bytes.  Return codes are those of trt.h (TRT_EINVAL for bad
  * sizes or NULL pointers, checked before anything is enqueued; TRT_ECUDA for a launch
  * error).  A kernel whose wait on a tensor-core completion exceeds one second records
  * TRT_ETIMEOUT in the error word read by trt_mlp_status.
@@ -80,8 +82,8 @@ int trt_mlp_forward(int rows, const float *x, const float *params, const void *w
  * iteration as two 128-row groups half a period apart, both hidden layers on the tensor
  * cores with the activations kept in shared memory and the weights streamed in 32-wide K
  * chunks from the image trt_mlp_refresh keeps in w16); same arithmetic and result as
- * trt_mlp_forward up to the order of the FP32 accumulation.  Needs no scratch.  params must be 16-byte aligned (the
- * biases and the first and last layers' weights are read as float4): TRT_EINVAL otherwise. */
+ * trt_mlp_forward up to the order of the FP32 accumulation.  Needs no scratch.  params must
+ * be 16-byte aligned: TRT_EINVAL otherwise. */
 int trt_mlp_forward_fused(int rows, const float *x, const float *params, const void *w16,
                           float *y, void *stream);
 

@@ -1329,7 +1329,6 @@ cudaError_t mlp_fused(int rows, const float *x, const float *P, const bf16 *W, f
         cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
         attr = true;
     }
-    if (reinterpret_cast<uintptr_t>(P) & 15) return cudaErrorMisalignedAddress;   // float4 loads
     // one persistent CTA per SM, no more CTAs than row tiles (a CTA left for a second wave
     // would double the time)
     const int ntiles = (rows + 255) / 256;
@@ -1514,7 +1513,7 @@ int trt_mlp_forward_fused(int rows, const float *x, const float *params, const v
                           float *y, void *stream)
 {
     if (rows < 1 || !x || !params || !w16 || !y) return TRT_EINVAL;
-    if (reinterpret_cast<uintptr_t>(params) & 15) return TRT_EINVAL;
+    if (!al16(params) || !al16(w16)) return TRT_EINVAL;   // w16: 16-byte pieces of the bulk copies
     return mlp_fused(rows, x, params, reinterpret_cast<const bf16 *>(w16), y,
                      reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess
                ? TRT_OK
@@ -1526,7 +1525,7 @@ int trt_mlp_forward(int rows, const float *x, const float *params, const void *w
 {
     if (rows < 1 || !x || !params || !w16 || !scratch || !y) return TRT_EINVAL;
     Scratch s = carve_scratch(scratch, rows, 0);
-    if (scratch_bytes < s.bytes || !al16(scratch)) return TRT_EINVAL;
+    if (scratch_bytes < s.bytes || !al16(scratch) || !al16(w16)) return TRT_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const bf16 *W = reinterpret_cast<const bf16 *>(w16);
     k_layer1<<<(rows + 127) / 128, 128, 0, st>>>(rows, x, params, s.h1);
@@ -1554,10 +1553,9 @@ int trt_mlp_grad(int rows, const float *x, const float *target, const float *par
         !loss)
         return TRT_EINVAL;
     Scratch s = carve_scratch(scratch, rows, 1);
-    if (scratch_bytes < s.bytes || !al16(scratch)) return TRT_EINVAL;
+    if (scratch_bytes < s.bytes || !al16(scratch) || !al16(w16)) return TRT_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const bf16 *img = reinterpret_cast<const bf16 *>(w16) + 4 * 65536;
-    if (!al16(w16)) return TRT_EINVAL;
     const int nt = rows / 128;
     CUtensorMap map;
     if (image_map(img, &map) != cudaSuccess ||

@@ -95,6 +95,18 @@ def test_create_rejects_missing_workspace(L):
     assert L.trt_destroy(None) == trt.TRT_OK
 
 
+@pytest.mark.parametrize("off", [2, 4, 8])
+def test_network_rejects_unaligned_weight_copies(L, off):
+    """The kernels copy the BF16 weights in 16-byte pieces: a w16 that is not aligned to them is
+    refused before anything is enqueued (the addresses here are never followed)."""
+    from paper_2011_05427_gb300 import trt
+    a, w = 1 << 20, (1 << 20) + off
+    big = 1 << 40
+    assert L.trt_mlp_forward_fused(128, a, a, w, a, None) == trt.TRT_EINVAL
+    assert L.trt_mlp_forward(128, a, a, w, a, big, a, None) == trt.TRT_EINVAL
+    assert L.trt_mlp_grad(128, a, a, a, w, a, big, a, a, None) == trt.TRT_EINVAL
+
+
 def test_binding_fails_loudly_without_library(monkeypatch, tmp_path):
     from paper_2011_05427_gb300 import trt
     monkeypatch.setattr(trt, "LIB_PATH", str(tmp_path / "missing.so"))

@@ -68,3 +68,19 @@ def test_removing_the_closure_restores_the_plain_path(trained, env):
         sb = b.step(cfg.dt, "V", 4, 1e-8)
         assert (sa["n_ti"], sa["n_c"]) == (sb["n_ti"], sb["n_c"])
     assert np.array_equal(a.moments()["T"], b.moments()["T"])
+
+
+def test_closure_rejects_unaligned_weight_copies(env):
+    """trt_set_closure refuses BF16 weights that the network kernel's 16-byte copies cannot read."""
+    torch, closure, mlp, trt = env
+    cfg = W.scaled(W.fc_small(), 12, 4, 17, levels=[17, 1])
+    s = trt.Solver.from_slab(cfg)
+    net = mlp.MLP(device="cuda:0")
+    rows = s.G * s.nx
+    b = torch.empty(1 << 20, dtype=torch.float32, device="cuda")
+    n = trt.lib().trt_mlp_scratch_bytes(rows, 0)
+    args = (b.data_ptr(), n, b.data_ptr() + (2 << 20), b.data_ptr() + (3 << 20))
+    call = lambda w: trt.lib().trt_set_closure(s.h, net.params.data_ptr(), w, *args)  # noqa: E731
+    assert call(net.w16.data_ptr() + 2) == trt.TRT_EINVAL
+    assert call(net.w16.data_ptr()) == trt.TRT_OK
+    s.close()
