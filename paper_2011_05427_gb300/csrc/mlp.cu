@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
     float *sdot = reinterpret_cast<float *>(bar + F_NBAR) + 8;   // [2][128] head sums of columns 128 ..
 
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int ntiles = (rows + 255) / 256;
+    const int ntiles = (rows - 1) / 256 + 1;
     const int mine = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
     if (tid == 0) {
@@ -644,21 +644,23 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
         // layer 1: rows lane + 32 j, columns 32 w8 .. 32 w8 + 31 (w8: the warp within its group)
         const int lane = tid & 31, w8 = warp & 7;
         float xn[4][3];   // the tile's inputs (0 past the last row)
-        auto load_x = [&](int base) {
+        // rows unsigned: a tile's last may lie past 2^31, and three values a row past 2^32
+        auto load_x = [&](unsigned base) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int row = base + lane + 32 * j;
+                const unsigned row = base + lane + 32 * j;
+                const float *xr = x + 3 * (size_t)row;
 #pragma unroll
-                for (int k = 0; k < 3; ++k) xn[j][k] = row < rows ? x[3 * row + k] : 0.f;
+                for (int k = 0; k < 3; ++k) xn[j][k] = row < (unsigned)rows ? xr[k] : 0.f;
             }
         };
-        if (mine > 0) load_x((int)blockIdx.x * 256 + g * 128);
+        if (mine > 0) load_x(blockIdx.x * 256 + g * 128);
         for (int it = 0; it < mine && ok; ++it) {
-            const int base = ((int)blockIdx.x + it * (int)gridDim.x) * 256 + g * 128, row = base + r;
-            const bool rv = row < rows;
+            const unsigned base = (blockIdx.x + it * gridDim.x) * 256 + g * 128, row = base + r;
+            const bool rv = row < (unsigned)rows;
             layer1_rows4<false>(sP, xn, myA, lane, 4 * w8, 4 * w8 + 4);
             // the next tile's inputs, in flight during the two layers
-            if (it + 1 < mine) load_x(base + (int)gridDim.x * 256);
+            if (it + 1 < mine) load_x(base + gridDim.x * 256);
             hand_off();
             if (!(ok = wait_acc())) break;
             // ---- epilogue of layer 2: h2 = relu(acc + b2) over h1 ----
@@ -1331,7 +1333,7 @@ cudaError_t mlp_fused(int rows, const float *x, const float *P, const bf16 *W, f
     }
     // one persistent CTA per SM, no more CTAs than row tiles (a CTA left for a second wave
     // would double the time)
-    const int ntiles = (rows + 255) / 256;
+    const int ntiles = (rows - 1) / 256 + 1;
     const int grid = std::max(1, std::min(ntiles, g_num_sms > 0 ? g_num_sms : 148));
     k_mlp_fused<<<grid, F_THREADS, F_SMEM, st>>>(rows, x, P, (const bf16 *)(W + 4 * 65536), y);
     return cudaGetLastError();

@@ -110,6 +110,31 @@ def test_mlp_fused_row_edges(env, rows):
     assert mlp.MLP.status() == 0
 
 
+def test_mlp_fused_many_rows(env):
+    """More rows than 2^31 / 3, so that the inputs' indices pass 2^31: rows on both sides of that
+    point and the last ones are those of small calls bit for bit (a row's result does not
+    depend on the others)."""
+    torch, mlp = env
+    rows = (1 << 31) // 3 + 70001
+    if torch.cuda.mem_get_info()[0] < 16 * rows + (4 << 30):
+        pytest.skip("needs 16 GB of device memory")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(65)
+    small = torch.randn(100000, 3, generator=g, device="cuda")
+    net = mlp.MLP(OM.init_params(66).astype(np.float32).astype(np.float64))
+    x = torch.zeros(rows, 3, device="cuda")
+    at = [0, (1 << 31) // 3 - 50000, rows - 20000]
+    for k, a in enumerate(at):
+        n = min(100000, rows - a)
+        x[a:a + n] = small[:n]
+    y = net.forward_fused(x)
+    ref = net.forward_fused(small)
+    for a in at:
+        n = min(100000, rows - a, *[b - a for b in at if b > a])
+        assert torch.equal(y[a:a + n], ref[:n]), a
+    assert mlp.MLP.status() == 0
+
+
 def test_mlp_gradient_vs_oracle(env):
     """Gradients of the tensor-core backward pass against the oracle's backward pass with
     BF16 rounding at the same points, element by element: every element within 5e-4 of its
