@@ -322,7 +322,9 @@ __device__ inline double one_minus_exp(double x, double ex)
 // all over [x_g, min(x_{g+1}, x_g + 64)] and scaled by e^{x_g}, by the 8-point Gauss rule on
 // panels of width 2 or, for rho > 1, max(1/rho, a/2) from a panel start a below 4 (1 -
 // e^{-rho x} changes on the scale 1/rho near 0), the last panel taking the remainder up to
-// 1.5 widths.  Where e^{-x} and e^{-rho x} are both below e^{-40} and the group takes
+// 1.5 widths.  The panels are walked in x - x_g, where every step moves the start however
+// large x_g (nu/T_r beyond 2^54, where x_g + 2 = x_g) or rho (1/rho = 0) is: at most 1740
+// panels.  Where e^{-x} and e^{-rho x} are both below e^{-40} and the group takes
 // several panels, the factors are 1 and the four integrals are the T_r = T ones in closed
 // form.  Four lanes share a (cell, group): each takes one pair of nodes mid -/+ t of every
 // panel (they share e^{t}, e^{rho t} and their reciprocals) and the sums meet by shuffles.
@@ -348,18 +350,20 @@ __global__ void __launch_bounds__(256) k_opacity_tr(OpacityArgs a)
     const bool binf = isinf(nu_b);
     const double rho = v.rho, iTr = 1.0 / v.Tr;
     const double xa = nu_a * iTr, xb = binf ? 0.0 : nu_b * iTr;
-    const double hi = binf ? xa + 64.0 : fmin(xb, xa + 64.0);
+    const double w = binf ? 64.0 : fmin((nu_b - nu_a) * iTr, 64.0);
     const double gx = c_ser.g8x[4 + j], gw = c_ser.g8w[4 + j];
     double J = 0.0, P = 0.0, N = 0.0, D = 0.0;
-    const bool closed = xa >= 40.0 && rho * xa >= 40.0 && hi - xa > 3.0;
+    const bool closed = xa >= 40.0 && rho * xa >= 40.0 && w > 3.0;
     if (!closed) {
         const double exa = mx.ex(-xa);
-        double lo = xa;
-        while (lo < hi) {
-            const double wmax = (rho > 1.0) ? fmin(2.0, fmax(rcp64(rho), 0.5 * lo)) : 2.0;
-            const double up = (hi - lo <= 1.5 * wmax) ? hi : lo + wmax;
-            const double hw = 0.5 * (up - lo), mid = 0.5 * (up + lo), t = hw * gx;
-            const double E0 = mx.ex(xa - mid), ep = mx.ex(t), em = rcp64(ep);
+        double ulo = 0.0;   // the panel's start less x_g
+        while (ulo < w) {
+            const double lo = xa + ulo;
+            const double wmax =
+                (rho > 1.0) ? fmin(2.0, fmax(rcp64(fmin(rho, 1e300)), 0.5 * lo)) : 2.0;
+            const double uup = (w - ulo <= 1.5 * wmax) ? w : ulo + wmax;
+            const double hw = 0.5 * (uup - ulo), um = 0.5 * (uup + ulo), mid = xa + um, t = hw * gx;
+            const double E0 = mx.ex(-um), ep = mx.ex(t), em = rcp64(ep);
             const bool warm = lo < 37.0, rwarm = rho * lo < 37.0;   // some factor is not 1
             const double Em = warm ? E0 * exa : 0.0;
             double R0 = 0.0, rp = 0.0, rm = 0.0;
@@ -384,7 +388,7 @@ __global__ void __launch_bounds__(256) k_opacity_tr(OpacityArgs a)
                 N = fma(q3 * x, io, N);
                 D = fma(q3 * x2 * x2, iq, D);
             }
-            lo = up;
+            ulo = uup;
         }
     }
     __syncwarp();

@@ -53,6 +53,30 @@ def test_opacity_tr_parity(trt, orc, G, nx):
     s.close()
 
 
+def test_opacity_tr_at_extreme_radiation_temperatures(trt):
+    """T_r so far below T that x = nu/T_r is beyond 2^54 (a panel's width is below x's spacing),
+    and T_r / T above FP64's range: every panel walk ends.  With T_r -> 0 the weights of a group
+    shrink to its lower edge (corrections 7 T_r/nu <= 7e-15): sigma_E and sigma_R are 27 s
+    (1 - e^{-nu/T})/nu^3 there; the group from 0 has the integrals of rho x in closed form."""
+    G = 17
+    edges = W.group_edges(G, 1e-5, 1e2)
+    cfg = W.scaled(W.fc_small(), 4, 2, G, levels=[G, 1])
+    s = trt.Solver(4, 6.0, 2, edges, [G, 1], 1.3, W.CV_FC, 1e-3, 1.0, 0.0, tr_mode=True)
+    T = np.array([0.3, 1e-3, 2.0, 1e-300])
+    Tr = np.array([1e-20, 1e-22, 3e-21, 1e10])
+    sig, em, sR = (x.cpu().numpy() for x in s.k_opacity_tr(T, AR * Tr ** 4))
+    assert np.isfinite(sig).all() and np.isfinite(sR).all() and np.isfinite(em).all()
+    nu = edges[1:-1]
+    z6 = np.pi ** 6 / 945
+    for i in range(3):
+        ref = 27 * 1.3 * -np.expm1(-nu / T[i]) / nu ** 3
+        assert rel(sig[1:, i], ref) < 1e-11 and rel(sR[1:, i], ref) < 1e-11, i
+        k = 27 * 1.3 / (Tr[i] ** 2 * T[i])   # 27 s rho / T_r^3
+        assert rel(sig[0, i], k * (np.pi ** 2 / 6) * 15 / np.pi ** 4) < 1e-11, i
+        assert rel(sR[0, i], k * (4 * np.pi ** 4 / 15) / (720 * z6)) < 1e-11, i
+    s.close()
+
+
 CASES = [("tr_small", dataclasses.replace(W.scaled(W.fc_small(), 30, 4, 17, levels=[17, 1]),
                                           T0=0.05), "V", 2),
          ("tr_w", dataclasses.replace(W.scaled(W.fc_small(), 24, 4, 32, levels=[32, 8, 2, 1]),
