@@ -228,6 +228,12 @@ def sweep_kernel(fp32, D, shape):
     return k + " + k_sweep_finalize<float>"
 
 
+def sweep_tile(fp32, D, shape):
+    """The tile a solver's steps sweep with, (D, shape) of Solver.sweep_tile()."""
+    kernel = [k for k in sweep_kernel(fp32, D, shape).split(" + ") if k.startswith("k_sweep")][0]
+    return {"D": D if D else "default", "shape": shape, "kernel": kernel}
+
+
 def sweep_roofline(trt, s, cfg, fp32=False, local=0, reps=20):
     """Time the step's own sweep (K2 + its moment finalize; FP32 mode: the pre-scaled FP32
     inputs) with CUDA events on the solver's stream, `reps` launches after a warm-up, the
@@ -236,11 +242,10 @@ def sweep_roofline(trt, s, cfg, fp32=False, local=0, reps=20):
     HBM; algorithmic bytes per launch = updates x 4 intensity values (2 corners read, 2
     written) + per (cell, group) sigma_t h/2 and h e/2 read and f written."""
     own = s is None
-    tile = None
     if own:
         s = trt.Solver.from_slab(cfg, precision="sweep32" if fp32 else "fp64",
                                  device=f"cuda:{local}")
-        tile = s.autotune(cfg.dt, reps=10)
+        s.autotune(cfg.dt, reps=10)
     D, shape = s.sweep_tile()
     if D == 0 and fp32:   # the library default: the largest power of two <= 8 dividing N
         D = max(d for d in (1, 2, 4, 8) if cfg.N % d == 0)
@@ -274,8 +279,7 @@ def sweep_roofline(trt, s, cfg, fp32=False, local=0, reps=20):
                 "fp64_inst_frac": FP64_INST_PER_UPDATE[kind64] * upd / (ms * 1e-3) /
                                   (pk * 1e12 / 2),
                 "updates_per_s": upd / (ms * 1e-3)}
-    if tile:
-        roof["tile"] = {"D": tile[0], "S": tile[1], "NS": tile[2], "shape": shape}
+    roof["tile"] = sweep_tile(fp32, D, shape)
     return {"roofline": roof, "ms": ms}
 
 
@@ -296,7 +300,7 @@ def timed_steps(trt, cfg, precision, cycle, steps, warmup, local, ws, clocks=Fal
     of the timed steps (max over ranks), their stats, the clock record and the solver."""
     import torch
     s = trt.Solver.from_slab(cfg, precision=precision, device=f"cuda:{local}")
-    s.tile = s.autotune(cfg.dt, reps=10)   # sweep tile for this problem (state unchanged)
+    s.autotune(cfg.dt, reps=10)   # sweep tile for this problem (state unchanged)
     if l_max is None:
         l_max = tuned_lmax(precision, cycle)
     s.l_max = l_max
@@ -812,14 +816,12 @@ def run_ours(args):
         if args.large and ws == 1:
             extra["fc_4096"] = fc4096_bench(local)
 
-    tile = s.tile
+    tile = sweep_tile(args.precision not in ("fp64", "lo32", "lopair"), *s.sweep_tile())
     if args.precision in ("fp64", "lo32"):
         roof = sweep_roofline(trt, s, cfg, fp32=False)
-        roof["roofline"]["tile"] = {"D": tile[0], "S": tile[1], "NS": tile[2]}
         roof32 = sweep_roofline(trt, None, cfg, fp32=True, local=local)
     else:
         roof32 = sweep_roofline(trt, s, cfg, fp32=True)
-        roof32["roofline"]["tile"] = {"D": tile[0], "S": tile[1], "NS": tile[2]}
         roof = sweep_roofline(trt, None, cfg, fp32=False, local=local)
     if rank != 0:
         s.close()
@@ -843,8 +845,7 @@ def run_ours(args):
                                f"l_max {lm}, dt 1e-3 sh, eps 1e-8, {args.precision}",
                    "l_max": lm,
                    "parallelism": f"replicas x{ws}",
-                   "sweep_tile": {"D": tile[0], "S": tile[1], "NS": tile[2],
-                                  "picked_by": "trt_autotune"},
+                   "sweep_tile": {**tile, "picked_by": "trt_autotune"},
                    "l2": "inputs larger than L2 (intensity arrays 1 GB each in FP64)",
                    **{k + "_per_step": v for k, v in counters(stats, args.steps).items()}},
         "e2e": {"value": e2e_val, "unit": "updates/s", "h2d_bytes_per_step": h2d / args.steps,

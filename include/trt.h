@@ -273,22 +273,26 @@ const char *trt_batch_last_error(const trt_batch *b);
  * launches (after one warm-up), CUDA events on the handle's stream.  The state (T, E_g,
  * F_g, I, QD factors) is left unchanged; call it between steps.  Needs n_cells >= 3.
  *   *ms: milliseconds per sweep (K2 + its moment finalize).
- * trt_autotune: times every candidate (D, S, NS) with trt_sweep_time and keeps the
- * fastest for later steps.  D, S, NS (may be NULL) receive the choice.
+ * trt_autotune: times every candidate (D, S, NS) with trt_sweep_time, on an FP64 handle the
+ * library's default too (the paired sweep at 1 or 2 |mu| per CTA, which no D, S, NS of
+ * trt_set_sweep_tile names), and keeps the fastest for later steps.  D, S, NS (may be NULL)
+ * receive the fastest of the candidates: the tile that is kept unless the default was
+ * faster still.  What is kept is trt_get_sweep_tile's (D, shape), with D = 0 for the
+ * default; trt_set_sweep_tile takes that pair, on this handle or another one.
  * Both return TRT_EINVAL on bad arguments, TRT_ECUDA on a launch error. */
 int trt_sweep_time(trt_handle *h, double dt, int reps, float *ms);
 int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS);
 /* Set the sweep tile explicitly: D directions per CTA (a candidate of trt_autotune: the
  * largest power of two <= 4 dividing N, its double if <= 8 and dividing N, and with FP32
- * sweeps 16 if it divides N) and a shape index in [0, trt_sweep_shapes(h)); returns
+ * sweeps 16 if it divides N) and a shape index in [0, trt_sweep_shapes(h)), or (0, 0), the
+ * library's default for this problem, which a new handle has; returns
  * TRT_EINVAL otherwise, and for a pair with no kernel (D = 16 runs on the lean FP32 shapes
  * only) or whose kernel would exceed the shared memory of a CTA; trt_autotune skips such
  * pairs. */
 int trt_sweep_shapes(const trt_handle *h);
 int trt_set_sweep_tile(trt_handle *h, int D, int shape);
 /* The sweep tile the next step uses (after trt_autotune, trt_set_sweep_tile or neither):
- * *D = directions per CTA (0: the library's default for this problem, which trt_autotune
- * times too on an FP64 handle and may keep), *shape = shape index.
+ * *D = directions per CTA (0: the library's default for this problem), *shape = shape index.
  * Either pointer may be NULL.  TRT_EINVAL for a NULL handle. */
 int trt_get_sweep_tile(const trt_handle *h, int *D, int *shape);
 

@@ -846,6 +846,10 @@ int trt_set_sweep_tile(trt_handle *h, int D, int shape)
     int cand[3];
     const int nc = sweep_D_candidates(h->p, cand);
     bool ok = false;
+    if (D == 0 && shape == 0) {   // the library's default again
+        h->p.sweep_D = h->p.sweep_shape = 0;
+        return TRT_OK;
+    }
     for (int i = 0; i < nc; ++i) ok = ok || cand[i] == D;
     if (!ok || !sweep_tile_ok(h->p.precision, D, shape))
         return fail(h, TRT_EINVAL, "trt_set_sweep_tile: D or shape not a candidate");
@@ -902,8 +906,9 @@ int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS)
     const int nc = sweep_D_candidates(h->p, cand);
     const int ns = sweep_shape_count(h->p.precision);
     const int D0 = h->p.sweep_D, sh0 = h->p.sweep_shape;
-    float best = 1e30f;
+    float best = 1e30f, best_set = 1e30f;
     int bD = D0, bsh = sh0;
+    int rD = cand[0], rsh = 0;   // the fastest tile with D >= 1: what D, S, NS receive
     // the library's default (D = 0) first: the paired FP64 sweep at its own tile height
     for (int i = h->p.pair64 ? -1 : 0; i < nc; ++i) {
         for (int k = 0; k < (i < 0 ? 1 : ns); ++k) {
@@ -933,13 +938,18 @@ int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS)
                 bD = h->p.sweep_D;
                 bsh = k;
             }
+            if (i >= 0 && ms < best_set) {
+                best_set = ms;
+                rD = cand[i];
+                rsh = k;
+            }
         }
     }
     h->p.sweep_D = bD;
     h->p.sweep_shape = bsh;
     int s_ = 0, ns_ = 0;
-    sweep_shape_info(h->p.precision, bsh, &s_, &ns_);
-    if (D) *D = bD > 0 ? bD : cand[0];
+    sweep_shape_info(h->p.precision, rsh, &s_, &ns_);
+    if (D) *D = rD;
     if (S) *S = s_;
     if (NS) *NS = ns_;
     return TRT_OK;

@@ -481,13 +481,16 @@ class Solver:
         return ms.value
 
     def autotune(self, dt, reps=5):
-        """Time every candidate sweep tile and keep the fastest; returns (D, S, NS)."""
+        """Time every candidate sweep tile (FP64: the library's default too) and keep the
+        fastest, which sweep_tile() then gives; returns (D, S, NS) of the fastest tile that
+        set_sweep_tile takes with D >= 1 (the one kept unless the default was faster)."""
         D, S, NS = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         self._check(lib().trt_autotune(self.h, float(dt), int(reps), ctypes.byref(D),
                                        ctypes.byref(S), ctypes.byref(NS)))
         return D.value, S.value, NS.value
 
     def set_sweep_tile(self, D, shape):
+        """Use tile (D, shape) in later steps; (0, 0) is the library default."""
         self._check(lib().trt_set_sweep_tile(self.h, int(D), int(shape)))
 
     def sweep_shapes(self) -> int:

@@ -40,6 +40,13 @@ def test_sweep_kernel_names_follow_the_shape_table():
                for k in range(7))
 
 
+def test_sweep_tile_names_what_runs():
+    assert bench.sweep_tile(False, 0, 0) == {"D": "default", "shape": 0,
+                                             "kernel": "k_sweep_pair<default>"}
+    assert bench.sweep_tile(False, 4, 4)["kernel"] == "k_sweep_pair<4,2>"
+    assert bench.sweep_tile(True, 16, 0) == {"D": 16, "shape": 0, "kernel": "k_sweepf<1,8,4,16>"}
+
+
 def test_traffic_is_reported_only_for_the_captured_tile_and_code():
     key = "sweep_fp32"
     t = dict(bench.TRAFFIC[key])

@@ -374,6 +374,39 @@ def test_autotune_keeps_state(trt):
     assert np.max(np.abs(ma["T"] - mb["T"]) / mb["T"]) < 1e-12
 
 
+@pytest.mark.parametrize("precision", ["fp64", "sweep32"])
+def test_autotuned_tile_carries_over(trt, orc, precision):
+    """autotune, sweep_tile and set_sweep_tile agree: the returned (D, S, NS) are a settable
+    tile's (the kept one unless the default was faster), sweep_tile() is what runs, and the
+    same pair on another handle, also after another tile, gives the same sweep bit for bit;
+    (0, 0) is a new handle's sweep, and D = 0 goes with shape 0 only."""
+    nx, N, G = 30, 8, 40
+    r, h, sig, em, I_old, TL = sweep_inputs(orc, 3300, nx, N, G, thick=True)
+    edges = W.group_edges(G, 1e-5, 1e2)
+    a, b = (solver(trt, nx=nx, N=N, G=G, h=h, edges=edges, TL=TL, TR=0.3, precision=precision)
+            for _ in range(2))
+    sweep = lambda s: [x.cpu().numpy() for x in s.k_sweep(1.7e-3, sig, em, I_old)]  # noqa: E731
+    new = sweep(b)
+    D, S, NS = a.autotune(1.7e-3, reps=3)
+    tile, want = a.sweep_tile(), sweep(a)
+    shapes = {"fp64": [(8, 2), (16, 2), (8, 3), (8, 2), (4, 2)],
+              "sweep32": [(8, 4), (16, 2), (8, 3), (8, 2), (8, 2), (8, 4), (16, 2)]}[precision]
+    assert D in (4, 8) and (S, NS) in shapes
+    if tile[0]:   # a settable tile was the fastest: the returned one
+        assert (tile[0],) + shapes[tile[1]] == (D, S, NS)
+    b.set_sweep_tile(8, 1)
+    b.set_sweep_tile(*tile)
+    assert b.sweep_tile() == tile
+    for x, y in zip(want, sweep(b)):
+        assert np.array_equal(x, y)
+    b.set_sweep_tile(0, 0)
+    assert b.sweep_tile() == (0, 0)
+    for x, y in zip(new, sweep(b)):
+        assert np.array_equal(x, y)
+    with pytest.raises(trt.TRTError):
+        b.set_sweep_tile(0, 1)
+
+
 # ---------------------------------------------------------------------------- K3 / K4
 def random_level(r, ng, nx, eta=True):
     z = lambda shape: r.uniform(0, 0.2, shape) * (r.uniform(size=shape) < 0.5)
