@@ -237,7 +237,8 @@ int trt_fp64_peak(int reps, void *stream, double *tflops);
  * Newton, state copies) covers all slabs taking part in it, through device-side work lists
  * built from per-slab flags; each stage of a step is captured once in a CUDA graph and
  * replayed (a graph needs a non-legacy stream).  Every slab's result is that of
- * trt_step on the same slab.  The learned closure is not available in a batch.
+ * trt_step on the same slab with the batch's sweep tile.  The learned closure is not
+ * available in a batch.
  *   - workspace: one caller-owned device buffer of trt_batch_workspace_bytes; slab s owns
  *     a slice; the batch allocates only pinned host staging buffers;
  *   - stats: n entries (or NULL); the return value is the first failing slab's status;

@@ -104,7 +104,7 @@ void carve(trt_handle *h, Carver &c)
     if (sweep_fp32(p.precision)) {
         h->sig32 = c.take<float>(G * nx);
         h->emis32 = c.take<float>(G * nx + nx);   // then h/(2 c dt) per cell (kap32)
-    } else {   // the paired FP64 sweep's t, s, sums, pre-scaled inputs and hand-over slots
+    } else if (!h->batched) {   // the paired FP64 sweep's t, s, sums, pre-scaled inputs and hand-over slots
         p.ts64 = c.take<double>((size_t)p.N * nx * 3 * p.ldG);
         p.tab64 = c.take<double>(2 * nx * (size_t)p.ldG + nx);
         p.hand64 = c.take<double>(pair_hand_doubles());
@@ -123,7 +123,7 @@ void carve(trt_handle *h, Carver &c)
         h->crs_Eold[l] = l == 1 ? h->crs.Eold : c.take<double>((size_t)p.levels[l] * nx);
         h->crs_Fold[l] = l == 1 ? h->crs.Fold : c.take<double>((size_t)p.levels[l] * (nx + 1));
         // (a W cycle visits every grid but the finest coarse one again)
-        h->crs_fix[l] = l >= 2 ? c.take<double>(restrict_fix_doubles((int)nx, p.levels[l])) : nullptr;
+        h->crs_fix[l] = l >= 2 && !h->batched ? c.take<double>(restrict_fix_doubles((int)nx, p.levels[l])) : nullptr;
     }
     carve_level(c, h->grey, 1, p.nx);
     h->flags = c.take<double>(10);
@@ -287,12 +287,11 @@ cudaError_t d2d(trt_handle *h, double *dst, const double *src, size_t n)
 
 }  // namespace
 
-extern "C" {
-
-size_t trt_workspace_bytes(const trt_grid *grid, const trt_angles *angles,
-                           const trt_groups *groups, const trt_options *opt)
+size_t handle_bytes(const trt_grid *grid, const trt_angles *angles, const trt_groups *groups,
+                    const trt_options *opt, bool batched)
 {
     trt_handle tmp{};
+    tmp.batched = batched;
     std::vector<double> xe, ed;
     std::string err;
     if (!validate(grid, angles, groups, opt, tmp.p, xe, ed, err)) return 0;
@@ -301,14 +300,16 @@ size_t trt_workspace_bytes(const trt_grid *grid, const trt_angles *angles,
     return (c.off + 255) / 256 * 256;
 }
 
-int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups *groups,
-               const trt_opacity *opacity, double cv, const trt_options *opt, trt_handle **out)
+int create_handle(const trt_grid *grid, const trt_angles *angles, const trt_groups *groups,
+                  const trt_opacity *opacity, double cv, const trt_options *opt, bool batched,
+                  trt_handle **out)
 {
     if (!out) return fail(nullptr, TRT_EINVAL, "out is null");
     *out = nullptr;
     (void)cudaGetLastError();   // an error left by another library is not ours to report
     trt_handle *h = nullptr;   // errors during creation go to the global message (CK)
     std::unique_ptr<trt_handle> hp(new trt_handle());
+    hp->batched = batched;
     std::vector<double> xe, edges;
     std::string err;
     if (!validate(grid, angles, groups, opt, hp->p, xe, edges, err))
@@ -455,6 +456,20 @@ int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups 
     CK(cudaStreamSynchronize(p.stream));
     *out = hp.release();
     return TRT_OK;
+}
+
+extern "C" {
+
+size_t trt_workspace_bytes(const trt_grid *grid, const trt_angles *angles,
+                           const trt_groups *groups, const trt_options *opt)
+{
+    return handle_bytes(grid, angles, groups, opt, false);
+}
+
+int trt_create(const trt_grid *grid, const trt_angles *angles, const trt_groups *groups,
+               const trt_opacity *opacity, double cv, const trt_options *opt, trt_handle **out)
+{
+    return create_handle(grid, angles, groups, opacity, cv, opt, false, out);
 }
 
 int trt_destroy(trt_handle *h)
@@ -851,7 +866,7 @@ int trt_set_sweep_tile(trt_handle *h, int D, int shape)
         return TRT_OK;
     }
     for (int i = 0; i < nc; ++i) ok = ok || cand[i] == D;
-    if (!ok || !sweep_tile_ok(h->p.precision, D, shape))
+    if (!ok || !sweep_tile_ok(h->p.precision, D, shape, h->batched))
         return fail(h, TRT_EINVAL, "trt_set_sweep_tile: D or shape not a candidate");
     h->p.sweep_D = D;
     h->p.sweep_shape = shape;
@@ -912,7 +927,7 @@ int trt_autotune(trt_handle *h, double dt, int reps, int *D, int *S, int *NS)
     // the library's default (D = 0) first: the paired FP64 sweep at its own tile height
     for (int i = h->p.pair64 ? -1 : 0; i < nc; ++i) {
         for (int k = 0; k < (i < 0 ? 1 : ns); ++k) {
-            if (i >= 0 && !sweep_tile_ok(h->p.precision, cand[i], k)) continue;
+            if (i >= 0 && !sweep_tile_ok(h->p.precision, cand[i], k, h->batched)) continue;
             h->p.sweep_D = i < 0 ? 0 : cand[i];
             h->p.sweep_shape = k;
             float ms = 0;

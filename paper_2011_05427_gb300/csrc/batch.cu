@@ -395,7 +395,7 @@ size_t trt_batch_workspace_bytes(int n, const trt_grid *grids, const trt_angles 
     size_t tot = 0;
     int nlev_max = 2, nx_max = 1;
     for (int s = 0; s < n; ++s) {
-        const size_t w = trt_workspace_bytes(&grids[s], &angles[s], &groups[s], opt);
+        const size_t w = handle_bytes(&grids[s], &angles[s], &groups[s], opt, true);
         if (w == 0) return 0;
         tot += (w + 255) / 256 * 256;
         nlev_max = std::max(nlev_max, groups[s].n_levels);
@@ -433,11 +433,11 @@ int trt_create_batch(int n, const trt_grid *grids, const trt_angles *angles,
         if (opacities[s].tr_mode) return TRT_EINVAL;
     for (int s = 0; s < n; ++s) {
         trt_options o = *opt;
-        const size_t w = trt_workspace_bytes(&grids[s], &angles[s], &groups[s], opt);
+        const size_t w = handle_bytes(&grids[s], &angles[s], &groups[s], opt, true);
         o.workspace = base + off;
         o.workspace_bytes = w;
         trt_handle *x = nullptr;
-        const int rc = trt_create(&grids[s], &angles[s], &groups[s], &opacities[s], cv[s], &o, &x);
+        const int rc = create_handle(&grids[s], &angles[s], &groups[s], &opacities[s], cv[s], &o, true, &x);
         if (rc != TRT_OK) return rc;
         b->h.push_back(x);
         off += (w + 255) / 256 * 256;

@@ -7,6 +7,7 @@
 
 struct trt_handle {
     trt::Problem p;
+    bool batched = false;   // a slab of a batch: no scratch of kernels that batches don't run
     double *T, *Told, *Tcyc, *Tphase, *Ttil, *Tnew, *sig_prev, *T_prev;
     double *Eg, *Fg, *Eg_old, *Fg_old;
     void *I_cur, *I_alt;
@@ -37,6 +38,13 @@ struct trt_handle {
         if (ev_flags) cudaEventDestroy(ev_flags);
     }
 };
+
+// trt_workspace_bytes and trt_create for a single slab or a slab of a batch
+size_t handle_bytes(const trt_grid *grid, const trt_angles *angles, const trt_groups *groups,
+                    const trt_options *opt, bool batched);
+int create_handle(const trt_grid *grid, const trt_angles *angles, const trt_groups *groups,
+                  const trt_opacity *opacity, double cv, const trt_options *opt, bool batched,
+                  trt_handle **out);
 
 // cycle schedule S of Sec. 4 (grid indices 2..Gamma-1 visited between grey solves)
 inline void schedule(int type, int Gamma, std::vector<int> &S)

@@ -82,6 +82,25 @@ def test_workspace_bytes_and_validation(L):
         assert L.trt_last_error(None)
 
 
+@pytest.mark.parametrize("prec", ["TRT_FP64", "TRT_SWEEP_FP32"])
+def test_batch_slabs_carry_no_single_slab_scratch(L, prec):
+    """A batch runs neither the paired FP64 sweep, whose t, s and sums are three doubles per
+    (|mu|, cell, group), nor the restriction that keeps sums between visits: its workspace is
+    smaller than its slabs' own ones by at least the former in FP64, less the batch's argument
+    blocks (under 4 MB for these 8 slabs)."""
+    from paper_2011_05427_gb300 import trt
+    n, nx, N, lv = 8, 140, 16, (256, 64, 16, 4, 1)
+    slabs = [_args(trt, nx=nx, N=N, G=lv[0], levels=lv, precision=getattr(trt, prec)) for _ in range(n)]
+    opt = slabs[0][3]
+    one = L.trt_workspace_bytes(*[ctypes.byref(x) for x in slabs[0][:4]])
+    arr = [(type(slabs[0][k]) * n)(*[s[k] for s in slabs]) for k in range(3)]
+    got = L.trt_batch_workspace_bytes(n, *arr, ctypes.byref(opt))
+    pair = 3 * 8 * N * nx * lv[0] if prec == "TRT_FP64" else 0
+    assert one > 0 and got > 0
+    assert got < n * (one - pair) + (4 << 20)
+    assert got > n * (one - 2 * pair) - (4 << 20)
+
+
 def test_create_rejects_missing_workspace(L):
     from paper_2011_05427_gb300 import trt
     grid, ang, grp, opt, keep = _args(trt)
