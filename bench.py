@@ -178,12 +178,12 @@ FP64_INST_PER_UPDATE = {"strip": 17.6, "pair": 13.0}
 # sweep and its finalize on the fc_1024 workload), valid while the kernel sources hash to
 # `sha` and the tuned tile (D, shape) is the captured one.
 TRAFFIC = {
-    # k_prescale64 + k_sweep_pair<4,2> + k_sweep_finalize<double>: the t, s scratch and the
-    # 16 partial-moment tiles make it 1.70 x the algorithmic bytes (FP64-bound, not HBM)
-    "sweep_fp64": {"files": ("sweep64.cu", "sweep.cu"), "sha": "f4740f50793cb9cb", "tile": (4, 4),
-                   "bytes": 8202496 + 785604096 + 881712128 + 131672320 + 1171712},
-    "sweep_fp32": {"files": ("sweepf.cu", "sweep.cu"), "sha": "1c55093d94e37681", "tile": (16, 0),
-                   "bytes": 270072576 + 243014656 + 33098752 + 0},
+    # k_prescale64 + k_sweep_pair<2,4,2> + k_sweep_finalize<double>: the t, s, sum scratch and
+    # the 16 partial-moment tiles make it 1.98 x the algorithmic bytes (FP64-bound, not HBM)
+    "sweep_fp64": {"files": ("sweep64.cu", "sweep.cu"), "sha": "0d77d5ba888c02d3", "tile": (0, 0),
+                   "bytes": 8202752 + 934280960 + 1022310400 + 131683840 + 1169152},
+    "sweep_fp32": {"files": ("sweepf.cu", "sweep.cu"), "sha": "17da4f1c2f84dad2", "tile": (16, 0),
+                   "bytes": 270011648 + 242992896 + 33100032 + 0},
 }
 
 

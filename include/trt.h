@@ -355,8 +355,9 @@ int trt_k_grey_newton(trt_handle *h, double dt, const double *Tstar, const doubl
  * not allocate device memory -- a plug-in inside an application that owns every device
  * allocation and lends it no allocator, or a time loop that must not call cudaMalloc (nor
  * pay its device-wide synchronisation) once it is running.  trt_sweep_noalloc does the
- * work of trt_k_sweep (same kernels, the library's default sweep tile) with no handle and
- * no workspace: every input and output is a plain device pointer of the caller, and the
+ * work of trt_k_sweep with no handle and no workspace (FP32 sweeps: the same kernels and
+ * default tile, the same bits; FP64: the strip sweep, where a handle's default is the paired
+ * sweep, whose scratch the array below does not hold: the same values to round-off): every input and output is a plain device pointer of the caller, and the
  * scratch the sweep needs (per-direction-tile angular partial sums, exit intensities and,
  * for FP32 sweeps, the per-direction FP32 constants and the pre-scaled FP32 inputs
  * (sigma_E + 1/(c dt)) h/2, h e/2 that trt_k_sweep forms on an FP32 handle) lives in one

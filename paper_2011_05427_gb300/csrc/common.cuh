@@ -203,9 +203,8 @@ struct GreyArgs {
     const double *e2;
     ExpConsts ec;
     // the per-cell Newton terms w c sig*, w Q* - (1 - w) c_v (T* - Told)/dt and 1/Lambda,
-    // [3][nx], when the restriction to the grey level already formed them (its second
-    // stage, from the same values with the same operations); null: the grey kernel forms
-    // them
+    // [3][nx], when the restriction to the grey level already formed them (from the same
+    // values with the same operations); null: the grey kernel forms them
     const double *pre;
 };
 

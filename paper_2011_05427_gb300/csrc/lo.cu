@@ -465,9 +465,9 @@ __device__ void lo_one_cell(const LoCtx &x, int q, int ks = 0)
 }
 
 // FP32 group solve refined to FP64 accuracy (mixed-precision iterative refinement).  The
-// rows are staged in FP64 (s64, by the whole CTA); warp `sw` converts them to FP32 (s32),
-// eliminates in FP32 (x0), then kLoRefine times forms the residual r = b - A x of the FP64
-// rows in FP64, eliminates A d = r in FP32 and adds d to x in FP64; E = x, and the fluxes
+// rows are staged in FP64 (s64) and converted to FP32 (s32), eliminated in FP32 (x0), then
+// kLoRefine times the residual r = b - A x of the FP64 rows is formed in FP64, A d = r
+// eliminated in FP32 and d added to x in FP64, all by the whole CTA; E = x, and the fluxes
 // follow with the FP64 face coefficients.  Each step multiplies the error by about
 // cond(A) eps_32 (the plain FP32 solve's error: 3.6e-6 in T on fc_1024, ~5e-5 in E on a
 // 1000-cell random level, where one step left 2.6e-9); the eliminations, the part that is
@@ -535,8 +535,8 @@ __device__ void lo_solve_refined(const LoCtx &x, int q)
     lo_outputs_cta<double>(x, q, s64, S, 0);
 }
 
-// One system per CTA of 128 threads: all stage the rows (global loads and the face
-// coefficients), eliminate, and form and store the outputs.
+// One system per CTA (128 to 512 threads): all stage the rows (global loads and the face
+// coefficients) and form and store the outputs, the first P eliminate.
 template <typename R>
 __device__ void lo_solve_body(const LoCtx &x, int q)
 {
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(128) k_lo_solve_b(const int *__restrict__ meta
 // Per-cell terms of the grey Newton step (Sec. 5, eqs. eb-Gamma and f-derivative-d): from the
 // grey opacity sig*, Q* = 2 e* and the group energy sum Esum of cell i at T*, the
 // absorption w c sig*, the source w Q* - (1 - w) c_v (T* - Told)/dt and 1/Lambda.  Called
-// by the grey kernel on the grey level's arrays, or by the restriction's second stage on
+// by the grey kernel on the grey level's arrays, or by the restriction to that level on
 // the same values it writes there (the same operations, the same bits).
 // In two parts: what does not need the restricted sums (base = c_v/dt + Q'(T*), mT = c_v (T* -
 // Told)/dt, rdT = 1/(T* - T_prev) or 0 without a secant), and the rest.

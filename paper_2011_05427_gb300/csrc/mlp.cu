@@ -361,11 +361,8 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const bf16 *_
 // them: without the epilogues' work the same MMA stream takes 67 us for 512,000 rows, without
 // the weight copies it takes as long as with them.  So layer 1 reads each parameter once for
 // four rows (a lane's rows 32 apart, 32 columns per warp) instead of once per row.  512,000
-// rows: 137 us with one row per parameter read, four warps per group, four slots and every
-// MMA operand moved from one thread's registers; 121 us with eight warps, five slots and the
-// byte counts expected by the producer, 117 with the MMA warp's operands uniform, 102 with
-// the four-row layer 1 (floor at the measured BF16 GEMM rate 71 us).  Chunks of 16 K 152 us,
-// of 64 K with two slots 113.
+// rows: 104 us (floor at the measured BF16 GEMM rate 70); 117 with layer 1 reading its
+// parameters once per row, 113 with chunks of 64 K in two slots.
 //   Hand-offs: a group arrives on act[g] (256 arrivals) when A_g holds the next layer's
 // input (after a proxy fence: the MMAs read it through the async proxy); the MMA thread
 // commits the last MMA of a layer to acc[g], which the group waits on before it reads
@@ -767,11 +764,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(int rows, const floa
 // row's 256 terms in column order in one chain, as the inference GEMM's epilogue does.
 // What bounds it: 8192 rows are 64 CTAs of the 152 SMs, each a serial chain of 4 layer
 // products (1 us each at the tensor rate) with their epilogues; the floor at the measured
-// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 38.7 us against
+// BF16 GEMM rate is 3.4 us.  Measured (8192 rows, gradient and Adam step): 39 us, against
 // 1249 us for one GEMM launch per product, whose two weight gradients ran on two CTAs over K =
-// 8192 (500 us) and whose column sums ran on 8 and 1 CTAs (520 us); 46 us with the eight
-// warps doing everything and the backward weights copied as 512-byte pieces (6 us a layer),
-// 39.5 with layer 1 reading its parameters once per row.
+// 8192 (500 us) and whose column sums ran on 8 and 1 CTAs (520 us).
 constexpr int F_TSLOTS = 5;
 constexpr int F_TRING = F_TSLOTS * FW_BYTES;
 constexpr int T_THREADS = 576;
