@@ -22,11 +22,30 @@
 #include <cstdio>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 #include "handle.cuh"
 #include "tri_layout.cuh"
 #include "../../include/trt_mlp.h"
+
+namespace trt {
+
+cudaError_t allow_smem(const void *kernel, size_t bytes)
+{
+    static std::mutex mu;
+    static std::unordered_map<const void *, size_t> limit;   // an entry per kernel
+    std::lock_guard<std::mutex> lk(mu);
+    size_t &l = limit[kernel];
+    const size_t want = std::max(l, bytes);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)want);
+    if (e == cudaSuccess) l = want;
+    return e;
+}
+
+}  // namespace trt
 
 using namespace trt;
 

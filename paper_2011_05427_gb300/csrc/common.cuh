@@ -124,6 +124,11 @@ __device__ inline double widen_f32(float q)
 #ifdef __CUDACC__
 __device__ inline void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
+// Dynamic shared memory of `bytes` for the next launches of a kernel whose need depends on the
+// problem: the limit only grows, and under a lock, so that a launch of a smaller problem on
+// another thread cannot lower it between this call and the launch.
+cudaError_t allow_smem(const void *kernel, size_t bytes);
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        Args &&...args)

@@ -1596,7 +1596,7 @@ static cudaError_t lo_launch(const LoCtx &x, const OpacityArgs &a, int op, unsig
                              cudaStream_t st)
 {
     const auto go = [&](auto kern, auto... more) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        const cudaError_t e = allow_smem((const void *)kern, sm);
         return e != cudaSuccess ? e : launch_pdl(kern, dim3(nb), dim3(T), sm, st, x, more...);
     };
     return op == OP_NONE ? go(k_lo_solve<R, T>) : go(k_lo_solve_opac<R, T>, a, op);
@@ -1644,18 +1644,15 @@ cudaError_t launch_lo_solve_b(int precision, const BatchSmem &bs, const int *met
     const size_t sm = bs.lo;
     cudaError_t e;
     if (lo_pair(precision)) {
-        e = cudaFuncSetAttribute(k_lo_solve_b<fpair>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
+        e = allow_smem((const void *)k_lo_solve_b<fpair>, sm);
         if (e != cudaSuccess) return e;
         k_lo_solve_b<fpair><<<grid, 128, sm, st>>>(meta, N, xs);
     } else if (!lo_fp32(precision)) {
-        e = cudaFuncSetAttribute(k_lo_solve_b<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
+        e = allow_smem((const void *)k_lo_solve_b<double>, sm);
         if (e != cudaSuccess) return e;
         k_lo_solve_b<double><<<grid, 128, sm, st>>>(meta, N, xs);
     } else {
-        e = cudaFuncSetAttribute(k_lo_solve_b<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sm);
+        e = allow_smem((const void *)k_lo_solve_b<float>, sm);
         if (e != cudaSuccess) return e;
         k_lo_solve_b<float><<<grid, 128, sm, st>>>(meta, N, xs);
     }
@@ -1795,8 +1792,7 @@ cudaError_t launch_grey(const Problem &p, const Level &g, const GreyArgs &a)
 {
     const GreyCtx x = make_grey_ctx(p, g, a);
     const size_t sm = grey_smem(p.nx);
-    cudaError_t e = cudaFuncSetAttribute(k_grey, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
+    cudaError_t e = allow_smem((const void *)k_grey, sm);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_grey, dim3(1), dim3(grey_threads(p.nx)), sm, p.stream, x);
 }
@@ -1805,8 +1801,7 @@ cudaError_t launch_grey_b(const BatchSmem &bs, const int *meta, int N, const Gre
                           cudaStream_t st)
 {
     const size_t sm = bs.grey;
-    cudaError_t e = cudaFuncSetAttribute(k_grey_b, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
+    cudaError_t e = allow_smem((const void *)k_grey_b, sm);
     if (e != cudaSuccess) return e;
     k_grey_b<<<grid, grey_threads(bs.max_nx), sm, st>>>(meta, N, xs);
     return cudaGetLastError();

@@ -446,13 +446,11 @@ cudaError_t launch_shape(const SweepArgs *a, int M, int ldG, int D, const int *m
     const size_t sm = SweepSmem<R, SR, S, NS>(D).total;
     if (sm > 227 * 1024) return cudaErrorInvalidConfiguration;
     if (a) {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep<R, SR, S, NS>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem((const void *)k_sweep<R, SR, S, NS>, sm);
         if (e != cudaSuccess) return e;
         return launch_pdl(k_sweep<R, SR, S, NS>, dim3(M / D, ldG / 32), dim3(32 * D), sm, st, *a);
     } else {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep_b<R, SR, S, NS>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem((const void *)k_sweep_b<R, SR, S, NS>, sm);
         if (e != cudaSuccess) return e;
         k_sweep_b<R, SR, S, NS><<<grid, 32 * D, sm, st>>>(meta, N, xs);
     }

@@ -326,3 +326,39 @@ def test_lean_sweep_matches_strip_sweep(trt, D, shape):
     assert np.max(np.abs(ma["Eg"] - mb["Eg"]) / E[None, :]) < 1e-6
     a.close()
     b.close()
+
+
+def test_solvers_on_threads(trt):
+    """Solvers of different sizes stepping at the same time, each on a thread and a stream of its
+    own: the results of the same steps one solver after the other, bit for bit.  The kernels'
+    shared-memory needs differ (10 to 40 KB in the grey solve), and three of the solvers deal
+    their sweeps out over the resident CTAs of a cooperative launch."""
+    import threading
+
+    import torch
+    cfgs = [W.scaled(W.fc_1024(), 300, 32, 640, levels=[640, 160, 10, 1]),
+            W.scaled(W.fc_1024(), 200, 32, 320, levels=[320, 32, 1]),
+            W.scaled(W.fc_1024(), 101, 16, 640, levels=[640, 64, 1]), W.fc_small()]
+
+    def run(k, out, stream):
+        try:
+            s = trt.Solver.from_slab(cfgs[k], stream=stream)
+            for _ in range(12):
+                s.step(1e-3, "W", 1, 1e-8)
+            out[k] = s.moments()
+            s.close()
+        except Exception as e:   # reported by the assertion below
+            out[k] = e
+
+    ref, got = {}, {}
+    for k in range(len(cfgs)):
+        run(k, ref, torch.cuda.Stream())
+    th = [threading.Thread(target=run, args=(k, got, torch.cuda.Stream())) for k in range(len(cfgs))]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    for k in range(len(cfgs)):
+        assert isinstance(got[k], dict), got[k]
+        for f in ref[k]:
+            assert np.array_equal(got[k][f], ref[k][f]), (k, f)
